@@ -314,18 +314,18 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 
   if (warp == WARP_MMA) {
     // =========================== tensor-core issue warp ===========================
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      const uint32_t par = ch & 1;
-      // MMA1: [Kt;Qt] Kh^T.  M is padded to 128: rows 64-127 of the A tile are whatever follows it in
-      // shared memory, and land in TMEM lanes 64-127 that nobody reads.
-      if (lane == 0) {
+    if (elect_one()) {
+      for (int ch = 0; ch < n_chunks; ++ch) {
+        const uint32_t par = ch & 1;
+        // MMA1: [Kt;Qt] Kh^T.  M is padded to 128: rows 64-127 of the A tile are whatever follows it in
+        // shared memory, and land in TMEM lanes 64-127 that nobody reads.
         if (ch == 0 && a.poll_limit_first_wait)
           wait_bar_short(&misc->rdy_prep, par, misc, err, a.poll_limit_first_wait);
         else
           wait_bar(&misc->rdy_prep, par, misc, err);
         tc_fence_after_sync();
         if constexpr (KDA) {
-#pragma unroll 1
+#pragma unroll
           for (int kk = 0; kk < 16; ++kk)  // K = 128 in slices of 8: block kk / 4, 32 bytes per slice inside a block
             mma_ss(tm + COL_AP, desc_kmajor(sbase + OFF_KQ + (kk >> 2) * (64 * 128) + (kk & 3) * 32),
                    desc_kmajor(sbase + OFF_KH + (kk >> 2) * (32 * 128) + (kk & 3) * 32), ID_N32, kk != 0);
@@ -333,35 +333,26 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
           // GDN: the decay is one scalar per token, so it is applied to A and P after the product, and the product
           // itself is [k; q] k^T on the raw bf16 inputs: exact operands, K = 16 per instruction.  A and B come from
           // the same tile (B = its first 32 rows).
-#pragma unroll 1
+#pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
             const uint64_t d = desc_kmajor(sbase + OFF_KQ16 + (kk >> 2) * (64 * 128) + (kk & 3) * 32);
             mma_ss_bf16(tm + COL_AP, d, d, ID_BF16_N32, kk != 0);
           }
         }
         mma_commit(&misc->bar_ap);
-      }
-      __syncwarp();
-      // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
-      if (lane == 0) wait_bar(&misc->rdy_state, par, misc, err);
-      __syncwarp();
-      if (lane == 0) {
+        // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
+        wait_bar(&misc->rdy_state, par, misc, err);
         tc_fence_after_sync();
-#pragma unroll 1
+#pragma unroll
         for (int kk = 0; kk < 16; ++kk)
           mma_ts(tm + COL_RO, tm + COL_S + kk * 8, desc_kmajor(sbase + OFF_KQ + (kk >> 2) * (64 * 128) + (kk & 3) * 32),
                  WITH_O ? ID_N64 : ID_N32, kk != 0);  // without outputs only the Kt rows are needed
         mma_commit(&misc->bar_ro);
-      }
-      // MMA3: U^T = RHS^T T^T; RHS^T is a tf32 pair (high part over R^T, low part in the A|P columns)
-      if (lane == 0) {
+        // MMA3: U^T = RHS^T T^T; RHS^T is a tf32 pair (high part over R^T, low part in the A|P columns)
         wait_bar(&misc->rdy_t, par, misc, err);
         wait_bar(&misc->rdy_rhs, par, misc, err);
-      }
-      __syncwarp();
-      if (lane == 0) {
         tc_fence_after_sync();
-#pragma unroll 1
+#pragma unroll
         for (int kk = 0; kk < 8; ++kk)
           mma_ts(tm + COL_U, tm + (kk < 4 ? COL_RO : COL_AP) + (kk & 3) * 8, desc_kmajor(sbase + OFF_TM + (kk & 3) * 32),
                  ID_N32, kk != 0);
@@ -371,37 +362,33 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         // once, behind MMA3 in the tensor pipe's issue order, without a round trip through the chain warps:
         // MMA4 (high): O^T += U_hi^T P^T;  MMA5 (high): S'^T += U_hi^T Kh
         if (WITH_O) {
-#pragma unroll 1
+#pragma unroll
           for (int kk = 0; kk < 4; ++kk)
             mma_ts(tm + COL_RO + 32, tm + COL_U + kk * 8, desc_kmajor(sbase + OFF_PM + kk * 32), ID_N32, true);
         }
-#pragma unroll 1
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           mma_ts(tm + COL_S, tm + COL_U + kk * 8, desc_mn32(sbase + OFF_KHT + par * (128 * 128) + kk * 1024, 32 * 128), ID_N128_MN, true);
-      }
-      // MMA4 (low), MMA5 (low): the same with U_lo^T, which the chain warps wrote over the consumed RHS^T
-      if (lane == 0) wait_bar(&misc->rdy_u, par, misc, err);
-      __syncwarp();
-      if (lane == 0) {
+        // MMA4 (low), MMA5 (low): the same with U_lo^T, which the chain warps wrote over the consumed RHS^T
+        wait_bar(&misc->rdy_u, par, misc, err);
         tc_fence_after_sync();
         if (WITH_O) {
-#pragma unroll 1
+#pragma unroll
           for (int kk = 0; kk < 4; ++kk)
             mma_ts(tm + COL_RO + 32, tm + COL_RO + kk * 8, desc_kmajor(sbase + OFF_PM + kk * 32), ID_N32, true);
         }
         mma_commit(&misc->bar_o);
-#pragma unroll 1
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           mma_ts(tm + COL_S, tm + COL_RO + kk * 8, desc_mn32(sbase + OFF_KHT + par * (128 * 128) + kk * 1024, 32 * 128), ID_N128_MN, true);
         mma_commit(&misc->bar_s);
       }
-      __syncwarp();
-    }
-    // After a time-out the other roles no longer wait for the products: make sure none is still in flight when the
-    // tensor memory is given back (a real wait, bounded like the others).
-    if (lane == 0 && misc->abort_flag) {
-      mma_commit(&misc->drain);
-      mbar_wait_bounded(&misc->drain, 0, kMaxPolls);
+      // After a time-out the other roles no longer wait for the products: make sure none is still in flight when the
+      // tensor memory is given back (a real wait, bounded like the others).
+      if (misc->abort_flag) {
+        mma_commit(&misc->drain);
+        mbar_wait_bounded(&misc->drain, 0, kMaxPolls);
+      }
     }
     __syncwarp();
   } else if (warp == WARP_T) {

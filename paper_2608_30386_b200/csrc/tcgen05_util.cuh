@@ -72,6 +72,19 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst_smem, const void *tmap,
       : "memory");
 }
 
+// One lane of a converged warp.  The compiler knows that a branch on this predicate runs with a single active thread, so the
+// tcgen05 instructions below it take their descriptors straight from uniform registers; behind `lane == 0` it has to allow
+// for several active threads with different operands and serialises every one of them in a loop.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ---- proxies and tcgen05 fences -------------------------------------------------------------
 // Generic-proxy shared-memory writes -> visible to the tensor core (async proxy).
 __device__ __forceinline__ void fence_smem_to_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
