@@ -71,7 +71,7 @@ constexpr uint32_t OFF_MISC = OFF_BTE1 + 4 * C * 4;     // barriers, tmem base, 
 // GDN only: raw k (rows 0-31) and q (rows 32-63) as bf16, [2][64 rows][128 B], in the place of the K-major Kh tile
 constexpr uint32_t OFF_KQ16 = OFF_KH;
 constexpr uint32_t SMEM_BYTES = OFF_MISC + 192;
-constexpr uint32_t SMEM_ALLOC = SMEM_BYTES + 1024;      // slack to align the base to 1024 bytes
+constexpr uint32_t SMEM_ALLOC = SMEM_BYTES;
 static_assert(SMEM_ALLOC <= 113 * 1024, "two CTAs per SM");
 
 constexpr uint32_t kMaxPolls = 1u << 22;
@@ -137,24 +137,39 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // barrier among the 256 chain threads only
 __device__ __forceinline__ void sync_chain() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-// Bounded wait; after one time-out every later wait of this CTA returns at once.
-__device__ __forceinline__ void wait_bar(uint64_t *bar, uint32_t parity, Misc *misc, uint32_t *err) {
-  if (misc->abort_flag) return;
-  if (!mbar_wait_bounded(bar, parity, kMaxPolls)) {
-    misc->abort_flag = 1;
-    if (err) atomicExch(err, 1u);
-  }
+// What comes out of a broadcast shuffle the compiler may keep in uniform registers.
+__device__ __forceinline__ int uni(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// Bounded wait; after one time-out no wait of this CTA lasts longer than 8 polls.  Inlined at some thirty places, so it is
+// written as the smallest loop there is: the roles' code together has to stay within reach of the instruction caches.
+__device__ __forceinline__ void wait_bar(uint64_t *bar, uint32_t parity, Misc *misc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 n, f;\n\t"
+      "mov.b32 n, 0;\n"
+      "POLL:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n\t"
+      "@p bra DONE;\n\t"
+      "add.u32 n, n, 1;\n\t"
+      "and.b32 f, n, 7;\n\t"
+      "setp.ne.b32 p, f, 0;\n\t"
+      "@p bra POLL;\n\t"
+      "ld.volatile.shared.b32 f, [%2];\n\t"
+      "setp.ne.b32 p, f, 0;\n\t"
+      "@p bra DONE;\n\t"
+      "setp.ne.b32 p, n, %3;\n\t"
+      "@p bra POLL;\n\t"
+      "st.volatile.shared.b32 [%2], 1;\n"
+      "DONE:\n\t}" ::"r"(smem_u32(bar)),
+      "r"(parity), "r"(smem_u32(const_cast<uint32_t *>(&misc->abort_flag))), "n"(kMaxPolls)
+      : "memory");
 }
 
 // The test hook's wait (one call site): `max_polls` non-blocking looks at the barrier, so that a short limit runs out
 // whatever the time slice of a blocking poll is.
-__device__ __forceinline__ void wait_bar_short(uint64_t *bar, uint32_t parity, Misc *misc, uint32_t *err, uint32_t max_polls) {
+__device__ __forceinline__ void wait_bar_short(uint64_t *bar, uint32_t parity, Misc *misc, uint32_t max_polls) {
   bool done = false;
   for (uint32_t i = 0; i < max_polls && !done; ++i) done = mbar_test_wait(bar, parity);
-  if (!done) {
-    misc->abort_flag = 1;
-    if (err) atomicExch(err, 1u);
-  }
+  if (!done) misc->abort_flag = 1;
 }
 
 // This CTA does not (or could not) replay its unit: put the unit on the list that the token-by-token kernel walks
@@ -234,8 +249,8 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 // output product are left out.
 template <bool KDA, typename OT, bool WITH_O>
 __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_g) {
-  extern __shared__ unsigned char smem_dyn[];
-  unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t{1023});
+  // The base is a link-time constant (there is no static shared memory), so every operand descriptor is an immediate.
+  extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sbase = smem_u32(smem);
   float *Lm = reinterpret_cast<float *>(smem + OFF_L);
   float *Xm = reinterpret_cast<float *>(smem + OFF_X);
@@ -247,23 +262,22 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   float *bte1_s = reinterpret_cast<float *>(smem + OFF_BTE1);
   const __nv_bfloat16 *Vs = reinterpret_cast<const __nv_bfloat16 *>(smem + OFF_V);
   Misc *misc = reinterpret_cast<Misc *>(smem + OFF_MISC);
-  uint32_t *err = static_cast<uint32_t *>(a.workspace);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uni(tid >> 5), lane = tid & 31;
   const int h = blockIdx.x % a.H_v;
   const int lc = (blockIdx.x / a.H_v) % a.n_layers_in_call;
   const int r = blockIdx.x / (a.H_v * a.n_layers_in_call);
   const int hk = h / (a.H_v / a.H_k);
   const int layer = a.layer_begin + lc;
-  const int64_t t_begin = a.tok_begin ? a.tok_begin[r] : a.cu_seqlens[r];
-  const int n_tok = static_cast<int>(a.cu_seqlens[r + 1] - t_begin);
+  const int t_begin = uni(a.tok_begin ? a.tok_begin[r] : a.cu_seqlens[r]);
+  const int n_tok = uni(a.cu_seqlens[r + 1] - t_begin);
   if (n_tok <= 0 && a.mode == DASC_REFRESH_CONTINUE) return;
   if (n_tok <= a.short_thr) {  // left to the exact kernel (short_thr = -1: never)
     if (tid == 0) hand_over(a, false);
     return;
   }
 
-  float *st = a.state + static_cast<int64_t>(a.req_idx[r]) * a.req_stride + static_cast<int64_t>(layer) * a.layer_stride +
+  float *st = a.state + static_cast<int64_t>(uni(a.req_idx[r])) * a.req_stride + static_cast<int64_t>(layer) * a.layer_stride +
               static_cast<int64_t>(h) * D * D;
   const int64_t tok0 = static_cast<int64_t>(lc) * a.total_tokens + t_begin;
   const __nv_bfloat16 *gq = static_cast<const __nv_bfloat16 *>(a.q) + (tok0 * a.H_k + hk) * D;
@@ -303,7 +317,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  const uint32_t tm = misc->tmem_base;
+  const uint32_t tm = static_cast<uint32_t>(uni(static_cast<int>(misc->tmem_base)));
   const int n_chunks = (n_tok + C - 1) / C;
   constexpr float LOG2E = 1.4426950408889634f;
 
@@ -320,9 +334,9 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         // MMA1: [Kt;Qt] Kh^T.  M is padded to 128: rows 64-127 of the A tile are whatever follows it in
         // shared memory, and land in TMEM lanes 64-127 that nobody reads.
         if (ch == 0 && a.poll_limit_first_wait)
-          wait_bar_short(&misc->rdy_prep, par, misc, err, a.poll_limit_first_wait);
+          wait_bar_short(&misc->rdy_prep, par, misc, a.poll_limit_first_wait);
         else
-          wait_bar(&misc->rdy_prep, par, misc, err);
+          wait_bar(&misc->rdy_prep, par, misc);
         tc_fence_after_sync();
         if constexpr (KDA) {
 #pragma unroll
@@ -341,7 +355,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         }
         mma_commit(&misc->bar_ap);
         // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
-        wait_bar(&misc->rdy_state, par, misc, err);
+        wait_bar(&misc->rdy_state, par, misc);
         tc_fence_after_sync();
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk)
@@ -349,8 +363,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
                  WITH_O ? ID_N64 : ID_N32, kk != 0);  // without outputs only the Kt rows are needed
         mma_commit(&misc->bar_ro);
         // MMA3: U^T = RHS^T T^T; RHS^T is a tf32 pair (high part over R^T, low part in the A|P columns)
-        wait_bar(&misc->rdy_t, par, misc, err);
-        wait_bar(&misc->rdy_rhs, par, misc, err);
+        wait_bar(&misc->rdy_t, par, misc);
+        wait_bar(&misc->rdy_rhs, par, misc);
         tc_fence_after_sync();
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
@@ -358,9 +372,13 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
                  ID_N32, kk != 0);
         mma_commit(&misc->bar_u);
         // U^T stays where MMA3 leaves it: read as an operand, each fp32 value gives its high (truncated) part, and
-        // the chain warps supply the exact remainder afterwards (U = U_hi + U_lo).  The high-part products go out at
-        // once, behind MMA3 in the tensor pipe's issue order, without a round trip through the chain warps:
+        // the chain warps supply the exact remainder afterwards (U = U_hi + U_lo).  The high-part products go out
+        // without a round trip through the chain warps:
         // MMA4 (high): O^T += U_hi^T P^T;  MMA5 (high): S'^T += U_hi^T Kh
+        // U must have arrived in tensor memory before another product reads it as its A operand: the tensor pipe's issue
+        // order does not see to that (it orders accumulators only).
+        wait_bar(&misc->bar_u, par, misc);
+        tc_fence_after_sync();
         if (WITH_O) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
@@ -370,7 +388,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         for (int kk = 0; kk < 4; ++kk)
           mma_ts(tm + COL_S, tm + COL_U + kk * 8, desc_mn32(sbase + OFF_KHT + par * (128 * 128) + kk * 1024, 32 * 128), ID_N128_MN, true);
         // MMA4 (low), MMA5 (low): the same with U_lo^T, which the chain warps wrote over the consumed RHS^T
-        wait_bar(&misc->rdy_u, par, misc, err);
+        wait_bar(&misc->rdy_u, par, misc);
         tc_fence_after_sync();
         if (WITH_O) {
 #pragma unroll
@@ -399,7 +417,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     for (int ch = 0; ch < n_chunks; ++ch) {
       const uint32_t par = ch & 1;
       const float *beta_c = beta_s + (ch & 3) * C;
-      wait_bar(&misc->bar_ap, par, misc, err);
+      wait_bar(&misc->bar_ap, par, misc);
       tc_fence_after_sync();
       uint32_t x[32];
       tmem_ld32(tlane + COL_AP, x);
@@ -456,7 +474,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       __syncwarp();
       // the T tile's storage (shared with the P tile and the chain warps' output tile) is free once the chain
       // warps have copied the previous chunk's outputs out
-      if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc, err);
+      if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
       // T (lower triangle of X, unit diagonal) -> tf32 operand tile; lane = row
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
@@ -503,7 +521,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         if (!KDA) gsc_next = v1 ? gg[(t0 + C + ptid) * g_stride] : 0.f;
       }
       // (a) raw log-decay -> Kh tile, free once MMA1 of the previous chunk has completed
-      if (ch > 0) wait_bar(&misc->bar_ap, par ^ 1, misc, err);
+      if (ch > 0) wait_bar(&misc->bar_ap, par ^ 1, misc);
       if constexpr (KDA) {
         if (ptid == 0 && !misc->abort_flag) {
           mbar_expect_tx(&misc->g_full, C * D * 4);
@@ -517,7 +535,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
       // (b) raw k, q -> Kt/Qt tile, free once MMA2 of the previous chunk has completed; by then the chain warps
       //     have also left the chunk before that one, whose parity buffers (post, the MN-major Kh tile) are reused
-      if (ch > 0) wait_bar(&misc->bar_ro, par ^ 1, misc, err);
+      if (ch > 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
 #pragma unroll
       for (int jj = 0; jj < 8; ++jj) {
         const int t = (jj >> 2) * 16 + tg * 4 + (jj & 3);
@@ -529,7 +547,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       asm volatile("cp.async.commit_group;" ::: "memory");
       if constexpr (KDA) {
         {
-          wait_bar(&misc->g_full, par, misc, err);  // the log-decay has landed
+          wait_bar(&misc->g_full, par, misc);  // the log-decay has landed
           if (ntok < C) {
             // the box reached past the request's last token: those rows hold the decay of other tokens (or the
             // zeros past the end of the stream) and are cleared, each lane its own vectors
@@ -743,8 +761,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       const float *fac_c = fac_s + par * D;
 
       // ---- (1) the previous chunk's state update is complete; this chunk's factors and tiles are ready ----
-      if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc, err);
-      wait_bar(&misc->rdy_fac[par], (ch >> 1) & 1, misc, err);
+      if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
+      wait_bar(&misc->rdy_fac[par], (ch >> 1) & 1, misc);
       tc_fence_after_sync();
 
       // ---- (2) state pass: thread = (value column v, half of the channels); scale the state to this chunk's midpoint ----
@@ -771,7 +789,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 
       // ---- (3) P out of TMEM, by warp 1 (lanes 32-63 are its quadrant); A and T are the triangular warp's ----
       if (WITH_O && warp == 1) {
-        wait_bar(&misc->bar_ap, par, misc, err);
+        wait_bar(&misc->bar_ap, par, misc);
         tc_fence_after_sync();
         uint32_t x[32];
         tmem_ld32(tlane + COL_AP, x);
@@ -797,10 +815,10 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
 
       // ---- (4) RHS^T = beta (V - R)^T as a tf32 pair: high over R^T, low in the consumed A|P columns ----
-      wait_bar(&misc->bar_ro, par, misc, err);
+      wait_bar(&misc->bar_ro, par, misc);
       tc_fence_after_sync();
       asm volatile("cp.async.wait_all;" ::: "memory");  // V of this chunk
-      wait_bar(&misc->a_taken, par, misc, err);         // the A|P columns are about to be overwritten
+      wait_bar(&misc->a_taken, par, misc);         // the A|P columns are about to be overwritten
       sync_chain();
       {
         const int tb = colh * 16;
@@ -827,7 +845,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 
       // ---- (5) the part of U^T the tensor core drops when it reads it (the low 13 mantissa bits), written over
       //          the consumed RHS^T: U = U_hi + U_lo exactly ----
-      wait_bar(&misc->bar_u, par, misc, err);
+      wait_bar(&misc->bar_u, par, misc);
       tc_fence_after_sync();
       {
         const int tb = colh * 16;
@@ -844,7 +862,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       mbar_arrive(&misc->rdy_u);  // -> MMA4, MMA5
 
       // ---- (6) outputs of this chunk ----
-      wait_bar(&misc->bar_o, par, misc, err);
+      wait_bar(&misc->bar_o, par, misc);
       tc_fence_after_sync();
       if (WITH_O) {
         const int tb = colh * 16;
@@ -882,8 +900,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 
     // ---- final state: the factor still owed, then write back ----
     if (n_chunks > 0) {
-      wait_bar(&misc->rdy_prep, (n_chunks - 1) & 1, misc, err);  // the last chunk's post_s
-      wait_bar(&misc->bar_s, (n_chunks - 1) & 1, misc, err);
+      wait_bar(&misc->rdy_prep, (n_chunks - 1) & 1, misc);  // the last chunk's post_s
+      wait_bar(&misc->bar_s, (n_chunks - 1) & 1, misc);
     }
     // fac_s is free: the producer has finished (its last arrival was waited for above)
     if (tid < D) fac_s[tid] = n_chunks > 0 ? ex2f(post_s[((n_chunks - 1) & 1) * D + tid] * LOG2E) : 1.f;
@@ -918,6 +936,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   tc_fence_before_sync();
   __syncthreads();
   if (warp == WARP_MMA) tmem_dealloc(tm, TMEM_COLS);
+  if (tid == 0 && misc->abort_flag) atomicExch(static_cast<uint32_t *>(a.workspace), 1u);  // a wait ran out
 }
 
 // cuTensorMapEncodeTiled is a driver entry point.  It is looked up through the runtime at first use, so that the library
