@@ -58,8 +58,8 @@ constexpr uint32_t OFF_KH = OFF_KHT + 2 * 128 * 128;    // [4][32 rows][128 B]  
 constexpr uint32_t OFF_TM = OFF_KH + 4 * 32 * 128;      // [1][32 rows][128 B]  T[t][i]; TM|PM later the bf16 O tile
 constexpr uint32_t OFF_PM = OFF_TM + 32 * 128;          // [1][32 rows][128 B]  P[t][i]
 constexpr uint32_t OFF_V = OFF_PM + 32 * 128;           // [32][128] bf16 v
-constexpr uint32_t OFF_L = OFF_V + C * D * 2;           // [32][LDX] fp32
-constexpr uint32_t OFF_X = OFF_L + C * LDX * 4;         // [32][LDX] fp32
+constexpr uint32_t OFF_L = OFF_V + C * D * 2;           // [32][LDX] fp32 A^T (entries on and above A's diagonal are not used)
+constexpr uint32_t OFF_X = OFF_L + C * LDX * 4;         // [32][LDX] fp32 X = (I + A)^-1
 constexpr uint32_t OFF_FAC = OFF_X + C * LDX * 4;       // [2][128] fp32 state factor per channel, by chunk parity
 constexpr uint32_t OFF_POST = OFF_FAC + 2 * D * 4;      // [2][128] fp32 log-factor owed after a chunk, by chunk parity
 constexpr uint32_t OFF_BETA = OFF_POST + 2 * D * 4;     // [4][32] fp32, by chunk index mod 4 (written well ahead)
@@ -106,8 +106,8 @@ struct Misc {
   uint64_t tp_free;
   // issuing thread, only after a wait has run out: arrives once every tensor-core product issued so far has completed
   uint64_t drain;
-  // TMA -> producer warps: the log-decay tile of a chunk has landed in the Kh tile (KDA)
-  uint64_t g_full;
+  // TMA -> producer warps: the log-decay of a chunk has landed in the Kh tile (KDA); its raw k, q have landed
+  uint64_t g_full, kq_full;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;   // a bounded wait ran out: every later wait of this CTA returns at once
   volatile uint32_t domain_flag;  // a half-chunk decay sum left the range the midpoint factors can carry
@@ -125,13 +125,14 @@ __device__ __forceinline__ void cp_async16_zfill(uint32_t smem, const void *gmem
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem), "l"(gmem), "r"(n) : "memory");
 }
 
-__device__ __forceinline__ void cp_async8_zfill(uint32_t smem, const void *gmem, bool valid) {
-  const uint32_t n = valid ? 8u : 0u;
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem), "l"(gmem), "r"(n) : "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// One arrival for the whole warp, behind whatever its lanes did before.
+__device__ __forceinline__ void arrive_warp(uint64_t *bar, int lane) {
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar);
 }
 
 // barrier among the 256 chain threads only
@@ -189,16 +190,18 @@ __device__ __forceinline__ void mma_tf32_16x8x8(float (&d)[4], const uint32_t (&
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// One warp: acc (16x16) += A (16x16) * B (16x16), blocks in shared memory with pitch LDX.
+// One warp: acc (16x16) += A (16x16) * B (16x16), blocks in shared memory with pitch LDX; A row-major or its transpose.
+template <bool A_TRANSPOSED>
 __device__ __forceinline__ void warp_mm_acc(float (&acc)[2][4], const float *A, const float *B, int lane) {
   const int g = lane >> 2, tig = lane & 3;
 #pragma unroll
   for (int kh = 0; kh < 2; ++kh) {
     uint32_t af[4];
-    af[0] = tf32_pre(A[g * LDX + 8 * kh + tig]);
-    af[1] = tf32_pre(A[(g + 8) * LDX + 8 * kh + tig]);
-    af[2] = tf32_pre(A[g * LDX + 8 * kh + tig + 4]);
-    af[3] = tf32_pre(A[(g + 8) * LDX + 8 * kh + tig + 4]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = g + (i & 1) * 8, k = 8 * kh + tig + (i >> 1) * 4;
+      af[i] = tf32_pre(A_TRANSPOSED ? A[k * LDX + r] : A[r * LDX + k]);
+    }
 #pragma unroll
     for (int nh = 0; nh < 2; ++nh) {
       uint32_t bf[2];
@@ -245,14 +248,53 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   return r;
 }
 
+// 8 x 8 blocks of 16-bit values, transposed on the way: lane's row address; register m of the result belongs to block m.
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+  uint32_t w;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(hi), "f"(lo));
+  return w;
+}
+
+// Rows row0 .. row0 + 15 of A = strict_lower(Kt Kh^T) * beta out of tensor memory (`taddr`: first lane of the warp's quadrant),
+// transposed into LT.  KDA: the decay is inside the product, whose Kt rows carry the truncation compensation; `rowf` = beta.
+// GDN: the product is the raw k_t . k_j and the decay exp(G_t - G_j) = e1_t e2_j is applied here; `rowf` = beta e1, `colf` = e2.
+template <bool KDA>
+__device__ __forceinline__ void take_a_rows(uint32_t taddr, int row0, const float *rowf, const float *colf, float *LT, int lane) {
+  const int g = lane >> 2, tig = lane & 3;
+  uint32_t x[16];
+  tmem_ld_16x256b(taddr, x);
+  const float f0 = rowf[row0 + g] * (KDA ? kInvTruncComp : 1.f), f1 = rowf[row0 + g + 8] * (KDA ? kInvTruncComp : 1.f);
+  tmem_ld_wait();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float2 e = make_float2(1.f, 1.f);
+    if constexpr (!KDA) e = *reinterpret_cast<const float2 *>(colf + 8 * i + 2 * tig);
+    float *d = LT + (8 * i + 2 * tig) * LDX + row0 + g;
+    d[0] = __uint_as_float(x[4 * i]) * (f0 * e.x);
+    d[LDX] = __uint_as_float(x[4 * i + 1]) * (f0 * e.y);
+    d[8] = __uint_as_float(x[4 * i + 2]) * (f1 * e.x);
+    d[LDX + 8] = __uint_as_float(x[4 * i + 3]) * (f1 * e.y);
+  }
+}
+
 // WITH_O = false is the state-only variant (no outputs wanted): q is never read, the Qt rows, P and the
 // output product are left out.
 template <bool KDA, typename OT, bool WITH_O>
-__global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_g) {
+__global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
+                                                                const __grid_constant__ CUtensorMap tmap_k,
+                                                                const __grid_constant__ CUtensorMap tmap_g) {
   // The base is a link-time constant (there is no static shared memory), so every operand descriptor is an immediate.
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sbase = smem_u32(smem);
-  float *Lm = reinterpret_cast<float *>(smem + OFF_L);
+  float *LT = reinterpret_cast<float *>(smem + OFF_L);
   float *Xm = reinterpret_cast<float *>(smem + OFF_X);
   float *fac_s = reinterpret_cast<float *>(smem + OFF_FAC);
   float *post_s = reinterpret_cast<float *>(smem + OFF_POST);
@@ -260,7 +302,6 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   float *e1c_s = reinterpret_cast<float *>(smem + OFF_E1C);
   float *e2_s = reinterpret_cast<float *>(smem + OFF_E2);
   float *bte1_s = reinterpret_cast<float *>(smem + OFF_BTE1);
-  const __nv_bfloat16 *Vs = reinterpret_cast<const __nv_bfloat16 *>(smem + OFF_V);
   Misc *misc = reinterpret_cast<Misc *>(smem + OFF_MISC);
 
   const int tid = threadIdx.x, warp = uni(tid >> 5), lane = tid & 31;
@@ -280,12 +321,10 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   float *st = a.state + static_cast<int64_t>(uni(a.req_idx[r])) * a.req_stride + static_cast<int64_t>(layer) * a.layer_stride +
               static_cast<int64_t>(h) * D * D;
   const int64_t tok0 = static_cast<int64_t>(lc) * a.total_tokens + t_begin;
-  const __nv_bfloat16 *gq = static_cast<const __nv_bfloat16 *>(a.q) + (tok0 * a.H_k + hk) * D;
-  const __nv_bfloat16 *gk = static_cast<const __nv_bfloat16 *>(a.k) + (tok0 * a.H_k + hk) * D;
   const float *gg = a.g + (tok0 * a.H_v + h) * (KDA ? D : 1);
   const float *gb = a.beta + tok0 * a.H_v + h;
   OT *const go = WITH_O ? static_cast<OT *>(a.o) + (tok0 * a.H_v + h) * D : nullptr;
-  const int64_t qk_stride = static_cast<int64_t>(a.H_k) * D, v_stride = static_cast<int64_t>(a.H_v) * D;
+  const int64_t v_stride = static_cast<int64_t>(a.H_v) * D;
   const int64_t g_stride = static_cast<int64_t>(a.H_v) * (KDA ? D : 1), b_stride = a.H_v;
 
   // ---- set-up: barriers and tensor memory ----
@@ -295,17 +334,18 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     mbar_init(&misc->bar_u, 1);
     mbar_init(&misc->bar_o, 1);
     mbar_init(&misc->bar_s, 1);
-    mbar_init(&misc->rdy_prep, NP);
-    mbar_init(&misc->rdy_fac[0], NP);
-    mbar_init(&misc->rdy_fac[1], NP);
-    mbar_init(&misc->rdy_state, NCH);
-    mbar_init(&misc->rdy_rhs, NCH);
-    mbar_init(&misc->rdy_u, NCH);
-    mbar_init(&misc->a_taken, 32);
-    mbar_init(&misc->rdy_t, 32);
-    mbar_init(&misc->tp_free, NCH);
+    mbar_init(&misc->rdy_prep, NP / 32);
+    mbar_init(&misc->rdy_fac[0], NP / 32);
+    mbar_init(&misc->rdy_fac[1], NP / 32);
+    mbar_init(&misc->rdy_state, NCH / 32);
+    mbar_init(&misc->rdy_rhs, NCH / 32);
+    mbar_init(&misc->rdy_u, NCH / 32);
+    mbar_init(&misc->a_taken, 1);
+    mbar_init(&misc->rdy_t, 1);
+    mbar_init(&misc->tp_free, NCH / 32);
     mbar_init(&misc->drain, 1);
     mbar_init(&misc->g_full, 1);
+    mbar_init(&misc->kq_full, 1);
     misc->abort_flag = 0;
     misc->domain_flag = 0;
     fence_mbar_init();
@@ -322,27 +362,27 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   constexpr float LOG2E = 1.4426950408889634f;
 
   constexpr uint32_t ID_N32 = idesc_tf32(128, 32, false, false);
-  constexpr uint32_t ID_BF16_N32 = idesc_bf16(128, 32);
+  constexpr uint32_t ID_M64 = idesc_tf32(64, 32, false, false), ID_BF16_M64 = idesc_bf16(64, 32);
   constexpr uint32_t ID_N64 = idesc_tf32(128, 64, false, false);
   constexpr uint32_t ID_N128_MN = idesc_tf32(128, 128, false, true);  // B = Kh[t][c]: the channel index N is the contiguous one
 
   if (warp == WARP_MMA) {
     // =========================== tensor-core issue warp ===========================
-    if (elect_one()) {
-      for (int ch = 0; ch < n_chunks; ++ch) {
-        const uint32_t par = ch & 1;
-        // MMA1: [Kt;Qt] Kh^T.  M is padded to 128: rows 64-127 of the A tile are whatever follows it in
-        // shared memory, and land in TMEM lanes 64-127 that nobody reads.
-        if (ch == 0 && a.poll_limit_first_wait)
-          wait_bar_short(&misc->rdy_prep, par, misc, a.poll_limit_first_wait);
-        else
-          wait_bar(&misc->rdy_prep, par, misc);
-        tc_fence_after_sync();
+    // The whole warp walks the chunks and waits; an elected lane issues.
+    for (int ch = 0; ch < n_chunks; ++ch) {
+      const uint32_t par = ch & 1;
+      // MMA1: [Kt;Qt] Kh^T, M = 64: 16 rows in each TMEM quadrant, A's in the first two, P's in the last two.
+      if (ch == 0 && a.poll_limit_first_wait)
+        wait_bar_short(&misc->rdy_prep, par, misc, a.poll_limit_first_wait);
+      else
+        wait_bar(&misc->rdy_prep, par, misc);
+      tc_fence_after_sync();
+      if (elect_one()) {
         if constexpr (KDA) {
 #pragma unroll
           for (int kk = 0; kk < 16; ++kk)  // K = 128 in slices of 8: block kk / 4, 32 bytes per slice inside a block
             mma_ss(tm + COL_AP, desc_kmajor(sbase + OFF_KQ + (kk >> 2) * (64 * 128) + (kk & 3) * 32),
-                   desc_kmajor(sbase + OFF_KH + (kk >> 2) * (32 * 128) + (kk & 3) * 32), ID_N32, kk != 0);
+                   desc_kmajor(sbase + OFF_KH + (kk >> 2) * (32 * 128) + (kk & 3) * 32), ID_M64, kk != 0);
         } else {
           // GDN: the decay is one scalar per token, so it is applied to A and P after the product, and the product
           // itself is [k; q] k^T on the raw bf16 inputs: exact operands, K = 16 per instruction.  A and B come from
@@ -350,35 +390,49 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
             const uint64_t d = desc_kmajor(sbase + OFF_KQ16 + (kk >> 2) * (64 * 128) + (kk & 3) * 32);
-            mma_ss_bf16(tm + COL_AP, d, d, ID_BF16_N32, kk != 0);
+            mma_ss_bf16(tm + COL_AP, d, d, ID_BF16_M64, kk != 0);
           }
         }
         mma_commit(&misc->bar_ap);
-        // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
-        wait_bar(&misc->rdy_state, par, misc);
-        tc_fence_after_sync();
+      }
+      __syncwarp();
+      // rows 16-31 of A are in this warp's quadrant: hand them to the triangular warp
+      wait_bar(&misc->bar_ap, par, misc);
+      tc_fence_after_sync();
+      take_a_rows<KDA>(tm + (32u << 16) + COL_AP, 16, (KDA ? beta_s : bte1_s) + (ch & 3) * C, e2_s + (ch & 3) * C, LT, lane);
+      asm volatile("bar.arrive 3, 64;" ::: "memory");
+      // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
+      wait_bar(&misc->rdy_state, par, misc);
+      tc_fence_after_sync();
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk)
           mma_ts(tm + COL_RO, tm + COL_S + kk * 8, desc_kmajor(sbase + OFF_KQ + (kk >> 2) * (64 * 128) + (kk & 3) * 32),
                  WITH_O ? ID_N64 : ID_N32, kk != 0);  // without outputs only the Kt rows are needed
         mma_commit(&misc->bar_ro);
-        // MMA3: U^T = RHS^T T^T; RHS^T is a tf32 pair (high part over R^T, low part in the A|P columns)
-        wait_bar(&misc->rdy_t, par, misc);
-        wait_bar(&misc->rdy_rhs, par, misc);
-        tc_fence_after_sync();
+      }
+      __syncwarp();
+      // MMA3: U^T = RHS^T T^T; RHS^T is a tf32 pair (high part over R^T, low part in the A|P columns)
+      wait_bar(&misc->rdy_t, par, misc);
+      wait_bar(&misc->rdy_rhs, par, misc);
+      tc_fence_after_sync();
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
           mma_ts(tm + COL_U, tm + (kk < 4 ? COL_RO : COL_AP) + (kk & 3) * 8, desc_kmajor(sbase + OFF_TM + (kk & 3) * 32),
                  ID_N32, kk != 0);
         mma_commit(&misc->bar_u);
-        // U^T stays where MMA3 leaves it: read as an operand, each fp32 value gives its high (truncated) part, and
-        // the chain warps supply the exact remainder afterwards (U = U_hi + U_lo).  The high-part products go out
-        // without a round trip through the chain warps:
-        // MMA4 (high): O^T += U_hi^T P^T;  MMA5 (high): S'^T += U_hi^T Kh
-        // U must have arrived in tensor memory before another product reads it as its A operand: the tensor pipe's issue
-        // order does not see to that (it orders accumulators only).
-        wait_bar(&misc->bar_u, par, misc);
-        tc_fence_after_sync();
+      }
+      __syncwarp();
+      // U^T stays where MMA3 leaves it: read as an operand, each fp32 value gives its high (truncated) part, and
+      // the chain warps supply the exact remainder afterwards (U = U_hi + U_lo).  The high-part products go out
+      // without a round trip through the chain warps:
+      // MMA4 (high): O^T += U_hi^T P^T;  MMA5 (high): S'^T += U_hi^T Kh
+      // U must have arrived in tensor memory before another product reads it as its A operand: the tensor pipe's issue
+      // order does not see to that (it orders accumulators only).
+      wait_bar(&misc->bar_u, par, misc);
+      tc_fence_after_sync();
+      if (elect_one()) {
         if (WITH_O) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
@@ -387,9 +441,12 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           mma_ts(tm + COL_S, tm + COL_U + kk * 8, desc_mn32(sbase + OFF_KHT + par * (128 * 128) + kk * 1024, 32 * 128), ID_N128_MN, true);
-        // MMA4 (low), MMA5 (low): the same with U_lo^T, which the chain warps wrote over the consumed RHS^T
-        wait_bar(&misc->rdy_u, par, misc);
-        tc_fence_after_sync();
+      }
+      __syncwarp();
+      // MMA4 (low), MMA5 (low): the same with U_lo^T, which the chain warps wrote over the consumed RHS^T
+      wait_bar(&misc->rdy_u, par, misc);
+      tc_fence_after_sync();
+      if (elect_one()) {
         if (WITH_O) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
@@ -401,61 +458,47 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
           mma_ts(tm + COL_S, tm + COL_RO + kk * 8, desc_mn32(sbase + OFF_KHT + par * (128 * 128) + kk * 1024, 32 * 128), ID_N128_MN, true);
         mma_commit(&misc->bar_s);
       }
-      // After a time-out the other roles no longer wait for the products: make sure none is still in flight when the
-      // tensor memory is given back (a real wait, bounded like the others).
-      if (misc->abort_flag) {
-        mma_commit(&misc->drain);
-        mbar_wait_bounded(&misc->drain, 0, kMaxPolls);
-      }
+      __syncwarp();
+    }
+    // After a time-out the other roles no longer wait for the products: make sure none is still in flight when the
+    // tensor memory is given back (a real wait, bounded like the others).
+    if (misc->abort_flag) {
+      if (elect_one()) mma_commit(&misc->drain);
+      __syncwarp();
+      mbar_wait_bounded(&misc->drain, 0, kMaxPolls);
     }
     __syncwarp();
   } else if (warp == WARP_T) {
     // ================================ triangular warp ================================
-    // T = (I + A)^-1 depends on the token inputs only, so it is formed off the chain: A out of TMEM (lanes 0-31 are
-    // this warp's quadrant), 16x16 diagonal blocks by fp32 substitution, the off-diagonal block by mma.sync products.
-    const uint32_t tlane = tm;  // TMEM lanes 0-31
+    // T = (I + A)^-1 depends on the token inputs only, so it is formed off the chain: rows 0-15 of A out of TMEM (this
+    // warp's quadrant; the issuing warp brings rows 16-31), 16x16 diagonal blocks by fp32 substitution, the off-diagonal
+    // block by mma.sync products.
     for (int ch = 0; ch < n_chunks; ++ch) {
       const uint32_t par = ch & 1;
-      const float *beta_c = beta_s + (ch & 3) * C;
       wait_bar(&misc->bar_ap, par, misc);
       tc_fence_after_sync();
-      uint32_t x[32];
-      tmem_ld32(tlane + COL_AP, x);
-      tmem_ld_wait();
+      take_a_rows<KDA>(tm + COL_AP, 0, (KDA ? beta_s : bte1_s) + (ch & 3) * C, e2_s + (ch & 3) * C, LT, lane);
       tc_fence_before_sync();
-      mbar_arrive(&misc->a_taken);  // the chain warps may reuse the A|P columns
-      const int t = lane;
-      // row t of A = strict_lower(Kt Kh^T) * beta_t, kept in fp32 for the inverse
-      // KDA: the decay is inside the product, whose Kt rows carry the truncation compensation.  GDN: the product is
-      // the raw k_t . k_j and the decay exp(G_t - G_j) = e1_t e2_j is applied here.
-      const float bt = KDA ? beta_c[t] * kInvTruncComp : bte1_s[(ch & 3) * C + t];
-#pragma unroll
-      for (int j = 0; j < 32; j += 4) {
-        float4 e2 = make_float4(1.f, 1.f, 1.f, 1.f);
-        if constexpr (!KDA) e2 = *reinterpret_cast<const float4 *>(e2_s + (ch & 3) * C + j);
-        float4 o;
-        o.x = (j + 0 < t) ? bt * e2.x * __uint_as_float(x[j + 0]) : 0.f;
-        o.y = (j + 1 < t) ? bt * e2.y * __uint_as_float(x[j + 1]) : 0.f;
-        o.z = (j + 2 < t) ? bt * e2.z * __uint_as_float(x[j + 2]) : 0.f;
-        o.w = (j + 3 < t) ? bt * e2.w * __uint_as_float(x[j + 3]) : 0.f;
-        *reinterpret_cast<float4 *>(Lm + t * LDX + j) = o;
-      }
-      __syncwarp();
-      // diagonal 16x16 blocks: lane (block b, column cc) solves (I + L_bb) x = e_cc by forward substitution
+      asm volatile("bar.sync 3, 64;" ::: "memory");
+      arrive_warp(&misc->a_taken, lane);  // the chain warps may reuse the A|P columns
+      // diagonal 16x16 blocks: lane (block b, column cc) solves (I + L_bb) x = e_cc, column by column: every row that a new
+      // entry of x acts on is updated at once, so the serial chain is one multiply-add per row
       {
         const int b = lane >> 4, cc = lane & 15;
-        const float *Lb = Lm + (b * 16) * LDX + b * 16;
+        const float *Lb = LT + (b * 16) * LDX + b * 16;
         float xs[16];
 #pragma unroll
-        for (int rr = 0; rr < 16; ++rr) {
-          float acc0 = (rr == cc) ? 1.f : 0.f, acc1 = 0.f;
+        for (int i = 0; i < 16; ++i) xs[i] = i == cc ? 1.f : 0.f;
 #pragma unroll
-          for (int j = 0; j + 1 < rr; j += 2) {
-            acc0 = fmaf(-Lb[rr * LDX + j], xs[j], acc0);
-            acc1 = fmaf(-Lb[rr * LDX + j + 1], xs[j + 1], acc1);
+        for (int j = 0; j < 15; ++j) {
+#pragma unroll
+          for (int r4 = (j + 1) / 4 * 4; r4 < 16; r4 += 4) {
+            const float4 l4 = *reinterpret_cast<const float4 *>(Lb + j * LDX + r4);
+            if (r4 + 0 > j) xs[r4 + 0] = fmaf(-l4.x, xs[j], xs[r4 + 0]);
+            if (r4 + 1 > j) xs[r4 + 1] = fmaf(-l4.y, xs[j], xs[r4 + 1]);
+            if (r4 + 2 > j) xs[r4 + 2] = fmaf(-l4.z, xs[j], xs[r4 + 2]);
+            if (r4 + 3 > j) xs[r4 + 3] = fmaf(-l4.w, xs[j], xs[r4 + 3]);
           }
-          if (rr & 1) acc0 = fmaf(-Lb[rr * LDX + rr - 1], xs[rr - 1], acc0);
-          xs[rr] = acc0 + acc1;
         }
 #pragma unroll
         for (int rr = 0; rr < 16; ++rr) Xm[(b * 16 + rr) * LDX + b * 16 + cc] = xs[rr];
@@ -464,11 +507,11 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       // off-diagonal block: X_10 = -X_11 (L_10 X_00); the product L_10 X_00 is parked in the unused block (0,1)
       {
         float acc[2][4] = {};
-        warp_mm_acc(acc, Lm + 16 * LDX, Xm, lane);
+        warp_mm_acc<true>(acc, LT + 16, Xm, lane);
         warp_mm_store(Xm + 16, acc, 1.f, lane);
         __syncwarp();
         float acc2[2][4] = {};
-        warp_mm_acc(acc2, Xm + 16 * LDX + 16, Xm + 16, lane);
+        warp_mm_acc<false>(acc2, Xm + 16 * LDX + 16, Xm + 16, lane);
         warp_mm_store(Xm + 16 * LDX, acc2, -1.f, lane);
       }
       __syncwarp();
@@ -476,6 +519,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       // warps have copied the previous chunk's outputs out
       if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
       // T (lower triangle of X, unit diagonal) -> tf32 operand tile; lane = row
+      const int t = lane;
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
         const float4 xv = *reinterpret_cast<const float4 *>(Xm + t * LDX + j);
@@ -487,23 +531,48 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         *reinterpret_cast<uint4 *>(smem + OFF_TM + sw128_offset(32, t, j)) = o;
       }
       fence_smem_to_async();
-      mbar_arrive(&misc->rdy_t);  // -> MMA3
+      arrive_warp(&misc->rdy_t, lane);  // -> MMA3
       __syncwarp();
     }
   } else if (warp >= 8) {
     // =============================== producer warps ===============================
     // warp = block of 32 channels; per half of the chunk, lane = (4 adjacent channels, 4 consecutive tokens), a 4 x 4
-    // tile.  The midpoint is the end of the first half: first-half
-    // exponents are (local sum - the half's total), second-half exponents the local sums themselves.
+    // tile.  The midpoint is the end of the first half: first-half exponents are (local sum - the half's total),
+    // second-half exponents the local sums themselves, so the halves are independent of one another.
     const int pw = warp - 8, ptid = tid - NCH;
     const int cq = lane & 7, tg = lane >> 3;
     const int c0 = pw * 32 + cq * 4;
-    // Inputs land IN the operand tiles they will be overwritten with.  The raw log-decay of a chunk comes by TMA
-    // (KDA: four boxes of 32 tokens x 32 channels, 128-byte swizzle, i.e. exactly the layout of the Kh tile, so that
-    // the decay of (token t, channels c0..c0+3) sits where Kh[t][c0..] goes).  Raw k and q come by cp.async, each lane
-    // copying the 8-byte vectors of its own 4 x 4 tiles into the first half of the Kt / Qt vectors: a lane only ever
-    // reads what it copied itself, so no barrier is needed for them, and no register holds data in flight.
-    int g_issued = 0;
+    // Inputs come by TMA a chunk ahead, one issuing thread, into tiles they will be overwritten with (KDA) or that are
+    // operands as they are (GDN): shared memory holds no staging buffers, and no load or store instruction moves them.
+    //   log-decay (KDA, the largest stream): four boxes of 32 tokens x 32 channels with the 128-byte swizzle, i.e. exactly
+    //   the layout of the Kh tile, so that a lane finds the decay of its vectors where its Kh vectors go;
+    //   raw k, q: two boxes each of 32 tokens x 64 channels.  KDA: into the MN-major Kh tile of the chunk's parity, written
+    //   half by half once all producers have read that half (both layouts keep 16 tokens in 2 KB of every 4 KB).  GDN:
+    //   the operand tile of MMA1 itself.
+    constexpr uint32_t RAW_ROWS = KDA ? 32 : 64, OFF_RAW_Q = KDA ? 2 * 32 * 128 : 32 * 128;
+    int g_issued = 0, kq_issued = 0;
+    auto stage_kq = [&](int ch) {
+      const uint32_t dst = sbase + (KDA ? OFF_KHT + (ch & 1) * (128 * 128) : OFF_KQ16);
+      const int32_t z = static_cast<int32_t>(tok0 + ch * C);
+      mbar_expect_tx(&misc->kq_full, C * D * 2 * (WITH_O ? 2 : 1));
+#pragma unroll 1
+      for (int b = 0; b < 2; ++b) {
+        tma_load_3d(dst + b * (RAW_ROWS * 128), &tmap_k, b * 64, hk, z, &misc->kq_full);
+        if (WITH_O) tma_load_3d(dst + OFF_RAW_Q + b * (RAW_ROWS * 128), &tmap_q, b * 64, hk, z, &misc->kq_full);
+      }
+      ++kq_issued;
+    };
+    auto stage_g = [&](int ch) {
+      mbar_expect_tx(&misc->g_full, C * D * 4);
+#pragma unroll 1
+      for (int blk = 0; blk < 4; ++blk)
+        tma_load_3d(sbase + OFF_KH + blk * (C * 128), &tmap_g, blk * 32, h, static_cast<int32_t>(tok0 + ch * C), &misc->g_full);
+      ++g_issued;
+    };
+    if (ptid == 0 && n_chunks > 0) {
+      if (KDA) stage_g(0);
+      stage_kq(0);
+    }
     float beta_next = (n_chunks > 0 && ptid < min(C, n_tok)) ? gb[ptid * b_stride] : 0.f;
     float gsc_next = (!KDA && n_chunks > 0 && ptid < min(C, n_tok)) ? gg[ptid * g_stride] : 0.f;
     float gsc_cur = 0.f, post_prev = 0.f;  // GDN, first producer warp: this chunk's log-decay, the factor owed by the previous chunk
@@ -511,6 +580,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       const uint32_t par = ch & 1;
       const int t0 = ch * C, ntok = min(C, n_tok - t0);
       unsigned char *kht_tile = smem + OFF_KHT + par * (128 * 128);
+      unsigned char *raw = KDA ? kht_tile : smem + OFF_KQ16;
       // per-token scalars: this chunk's go to their ring slots (the chain warps are at most two chunks behind),
       // the next chunk's are fetched now and stored one iteration later
       if (ptid < C) {
@@ -520,146 +590,13 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         beta_next = v1 ? gb[(t0 + C + ptid) * b_stride] : 0.f;
         if (!KDA) gsc_next = v1 ? gg[(t0 + C + ptid) * g_stride] : 0.f;
       }
-      // (a) raw log-decay -> Kh tile, free once MMA1 of the previous chunk has completed
-      if (ch > 0) wait_bar(&misc->bar_ap, par ^ 1, misc);
-      if constexpr (KDA) {
-        if (ptid == 0 && !misc->abort_flag) {
-          mbar_expect_tx(&misc->g_full, C * D * 4);
-#pragma unroll
-          for (int blk = 0; blk < 4; ++blk)
-            tma_load_3d(sbase + OFF_KH + blk * (C * 128), &tmap_g, blk * 32, h, static_cast<int32_t>(tok0 + t0), &misc->g_full);
-          ++g_issued;
-        }
-      } else {
-        asm volatile("cp.async.commit_group;" ::: "memory");
-      }
-      // (b) raw k, q -> Kt/Qt tile, free once MMA2 of the previous chunk has completed; by then the chain warps
-      //     have also left the chunk before that one, whose parity buffers (post, the MN-major Kh tile) are reused
-      if (ch > 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj) {
-        const int t = (jj >> 2) * 16 + tg * 4 + (jj & 3);
-        const bool valid = t < ntok;
-        const int64_t tt = t0 + (valid ? t : 0);
-        cp_async8_zfill(sbase + OFF_KQ + sw128_offset(64, t, c0), gk + tt * qk_stride + c0, valid);
-        if (WITH_O) cp_async8_zfill(sbase + OFF_KQ + sw128_offset(64, 32 + t, c0), gq + tt * qk_stride + c0, valid);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      if constexpr (KDA) {
-        {
-          wait_bar(&misc->g_full, par, misc);  // the log-decay has landed
-          if (ntok < C) {
-            // the box reached past the request's last token: those rows hold the decay of other tokens (or the
-            // zeros past the end of the stream) and are cleared, each lane its own vectors
-  #pragma unroll
-            for (int jj = 0; jj < 8; ++jj) {
-              const int t = (jj >> 2) * 16 + tg * 4 + (jj & 3);
-              if (t >= ntok) *reinterpret_cast<float4 *>(smem + OFF_KH + sw128_offset(32, t, c0)) = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-          }
-        }
-        // sums: this lane's total, the prefix over the four token groups of the warp (lanes 8 apart), the half's total
-        float run0[2][4], refL[4];
-        bool out_of_range = false;
-  #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          float own[4] = {0.f, 0.f, 0.f, 0.f};
-  #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = half * 16 + tg * 4 + j;
-            const float4 g4 = *reinterpret_cast<const float4 *>(smem + OFF_KH + sw128_offset(32, t, c0));
-            own[0] += g4.x; own[1] += g4.y; own[2] += g4.z; own[3] += g4.w;
-          }
-          float tot[4];
-  #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            float incl = own[i];
-            float x = __shfl_up_sync(0xffffffffu, incl, 8);
-            if (tg >= 1) incl += x;
-            x = __shfl_up_sync(0xffffffffu, incl, 16);
-            if (tg >= 2) incl += x;
-            run0[half][i] = incl - own[i];                      // accumulated before this lane's first token
-            tot[i] = __shfl_sync(0xffffffffu, incl, cq + 24);    // the half's total
-            if (half == 0) refL[i] = -tot[i] * LOG2E;            // minus the midpoint reference, in log2 units
-            out_of_range |= !(fabsf(tot[i]) <= kMaxHalfDecay);   // also true for NaN
-          }
-          if (half == 0) {
-            // The factor that takes the state from where the previous chunk left it to this chunk's midpoint needs
-            // the first half's sums only: it is handed to the chain warps before the tiles are built.
-            if (tg == 0) {
-              const float4 post_prev = ch > 0 ? *reinterpret_cast<const float4 *>(post_s + (par ^ 1) * D + c0)
-                                              : make_float4(0.f, 0.f, 0.f, 0.f);
-              *reinterpret_cast<float4 *>(fac_s + par * D + c0) =
-                  make_float4(ex2f((post_prev.x + tot[0]) * LOG2E), ex2f((post_prev.y + tot[1]) * LOG2E),
-                              ex2f((post_prev.z + tot[2]) * LOG2E), ex2f((post_prev.w + tot[3]) * LOG2E));
-            }
-            mbar_arrive(&misc->rdy_fac[par]);
-          } else if (tg == 0) {
-            *reinterpret_cast<float4 *>(post_s + par * D + c0) = make_float4(tot[0], tot[1], tot[2], tot[3]);  // G_C - G_m
-          }
-        }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");  // k and q have landed
-        const uint64_t l2e2 = pack2(LOG2E, LOG2E), comp2 = pack2(kLog2TruncComp, kLog2TruncComp);
-        const uint64_t qs2 = pack2(a.q_scale, a.q_scale);
-  #pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
-          const int t4 = half * 16 + tg * 4;
-          uint64_t run01 = half == 0 ? pack2(run0[0][0], run0[0][1]) : pack2(run0[1][0], run0[1][1]);
-          uint64_t run23 = half == 0 ? pack2(run0[0][2], run0[0][3]) : pack2(run0[1][2], run0[1][3]);
-          const uint64_t ref01 = half == 0 ? pack2(refL[0], refL[1]) : 0ull, ref23 = half == 0 ? pack2(refL[2], refL[3]) : 0ull;
-  #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = t4 + j;
-            const uint32_t off_k = OFF_KQ + sw128_offset(64, t, c0), off_q = OFF_KQ + sw128_offset(64, 32 + t, c0);
-            const uint32_t off_h = OFF_KH + sw128_offset(32, t, c0);
-            const uint2 kw = *reinterpret_cast<const uint2 *>(smem + off_k);
-            const float4 g4 = *reinterpret_cast<const float4 *>(smem + off_h);
-            const uint64_t g01 = pack2(g4.x, g4.y), g23 = pack2(g4.z, g4.w);
-            const uint64_t k01 = pack2(bf16lo(kw.x), bf16hi(kw.x)), k23 = pack2(bf16lo(kw.y), bf16hi(kw.y));
-            run01 = add2(run01, g01);
-            run23 = add2(run23, g23);
-            const uint64_t d01 = fma2(run01, l2e2, ref01), d23 = fma2(run23, l2e2, ref23);  // (G_t - G_m) log2(e)
-            float d[4], dc[4];
-            unpack2(d01, d[0], d[1]);
-            unpack2(d23, d[2], d[3]);
-            unpack2(add2(d01, comp2), dc[0], dc[1]);
-            unpack2(add2(d23, comp2), dc[2], dc[3]);
-            const uint64_t e1_01 = pack2(ex2f(dc[0]), ex2f(dc[1])), e1_23 = pack2(ex2f(dc[2]), ex2f(dc[3]));
-            const uint64_t e2_01 = pack2(ex2f(-d[0]), ex2f(-d[1])), e2_23 = pack2(ex2f(-d[2]), ex2f(-d[3]));
-            float kt[4], kh[4];
-            unpack2(mul2(k01, e1_01), kt[0], kt[1]);
-            unpack2(mul2(k23, e1_23), kt[2], kt[3]);
-            unpack2(mul2(k01, e2_01), kh[0], kh[1]);
-            unpack2(mul2(k23, e2_23), kh[2], kh[3]);
-            if (WITH_O) {
-              const uint2 qw = *reinterpret_cast<const uint2 *>(smem + off_q);
-              const uint64_t q01 = pack2(bf16lo(qw.x), bf16hi(qw.x)), q23 = pack2(bf16lo(qw.y), bf16hi(qw.y));
-              float qt[4];
-              unpack2(mul2(q01, mul2(e1_01, qs2)), qt[0], qt[1]);
-              unpack2(mul2(q23, mul2(e1_23, qs2)), qt[2], qt[3]);
-              *reinterpret_cast<uint4 *>(smem + off_q) =
-                  make_uint4(tf32_pre(qt[0]), tf32_pre(qt[1]), tf32_pre(qt[2]), tf32_pre(qt[3]));
-            }
-            *reinterpret_cast<uint4 *>(smem + off_k) =
-                make_uint4(tf32_pre(kt[0]), tf32_pre(kt[1]), tf32_pre(kt[2]), tf32_pre(kt[3]));
-            // Kh goes out twice, the same four values in both places: K-major (MMA1 contracts over the channels) and
-            // MN-major (MMA5 contracts over the tokens).  A tf32 MN-major operand has a swizzle of its own, so the two
-            // tiles differ in where a vector lands, not in what it holds.
-            const uint4 khv = make_uint4(tf32_pre(kh[0]), tf32_pre(kh[1]), tf32_pre(kh[2]), tf32_pre(kh[3]));
-            *reinterpret_cast<uint4 *>(smem + off_h) = khv;
-            *reinterpret_cast<uint4 *>(kht_tile + mn32_offset(32, t, c0)) = khv;
-          }
-        }
-        // the exponents of this chunk may have overflowed: the unit will not be written back.  (Every lane of a channel
-        // quad holds the same totals; having only the first token group store keeps the producer loop free of spills.)
-        if (out_of_range && tg == 0) misc->domain_flag = 1;
-      } else {
+      bool out_of_range = false;
+      if constexpr (!KDA) {
         // ---- GDN: one scalar log-decay per token.  The first producer warp (lane = token) forms the running sums and
         // the per-token factors; nothing per channel needs an exponential, and k, q stay exactly their bf16 values:
         //   e1_t = exp(G_t - G_m), e2_t = exp(G_m - G_t) with m the end of the first half;
         //   MMA1 works on raw k, q (bf16 tile), MMA2 on raw k, q widened to tf32 containers, MMA5 on k_t e2_t;
         //   e1_t goes onto the rows of A, R and the outputs where they leave tensor memory, e2_j onto the columns of A, P.
-        bool out_of_range = false;
         if (ptid < C) {
           const int slot = (ch & 3) * C + lane;
           float incl = gsc_cur;
@@ -683,53 +620,163 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
           *reinterpret_cast<float4 *>(fac_s + par * D + lane * 4) = make_float4(f, f, f, f);
           *reinterpret_cast<float4 *>(post_s + par * D + lane * 4) = make_float4(tot1, tot1, tot1, tot1);
         }
-        mbar_arrive(&misc->rdy_fac[par]);
+        arrive_warp(&misc->rdy_fac[par], lane);
         asm volatile("bar.sync 2, 128;" ::: "memory");   // the factors are visible to all producer warps
-        asm volatile("cp.async.wait_group 0;" ::: "memory");  // k and q have landed
+      }
+      wait_bar(&misc->kq_full, par, misc);
+      if (KDA) wait_bar(&misc->g_full, par, misc);
+      const uint64_t l2e2 = pack2(LOG2E, LOG2E), comp2 = pack2(kLog2TruncComp, kLog2TruncComp);
+      const uint64_t qs2 = pack2(a.q_scale, a.q_scale);
 #pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
+      for (int half = 0; half < 2; ++half) {
+        const int tr = half * 16 + tg * 4;
+        // This lane's vectors (token tr + j): tr is a multiple of 4, so the row's part of a swizzle is an exclusive or with j.
+        const uint32_t or0 = sw128_offset_bf16(RAW_ROWS, tr, c0), ok0 = sw128_offset(64, tr, c0), oh0 = sw128_offset(32, tr, c0),
+                       om0 = mn32_offset(32, tr, c0);
+        const int left = ntok - tr;  // tokens of this request from this lane's first on
+        uint2 kw[4], qw[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          unsigned char *p = raw + (or0 ^ (j << 4)) + j * 128;
+          kw[j] = *reinterpret_cast<const uint2 *>(p);
+          if (WITH_O) qw[j] = *reinterpret_cast<const uint2 *>(p + OFF_RAW_Q);
+          if (j >= left) {
+            // the boxes reached past the request's last token and brought in other tokens' values (zeros past the end of
+            // the stream): those keys are cleared, so that what they hold cannot matter
+            kw[j] = make_uint2(0u, 0u);
+            if (!KDA) *reinterpret_cast<uint2 *>(p) = kw[j];
+          }
+        }
+        if constexpr (KDA) {
+          float4 g4[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const int t = half * 16 + tg * 4 + j;
-            const uint32_t off_k = OFF_KQ + sw128_offset(64, t, c0), off_q = OFF_KQ + sw128_offset(64, 32 + t, c0);
-            const uint2 kw = *reinterpret_cast<const uint2 *>(smem + off_k);
-            const uint4 kf = make_uint4(kw.x << 16, kw.x & 0xFFFF0000u, kw.y << 16, kw.y & 0xFFFF0000u);  // exact
-            *reinterpret_cast<uint4 *>(smem + off_k) = kf;
-            *reinterpret_cast<uint2 *>(smem + OFF_KQ16 + sw128_offset_bf16(64, t, c0)) = kw;
-            if (WITH_O) {
-              const uint2 qw = *reinterpret_cast<const uint2 *>(smem + off_q);
-              *reinterpret_cast<uint4 *>(smem + off_q) = make_uint4(qw.x << 16, qw.x & 0xFFFF0000u, qw.y << 16, qw.y & 0xFFFF0000u);
-              *reinterpret_cast<uint2 *>(smem + OFF_KQ16 + sw128_offset_bf16(64, 32 + t, c0)) = qw;
+            g4[j] = *reinterpret_cast<const float4 *>(smem + OFF_KH + (oh0 ^ (j << 4)) + j * 128);
+            if (j >= left) g4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+          // sums: this lane's total, the prefix over the four token groups of the warp (lanes 8 apart), the half's total
+          float run0[4], tot[4];
+          const float own[4] = {(g4[0].x + g4[1].x) + (g4[2].x + g4[3].x), (g4[0].y + g4[1].y) + (g4[2].y + g4[3].y),
+                                (g4[0].z + g4[1].z) + (g4[2].z + g4[3].z), (g4[0].w + g4[1].w) + (g4[2].w + g4[3].w)};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float incl = own[i];
+            float x = __shfl_up_sync(0xffffffffu, incl, 8);
+            if (tg >= 1) incl += x;
+            x = __shfl_up_sync(0xffffffffu, incl, 16);
+            if (tg >= 2) incl += x;
+            run0[i] = incl - own[i];                            // accumulated before this lane's first token
+            tot[i] = __shfl_sync(0xffffffffu, incl, cq + 24);    // the half's total
+            out_of_range |= !(fabsf(tot[i]) <= kMaxHalfDecay);   // also true for NaN
+          }
+          uint64_t ref01 = 0ull, ref23 = 0ull;  // minus the midpoint reference, in log2 units
+          if (half == 0) {
+            // The factor that takes the state from where the previous chunk left it to this chunk's midpoint needs
+            // the first half's sums only: it is handed to the chain warps before the tiles are built.
+            if (tg == 0) {
+              const float4 pp = ch > 0 ? *reinterpret_cast<const float4 *>(post_s + (par ^ 1) * D + c0) : make_float4(0.f, 0.f, 0.f, 0.f);
+              *reinterpret_cast<float4 *>(fac_s + par * D + c0) =
+                  make_float4(ex2f((pp.x + tot[0]) * LOG2E), ex2f((pp.y + tot[1]) * LOG2E), ex2f((pp.z + tot[2]) * LOG2E),
+                              ex2f((pp.w + tot[3]) * LOG2E));
             }
-            const float e2 = e2_s[(ch & 3) * C + t];
-            *reinterpret_cast<uint4 *>(kht_tile + mn32_offset(32, t, c0)) =
+            arrive_warp(&misc->rdy_fac[par], lane);
+            ref01 = pack2(-tot[0] * LOG2E, -tot[1] * LOG2E);
+            ref23 = pack2(-tot[2] * LOG2E, -tot[3] * LOG2E);
+          } else if (tg == 0) {
+            *reinterpret_cast<float4 *>(post_s + par * D + c0) = make_float4(tot[0], tot[1], tot[2], tot[3]);  // G_C - G_m
+          }
+          asm volatile("bar.sync 2, 128;" ::: "memory");  // this half's raw k, q have been read: Kh may take their place
+          // the Kt/Qt tile is free once MMA2 of the previous chunk has completed
+          if (ch > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
+          uint64_t run01 = pack2(run0[0], run0[1]), run23 = pack2(run0[2], run0[3]);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint64_t k01 = pack2(bf16lo(kw[j].x), bf16hi(kw[j].x)), k23 = pack2(bf16lo(kw[j].y), bf16hi(kw[j].y));
+            run01 = add2(run01, pack2(g4[j].x, g4[j].y));
+            run23 = add2(run23, pack2(g4[j].z, g4[j].w));
+            const uint64_t d01 = fma2(run01, l2e2, ref01), d23 = fma2(run23, l2e2, ref23);  // (G_t - G_m) log2(e)
+            float d[4], dc[4];
+            unpack2(d01, d[0], d[1]);
+            unpack2(d23, d[2], d[3]);
+            unpack2(add2(d01, comp2), dc[0], dc[1]);
+            unpack2(add2(d23, comp2), dc[2], dc[3]);
+            const uint64_t e1_01 = pack2(ex2f(dc[0]), ex2f(dc[1])), e1_23 = pack2(ex2f(dc[2]), ex2f(dc[3]));
+            const uint64_t e2_01 = pack2(ex2f(-d[0]), ex2f(-d[1])), e2_23 = pack2(ex2f(-d[2]), ex2f(-d[3]));
+            float kt[4], kh[4];
+            unpack2(mul2(k01, e1_01), kt[0], kt[1]);
+            unpack2(mul2(k23, e1_23), kt[2], kt[3]);
+            unpack2(mul2(k01, e2_01), kh[0], kh[1]);
+            unpack2(mul2(k23, e2_23), kh[2], kh[3]);
+            unsigned char *pk = smem + OFF_KQ + (ok0 ^ (j << 4)) + j * 128;
+            if (WITH_O) {
+              const uint64_t q01 = pack2(bf16lo(qw[j].x), bf16hi(qw[j].x)), q23 = pack2(bf16lo(qw[j].y), bf16hi(qw[j].y));
+              float qt[4];
+              unpack2(mul2(q01, mul2(e1_01, qs2)), qt[0], qt[1]);
+              unpack2(mul2(q23, mul2(e1_23, qs2)), qt[2], qt[3]);
+              *reinterpret_cast<uint4 *>(pk + 32 * 128) = make_uint4(tf32_pre(qt[0]), tf32_pre(qt[1]), tf32_pre(qt[2]), tf32_pre(qt[3]));
+            }
+            *reinterpret_cast<uint4 *>(pk) = make_uint4(tf32_pre(kt[0]), tf32_pre(kt[1]), tf32_pre(kt[2]), tf32_pre(kt[3]));
+            // Kh goes out twice, the same four values in both places: K-major (MMA1 contracts over the channels) and
+            // MN-major (MMA5 contracts over the tokens).  A tf32 MN-major operand has a swizzle of its own, so the two
+            // tiles differ in where a vector lands, not in what it holds.
+            const uint4 khv = make_uint4(tf32_pre(kh[0]), tf32_pre(kh[1]), tf32_pre(kh[2]), tf32_pre(kh[3]));
+            *reinterpret_cast<uint4 *>(smem + OFF_KH + (oh0 ^ (j << 4)) + j * 128) = khv;
+            *reinterpret_cast<uint4 *>(kht_tile + (om0 ^ (j << 5)) + j * 128) = khv;
+          }
+        } else {
+          if (ch > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            unsigned char *pk = smem + OFF_KQ + (ok0 ^ (j << 4)) + j * 128;
+            const uint4 kf = make_uint4(kw[j].x << 16, kw[j].x & 0xFFFF0000u, kw[j].y << 16, kw[j].y & 0xFFFF0000u);  // exact
+            *reinterpret_cast<uint4 *>(pk) = kf;
+            if (WITH_O)
+              *reinterpret_cast<uint4 *>(pk + 32 * 128) = make_uint4(qw[j].x << 16, qw[j].x & 0xFFFF0000u, qw[j].y << 16, qw[j].y & 0xFFFF0000u);
+            const float e2 = e2_s[(ch & 3) * C + tr + j];
+            *reinterpret_cast<uint4 *>(kht_tile + (om0 ^ (j << 5)) + j * 128) =
                 make_uint4(tf32_pre(__uint_as_float(kf.x) * e2), tf32_pre(__uint_as_float(kf.y) * e2),
                            tf32_pre(__uint_as_float(kf.z) * e2), tf32_pre(__uint_as_float(kf.w) * e2));
           }
         }
-        if (out_of_range && lane == 0) misc->domain_flag = 1;
       }
+      // the exponents of this chunk may have overflowed: the unit will not be written back
+      if (out_of_range && (KDA ? tg == 0 : lane == 0)) misc->domain_flag = 1;
       fence_smem_to_async();
-      mbar_arrive(&misc->rdy_prep);  // -> MMA1
+      arrive_warp(&misc->rdy_prep, lane);  // -> MMA1
+      if (pw == 0 && ch + 1 < n_chunks) {
+        // The next raw k, q (KDA) land once MMA5 of the previous chunk has read the Kh tile of that parity; the next
+        // log-decay (KDA) or k, q (GDN) once MMA1 of this chunk has read the tile they go to.
+        if (KDA) {
+          if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
+          if (lane == 0 && !misc->abort_flag) stage_kq(ch + 1);
+        }
+        wait_bar(&misc->bar_ap, par, misc);
+        if (lane == 0 && !misc->abort_flag) {
+          if (KDA) stage_g(ch + 1); else stage_kq(ch + 1);
+        }
+      }
     }
-    // after a time-out the last log-decay copy may not have been waited for: it must have landed before the CTA leaves
-    if (KDA && ptid == 0 && misc->abort_flag && g_issued > 0) mbar_wait_bounded(&misc->g_full, (g_issued - 1) & 1, kMaxPolls);
+    // after a time-out the last copies may not have been waited for: they must have landed before the CTA leaves
+    if (ptid == 0 && misc->abort_flag) {
+      if (g_issued > 0) mbar_wait_bounded(&misc->g_full, (g_issued - 1) & 1, kMaxPolls);
+      if (kq_issued > 0) mbar_wait_bounded(&misc->kq_full, (kq_issued - 1) & 1, kMaxPolls);
+    }
   } else {
     // ================================= chain warps =================================
     const int quad = warp & 3, colh = warp >> 2;                           // TMEM lane quadrant, column half
     const uint32_t tlane = tm + (static_cast<uint32_t>(quad * 32) << 16);  // this warp's TMEM lanes
     const int vrow = quad * 32 + lane;                                     // the TMEM lane this thread owns
 
-    // V arrives by TMA, one box of 32 tokens x 128 values per chunk, started by one thread.  A box that reaches past
-    // the request's last token brings in the following tokens of the stream (zeros past its end): those columns are
-    // masked where V is used.
+    const int g = lane >> 2, tig = lane & 3;
+    // V arrives by cp.async, zeros past the request's last token; 16-byte vector j of token t sits at j ^ (t & 7) (no bank
+    // conflicts for the 8 x 8 blocks it is read in)
     const __nv_bfloat16 *gv = static_cast<const __nv_bfloat16 *>(a.v) + (tok0 * a.H_v + h) * D;
     auto stage_v = [&](int ch) {
       const int t0 = ch * C, ntok = min(C, n_tok - t0);
       for (int i = tid; i < C * 16; i += NCH) {
         const int t = i >> 4, j = i & 15;
         const bool valid = t < ntok;
-        cp_async16_zfill(sbase + OFF_V + t * 256 + j * 16,
+        cp_async16_zfill(sbase + OFF_V + t * 256 + ((j ^ (t & 7)) << 4),
                          reinterpret_cast<const char *>(gv + (t0 + (valid ? t : 0)) * v_stride) + j * 16, valid);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -765,51 +812,55 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       wait_bar(&misc->rdy_fac[par], (ch >> 1) & 1, misc);
       tc_fence_after_sync();
 
-      // ---- (2) state pass: thread = (value column v, half of the channels); scale the state to this chunk's midpoint ----
+      // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
       {
+        float2 f[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const float2 *>(fac_c + colh * 64 + 8 * i + 2 * tig);
 #pragma unroll 1
-        for (int c0 = colh * 64; c0 < colh * 64 + 64; c0 += 32) {
+        for (uint32_t hh = 0; hh < 2; ++hh) {  // lanes 0-15, 16-31 of the quadrant
+          const uint32_t addr = tlane + (hh << 20) + COL_S + colh * 64;
           uint32_t s[32];
-          tmem_ld32(tlane + COL_S + c0, s);
+          tmem_ld_16x256b(addr, s);
           tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const float4 f = *reinterpret_cast<const float4 *>(fac_c + c0 + j);
-            s[j + 0] = __float_as_uint(__uint_as_float(s[j + 0]) * f.x);
-            s[j + 1] = __float_as_uint(__uint_as_float(s[j + 1]) * f.y);
-            s[j + 2] = __float_as_uint(__uint_as_float(s[j + 2]) * f.z);
-            s[j + 3] = __float_as_uint(__uint_as_float(s[j + 3]) * f.w);
+          for (int i = 0; i < 8; ++i) {
+            s[4 * i + 0] = __float_as_uint(__uint_as_float(s[4 * i + 0]) * f[i].x);
+            s[4 * i + 1] = __float_as_uint(__uint_as_float(s[4 * i + 1]) * f[i].y);
+            s[4 * i + 2] = __float_as_uint(__uint_as_float(s[4 * i + 2]) * f[i].x);
+            s[4 * i + 3] = __float_as_uint(__uint_as_float(s[4 * i + 3]) * f[i].y);
           }
-          tmem_st32(tlane + COL_S + c0, s);
+          tmem_st_16x256b(addr, s);
         }
         tmem_st_wait();
       }
       tc_fence_before_sync();
-      mbar_arrive(&misc->rdy_state);  // -> MMA2
+      arrive_warp(&misc->rdy_state, lane);  // -> MMA2
 
-      // ---- (3) P out of TMEM, by warp 1 (lanes 32-63 are its quadrant); A and T are the triangular warp's ----
-      if (WITH_O && warp == 1) {
+      // ---- (3) P = lower_incl_diag(Qt Kh^T) out of TMEM (rows 0-15, 16-31 are in the third and fourth quadrant) straight to
+      //          its operand tile.  GDN: the raw q_t . k_j gets its column factor e2_j here, the row factor e1_t is applied
+      //          to the outputs ----
+      if (WITH_O && colh == 0 && quad >= 2) {
         wait_bar(&misc->bar_ap, par, misc);
         tc_fence_after_sync();
-        uint32_t x[32];
-        tmem_ld32(tlane + COL_AP, x);
+        uint32_t x[16];
+        tmem_ld_16x256b(tlane + COL_AP, x);
         tmem_ld_wait();
-        const int t = lane;
-        // row t of P = lower_incl_diag(Qt Kh^T), straight to its operand tile
-        // (GDN: the raw q_t . k_j gets its column factor e2_j here; the row factor e1_t is applied to the outputs)
+        const int t = (quad - 2) * 16 + g;
 #pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-          float4 e2 = make_float4(kInvTruncComp, kInvTruncComp, kInvTruncComp, kInvTruncComp);
+        for (int i = 0; i < 4; ++i) {
+          const int j = 8 * i + 2 * tig;
+          float2 e = make_float2(kInvTruncComp, kInvTruncComp);
           if constexpr (!KDA) {
-            e2 = *reinterpret_cast<const float4 *>(e2_s + (ch & 3) * C + j);
-            e2.x *= kInvTruncComp; e2.y *= kInvTruncComp; e2.z *= kInvTruncComp; e2.w *= kInvTruncComp;
+            const float2 e2 = *reinterpret_cast<const float2 *>(e2_s + (ch & 3) * C + j);
+            e.x *= e2.x;
+            e.y *= e2.y;
           }
-          uint4 o;
-          o.x = (j + 0 <= t) ? tf32_pre(__uint_as_float(x[j + 0]) * e2.x) : 0u;
-          o.y = (j + 1 <= t) ? tf32_pre(__uint_as_float(x[j + 1]) * e2.y) : 0u;
-          o.z = (j + 2 <= t) ? tf32_pre(__uint_as_float(x[j + 2]) * e2.z) : 0u;
-          o.w = (j + 3 <= t) ? tf32_pre(__uint_as_float(x[j + 3]) * e2.w) : 0u;
-          *reinterpret_cast<uint4 *>(smem + OFF_PM + sw128_offset(32, t, j)) = o;
+          unsigned char *const p = smem + OFF_PM + sw128_offset(32, t, j);
+          *reinterpret_cast<uint2 *>(p) = make_uint2(j <= t ? tf32_pre(__uint_as_float(x[4 * i]) * e.x) : 0u,
+                                                     j + 1 <= t ? tf32_pre(__uint_as_float(x[4 * i + 1]) * e.y) : 0u);
+          *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(j <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 2]) * e.x) : 0u,
+                                                            j + 1 <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 3]) * e.y) : 0u);
         }
         fence_smem_to_async();
       }
@@ -822,24 +873,35 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       sync_chain();
       {
         const int tb = colh * 16;
-        uint32_t x[16], lo[16];
-        tmem_ld16(tlane + COL_RO + tb, x);
-        tmem_ld_wait();
+        // blocks of one ldmatrix: tokens 0-7 of the half with values 0-7, 8-15, tokens 8-15 with the same
+        const int vt = tb + (lane >> 4) * 8 + (lane & 7);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float vv = __bfloat162float(Vs[(tb + j) * D + vrow]);
-          // GDN: the product is k_t S' on the raw keys; its row factor e1_t (with the truncation compensation) comes here
-          const float r = KDA ? __uint_as_float(x[j]) : e1c_s[(ch & 3) * C + tb + j] * __uint_as_float(x[j]);
-          const float rhs = beta_c[tb + j] * (vv - r);
-          x[j] = to_tf32(rhs);
-          lo[j] = tf32_pre(rhs - __uint_as_float(x[j]));
+        for (uint32_t hh = 0; hh < 2; ++hh) {
+          uint32_t x[8], lo[8], vv[4];
+          tmem_ld_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
+          ldmatrix_x4_trans(vv, sbase + OFF_V + vt * 256 + (((quad * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (vt & 7)) << 4));
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int t = tb + (i >> 1) * 8 + 2 * tig;
+            const float2 b2 = *reinterpret_cast<const float2 *>(beta_c + t);
+            float2 e = make_float2(1.f, 1.f);
+            // GDN: the product is k_t S' on the raw keys; its row factor e1_t (with the truncation compensation) comes here
+            if constexpr (!KDA) e = *reinterpret_cast<const float2 *>(e1c_s + (ch & 3) * C + t);
+            const float r0 = b2.x * (bf16lo(vv[i]) - e.x * __uint_as_float(x[2 * i]));
+            const float r1 = b2.y * (bf16hi(vv[i]) - e.y * __uint_as_float(x[2 * i + 1]));
+            x[2 * i] = to_tf32(r0);
+            x[2 * i + 1] = to_tf32(r1);
+            lo[2 * i] = tf32_pre(r0 - __uint_as_float(x[2 * i]));
+            lo[2 * i + 1] = tf32_pre(r1 - __uint_as_float(x[2 * i + 1]));
+          }
+          tmem_st_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
+          tmem_st_16x256b(tlane + (hh << 20) + COL_AP + tb, lo);
         }
-        tmem_st16(tlane + COL_RO + tb, x);
-        tmem_st16(tlane + COL_AP + tb, lo);
         tmem_st_wait();
       }
       tc_fence_before_sync();
-      mbar_arrive(&misc->rdy_rhs);  // -> MMA3 (T tile and RHS^T are ready)
+      arrive_warp(&misc->rdy_rhs, lane);  // -> MMA3 (T tile and RHS^T are ready)
       sync_chain();                 // everyone is done with V: the next chunk's V may land
       if (more) stage_v(ch + 1);
 
@@ -859,42 +921,57 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         tmem_st_wait();
       }
       tc_fence_before_sync();
-      mbar_arrive(&misc->rdy_u);  // -> MMA4, MMA5
+      arrive_warp(&misc->rdy_u, lane);  // -> MMA4, MMA5
 
       // ---- (6) outputs of this chunk ----
       wait_bar(&misc->bar_o, par, misc);
       tc_fence_after_sync();
       if (WITH_O) {
         const int tb = colh * 16;
-        uint32_t x[16];
-        tmem_ld16(tlane + COL_RO + 32 + tb, x);
-        tmem_ld_wait();
-        if constexpr (!KDA) {
-          // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
-          // the truncation compensation
+        const int ot = tb + (lane >> 4) * 8 + (lane & 7);  // blocks of one stmatrix: as for V
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            x[j] = __float_as_uint(__uint_as_float(x[j]) * (e1c_s[(ch & 3) * C + tb + j] * a.q_scale));
+        for (uint32_t hh = 0; hh < 2; ++hh) {
+          uint32_t x[8];
+          tmem_ld_16x256b(tlane + (hh << 20) + COL_RO + 32 + tb, x);
+          tmem_ld_wait();
+          if constexpr (!KDA) {
+            // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
+            // the truncation compensation
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const float2 e = *reinterpret_cast<const float2 *>(e1c_s + (ch & 3) * C + tb + 8 * i + 2 * tig);
+              x[4 * i + 0] = __float_as_uint(__uint_as_float(x[4 * i + 0]) * (e.x * a.q_scale));
+              x[4 * i + 1] = __float_as_uint(__uint_as_float(x[4 * i + 1]) * (e.y * a.q_scale));
+              x[4 * i + 2] = __float_as_uint(__uint_as_float(x[4 * i + 2]) * (e.x * a.q_scale));
+              x[4 * i + 3] = __float_as_uint(__uint_as_float(x[4 * i + 3]) * (e.y * a.q_scale));
+            }
+          }
+          if constexpr (sizeof(OT) == 2) {
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = pack_bf16x2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+            stmatrix_x4_trans(sbase + OFF_TM + ot * 256 + (((quad * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (ot & 7)) << 4), w[0], w[1], w[2], w[3]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int t = tb + (i >> 1) * 8 + 2 * tig, v = quad * 32 + hh * 16 + (i & 1) * 8 + g;
+              if (t < ntok) go[(t0 + t) * v_stride + v] = __uint_as_float(x[2 * i]);
+              if (t + 1 < ntok) go[(t0 + t + 1) * v_stride + v] = __uint_as_float(x[2 * i + 1]);
+            }
+          }
         }
         if constexpr (sizeof(OT) == 2) {
           // through shared memory (the T and P tiles are free now) so that global stores are 16 bytes wide
-          __nv_bfloat16 *Os = reinterpret_cast<__nv_bfloat16 *>(smem + OFF_TM);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) Os[(tb + j) * D + vrow] = __float2bfloat16_rn(__uint_as_float(x[j]));
           sync_chain();
           for (int i = tid; i < ntok * 16; i += NCH) {
             const int t = i >> 4, j = i & 15;
             *reinterpret_cast<uint4 *>(reinterpret_cast<char *>(go + (t0 + t) * v_stride) + j * 16) =
-                *reinterpret_cast<const uint4 *>(smem + OFF_TM + t * 256 + j * 16);
+                *reinterpret_cast<const uint4 *>(smem + OFF_TM + t * 256 + ((j ^ (t & 7)) << 4));
           }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (tb + j < ntok) go[(t0 + tb + j) * v_stride + vrow] = __uint_as_float(x[j]);
         }
       }
       tc_fence_before_sync();
-      mbar_arrive(&misc->tp_free);  // this thread is done with the T|P|O tile region
+      arrive_warp(&misc->tp_free, lane);  // this thread is done with the T|P|O tile region
       sync_chain();  // every chain thread is done with this chunk's P and O tiles before they are rewritten
     }
 
@@ -966,23 +1043,25 @@ int launch(const DascRefreshArgs &a, void *stream) {
   if (n_units > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
   e = cudaMemsetAsync(a.workspace, 0, 16, static_cast<cudaStream_t>(stream));  // clear the four header words
   if (e != cudaSuccess) return static_cast<int>(e);
-  // tensor map of the KDA log-decay [Lc*T tokens][H_v][128] fp32: boxes of 32 tokens x one head x 32 channels with the
-  // 128-byte swizzle, which is the layout of one block of the Kh operand tile (GDN has one scalar per token: no map)
-  CUtensorMap tmap_g{};
-  if (KDA) {
-    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(a.H_v),
+  // tensor maps of the token streams [Lc*T tokens][heads][128]: boxes of 32 tokens x one head x 128 bytes of channels with
+  // the 128-byte swizzle, which is the layout of one block of an operand tile
+  CUtensorMap tmap_q{}, tmap_k{}, tmap_g{};
+  const EncodeTiledFn encode = encode_tiled_fn();
+  if (!encode) return static_cast<int>(cudaErrorNotSupported);
+  auto make_map = [&](CUtensorMap *m, CUtensorMapDataType type, const void *base, int heads, cuuint64_t esz) {
+    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(heads),
                                 static_cast<cuuint64_t>(a.n_layers_in_call) * static_cast<cuuint64_t>(a.total_tokens)};
-    const cuuint64_t strides[2] = {static_cast<cuuint64_t>(D) * 4, static_cast<cuuint64_t>(a.H_v) * D * 4};
-    const cuuint32_t box[3] = {32, 1, static_cast<cuuint32_t>(C)};
+    const cuuint64_t strides[2] = {D * esz, static_cast<cuuint64_t>(heads) * D * esz};
+    const cuuint32_t box[3] = {static_cast<cuuint32_t>(128 / esz), 1, static_cast<cuuint32_t>(C)};
     const cuuint32_t ones[3] = {1, 1, 1};
-    const EncodeTiledFn encode = encode_tiled_fn();
-    if (!encode) return static_cast<int>(cudaErrorNotSupported);
-    if (encode(&tmap_g, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(a.g), dims, strides, box, ones,
-                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return static_cast<int>(cudaErrorInvalidValue);
-  }
-  kern<<<static_cast<unsigned>(n_units), NT, SMEM_ALLOC, static_cast<cudaStream_t>(stream)>>>(a, tmap_g);
+    return encode(m, type, 3, const_cast<void *>(base), dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  if (!make_map(&tmap_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.k, a.H_k, 2) ||
+      (WITH_O && !make_map(&tmap_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.q, a.H_k, 2)) ||
+      (KDA && !make_map(&tmap_g, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.g, a.H_v, 4)))
+    return static_cast<int>(cudaErrorInvalidValue);
+  kern<<<static_cast<unsigned>(n_units), NT, SMEM_ALLOC, static_cast<cudaStream_t>(stream)>>>(a, tmap_q, tmap_k, tmap_g);
   return static_cast<int>(cudaGetLastError());
 }
 
