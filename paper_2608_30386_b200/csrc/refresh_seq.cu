@@ -3,17 +3,28 @@
 // log-decay g <= 0; it is the reference point for the chunked tensor-core kernel
 // and the path for shapes that kernel does not take.
 //
-// One CTA per (request, layer, value head).  The d_k x d_v state lives in
-// registers: thread (s, v) owns column v of row slice s (DK/RS rows).  Per token
+// One CTA per (request, layer, value head), or per part of its columns.  Columns of the state do not interact, so there is no
+// barrier between tokens: a column's d_k entries live in the registers of SL adjacent lanes, and S^T k, S^T q are shuffles.
+// Per token
 //   S   <- Diag(alpha_t) S                       (decay on the key-channel index)
-//   r   <- S^T k_t                               (reduced over the row slices via shared memory)
+//   r   <- S^T k_t
 //   u   <- beta_t (v_t - r)
 //   S   <- S + k_t u^T
 //   o_t <- q_scale * S^T q_t
+// A lane holds rows 4 (i SL + slice) ... + 3, i = 0, 1, ..., of COLS columns: the SL lanes of a column read one contiguous
+// stretch of k, q, alpha, and row pairs are the operand pairs of the packed fp32 instructions.  Bound: when units are few the
+// serial chain (a dot product and its shuffles per token; the next token's is started before this token's update, see
+// below), else instruction issue and the registers' share of the shared-memory bandwidth (128 bytes per cycle whatever is
+// broadcast, hence 4 columns per lane in the wide variants).
+// Measured on B200 (the form before: one column per thread and row half, a block barrier per token): 4 units of 64 x 64, 64 fp32
+// tokens 26.7 -> 15.8 us; 4 of 128 x 128 54 -> 18.5 us; 256 of 128 x 128, 256 tokens 407 -> 345 us; 8192 of them 11.2 -> 9.5 ms.
 // Token inputs are staged TB tokens at a time: raw rows by cp.async into a double
-// buffer, then converted once (bf16 -> fp32, alpha = exp(g)) for all threads.
+// buffer, then converted once (bf16 -> fp32, alpha = exp(g)); outputs leave a group later, 16 bytes per store.  With NHELP > 0
+// that many extra threads do both, a group ahead of and a group behind the tokens being replayed.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "dasc_internal.h"
 
@@ -30,6 +41,13 @@ __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all committed groups, or all but the last one
+__device__ __forceinline__ void cp_async_wait_but(bool one) {
+  if (one)
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+  else
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <typename IO>
@@ -46,37 +64,91 @@ __device__ __forceinline__ float float_to_io<float>(float x) { return x; }
 template <>
 __device__ __forceinline__ __nv_bfloat16 float_to_io<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
 
-template <int DK, int DV, typename IO, bool KDA>
+// packed pairs of fp32 (one instruction per pair)
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float sum2(uint64_t v) {
+  float lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+  return lo + hi;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+template <int DK, int NCOL, int NOP, bool AHEAD, typename IO, bool KDA>
 struct SeqSmem {
   // raw staging, double buffered
   alignas(16) IO q[2][TB][DK];
   alignas(16) IO k[2][TB][DK];
-  alignas(16) IO v[2][TB][DV];
+  alignas(16) IO v[2][TB][NCOL];
   alignas(16) float g[2][TB][KDA ? DK : 4];
   alignas(16) float beta[2][TB];
-  // converted, current group
-  alignas(16) float kf[TB][DK];
-  alignas(16) float qf[TB][DK];
-  alignas(16) float af[TB][DK];
-  alignas(16) float vf[TB][DV];
-  float bf[TB];
+  // converted; two groups when extra warps convert the next one meanwhile
+  struct Group {
+    alignas(16) float kf[TB][DK];
+    alignas(16) float qf[TB][DK];
+    alignas(16) float af[TB][KDA ? DK : 4];
+    alignas(16) float vf[TB][NCOL];
+    alignas(16) float of[TB][NCOL][NOP];  // NOP shares of each of the group's outputs
+    float bf[TB], cf[TB];                     // beta;  c_t = (alpha_t k_t) . k_{t-1}
+  } grp[AHEAD ? 2 : 1];
 };
 
-// One (request, layer, value head) unit, replayed by the whole CTA.
-template <int DK, int DV, int RS, typename IO, typename OT, bool KDA>
-__device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, unsigned char *smem_raw) {
-  constexpr int NT = DV * RS;
-  constexpr int ROWS = DK / RS;  // rows of the state held by one thread
-  using Smem = SeqSmem<DK, DV, IO, KDA>;
+template <int COLS>
+__device__ __forceinline__ void load_cols(float (&x)[COLS], const float *p) {
+  if constexpr (COLS == 4) {
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+  } else if constexpr (COLS == 1) {
+    x[0] = *p;
+  } else {
+    const float2 v = *reinterpret_cast<const float2 *>(p);
+    x[0] = v.x; x[1] = v.y;
+  }
+}
+template <int COLS>
+__device__ __forceinline__ void store_cols(float *p, const float (&x)[COLS]) {
+  if constexpr (COLS == 4)
+    *reinterpret_cast<float4 *>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  else if constexpr (COLS == 1)
+    *p = x[0];
+  else
+    *reinterpret_cast<float2 *>(p) = make_float2(x[0], x[1]);
+}
+
+// One (request, layer, value head) unit, or NCOL of its DV columns, replayed by the whole CTA; COLS columns per lane, SL lanes per column.
+template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
+__device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int part, unsigned char *smem_raw) {
+  constexpr int NC = NCOL / COLS * SL;      // threads that replay tokens
+  constexpr int NT = NHELP > 0 ? NHELP : NC;  // threads that bring the tokens in and the outputs out
+  constexpr int NV = DK / SL / 4;  // groups of four rows held by one lane
+  constexpr int NOP = SL / COLS;
+  constexpr bool AHEAD = NHELP > 0;
+  using Smem = SeqSmem<DK, NCOL, NOP, AHEAD, IO, KDA>;
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
-  // partial sums across row slices, double buffered by token parity
-  float(*red_r)[RS][DV] = reinterpret_cast<float(*)[RS][DV]>(smem_raw + sizeof(Smem));
-  float(*red_o)[RS][DV] = red_r + 2;
 
   const int tid = threadIdx.x;
-  const int v_col = tid % DV;
-  const int slice = tid / DV;
-  const int row0 = slice * ROWS;
+  const bool helper = AHEAD && tid >= NC;
+  const int ht = AHEAD ? tid - NC : tid;  // index among the latter (negative: none of them)
+  const int slice = tid % SL;
+  const int col0 = tid / SL * COLS;
+  const int own = slice % COLS;  // the one of this lane's columns whose sums it ends up with
 
   const int h = unit % a.H_v;
   const int lc = (unit / a.H_v) % a.n_layers_in_call;
@@ -90,202 +162,355 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, uns
   if (n_tok <= 0 && a.mode == DASC_REFRESH_CONTINUE) return;
 
   float *st = a.state + static_cast<int64_t>(a.req_idx[r]) * a.req_stride + static_cast<int64_t>(layer) * a.layer_stride +
-              static_cast<int64_t>(h) * DK * DV;
-  float S[ROWS];
-  if (a.mode == DASC_REFRESH_CONTINUE) {
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) S[i] = st[(row0 + i) * DV + v_col];
-  } else {
-#pragma unroll
-    for (int i = 0; i < ROWS; ++i) S[i] = 0.f;
-  }
-
+              static_cast<int64_t>(h) * DK * DV + part * NCOL;
   const int64_t tok0 = static_cast<int64_t>(lc) * a.total_tokens + t_begin;
   const IO *gq = static_cast<const IO *>(a.q) + (tok0 * a.H_k + hk) * DK;
   const IO *gk = static_cast<const IO *>(a.k) + (tok0 * a.H_k + hk) * DK;
-  const IO *gv = static_cast<const IO *>(a.v) + (tok0 * a.H_v + h) * DV;
+  const IO *gv = static_cast<const IO *>(a.v) + (tok0 * a.H_v + h) * DV + part * NCOL;
   const float *gg = a.g + (tok0 * a.H_v + h) * (KDA ? DK : 1);
   const float *gb = a.beta + tok0 * a.H_v + h;
-  OT *go = a.o ? static_cast<OT *>(a.o) + (tok0 * a.H_v + h) * DV : nullptr;
+  OT *go = a.o ? static_cast<OT *>(a.o) + (tok0 * a.H_v + h) * DV + part * NCOL : nullptr;
   const int64_t qk_stride = static_cast<int64_t>(a.H_k) * DK, v_stride = static_cast<int64_t>(a.H_v) * DV;
   const int64_t g_stride = static_cast<int64_t>(a.H_v) * (KDA ? DK : 1), b_stride = a.H_v;
 
-  auto stage = [&](int grp, int buf) {
-    const int t_lo = grp * TB;
+  // raw rows of a group -> shared memory; consecutive threads take 16-byte vectors of all streams
+  auto stage = [&](int grp) {
+    const int t_lo = grp * TB, buf = grp & 1;
     const int cnt = min(TB, n_tok - t_lo);
-    constexpr int QV = DK * sizeof(IO) / 16, VV = DV * sizeof(IO) / 16, GV = KDA ? DK * 4 / 16 : 1;
-    for (int i = tid; i < cnt * QV; i += NT) {
+    constexpr int QV = DK * sizeof(IO) / 16, VV = NCOL * sizeof(IO) / 16, GV = KDA ? DK * 4 / 16 : 1;
+    for (int i = ht; i < cnt * QV; i += NT) {
       const int t = i / QV, j = i % QV;
       cp_async16(reinterpret_cast<char *>(&sm.q[buf][t][0]) + j * 16,
                  reinterpret_cast<const char *>(gq + (t_lo + t) * qk_stride) + j * 16);
       cp_async16(reinterpret_cast<char *>(&sm.k[buf][t][0]) + j * 16,
                  reinterpret_cast<const char *>(gk + (t_lo + t) * qk_stride) + j * 16);
     }
-    for (int i = tid; i < cnt * VV; i += NT) {
+    for (int i = ht; i < cnt * VV; i += NT) {
       const int t = i / VV, j = i % VV;
       cp_async16(reinterpret_cast<char *>(&sm.v[buf][t][0]) + j * 16,
                  reinterpret_cast<const char *>(gv + (t_lo + t) * v_stride) + j * 16);
     }
     if constexpr (KDA) {
-      for (int i = tid; i < cnt * GV; i += NT) {
+      for (int i = ht; i < cnt * GV; i += NT) {
         const int t = i / GV, j = i % GV;
         cp_async16(reinterpret_cast<char *>(&sm.g[buf][t][0]) + j * 16,
                    reinterpret_cast<const char *>(gg + (t_lo + t) * g_stride) + j * 16);
       }
     } else {
-      for (int t = tid; t < cnt; t += NT) cp_async4(&sm.g[buf][t][0], gg + (t_lo + t) * g_stride);
+      for (int t = ht; t < cnt; t += NT) cp_async4(&sm.g[buf][t][0], gg + (t_lo + t) * g_stride);
     }
-    for (int t = tid; t < cnt; t += NT) cp_async4(&sm.beta[buf][t], gb + (t_lo + t) * b_stride);
+    for (int t = ht; t < cnt; t += NT) cp_async4(&sm.beta[buf][t], gb + (t_lo + t) * b_stride);
     cp_async_commit();
   };
 
   const int n_grp = n_tok > 0 ? (n_tok + TB - 1) / TB : 0;
-  if (n_grp > 0) stage(0, 0);
-  int parity = 0;  // token parity for the reduction buffers
-  bool have_prev_o = false;
-  int prev_t = 0;
-  for (int grp = 0; grp < n_grp; ++grp) {
-    const int buf = grp & 1;
-    const int t_lo = grp * TB;
-    const int cnt = min(TB, n_tok - t_lo);
-    cp_async_wait_all();
-    __syncthreads();  // raw[buf] landed; everyone is past the previous group's converted buffers
-    if (grp + 1 < n_grp) stage(grp + 1, buf ^ 1);
-    for (int i = tid; i < cnt * DK; i += NT) {
+
+  // row pairs (4 (i SL + slice) + 2p, + 1) of column col0 + c
+  uint64_t S[NV][2][COLS];
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const float *row = st + (4 * (i * SL + slice) + 2 * p) * DV + col0;
+      float x[COLS] = {}, y[COLS] = {};
+      if (a.mode == DASC_REFRESH_CONTINUE && !helper) {
+        load_cols<COLS>(x, row);
+        load_cols<COLS>(y, row + DV);
+      }
+#pragma unroll
+      for (int c = 0; c < COLS; ++c) S[i][p][c] = pack2(x[c], y[c]);
+    }
+
+  // x[c] summed over the COLS lanes around this one, column `own` of it: COLS - 1 shuffles
+  auto scatter = [&](float (&x)[COLS]) {
+#pragma unroll
+    for (int w = COLS / 2; w > 0; w >>= 1) {
+      const bool up = (slice & w) != 0;
+#pragma unroll
+      for (int c = 0; c < w; ++c) {
+        const float give = up ? x[c] : x[c + w];
+        x[c] = (up ? x[c + w] : x[c]) + __shfl_xor_sync(0xffffffffu, give, w);
+      }
+    }
+    return x[0];
+  };
+  // column sums over the whole column's lanes, of column `own`
+  auto reduce = [&](const uint64_t (&acc)[COLS][2]) {
+    float x[COLS];
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) x[c] = sum2(add2(acc[c][0], acc[c][1]));
+    float r = scatter(x);
+#pragma unroll
+    for (int d = COLS; d < SL; d <<= 1) r += __shfl_xor_sync(0xffffffffu, r, d);
+    return r;
+  };
+  // raw -> converted
+  auto convert = [&](int grp) {
+    const int buf = grp & 1, cnt = min(TB, n_tok - grp * TB);
+    typename Smem::Group &G = sm.grp[AHEAD ? buf : 0];
+#pragma unroll 4
+    for (int i = ht; i < cnt * DK; i += NT) {
       const int t = i / DK, c = i % DK;
-      sm.kf[t][c] = io_to_float<IO>(sm.k[buf][t][c]);
-      sm.qf[t][c] = io_to_float<IO>(sm.q[buf][t][c]) * a.q_scale;
-      sm.af[t][c] = expf(sm.g[buf][t][KDA ? c : 0]);
+      G.kf[t][c] = io_to_float<IO>(sm.k[buf][t][c]);
+      if (go) G.qf[t][c] = io_to_float<IO>(sm.q[buf][t][c]) * a.q_scale;
+      if constexpr (KDA) G.af[t][c] = expf(sm.g[buf][t][c]);
     }
-    for (int i = tid; i < cnt * DV; i += NT) sm.vf[i / DV][i % DV] = io_to_float<IO>(sm.v[buf][i / DV][i % DV]);
-    for (int t = tid; t < cnt; t += NT) sm.bf[t] = sm.beta[buf][t];
-    __syncthreads();
-
-    for (int t = 0; t < cnt; ++t) {
-      // decay and the partial of r = S^T k over this thread's rows
-      float racc = 0.f;
+    for (int i = ht; i < cnt * NCOL; i += NT) G.vf[i / NCOL][i % NCOL] = io_to_float<IO>(sm.v[buf][i / NCOL][i % NCOL]);
+    for (int t = ht; t < cnt; t += NT) {
+      G.bf[t] = sm.beta[buf][t];
+      if constexpr (!KDA) G.af[t][0] = expf(sm.g[buf][t][0]);
+    }
+    for (int t = ht / 32 + 1; t < cnt; t += NT / 32) {  // a warp per token
+      float c = 0.f;
 #pragma unroll
-      for (int i = 0; i < ROWS; i += 4) {
-        const float4 al = *reinterpret_cast<const float4 *>(&sm.af[t][row0 + i]);
-        const float4 kk = *reinterpret_cast<const float4 *>(&sm.kf[t][row0 + i]);
-        S[i + 0] *= al.x; racc = fmaf(kk.x, S[i + 0], racc);
-        S[i + 1] *= al.y; racc = fmaf(kk.y, S[i + 1], racc);
-        S[i + 2] *= al.z; racc = fmaf(kk.z, S[i + 2], racc);
-        S[i + 3] *= al.w; racc = fmaf(kk.w, S[i + 3], racc);
+      for (int i = ht % 32; i < DK; i += 32)
+        c = fmaf(io_to_float<IO>(sm.k[buf][t][i]) * (KDA ? expf(sm.g[buf][t][i]) : 1.f), io_to_float<IO>(sm.k[buf][t - 1][i]), c);
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
+      if constexpr (!KDA) c *= expf(sm.g[buf][t][0]);
+      if (ht % 32 == 0) G.cf[t] = c;
+    }
+  };
+  // the outputs of a group, 16 bytes of `OT` per store
+  auto flush = [&](int grp) {
+    if (!go) return;
+    constexpr int OV = 16 / sizeof(OT);
+    const int t_lo = grp * TB, cnt = min(TB, n_tok - t_lo);
+    const typename Smem::Group &G = sm.grp[AHEAD ? grp & 1 : 0];
+    for (int i = ht; i < cnt * (NCOL / OV); i += NT) {
+      const int t = i / (NCOL / OV), j = i % (NCOL / OV) * OV;
+      alignas(16) OT w[OV];
+#pragma unroll
+      for (int e = 0; e < OV; ++e) {
+        const float2 *p = reinterpret_cast<const float2 *>(G.of[t][j + e]);
+        float x = 0.f, y = 0.f;
+#pragma unroll
+        for (int sl = 0; sl < NOP / 2; ++sl) {
+          x += p[sl].x;
+          y += p[sl].y;
+        }
+        w[e] = float_to_io<OT>(x + y);
       }
-      if (RS > 1) red_r[parity][slice][v_col] = racc;
+      *reinterpret_cast<uint4 *>(go + (t_lo + t) * v_stride + j) = *reinterpret_cast<const uint4 *>(w);
+    }
+  };
+  auto sync_helpers = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };
+
+  // Group 0 is converted by the helpers (or by everyone) before the loop.
+  if (n_grp > 0 && ht >= 0) {
+    stage(0);
+    if (AHEAD) {
+      cp_async_wait_all();
+      sync_helpers();
+      if (n_grp > 1) stage(1);
+      convert(0);
+    }
+  }
+  if (AHEAD) __syncthreads();
+  for (int grp = 0; grp < n_grp; ++grp) {
+    const int cnt = min(TB, n_tok - grp * TB);
+    if constexpr (AHEAD) {
+      // extra warps: the group before goes out, the next one is converted, the one after that is fetched
+      if (helper) {
+        if (grp + 1 < n_grp) {
+          if (grp + 2 < n_grp) stage(grp + 2);
+          cp_async_wait_but(grp + 2 < n_grp);
+          sync_helpers();
+          convert(grp + 1);
+        }
+        if (grp > 0) flush(grp - 1);
+        __syncthreads();
+        continue;
+      }
+    } else {
+      cp_async_wait_all();
+      __syncthreads();  // the raw rows have landed; everyone is past the previous group's converted rows
+      if (grp + 1 < n_grp) stage(grp + 1);
+      if (grp > 0) flush(grp - 1);
+      convert(grp);
       __syncthreads();
-      // the previous token's read-out partials are complete now as well
-      if (RS > 1 && have_prev_o && slice == 0 && go) {
-        float o = 0.f;
-#pragma unroll
-        for (int s = 0; s < RS; ++s) o += red_o[parity ^ 1][s][v_col];
-        go[prev_t * v_stride + v_col] = float_to_io<OT>(o);
-      }
-      float rsum = racc;
-      if (RS > 1) {
-        rsum = 0.f;
-#pragma unroll
-        for (int s = 0; s < RS; ++s) rsum += red_r[parity][s][v_col];
-      }
-      const float u = sm.bf[t] * (sm.vf[t][v_col] - rsum);
-      float oacc = 0.f;
-#pragma unroll
-      for (int i = 0; i < ROWS; i += 4) {
-        const float4 kk = *reinterpret_cast<const float4 *>(&sm.kf[t][row0 + i]);
-        const float4 qq = *reinterpret_cast<const float4 *>(&sm.qf[t][row0 + i]);
-        S[i + 0] = fmaf(kk.x, u, S[i + 0]); oacc = fmaf(qq.x, S[i + 0], oacc);
-        S[i + 1] = fmaf(kk.y, u, S[i + 1]); oacc = fmaf(qq.y, S[i + 1], oacc);
-        S[i + 2] = fmaf(kk.z, u, S[i + 2]); oacc = fmaf(qq.z, S[i + 2], oacc);
-        S[i + 3] = fmaf(kk.w, u, S[i + 3]); oacc = fmaf(qq.w, S[i + 3], oacc);
-      }
-      if (RS > 1) {
-        red_o[parity][slice][v_col] = oacc;
-        have_prev_o = true;
-        prev_t = t_lo + t;
-      } else if (go) {
-        go[(t_lo + t) * v_stride + v_col] = float_to_io<OT>(oacc);
-      }
-      parity ^= 1;
     }
-  }
-  if (RS > 1) {
-    __syncthreads();
-    if (have_prev_o && slice == 0 && go) {
-      float o = 0.f;
-#pragma unroll
-      for (int s = 0; s < RS; ++s) o += red_o[parity ^ 1][s][v_col];
-      go[prev_t * v_stride + v_col] = float_to_io<OT>(o);
-    }
-  }
+    const typename Smem::Group &G = sm.grp[AHEAD ? grp & 1 : 0];
 
-  if (a.mode == DASC_REFRESH_CONTINUE) {
+    // (alpha_t k_t)^T x over this lane's rows, x = the state before or behind the decay of the token before
+    uint64_t al2[NV][2];
+    auto dot = [&](int t, uint64_t (&acc)[COLS][2]) {
+      uint64_t as = 0ull;
+      if constexpr (!KDA) as = pack2(G.af[t][0], G.af[t][0]);
 #pragma unroll
-    for (int i = 0; i < ROWS; ++i) st[(row0 + i) * DV + v_col] = S[i];
-  } else {
-    const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * DK;
+      for (int i = 0; i < NV; ++i) {
+        const ulonglong2 kk = (reinterpret_cast<const ulonglong2 *>(G.kf[t]) + slice)[i * SL];
+        ulonglong2 al = make_ulonglong2(as, as);
+        if constexpr (KDA) al = (reinterpret_cast<const ulonglong2 *>(G.af[t]) + slice)[i * SL];
+        al2[i][0] = al.x;
+        al2[i][1] = al.y;
+        const uint64_t k0 = mul2(kk.x, al.x), k1 = mul2(kk.y, al.y);
 #pragma unroll
-    for (int i = 0; i < ROWS; ++i)
-      if (!keep[row0 + i]) st[(row0 + i) * DV + v_col] = S[i];
+        for (int c = 0; c < COLS; ++c) {
+          acc[c][0] = i == 0 ? mul2(k0, S[i][0][c]) : fma2(k0, S[i][0][c], acc[c][0]);
+          acc[c][1] = i == 0 ? mul2(k1, S[i][1][c]) : fma2(k1, S[i][1][c], acc[c][1]);
+        }
+      }
+    };
+    // u of one column in every lane that holds it; S <- alpha S (the decay of the token whose dot() came last)
+    auto decay = [&]() {
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) {
+          S[i][0][c] = mul2(S[i][0][c], al2[i][0]);
+          S[i][1][c] = mul2(S[i][1][c], al2[i][1]);
+        }
+    };
+    uint64_t acc[COLS][2];
+    dot(0, acc);
+    decay();
+    float u = G.bf[0] * (G.vf[0][col0 + own] - reduce(acc));
+    auto token = [&](int t, auto has_next) {
+      // S = Diag(alpha_t) S_{t-1} here.  The next token's r is split, r_{t+1} = (alpha k)_{t+1}^T Diag(alpha_t) S_{t-1} + c_{t+1} u_t,
+      // so that its dot product and shuffles run beside this token's update instead of behind it.
+      constexpr bool next = decltype(has_next)::value;
+      if constexpr (next) dot(t + 1, acc);
+      uint64_t uu[COLS];
+#pragma unroll
+      for (int c = 0; c < COLS; ++c) {
+        const float x = COLS == 1 ? u : __shfl_sync(0xffffffffu, u, (threadIdx.x & 31 & ~(COLS - 1)) + c);
+        uu[c] = pack2(x, x);
+      }
+      float p = 0.f;
+      if constexpr (next) p = reduce(acc);
+      uint64_t oa[COLS][2];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const ulonglong2 kk = (reinterpret_cast<const ulonglong2 *>(G.kf[t]) + slice)[i * SL];
+        const ulonglong2 qq = (reinterpret_cast<const ulonglong2 *>(G.qf[t]) + slice)[i * SL];
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) {
+          S[i][0][c] = fma2(kk.x, uu[c], S[i][0][c]);
+          S[i][1][c] = fma2(kk.y, uu[c], S[i][1][c]);
+          oa[c][0] = i == 0 ? mul2(qq.x, S[i][0][c]) : fma2(qq.x, S[i][0][c], oa[c][0]);
+          oa[c][1] = i == 0 ? mul2(qq.y, S[i][1][c]) : fma2(qq.y, S[i][1][c], oa[c][1]);
+        }
+      }
+      if constexpr (next) {
+        decay();
+        u = G.bf[t + 1] * (G.vf[t + 1][col0 + own] - fmaf(G.cf[t + 1], u, p));
+      }
+      if (go) {
+        float x[COLS];
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) x[c] = sum2(add2(oa[c][0], oa[c][1]));
+        const float o = scatter(x);
+        // no "memory" clobber: the loads of the next token may be moved above this store
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&G.of[t][col0 + own][slice / COLS]))), "f"(o));
+      }
+    };
+    // one straight block per token, so that the scheduler can interleave the two halves
+#pragma unroll 2
+    for (int t = 0; t + 1 < cnt; ++t) token(t, std::true_type{});
+    token(cnt - 1, std::false_type{});
+    if (AHEAD) __syncthreads();
   }
+  __syncthreads();
+  if (n_grp > 0 && (!AHEAD || helper)) flush(n_grp - 1);
+  if (helper) return;
+
+  const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * DK;
+  const bool all_rows = a.mode == DASC_REFRESH_CONTINUE;
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const int row = 4 * (i * SL + slice) + 2 * p;
+      float lo[COLS], hi[COLS];
+#pragma unroll
+      for (int c = 0; c < COLS; ++c) asm("mov.b64 {%0, %1}, %2;" : "=f"(lo[c]), "=f"(hi[c]) : "l"(S[i][p][c]));
+      float *d = st + row * DV + col0;
+      if (all_rows || !keep[row]) store_cols<COLS>(d, lo);
+      if (all_rows || !keep[row + 1]) store_cols<COLS>(d + DV, hi);
+    }
 }
 
-// grid = one CTA per unit (from_list == 0), or a fixed grid whose CTAs walk the list of units that the chunked kernel
-// handed over (from_list == 1; the list and its length are in the workspace, written earlier on the same stream).
-template <int DK, int DV, int RS, typename IO, typename OT, bool KDA>
-__global__ void __launch_bounds__(DV *RS) refresh_seq_kernel(DascRefreshArgs a) {
+// grid = one CTA per unit and column part (from_list == 0), or a fixed grid whose CTAs walk the list of units that the
+// chunked kernel handed over (from_list == 1; the list and its length are in the workspace, written earlier on the same stream).
+template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
+__global__ void __launch_bounds__(NCOL / COLS *SL + NHELP) refresh_seq_kernel(DascRefreshArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int PARTS = DV / NCOL;
   if (!a.from_list) {
-    seq_unit<DK, DV, RS, IO, OT, KDA>(a, static_cast<int>(blockIdx.x), smem_raw);
+    seq_unit<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x) / PARTS, static_cast<int>(blockIdx.x) % PARTS, smem_raw);
     return;
   }
   uint32_t *ws = static_cast<uint32_t *>(a.workspace);
   const uint32_t listed = ws[2];
   const int n_list = static_cast<int>(listed < static_cast<uint32_t>(a.unit_list_cap) ? listed : a.unit_list_cap);
-  for (int i = blockIdx.x; i < n_list; i += gridDim.x) {
-    seq_unit<DK, DV, RS, IO, OT, KDA>(a, a.unit_list[i], smem_raw);
-    if (threadIdx.x == 0) atomicAdd(ws + 3, 1u);
+  for (int i = blockIdx.x; i < n_list * PARTS; i += gridDim.x) {
+    seq_unit<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>(a, a.unit_list[i / PARTS], i % PARTS, smem_raw);
+    if (threadIdx.x == 0 && i % PARTS == 0) atomicAdd(ws + 3, 1u);
     __syncthreads();  // the next unit reuses the staging buffers
   }
 }
 
-template <int DK, int DV, int RS, typename IO, typename OT, bool KDA>
+template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
 int launch(const DascRefreshArgs &a, void *stream) {
-  const size_t smem = sizeof(SeqSmem<DK, DV, IO, KDA>) + sizeof(float) * 4 * RS * DV;
-  auto kern = refresh_seq_kernel<DK, DV, RS, IO, OT, KDA>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return static_cast<int>(e);
-  const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
-  if (n_units == 0) return cudaSuccess;
-  if (n_units > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
+  constexpr size_t smem = sizeof(SeqSmem<DK, NCOL, SL / COLS, (NHELP > 0), IO, KDA>);
+  auto kern = refresh_seq_kernel<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return static_cast<int>(e);
+  }
+  const int64_t n_ctas = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v * (DV / NCOL);
+  if (n_ctas == 0) return cudaSuccess;
+  if (n_ctas > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
   // a handed-over list is short (units outside the chunked kernel's range or below its length threshold): a grid
-  // of a few CTAs per SM walks it, and costs next to nothing when the list is empty
-  const int64_t grid = a.from_list ? (n_units < 444 ? n_units : 444) : n_units;
-  kern<<<static_cast<unsigned>(grid), DV * RS, smem, static_cast<cudaStream_t>(stream)>>>(a);
+  // of a CTA per SM walks it, and costs next to nothing when the list is empty
+  const int64_t grid = a.from_list ? (n_ctas < 148 ? n_ctas : 148) : n_ctas;
+  kern<<<static_cast<unsigned>(grid), NCOL / COLS * SL + NHELP, smem, static_cast<cudaStream_t>(stream)>>>(a);
   return static_cast<int>(cudaGetLastError());
 }
 
-template <int DK, int DV, int RS, typename IO, typename OT>
-int dispatch_kind(const DascRefreshArgs &a, void *stream) {
-  return a.kind == DASC_KDA ? launch<DK, DV, RS, IO, OT, true>(a, stream) : launch<DK, DV, RS, IO, OT, false>(a, stream);
+// Columns do not interact, so units that leave SMs idle are split by columns: parts of 8 (16 at d = 32) with 16 (8) lanes per
+// column and warps of their own for the conversions while that gives at most two CTAs per SM (beyond, the conversions, which
+// every part repeats, cost more than the shorter chain saves); at d = 128 halves while those fit one CTA per SM.
+// B200, 128 tokens, split / whole: d = 64, 16 units 25 / 49 us, 32 units 33 / 43 us, 64 units 62 / 43 us; d = 128, 16 units
+// 60 / 90 us, 32 units 115 / 90 us (halves 64 us).
+constexpr int64_t kSplitCtas = 296, kHalfCtas = 148;
+
+template <int D, typename IO, typename OT, bool KDA>
+int dispatch_split(const DascRefreshArgs &a, void *stream) {
+  const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
+  if constexpr (D == 32) {
+    if (!a.from_list && n_units * 2 <= kSplitCtas) return launch<32, 32, 16, 1, 8, 256, IO, OT, KDA>(a, stream);
+    return launch<32, 32, 32, 2, 8, 0, IO, OT, KDA>(a, stream);
+  } else if constexpr (D == 64) {
+    if (!a.from_list && n_units * 8 <= kSplitCtas) return launch<64, 64, 8, 1, 16, 256, IO, OT, KDA>(a, stream);
+    return launch<64, 64, 64, 4, 8, 128, IO, OT, KDA>(a, stream);
+  } else {
+    if (!a.from_list && n_units * 16 <= kSplitCtas) return launch<128, 128, 8, 1, 16, 256, IO, OT, KDA>(a, stream);
+    if (!a.from_list && n_units * 2 <= kHalfCtas) return launch<128, 128, 64, 4, 16, 128, IO, OT, KDA>(a, stream);
+    return launch<128, 128, 128, 4, 16, 0, IO, OT, KDA>(a, stream);
+  }
 }
 
-template <int DK, int DV, int RS>
+template <int D, typename IO, typename OT>
+int dispatch_kind(const DascRefreshArgs &a, void *stream) {
+  return a.kind == DASC_KDA ? dispatch_split<D, IO, OT, true>(a, stream) : dispatch_split<D, IO, OT, false>(a, stream);
+}
+
+template <int D>
 int dispatch(const DascRefreshArgs &a, void *stream) {
   const bool o_bf16 = a.o ? a.o_bf16 != 0 : a.io_bf16 != 0;  // no output: any instantiation will do
   if (a.io_bf16)
-    return o_bf16 ? dispatch_kind<DK, DV, RS, __nv_bfloat16, __nv_bfloat16>(a, stream)
-                  : dispatch_kind<DK, DV, RS, __nv_bfloat16, float>(a, stream);
-  return o_bf16 ? dispatch_kind<DK, DV, RS, float, __nv_bfloat16>(a, stream)
-                : dispatch_kind<DK, DV, RS, float, float>(a, stream);
+    return o_bf16 ? dispatch_kind<D, __nv_bfloat16, __nv_bfloat16>(a, stream) : dispatch_kind<D, __nv_bfloat16, float>(a, stream);
+  return o_bf16 ? dispatch_kind<D, float, __nv_bfloat16>(a, stream) : dispatch_kind<D, float, float>(a, stream);
 }
 
 }  // namespace
 
 // Returns a cudaError_t as int, or -1 if the shape has no instantiation.
 int dasc_launch_refresh_seq(const DascRefreshArgs &a, void *stream) {
-  if (a.d_k == 128 && a.d_v == 128) return dispatch<128, 128, 2>(a, stream);
-  if (a.d_k == 64 && a.d_v == 64) return dispatch<64, 64, 2>(a, stream);
-  if (a.d_k == 32 && a.d_v == 32) return dispatch<32, 32, 1>(a, stream);
+  if (a.d_k == 128 && a.d_v == 128) return dispatch<128>(a, stream);
+  if (a.d_k == 64 && a.d_v == 64) return dispatch<64>(a, stream);
+  if (a.d_k == 32 && a.d_v == 32) return dispatch<32>(a, stream);
   return -1;
 }
