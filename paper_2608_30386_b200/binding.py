@@ -1,12 +1,14 @@
-"""Thin ctypes binding of libdasc: the same four calls as the C ABI
+"""Thin binding of libdasc: the same four calls as the C ABI
 (``dasc_plan``, ``dasc_pack``, ``dasc_restore``, ``dasc_refresh``), taking torch
-tensors for device memory.  Argument marshalling only: every step runs in the
+tensors for device memory; ctypes, and for the device calls of a serving path the CPython
+module ``_dasccall`` (``csrc/pycall.c``), which marshals the same arguments in native code.  Argument marshalling only: every step runs in the
 library.  There is no fallback: if the shared library is missing or a call
 fails, an exception is raised.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -15,6 +17,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libdasc.so")
+CALL_PATH = os.path.join(_HERE, "_dasccall.so")
 
 KDA, GDN = 0, 1
 SEL_THRESHOLD, SEL_TOP_RATIO, SEL_EXPLICIT = 0, 1, 2
@@ -138,6 +141,29 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_native = None
+
+
+def _call():
+    """The native marshalling module, loaded behind the library it calls."""
+    global _native
+    if _native is None:
+        lib()
+        if not os.path.exists(CALL_PATH):
+            raise ImportError(f"{CALL_PATH} is missing: run `python -m paper_2608_30386_b200.build`")
+        spec = importlib.util.spec_from_file_location("_dasccall", CALL_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        if torch.cuda.is_available():
+            torch.cuda.init()
+            raw_stream, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        else:  # asking for the current stream raises, as it does in torch
+            raw_stream, device = (lambda _: torch.cuda.current_stream().cuda_stream), (lambda: 0)
+        mod.init(raw_stream, device, torch.bfloat16, lambda x: _ptr(x).value or 0)
+        _native = mod
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().dasc_status_string(int(status)).decode()
 
@@ -257,15 +283,15 @@ def dasc_plan_load(blob: bytes, device: int = 0) -> Plan:
 def dasc_pack(plan: Plan, state: torch.Tensor, layer_stride: int, req_stride: int, src_req: torch.Tensor,
               pool: torch.Tensor, dst_slot: torch.Tensor, slot_stride: int = 0, stream=None):
     """Gather the retained units of ``state`` (requests ``src_req``) into pool slots ``dst_slot``."""
-    _check(lib().dasc_pack(plan.handle, _ptr(state), layer_stride, req_stride, _ptr(src_req), _ptr(pool), slot_stride,
-                           _ptr(dst_slot), int(src_req.numel()), _stream_ptr(stream)), "dasc_pack")
+    _check((_native or _call()).pack(plan.handle, state, layer_stride, req_stride, src_req, pool, slot_stride, dst_slot, stream),
+           "dasc_pack")
 
 
 def dasc_restore(plan: Plan, pool: torch.Tensor, src_slot: torch.Tensor, state: torch.Tensor, layer_stride: int,
                  req_stride: int, dst_req: torch.Tensor, slot_stride: int = 0, stream=None):
     """Scatter pool slots ``src_slot`` into the dense states ``dst_req``; omitted units become +0.0."""
-    _check(lib().dasc_restore(plan.handle, _ptr(pool), slot_stride, _ptr(src_slot), _ptr(state), layer_stride,
-                              req_stride, _ptr(dst_req), int(src_slot.numel()), _stream_ptr(stream)), "dasc_restore")
+    _check((_native or _call()).restore(plan.handle, pool, slot_stride, src_slot, state, layer_stride, req_stride, dst_req, stream),
+           "dasc_restore")
 
 
 LAYOUT_RAGGED, LAYOUT_PADDED, LAYOUT_DENSE = 0, 1, 2
@@ -281,16 +307,14 @@ def dasc_padded_pool_floats(plan: Plan, n_slots: int) -> int:
 def dasc_pack_padded(plan: Plan, state: torch.Tensor, layer_stride: int, req_stride: int, src_req: torch.Tensor,
                      pool: torch.Tensor, n_slots: int, dst_slot: torch.Tensor, stream=None):
     """``dasc_pack`` into the padded pool; padding entries are not written."""
-    _check(lib().dasc_pack_padded(plan.handle, _ptr(state), layer_stride, req_stride, _ptr(src_req), _ptr(pool),
-                                  int(n_slots), _ptr(dst_slot), int(src_req.numel()), _stream_ptr(stream)),
+    _check((_native or _call()).pack_padded(plan.handle, state, layer_stride, req_stride, src_req, pool, n_slots, dst_slot, stream),
            "dasc_pack_padded")
 
 
 def dasc_restore_padded(plan: Plan, pool: torch.Tensor, n_slots: int, src_slot: torch.Tensor, state: torch.Tensor,
                         layer_stride: int, req_stride: int, dst_req: torch.Tensor, stream=None):
     """``dasc_restore`` from the padded pool."""
-    _check(lib().dasc_restore_padded(plan.handle, _ptr(pool), int(n_slots), _ptr(src_slot), _ptr(state), layer_stride,
-                                     req_stride, _ptr(dst_req), int(src_slot.numel()), _stream_ptr(stream)),
+    _check((_native or _call()).restore_padded(plan.handle, pool, n_slots, src_slot, state, layer_stride, req_stride, dst_req, stream),
            "dasc_restore_padded")
 
 
@@ -384,17 +408,15 @@ def dasc_int8_slot_bytes(plan: Plan) -> int:
 def dasc_pack_int8(plan: Plan, state: torch.Tensor, layer_stride: int, req_stride: int, src_req: torch.Tensor,
                    pool: torch.Tensor, dst_slot: torch.Tensor, slot_stride_bytes: int = 0, stream=None):
     """Like ``dasc_pack`` with the Appendix D quantiser fused in; ``pool`` is a byte (uint8) tensor."""
-    _check(lib().dasc_pack_int8(plan.handle, _ptr(state), layer_stride, req_stride, _ptr(src_req), _ptr(pool),
-                                slot_stride_bytes, _ptr(dst_slot), int(src_req.numel()), _stream_ptr(stream)),
+    _check((_native or _call()).pack_int8(plan.handle, state, layer_stride, req_stride, src_req, pool, slot_stride_bytes, dst_slot, stream),
            "dasc_pack_int8")
 
 
 def dasc_restore_int8(plan: Plan, pool: torch.Tensor, src_slot: torch.Tensor, state: torch.Tensor, layer_stride: int,
                       req_stride: int, dst_req: torch.Tensor, slot_stride_bytes: int = 0, stream=None):
     """Like ``dasc_restore`` with the dequantisation fused in; ``pool`` is a byte (uint8) tensor."""
-    _check(lib().dasc_restore_int8(plan.handle, _ptr(pool), slot_stride_bytes, _ptr(src_slot), _ptr(state),
-                                   layer_stride, req_stride, _ptr(dst_req), int(src_slot.numel()),
-                                   _stream_ptr(stream)), "dasc_restore_int8")
+    _check((_native or _call()).restore_int8(plan.handle, pool, slot_stride_bytes, src_slot, state, layer_stride, req_stride, dst_req, stream),
+           "dasc_restore_int8")
 
 
 def dasc_refresh_workspace_bytes(plan: Plan, n_req: int, n_layers_in_call: int, algo: int = ALGO_AUTO) -> int:
@@ -411,15 +433,10 @@ def dasc_refresh(plan: Plan, state: torch.Tensor, layer_stride: int, req_stride:
                  mode: int = REFRESH_CONTINUE, algo: int = ALGO_AUTO, workspace: torch.Tensor | None = None,
                  stream=None):
     """Replay the gated delta rule over each request's suffix, in place on ``state``."""
-    io = IO_BF16 if q.dtype == torch.bfloat16 else IO_FP32
-    o_io = IO_BF16 if (o is not None and o.dtype == torch.bfloat16) else IO_FP32
-    if layer_end is None:
-        layer_end = plan.info.n_layers
-    ws_bytes = int(workspace.numel() * workspace.element_size()) if workspace is not None else 0
-    _check(lib().dasc_refresh(plan.handle, _ptr(state), layer_stride, req_stride, _ptr(req_idx), _ptr(q), _ptr(k),
-                              _ptr(v), io, _ptr(g), _ptr(beta), _ptr(cu_seqlens), int(cu_seqlens.numel() - 1),
-                              int(total_tokens), int(max_seqlen), layer_begin, layer_end, float(q_scale), _ptr(o),
-                              o_io, mode, algo, _ptr(workspace), ws_bytes, _stream_ptr(stream)), "dasc_refresh")
+    _check((_native or _call()).refresh(
+        plan.handle, state, layer_stride, req_stride, req_idx, q, k, v, g, beta, cu_seqlens, total_tokens, max_seqlen,
+        layer_begin, plan.info.n_layers if layer_end is None else layer_end, q_scale, o, algo, workspace, stream, mode),
+        "dasc_refresh")
 
 
 def dasc_refresh_window(plan: Plan, state: torch.Tensor, layer_stride: int, req_stride: int, req_idx: torch.Tensor,
@@ -431,16 +448,10 @@ def dasc_refresh_window(plan: Plan, state: torch.Tensor, layer_stride: int, req_
     """The paper's suffix-refresh load policy: replay each request's last ``window`` prefix tokens (0 = the
     plan's W_replay) from a zero scratch state and merge only the omitted units.  ``window_begin`` (int32
     [n_req], device) receives the first replayed token of each request.  ``q`` may be None when ``o`` is."""
-    io = IO_BF16 if k.dtype == torch.bfloat16 else IO_FP32
-    o_io = IO_BF16 if (o is not None and o.dtype == torch.bfloat16) else IO_FP32
-    if layer_end is None:
-        layer_end = plan.info.n_layers
-    ws_bytes = int(workspace.numel() * workspace.element_size()) if workspace is not None else 0
-    _check(lib().dasc_refresh_window(plan.handle, _ptr(state), layer_stride, req_stride, _ptr(req_idx), _ptr(q),
-                                     _ptr(k), _ptr(v), io, _ptr(g), _ptr(beta), _ptr(cu_seqlens),
-                                     int(cu_seqlens.numel() - 1), int(total_tokens), int(window), layer_begin,
-                                     layer_end, float(q_scale), _ptr(o), o_io, algo, _ptr(window_begin),
-                                     _ptr(workspace), ws_bytes, _stream_ptr(stream)), "dasc_refresh_window")
+    _check((_native or _call()).refresh_window(
+        plan.handle, state, layer_stride, req_stride, req_idx, q, k, v, g, beta, cu_seqlens, total_tokens, window,
+        layer_begin, plan.info.n_layers if layer_end is None else layer_end, q_scale, o, algo, workspace, stream, window_begin),
+        "dasc_refresh_window")
 
 
 def dasc_refresh_status(workspace) -> int:

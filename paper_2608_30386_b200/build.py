@@ -4,11 +4,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdasc.so")
+CALL = os.path.join(HERE, "_dasccall.so")   # CPython entry to the library's device calls
+CALL_SOURCE = "pycall.c"
 SOURCES = ["dasc_api.cu", "plan_host.cpp", "pack_restore.cu", "codec_int8.cu", "refresh_seq.cu", "refresh_chunked.cu"]
 HEADERS = [os.path.join(ROOT, "include", "dasc.h"), os.path.join(CSRC, "dasc_internal.h"),
            os.path.join(CSRC, "tcgen05_util.cuh")]
@@ -27,10 +30,10 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS + [os.path.abspath(__file__)]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
+    deps = [os.path.join(CSRC, s) for s in SOURCES + [CALL_SOURCE]] + HEADERS + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -59,6 +62,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     link = [_nvcc(), "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
     subprocess.run(link, check=True)
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(ROOT, "include"), os.path.join(CSRC, CALL_SOURCE), "-o", CALL, "-L", HERE,
+                    "-l:libdasc.so", "-Wl,-rpath,$ORIGIN"], check=True)
     return LIB
 
 
