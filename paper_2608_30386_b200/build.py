@@ -14,7 +14,7 @@ CALL = os.path.join(HERE, "_dasccall.so")   # CPython entry to the library's dev
 CALL_SOURCE = "pycall.c"
 SOURCES = ["dasc_api.cu", "plan_host.cpp", "pack_restore.cu", "codec_int8.cu", "refresh_seq.cu", "refresh_chunked.cu"]
 HEADERS = [os.path.join(ROOT, "include", "dasc.h"), os.path.join(CSRC, "dasc_internal.h"),
-           os.path.join(CSRC, "tcgen05_util.cuh")]
+           os.path.join(CSRC, "tcgen05_util.cuh"), os.path.join(CSRC, "launch.cuh")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

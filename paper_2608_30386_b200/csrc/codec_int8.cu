@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include "dasc_internal.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -121,6 +122,7 @@ __global__ void __launch_bounds__(kThreads, DASC_INT8_PACK_MIN_BLOCKS) pack_int8
                                                              const DascRowSrc *__restrict__ row_src,
                                                              uint32_t packed_vecs, uint32_t packed_rows,
                                                              uint32_t lanes_per_row_arg, int32_t n_pairs) {
+  stream_order_begin();
   const uint32_t lanes_per_row = FULL_WARP_ROWS ? 32u : lanes_per_row_arg;
   const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
   for (int32_t pair = blockIdx.y; pair < n_pairs; pair += gridDim.y) {
@@ -214,6 +216,7 @@ __global__ void __launch_bounds__(kThreads, DASC_INT8_RESTORE_MIN_BLOCKS) restor
                                                                 const int32_t *__restrict__ row_pos, uint32_t layer_vecs,
                                                                 uint32_t rows_per_layer, uint32_t packed_rows,
                                                                 uint32_t lanes_per_row_arg, int32_t n_pairs) {
+  stream_order_begin();
   const uint32_t lanes_per_row = FULL_WARP_ROWS ? 32u : lanes_per_row_arg;
   const uint32_t base = blockIdx.x * (kThreads * kRUnroll) + threadIdx.x;
   const int32_t layer = blockIdx.y;
@@ -261,11 +264,10 @@ int dasc_launch_pack_int8(const dasc_plan_s *plan, const float *state, int64_t l
   dim3 grid(static_cast<uint32_t>((packed_vecs + per_block - 1) / per_block),
             static_cast<uint32_t>(n_pairs < 65535 ? n_pairs : 65535));
   auto kernel = lpr == 32 ? pack_int8_kernel<true> : pack_int8_kernel<false>;
-  kernel<<<grid, kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
+  return static_cast<int>(launch_in_order(kernel, grid, dim3(kThreads), 0, stream,
       reinterpret_cast<const uint4 *>(state), layer_stride / 4, req_stride / 4, src_req,
       static_cast<uint8_t *>(pool), slot_stride_bytes, dst_slot, plan->d_row_src, static_cast<uint32_t>(packed_vecs),
-      static_cast<uint32_t>(plan->packed_rows), lpr, n_pairs);
-  return static_cast<int>(cudaGetLastError());
+      static_cast<uint32_t>(plan->packed_rows), lpr, n_pairs));
 }
 
 int dasc_launch_restore_int8(const dasc_plan_s *plan, const void *pool, int64_t slot_stride_bytes,
@@ -278,9 +280,8 @@ int dasc_launch_restore_int8(const dasc_plan_s *plan, const void *pool, int64_t 
   dim3 grid(static_cast<uint32_t>((layer_vecs + per_block - 1) / per_block),
             static_cast<uint32_t>(plan->info.n_layers), static_cast<uint32_t>(n_pairs < 65535 ? n_pairs : 65535));
   auto kernel = lpr == 32 ? restore_int8_kernel<true> : restore_int8_kernel<false>;
-  kernel<<<grid, kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
+  return static_cast<int>(launch_in_order(kernel, grid, dim3(kThreads), 0, stream,
       static_cast<const uint8_t *>(pool), slot_stride_bytes, src_slot, reinterpret_cast<uint4 *>(state),
       layer_stride / 4, req_stride / 4, dst_req, plan->d_row_pos, static_cast<uint32_t>(layer_vecs),
-      static_cast<uint32_t>(plan->rows_per_layer), static_cast<uint32_t>(plan->packed_rows), lpr, n_pairs);
-  return static_cast<int>(cudaGetLastError());
+      static_cast<uint32_t>(plan->rows_per_layer), static_cast<uint32_t>(plan->packed_rows), lpr, n_pairs));
 }

@@ -116,17 +116,6 @@ dasc_status_t check_copy_args(const dasc_plan_t *plan, const void *state, int64_
   return DASC_OK;
 }
 
-// first replayed token of each request: max(cu[r], cu[r+1] - window)
-__global__ void window_begin_kernel(const int32_t *__restrict__ cu, int32_t n_req, int64_t window,
-                                    int32_t *__restrict__ out) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n_req) {
-    const int64_t lo = cu[r], hi = cu[r + 1];
-    const int64_t b = hi - window;
-    out[r] = static_cast<int32_t>(b > lo ? b : lo);
-  }
-}
-
 }  // namespace
 
 extern "C" {
@@ -593,7 +582,7 @@ struct RefreshRequest {
 // tok_begin: device array of first tokens (null = cu_seqlens[r]).  q may be null when o is null.
 dasc_status_t refresh_validate(const dasc_plan_t *plan, float *state_base, int64_t layer_stride, int64_t req_stride,
                                const int32_t *req_idx, const void *q, const void *k, const void *v, int32_t io_dtype,
-                               const float *g, const float *beta, const int32_t *cu_seqlens, const int32_t *tok_begin,
+                               const float *g, const float *beta, const int32_t *cu_seqlens, int32_t *tok_begin,
                                int32_t n_req, int64_t total_tokens, int32_t max_seqlen, int32_t layer_begin,
                                int32_t layer_end, float q_scale, void *o, int32_t o_dtype, int32_t mode, int32_t algo,
                                void *workspace, size_t workspace_bytes, RefreshRequest *out) {
@@ -674,7 +663,9 @@ dasc_status_t refresh_launch(const RefreshRequest &rq, void *cuda_stream) {
   DascRefreshArgs a = rq.args;
   int e;
   if (!rq.chunked) {
-    e = dasc_launch_refresh_seq(a, cuda_stream);
+    a.workspace = nullptr;  // the token-by-token kernel on its own keeps nothing there
+    e = a.window > 0 ? dasc_launch_refresh_prep(a, cuda_stream) : 0;
+    if (e == 0) e = dasc_launch_refresh_seq(a, cuda_stream);
   } else if (rq.algo == DASC_ALGO_CHUNKED) {
     a.domain_is_error = 1;
     e = dasc_launch_refresh_chunked(a, cuda_stream);
@@ -731,10 +722,16 @@ dasc_status_t dasc_refresh_window(const dasc_plan_t *plan, float *state_base, in
                        o_dtype, DASC_REFRESH_SCRATCH_MERGE_LOCAL, algo, workspace, workspace_bytes, &rq);
   if (st != DASC_OK) return st;
   if (const dasc_status_t ds = check_device(plan); ds != DASC_OK) return ds;
-  window_begin_kernel<<<(n_req + 255) / 256, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(cu_seqlens, n_req, window,
-                                                                                               window_begin);
-  if (cudaGetLastError() != cudaSuccess) return DASC_ERR_CUDA;
-  if (window == 0) return DASC_OK;  // nothing is omitted, so nothing needs a refresh
+  if (rq.nothing_to_do || window == 0) {
+    // only window_begin is written: nothing is replayed (window 0: nothing is omitted)
+    DascRefreshArgs a{};
+    a.cu_seqlens = cu_seqlens;
+    a.tok_begin = window_begin;
+    a.n_req = n_req;
+    a.window = static_cast<int32_t>(window);
+    return dasc_launch_refresh_prep(a, cuda_stream) == 0 ? DASC_OK : DASC_ERR_CUDA;
+  }
+  rq.args.window = static_cast<int32_t>(window);
   return refresh_launch(rq, cuda_stream);
 }
 

@@ -73,8 +73,11 @@ int dasc_launch_restore_int8(const dasc_plan_s *plan, const void *pool, int64_t 
 //   word 1  a unit left the chunked kernel's log-decay range and nothing replayed it (an error)
 //   word 2  units the chunked kernel handed over (out of range, or shorter than its threshold): length of the list
 //   word 3  units the token-by-token kernel replayed from the list
+//   bytes 16..255: uint8 per request, the order in which the chunked kernel takes the requests (kRefreshOrderMax at most)
 //   bytes 256...: int32 unit indices ((request * layers_in_call + layer) * H_v + head), in hand-over order
 constexpr size_t kRefreshWsHeader = 256;
+constexpr size_t kRefreshWsOrder = 16;
+constexpr int kRefreshOrderMax = static_cast<int>(kRefreshWsHeader - kRefreshWsOrder);
 // Requests of at most this many tokens are replayed by the exact kernel under DASC_ALGO_AUTO: with only a handful of
 // tokens every output is a sum of a few q.k products, so the tf32 rounding of one product can exceed the output
 // tolerance, and the tensor-core kernel has no speed to offer at that length anyway.
@@ -89,7 +92,8 @@ struct DascRefreshArgs {
   int32_t io_bf16;
   const float *g, *beta;
   const int32_t *cu_seqlens;
-  const int32_t *tok_begin;  // device, [n_req], or null: first token of each request (null = cu_seqlens[r])
+  int32_t *tok_begin;        // device, [n_req], or null: first token of each request (null = cu_seqlens[r])
+  int32_t window;            // > 0: tok_begin is written first, max(cu_seqlens[r], cu_seqlens[r+1] - window)
   int32_t n_req;
   int64_t total_tokens;
   int32_t max_seqlen;
@@ -106,9 +110,13 @@ struct DascRefreshArgs {
   int32_t unit_list_cap;    // entries the list can hold
   int32_t short_thr;        // chunked kernel: units of at most this many tokens are handed over; -1 = none
   int32_t from_list;        // token-by-token kernel: 1 = replay the listed units only, 0 = every unit of the grid
+  int32_t ordered;          // chunked kernel: the workspace header holds the order of the requests
   int32_t domain_is_error;  // chunked kernel: an out-of-range unit also sets word 1
   uint32_t poll_limit_first_wait;  // test hook: poll limit of the issuing warp's very first wait (0 = the normal limit)
 };
+// What has to be on the device before a refresh kernel: tok_begin (window > 0), cleared header words and the request order
+// (workspace).
+int dasc_launch_refresh_prep(const DascRefreshArgs &a, void *stream);
 int dasc_launch_refresh_seq(const DascRefreshArgs &a, void *stream);
 int dasc_launch_refresh_chunked(const DascRefreshArgs &a, void *stream);
 size_t dasc_refresh_chunked_workspace_bytes(int32_t n_req, int32_t n_layers_in_call, int32_t H_v);

@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "dasc_internal.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restri
                                                            const int32_t *__restrict__ layer_row_off,
                                                            uint32_t vecs_per_row, int32_t n_pairs,
                                                            const __grid_constant__ TpPools tp) {
+  stream_order_begin();
   const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
   const int32_t layer = blockIdx.y;
   const uint32_t first = static_cast<uint32_t>(__ldg(layer_row_off + layer));
@@ -118,6 +120,7 @@ __global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restri
                                                            uint32_t layer_vecs, uint32_t rows_per_layer,
                                                            uint32_t vecs_per_row, int32_t n_pairs,
                                                            const __grid_constant__ TpPools tp) {
+  stream_order_begin();
   const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
   const int32_t layer = blockIdx.y;
   const int32_t *pos_l = row_pos + static_cast<int64_t>(layer) * rows_per_layer;
@@ -160,6 +163,7 @@ __global__ void __launch_bounds__(kThreads) blob_copy_kernel(const uint4 *__rest
                                                              uint4 *__restrict__ dst, int64_t dst_stride4,
                                                              const int32_t *__restrict__ dst_idx, uint32_t vecs,
                                                              int32_t n_pairs) {
+  stream_order_begin();
   const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
   for (int32_t pair = blockIdx.y; pair < n_pairs; pair += gridDim.y) {
     const uint4 *s = src + static_cast<int64_t>(__ldg(src_idx + pair)) * src_stride4;
@@ -219,21 +223,20 @@ int dasc_launch_pack(const dasc_plan_s *plan, const float *state, int64_t layer_
   const int64_t entry_stride4 = plan->info.r_max * rows_per_unit * vpr;  // vectors of the fullest layer
   const dim3 grid = copy_grid(static_cast<uint64_t>(entry_stride4), plan, n_pairs);
   const TpPools tp = make_tp(placement, plan->info.unit_floats);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint4 *st = reinterpret_cast<const uint4 *>(state);
   uint4 *pl = reinterpret_cast<uint4 *>(pool);
+  auto launch = [&](auto kernel, uint4 *dst, int64_t dst_stride4, int64_t slots) {
+    return launch_in_order(kernel, grid, dim3(kThreads), 0, stream, st, layer_stride / 4, req_stride / 4, src_req, dst, dst_stride4,
+                           slots, dst_slot, plan->d_row_src, plan->d_layer_row_off, vpr, n_pairs, tp);
+  };
+  cudaError_t e;
   if (layout == 0)
-    pack_kernel<Layout::Ragged><<<grid, kThreads, 0, s>>>(st, layer_stride / 4, req_stride / 4, src_req, pl, pool_stride / 4, 0,
-                                                          dst_slot, plan->d_row_src, plan->d_layer_row_off, vpr, n_pairs, tp);
+    e = launch(pack_kernel<Layout::Ragged>, pl, pool_stride / 4, 0);
   else if (layout == 1)
-    pack_kernel<Layout::Padded><<<grid, kThreads, 0, s>>>(st, layer_stride / 4, req_stride / 4, src_req, pl, entry_stride4,
-                                                          n_slots, dst_slot, plan->d_row_src, plan->d_layer_row_off, vpr,
-                                                          n_pairs, tp);
+    e = launch(pack_kernel<Layout::Padded>, pl, entry_stride4, n_slots);
   else
-    pack_kernel<Layout::TpBalanced><<<grid, kThreads, 0, s>>>(st, layer_stride / 4, req_stride / 4, src_req, nullptr,
-                                                              pool_stride / 4, 0, dst_slot, plan->d_row_src,
-                                                              plan->d_layer_row_off, vpr, n_pairs, tp);
-  return static_cast<int>(cudaGetLastError());
+    e = launch(pack_kernel<Layout::TpBalanced>, nullptr, pool_stride / 4, 0);
+  return static_cast<int>(e);
 }
 
 int dasc_launch_restore(const dasc_plan_s *plan, const float *pool, int64_t pool_stride, int64_t n_slots,
@@ -247,23 +250,21 @@ int dasc_launch_restore(const dasc_plan_s *plan, const float *pool, int64_t pool
   const int64_t entry_stride4 = plan->info.r_max * rows_per_unit * vpr;
   const dim3 grid = copy_grid(layer_vecs, plan, n_pairs);
   const TpPools tp = make_tp(placement, plan->info.unit_floats);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint4 *pl = reinterpret_cast<const uint4 *>(pool);
   uint4 *st = reinterpret_cast<uint4 *>(state);
   const uint32_t lv = static_cast<uint32_t>(layer_vecs), rpl = static_cast<uint32_t>(plan->rows_per_layer);
+  auto launch = [&](auto kernel, const uint4 *src, int64_t src_stride4, int64_t slots) {
+    return launch_in_order(kernel, grid, dim3(kThreads), 0, stream, src, src_stride4, slots, src_slot, st, layer_stride / 4, req_stride / 4,
+                           dst_req, plan->d_row_pos, plan->d_layer_row_off, lv, rpl, vpr, n_pairs, tp);
+  };
+  cudaError_t e;
   if (layout == 0)
-    restore_kernel<Layout::Ragged><<<grid, kThreads, 0, s>>>(pl, pool_stride / 4, 0, src_slot, st, layer_stride / 4,
-                                                             req_stride / 4, dst_req, plan->d_row_pos,
-                                                             plan->d_layer_row_off, lv, rpl, vpr, n_pairs, tp);
+    e = launch(restore_kernel<Layout::Ragged>, pl, pool_stride / 4, 0);
   else if (layout == 1)
-    restore_kernel<Layout::Padded><<<grid, kThreads, 0, s>>>(pl, entry_stride4, n_slots, src_slot, st, layer_stride / 4,
-                                                             req_stride / 4, dst_req, plan->d_row_pos,
-                                                             plan->d_layer_row_off, lv, rpl, vpr, n_pairs, tp);
+    e = launch(restore_kernel<Layout::Padded>, pl, entry_stride4, n_slots);
   else
-    restore_kernel<Layout::TpBalanced><<<grid, kThreads, 0, s>>>(nullptr, pool_stride / 4, 0, src_slot, st, layer_stride / 4,
-                                                                 req_stride / 4, dst_req, plan->d_row_pos,
-                                                                 plan->d_layer_row_off, lv, rpl, vpr, n_pairs, tp);
-  return static_cast<int>(cudaGetLastError());
+    e = launch(restore_kernel<Layout::TpBalanced>, nullptr, pool_stride / 4, 0);
+  return static_cast<int>(e);
 }
 
 int dasc_launch_blob_copy(const void *src, int64_t src_stride_bytes, const int32_t *src_idx, void *dst,
@@ -273,8 +274,7 @@ int dasc_launch_blob_copy(const void *src, int64_t src_stride_bytes, const int32
   const uint64_t vecs = static_cast<uint64_t>(blob_bytes / 16);
   const uint32_t per_block = kThreads * kUnroll;
   dim3 grid(static_cast<uint32_t>((vecs + per_block - 1) / per_block), static_cast<uint32_t>(n_pairs < 65535 ? n_pairs : 65535));
-  blob_copy_kernel<<<grid, kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-      reinterpret_cast<const uint4 *>(src), src_stride_bytes / 16, src_idx, reinterpret_cast<uint4 *>(dst),
-      dst_stride_bytes / 16, dst_idx, static_cast<uint32_t>(vecs), n_pairs);
-  return static_cast<int>(cudaGetLastError());
+  return static_cast<int>(launch_in_order(blob_copy_kernel, grid, dim3(kThreads), 0, stream, reinterpret_cast<const uint4 *>(src),
+                                          src_stride_bytes / 16, src_idx, reinterpret_cast<uint4 *>(dst), dst_stride_bytes / 16,
+                                          dst_idx, static_cast<uint32_t>(vecs), n_pairs));
 }

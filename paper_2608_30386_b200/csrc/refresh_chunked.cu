@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 
 #include "dasc_internal.h"
+#include "launch.cuh"
 #include "tcgen05_util.cuh"
 
 namespace {
@@ -176,11 +177,11 @@ __device__ __forceinline__ void wait_bar_short(uint64_t *bar, uint32_t parity, M
 // This CTA does not (or could not) replay its unit: put the unit on the list that the token-by-token kernel walks
 // next on the same stream.  Without a list, or when it is full, or when the caller asked for this kernel alone, an
 // out-of-range unit is an error (word 1).
-__device__ __forceinline__ void hand_over(const DascRefreshArgs &a, bool out_of_range) {
+__device__ __forceinline__ void hand_over(const DascRefreshArgs &a, int unit, bool out_of_range) {
   uint32_t *ws = static_cast<uint32_t *>(a.workspace);
   const uint32_t idx = atomicAdd(ws + 2, 1u);
   const bool listed = a.unit_list && idx < static_cast<uint32_t>(a.unit_list_cap);
-  if (listed) a.unit_list[idx] = static_cast<int32_t>(blockIdx.x);
+  if (listed) a.unit_list[idx] = unit;
   if (!listed || (out_of_range && a.domain_is_error)) atomicExch(ws + 1, 1u);
 }
 
@@ -307,14 +308,17 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   const int tid = threadIdx.x, warp = uni(tid >> 5), lane = tid & 31;
   const int h = blockIdx.x % a.H_v;
   const int lc = (blockIdx.x / a.H_v) % a.n_layers_in_call;
-  const int r = blockIdx.x / (a.H_v * a.n_layers_in_call);
+  stream_order_begin();
+  int r = blockIdx.x / (a.H_v * a.n_layers_in_call);
+  if (a.ordered) r = uni(static_cast<const uint8_t *>(a.workspace)[kRefreshWsOrder + r]);
+  const int unit = (r * a.n_layers_in_call + lc) * a.H_v + h;
   const int hk = h / (a.H_v / a.H_k);
   const int layer = a.layer_begin + lc;
   const int t_begin = uni(a.tok_begin ? a.tok_begin[r] : a.cu_seqlens[r]);
   const int n_tok = uni(a.cu_seqlens[r + 1] - t_begin);
   if (n_tok <= 0 && a.mode == DASC_REFRESH_CONTINUE) return;
   if (n_tok <= a.short_thr) {  // left to the exact kernel (short_thr = -1: never)
-    if (tid == 0) hand_over(a, false);
+    if (tid == 0) hand_over(a, unit, false);
     return;
   }
 
@@ -988,7 +992,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     // the bits it had before the call, so that it can be replayed by the exact kernel (or by the caller).
     const bool bad = misc->abort_flag != 0 || misc->domain_flag != 0;
     if (bad) {
-      if (tid == 0 && misc->abort_flag == 0) hand_over(a, true);
+      if (tid == 0 && misc->abort_flag == 0) hand_over(a, unit, true);
     } else {
       const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * D;
       const bool merge = a.mode != DASC_REFRESH_CONTINUE;
@@ -1016,6 +1020,47 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   if (tid == 0 && misc->abort_flag) atomicExch(static_cast<uint32_t *>(a.workspace), 1u);  // a wait ran out
 }
 
+// Blocks are placed in index order, so the requests are taken longest first: a long one started last would run on while
+// the rest of the GPU is idle.  64 requests of 1 .. 1023 tokens x 32 heads (2048 units, 296 resident): 635 -> 610 us on B200.
+// Ties keep their order; up to 240 requests (the table lives in the workspace header), beyond which the units far outnumber
+// the resident ones.
+bool ordered(const DascRefreshArgs &a) { return a.n_req > 1 && a.n_req <= kRefreshOrderMax; }
+
+constexpr int kPrepThreads = 256;
+static_assert(kPrepThreads >= kRefreshOrderMax);
+// One thread per request; block 0 also clears the header words and ranks the requests.
+__global__ void __launch_bounds__(kPrepThreads) refresh_prep_kernel(uint32_t *ws, const int32_t *cu, int32_t n_req, int32_t window,
+                                                                    int32_t *tok_begin, bool order) {
+  stream_order_begin();
+  const int r = blockIdx.x * kPrepThreads + threadIdx.x;
+  if (ws && r < 4) ws[r] = 0;
+  int len = -1;
+  if (r < n_req && (tok_begin || order)) {
+    const int lo = cu[r], hi = cu[r + 1];
+    len = hi - lo;
+    if (tok_begin) {
+      const int64_t b = static_cast<int64_t>(hi) - window;
+      const int first = b > lo ? static_cast<int>(b) : lo;
+      tok_begin[r] = first;
+      len = hi - first;
+    }
+  }
+  if (!order) return;  // (one block when there is an order)
+  __shared__ __align__(16) int lens[kPrepThreads];
+  lens[threadIdx.x] = len;
+  __syncthreads();
+  if (r < n_req) {
+    int rank = 0;
+    for (int j = 0; j < n_req; j += 4) {
+      const int4 l4 = *reinterpret_cast<const int4 *>(lens + j);  // entries past n_req are -1: they rank below
+      const int l[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) rank += l[i] > len || (l[i] == len && j + i < r);
+    }
+    reinterpret_cast<uint8_t *>(ws)[kRefreshWsOrder + rank] = static_cast<uint8_t>(r);
+  }
+}
+
 // cuTensorMapEncodeTiled is a driver entry point.  It is looked up through the runtime at first use, so that the library
 // has no link-time dependency on libcuda and still loads (plan building, accessors) on a machine without a driver.
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -1034,15 +1079,16 @@ EncodeTiledFn encode_tiled_fn() {
 }
 
 template <bool KDA, typename OT, bool WITH_O>
-int launch(const DascRefreshArgs &a, void *stream) {
+int launch(DascRefreshArgs a, void *stream) {
   auto kern = refresh_chunked_kernel<KDA, OT, WITH_O>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(SMEM_ALLOC));
   if (e != cudaSuccess) return static_cast<int>(e);
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
   if (n_units == 0) return cudaSuccess;
   if (n_units > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
-  e = cudaMemsetAsync(a.workspace, 0, 16, static_cast<cudaStream_t>(stream));  // clear the four header words
-  if (e != cudaSuccess) return static_cast<int>(e);
+  a.ordered = ordered(a);
+  const int prep = dasc_launch_refresh_prep(a, stream);
+  if (prep != 0) return prep;
   // tensor maps of the token streams [Lc*T tokens][heads][128]: boxes of 32 tokens x one head x 128 bytes of channels with
   // the 128-byte swizzle, which is the layout of one block of an operand tile
   CUtensorMap tmap_q{}, tmap_k{}, tmap_g{};
@@ -1061,11 +1107,17 @@ int launch(const DascRefreshArgs &a, void *stream) {
       (WITH_O && !make_map(&tmap_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.q, a.H_k, 2)) ||
       (KDA && !make_map(&tmap_g, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.g, a.H_v, 4)))
     return static_cast<int>(cudaErrorInvalidValue);
-  kern<<<static_cast<unsigned>(n_units), NT, SMEM_ALLOC, static_cast<cudaStream_t>(stream)>>>(a, tmap_q, tmap_k, tmap_g);
-  return static_cast<int>(cudaGetLastError());
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(n_units)), dim3(NT), SMEM_ALLOC, stream, a, tmap_q, tmap_k, tmap_g));
 }
 
 }  // namespace
+
+int dasc_launch_refresh_prep(const DascRefreshArgs &a, void *stream) {
+  const int blocks = a.window > 0 || a.tok_begin ? (a.n_req + kPrepThreads - 1) / kPrepThreads : 1;
+  return static_cast<int>(launch_in_order(refresh_prep_kernel, dim3(static_cast<unsigned>(blocks)), dim3(kPrepThreads), 0, stream,
+                                          static_cast<uint32_t *>(a.workspace), a.cu_seqlens, a.n_req, a.window, a.tok_begin,
+                                          a.ordered != 0));
+}
 
 // Scratch the chunked kernel needs: the 256-byte header (flags and counters) and one list entry per unit of the call.
 size_t dasc_refresh_chunked_workspace_bytes(int32_t n_req, int32_t n_layers_in_call, int32_t H_v) {

@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "dasc_internal.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -436,6 +437,7 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
 template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
 __global__ void __launch_bounds__(NCOL / COLS *SL + NHELP) refresh_seq_kernel(DascRefreshArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  stream_order_begin();
   constexpr int PARTS = DV / NCOL;
   if (!a.from_list) {
     seq_unit<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x) / PARTS, static_cast<int>(blockIdx.x) % PARTS, smem_raw);
@@ -465,8 +467,7 @@ int launch(const DascRefreshArgs &a, void *stream) {
   // a handed-over list is short (units outside the chunked kernel's range or below its length threshold): a grid
   // of a CTA per SM walks it, and costs next to nothing when the list is empty
   const int64_t grid = a.from_list ? (n_ctas < 148 ? n_ctas : 148) : n_ctas;
-  kern<<<static_cast<unsigned>(grid), NCOL / COLS * SL + NHELP, smem, static_cast<cudaStream_t>(stream)>>>(a);
-  return static_cast<int>(cudaGetLastError());
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(grid)), dim3(NCOL / COLS * SL + NHELP), smem, stream, a));
 }
 
 // Columns do not interact, so units that leave SMs idle are split by columns: parts of 8 (16 at d = 32) with 16 (8) lanes per
