@@ -286,6 +286,14 @@ __device__ __forceinline__ void take_a_rows(uint32_t taddr, int row0, const floa
   }
 }
 
+// (a, b) *= f on fp32 bit patterns
+__device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
+  float x, y;
+  unpack2(mul2(pack2(__uint_as_float(a), __uint_as_float(b)), f), x, y);
+  a = __float_as_uint(x);
+  b = __float_as_uint(y);
+}
+
 // WITH_O = false is the state-only variant (no outputs wanted): q is never read, the Qt rows, P and the
 // output product are left out.
 template <bool KDA, typename OT, bool WITH_O>
@@ -644,19 +652,25 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
           unsigned char *p = raw + (or0 ^ (j << 4)) + j * 128;
           kw[j] = *reinterpret_cast<const uint2 *>(p);
           if (WITH_O) qw[j] = *reinterpret_cast<const uint2 *>(p + OFF_RAW_Q);
-          if (j >= left) {
-            // the boxes reached past the request's last token and brought in other tokens' values (zeros past the end of
-            // the stream): those keys are cleared, so that what they hold cannot matter
-            kw[j] = make_uint2(0u, 0u);
-            if (!KDA) *reinterpret_cast<uint2 *>(p) = kw[j];
-          }
+        }
+        if (left < 4) {
+          // the boxes reached past the request's last token and brought in other tokens' values (zeros past the end of
+          // the stream): those keys are cleared, so that what they hold cannot matter
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (j >= left) {
+              kw[j] = make_uint2(0u, 0u);
+              if (!KDA) *reinterpret_cast<uint2 *>(raw + (or0 ^ (j << 4)) + j * 128) = kw[j];
+            }
         }
         if constexpr (KDA) {
           float4 g4[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            g4[j] = *reinterpret_cast<const float4 *>(smem + OFF_KH + (oh0 ^ (j << 4)) + j * 128);
-            if (j >= left) g4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int j = 0; j < 4; ++j) g4[j] = *reinterpret_cast<const float4 *>(smem + OFF_KH + (oh0 ^ (j << 4)) + j * 128);
+          if (left < 4) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (j >= left) g4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
           }
           // sums: this lane's total, the prefix over the four token groups of the warp (lanes 8 apart), the half's total
           float run0[4], tot[4];
@@ -818,9 +832,9 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 
       // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
       {
-        float2 f[8];
+        uint64_t f[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const float2 *>(fac_c + colh * 64 + 8 * i + 2 * tig);
+        for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const uint64_t *>(fac_c + colh * 64 + 8 * i + 2 * tig);
 #pragma unroll 1
         for (uint32_t hh = 0; hh < 2; ++hh) {  // lanes 0-15, 16-31 of the quadrant
           const uint32_t addr = tlane + (hh << 20) + COL_S + colh * 64;
@@ -829,10 +843,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
           tmem_ld_wait();
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            s[4 * i + 0] = __float_as_uint(__uint_as_float(s[4 * i + 0]) * f[i].x);
-            s[4 * i + 1] = __float_as_uint(__uint_as_float(s[4 * i + 1]) * f[i].y);
-            s[4 * i + 2] = __float_as_uint(__uint_as_float(s[4 * i + 2]) * f[i].x);
-            s[4 * i + 3] = __float_as_uint(__uint_as_float(s[4 * i + 3]) * f[i].y);
+            scale2(s[4 * i + 0], s[4 * i + 1], f[i]);
+            scale2(s[4 * i + 2], s[4 * i + 3], f[i]);
           }
           tmem_st_16x256b(addr, s);
         }
@@ -894,10 +906,11 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
             if constexpr (!KDA) e = *reinterpret_cast<const float2 *>(e1c_s + (ch & 3) * C + t);
             const float r0 = b2.x * (bf16lo(vv[i]) - e.x * __uint_as_float(x[2 * i]));
             const float r1 = b2.y * (bf16hi(vv[i]) - e.y * __uint_as_float(x[2 * i + 1]));
-            x[2 * i] = to_tf32(r0);
-            x[2 * i + 1] = to_tf32(r1);
-            lo[2 * i] = tf32_pre(r0 - __uint_as_float(x[2 * i]));
-            lo[2 * i + 1] = tf32_pre(r1 - __uint_as_float(x[2 * i + 1]));
+            // the high part is the value itself, which the tensor core truncates on reading; the low part the exact rest
+            x[2 * i] = __float_as_uint(r0);
+            x[2 * i + 1] = __float_as_uint(r1);
+            lo[2 * i] = tf32_pre(r0 - __uint_as_float(x[2 * i] & 0xFFFFE000u));
+            lo[2 * i + 1] = tf32_pre(r1 - __uint_as_float(x[2 * i + 1] & 0xFFFFE000u));
           }
           tmem_st_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
           tmem_st_16x256b(tlane + (hh << 20) + COL_AP + tb, lo);
