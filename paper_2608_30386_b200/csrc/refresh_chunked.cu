@@ -356,8 +356,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     mbar_init(&misc->rdy_t, 1);
     mbar_init(&misc->tp_free, NCH / 32);
     mbar_init(&misc->drain, 1);
-    mbar_init(&misc->g_full, 1);
-    mbar_init(&misc->kq_full, 1);
+    mbar_init(&misc->g_full, NP / 32);
+    mbar_init(&misc->kq_full, WITH_O ? NP / 32 : NP / 64);
     misc->abort_flag = 0;
     misc->domain_flag = 0;
     fence_mbar_init();
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     const int pw = warp - 8, ptid = tid - NCH;
     const int cq = lane & 7, tg = lane >> 3;
     const int c0 = pw * 32 + cq * 4;
-    // Inputs come by TMA a chunk ahead, one issuing thread, into tiles they will be overwritten with (KDA) or that are
+    // Inputs come by TMA a chunk ahead into tiles they will be overwritten with (KDA) or that are
     // operands as they are (GDN): shared memory holds no staging buffers, and no load or store instruction moves them.
     //   log-decay (KDA, the largest stream): four boxes of 32 tokens x 32 channels with the 128-byte swizzle, i.e. exactly
     //   the layout of the Kh tile, so that a lane finds the decay of its vectors where its Kh vectors go;
@@ -563,25 +563,25 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     //   the operand tile of MMA1 itself.
     constexpr uint32_t RAW_ROWS = KDA ? 32 : 64, OFF_RAW_Q = KDA ? 2 * 32 * 128 : 32 * 128;
     int g_issued = 0, kq_issued = 0;
+    // Each warp's first lane starts one box of each stream: a copy takes its issuing thread 200 to 300 cycles, and the warp that
+    // issued all of them arrived 800 cycles behind the others.
     auto stage_kq = [&](int ch) {
-      const uint32_t dst = sbase + (KDA ? OFF_KHT + (ch & 1) * (128 * 128) : OFF_KQ16);
+      if (!WITH_O && pw >= 2) return;
+      const uint32_t dst = sbase + (KDA ? OFF_KHT + (ch & 1) * (128 * 128) : OFF_KQ16) + (pw & 1) * (RAW_ROWS * 128);
       const int32_t z = static_cast<int32_t>(tok0 + ch * C);
-      mbar_expect_tx(&misc->kq_full, C * D * 2 * (WITH_O ? 2 : 1));
-#pragma unroll 1
-      for (int b = 0; b < 2; ++b) {
-        tma_load_3d(dst + b * (RAW_ROWS * 128), &tmap_k, b * 64, hk, z, &misc->kq_full);
-        if (WITH_O) tma_load_3d(dst + OFF_RAW_Q + b * (RAW_ROWS * 128), &tmap_q, b * 64, hk, z, &misc->kq_full);
-      }
+      mbar_expect_tx(&misc->kq_full, C * 128);
+      if (pw < 2)
+        tma_load_3d(dst, &tmap_k, pw * 64, hk, z, &misc->kq_full);
+      else
+        tma_load_3d(dst + OFF_RAW_Q, &tmap_q, (pw & 1) * 64, hk, z, &misc->kq_full);
       ++kq_issued;
     };
     auto stage_g = [&](int ch) {
-      mbar_expect_tx(&misc->g_full, C * D * 4);
-#pragma unroll 1
-      for (int blk = 0; blk < 4; ++blk)
-        tma_load_3d(sbase + OFF_KH + blk * (C * 128), &tmap_g, blk * 32, h, static_cast<int32_t>(tok0 + ch * C), &misc->g_full);
+      mbar_expect_tx(&misc->g_full, C * 128);
+      tma_load_3d(sbase + OFF_KH + pw * (C * 128), &tmap_g, pw * 32, h, static_cast<int32_t>(tok0 + ch * C), &misc->g_full);
       ++g_issued;
     };
-    if (ptid == 0 && n_chunks > 0) {
+    if (lane == 0 && n_chunks > 0) {
       if (KDA) stage_g(0);
       stage_kq(0);
     }
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       if (out_of_range && (KDA ? tg == 0 : lane == 0)) misc->domain_flag = 1;
       fence_smem_to_async();
       arrive_warp(&misc->rdy_prep, lane);  // -> MMA1
-      if (pw == 0 && ch + 1 < n_chunks) {
+      if (ch + 1 < n_chunks) {
         // The next raw k, q (KDA) land once MMA5 of the previous chunk has read the Kh tile of that parity; the next
         // log-decay (KDA) or k, q (GDN) once MMA1 of this chunk has read the tile they go to.
         if (KDA) {
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
     }
     // after a time-out the last copies may not have been waited for: they must have landed before the CTA leaves
-    if (ptid == 0 && misc->abort_flag) {
+    if (lane == 0 && misc->abort_flag) {
       if (g_issued > 0) mbar_wait_bounded(&misc->g_full, (g_issued - 1) & 1, kMaxPolls);
       if (kq_issued > 0) mbar_wait_bounded(&misc->kq_full, (kq_issued - 1) & 1, kMaxPolls);
     }
