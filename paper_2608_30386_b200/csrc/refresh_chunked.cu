@@ -347,8 +347,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     mbar_init(&misc->bar_o, 1);
     mbar_init(&misc->bar_s, 1);
     mbar_init(&misc->rdy_prep, NP / 32);
-    mbar_init(&misc->rdy_fac[0], NP / 32);
-    mbar_init(&misc->rdy_fac[1], NP / 32);
+    mbar_init(&misc->rdy_fac[0], KDA ? NP / 32 : 1);
+    mbar_init(&misc->rdy_fac[1], KDA ? NP / 32 : 1);
     mbar_init(&misc->rdy_state, NCH / 32);
     mbar_init(&misc->rdy_rhs, NCH / 32);
     mbar_init(&misc->rdy_u, NCH / 32);
@@ -514,33 +514,32 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         }
 #pragma unroll
         for (int rr = 0; rr < 16; ++rr) Xm[(b * 16 + rr) * LDX + b * 16 + cc] = xs[rr];
-      }
-      __syncwarp();
-      // off-diagonal block: X_10 = -X_11 (L_10 X_00); the product L_10 X_00 is parked in the unused block (0,1)
-      {
+        __syncwarp();
+        // off-diagonal block: X_10 = -X_11 (L_10 X_00); the product L_10 X_00 is parked in the unused block (0,1)
         float acc[2][4] = {};
         warp_mm_acc<true>(acc, LT + 16, Xm, lane);
         warp_mm_store(Xm + 16, acc, 1.f, lane);
-        __syncwarp();
-        float acc2[2][4] = {};
-        warp_mm_acc<false>(acc2, Xm + 16 * LDX + 16, Xm + 16, lane);
-        warp_mm_store(Xm + 16 * LDX, acc2, -1.f, lane);
+        // T -> tf32 operand tile, straight from the registers.  Its storage (shared with the P tile and the chain warps'
+        // output tile) is free once the chain warps have copied the previous chunk's outputs out.
+        if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
+#pragma unroll
+        for (int rr = 0; rr < 16; ++rr)
+          *reinterpret_cast<uint32_t *>(smem + OFF_TM + sw128_offset(32, b * 16 + rr, b * 16 + cc)) = tf32_pre(xs[rr]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          *reinterpret_cast<uint4 *>(smem + OFF_TM + sw128_offset(32, i * 8 + (lane >> 2), 16 + (lane & 3) * 4)) = make_uint4(0u, 0u, 0u, 0u);
       }
       __syncwarp();
-      // the T tile's storage (shared with the P tile and the chain warps' output tile) is free once the chain
-      // warps have copied the previous chunk's outputs out
-      if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
-      // T (lower triangle of X, unit diagonal) -> tf32 operand tile; lane = row
-      const int t = lane;
+      {
+        float acc2[2][4] = {};
+        warp_mm_acc<false>(acc2, Xm + 16 * LDX + 16, Xm + 16, lane);
+        const int g = lane >> 2, tig = lane & 3;
 #pragma unroll
-      for (int j = 0; j < 32; j += 4) {
-        const float4 xv = *reinterpret_cast<const float4 *>(Xm + t * LDX + j);
-        uint4 o;
-        o.x = (j + 0 <= t) ? tf32_pre(xv.x) : 0u;
-        o.y = (j + 1 <= t) ? tf32_pre(xv.y) : 0u;
-        o.z = (j + 2 <= t) ? tf32_pre(xv.z) : 0u;
-        o.w = (j + 3 <= t) ? tf32_pre(xv.w) : 0u;
-        *reinterpret_cast<uint4 *>(smem + OFF_TM + sw128_offset(32, t, j)) = o;
+        for (int nh = 0; nh < 2; ++nh) {
+          unsigned char *const p = smem + OFF_TM + sw128_offset(32, 16 + g, 8 * nh + 2 * tig);
+          *reinterpret_cast<uint2 *>(p) = make_uint2(tf32_pre(-acc2[nh][0]), tf32_pre(-acc2[nh][1]));
+          *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(tf32_pre(-acc2[nh][2]), tf32_pre(-acc2[nh][3]));
+        }
       }
       fence_smem_to_async();
       arrive_warp(&misc->rdy_t, lane);  // -> MMA3
@@ -585,56 +584,58 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       if (KDA) stage_g(0);
       stage_kq(0);
     }
-    float beta_next = (n_chunks > 0 && ptid < min(C, n_tok)) ? gb[ptid * b_stride] : 0.f;
-    float gsc_next = (!KDA && n_chunks > 0 && ptid < min(C, n_tok)) ? gg[ptid * g_stride] : 0.f;
-    float gsc_cur = 0.f, post_prev = 0.f;  // GDN, first producer warp: this chunk's log-decay, the factor owed by the previous chunk
+    // Per-token scalars, by the first warp (lane = token): a chunk's go to their ring slots (the chain warps are at most two
+    // chunks behind) while MMA1 of the chunk before runs; the next chunk's are fetched then and stored one chunk later.
+    const float *gbp = gb + static_cast<int64_t>(lane) * b_stride, *ggp = gg + static_cast<int64_t>(lane) * g_stride;
+    float beta_next = (n_chunks > 0 && ptid < min(C, n_tok)) ? *gbp : 0.f;
+    float gsc_next = (!KDA && n_chunks > 0 && ptid < min(C, n_tok)) ? *ggp : 0.f;
+    float post_prev = 0.f;  // GDN: the factor owed by the previous chunk
+    auto scalars = [&](int ch) {
+      const int slot = (ch & 3) * C + lane;
+      const float beta = beta_next;
+      beta_s[slot] = beta;
+      if constexpr (!KDA) {
+        // ---- GDN: one scalar log-decay per token: the running sums and the per-token factors are formed here; nothing per
+        // channel needs an exponential, and k, q stay exactly their bf16 values:
+        //   e1_t = exp(G_t - G_m), e2_t = exp(G_m - G_t) with m the end of the first half;
+        //   MMA1 works on raw k, q (bf16 tile), MMA2 on raw k, q widened to tf32 containers, MMA5 on k_t e2_t;
+        //   e1_t goes onto the rows of A, R and the outputs where they leave tensor memory, e2_j onto the columns of A, P.
+        float incl = gsc_next;
+#pragma unroll
+        for (int dlt = 1; dlt < 32; dlt <<= 1) {
+          const float x = __shfl_up_sync(0xffffffffu, incl, dlt);
+          if (lane >= dlt) incl += x;
+        }
+        const float tot0 = __shfl_sync(0xffffffffu, incl, 15);          // G_m: the first half's total
+        const float tot1 = __shfl_sync(0xffffffffu, incl, 31) - tot0;   // G_C - G_m
+        const float d2 = (incl - tot0) * LOG2E;
+        const float e1 = ex2f(d2), e2 = ex2f(-d2);
+        e1c_s[slot] = e1 * kTruncComp;
+        e2_s[slot] = e2;
+        bte1_s[slot] = beta * e1;
+        if (lane == 0 && (!(fabsf(tot0) <= kMaxHalfDecay) || !(fabsf(tot1) <= kMaxHalfDecay))) misc->domain_flag = 1;  // also true for NaN
+        // state factor from where the previous chunk left the state to this chunk's midpoint, and the factor owed after
+        // it; scalars here, written for every channel so that the chain warps read them as they do for KDA
+        const float f = ex2f((post_prev + tot0) * LOG2E);
+        post_prev = tot1;
+        *reinterpret_cast<float4 *>(fac_s + (ch & 1) * D + lane * 4) = make_float4(f, f, f, f);
+        *reinterpret_cast<float4 *>(post_s + (ch & 1) * D + lane * 4) = make_float4(tot1, tot1, tot1, tot1);
+        arrive_warp(&misc->rdy_fac[ch & 1], lane);
+      }
+      const bool v1 = lane < n_tok - (ch + 1) * C;
+      gbp += C * b_stride;
+      ggp += C * g_stride;
+      beta_next = v1 ? *gbp : 0.f;
+      if (!KDA) gsc_next = v1 ? *ggp : 0.f;
+    };
+    if (pw == 0 && n_chunks > 0) scalars(0);
     for (int ch = 0; ch < n_chunks; ++ch) {
       const uint32_t par = ch & 1;
       const int t0 = ch * C, ntok = min(C, n_tok - t0);
       unsigned char *kht_tile = smem + OFF_KHT + par * (128 * 128);
       unsigned char *raw = KDA ? kht_tile : smem + OFF_KQ16;
-      // per-token scalars: this chunk's go to their ring slots (the chain warps are at most two chunks behind),
-      // the next chunk's are fetched now and stored one iteration later
-      if (ptid < C) {
-        beta_s[(ch & 3) * C + ptid] = beta_next;
-        if (!KDA) gsc_cur = gsc_next;
-        const bool v1 = ch + 1 < n_chunks && ptid < min(C, n_tok - t0 - C);
-        beta_next = v1 ? gb[(t0 + C + ptid) * b_stride] : 0.f;
-        if (!KDA) gsc_next = v1 ? gg[(t0 + C + ptid) * g_stride] : 0.f;
-      }
+      if (!KDA) asm volatile("bar.sync 2, 128;" ::: "memory");   // the per-token factors are visible to all producer warps
       bool out_of_range = false;
-      if constexpr (!KDA) {
-        // ---- GDN: one scalar log-decay per token.  The first producer warp (lane = token) forms the running sums and
-        // the per-token factors; nothing per channel needs an exponential, and k, q stay exactly their bf16 values:
-        //   e1_t = exp(G_t - G_m), e2_t = exp(G_m - G_t) with m the end of the first half;
-        //   MMA1 works on raw k, q (bf16 tile), MMA2 on raw k, q widened to tf32 containers, MMA5 on k_t e2_t;
-        //   e1_t goes onto the rows of A, R and the outputs where they leave tensor memory, e2_j onto the columns of A, P.
-        if (ptid < C) {
-          const int slot = (ch & 3) * C + lane;
-          float incl = gsc_cur;
-#pragma unroll
-          for (int dlt = 1; dlt < 32; dlt <<= 1) {
-            const float x = __shfl_up_sync(0xffffffffu, incl, dlt);
-            if (lane >= dlt) incl += x;
-          }
-          const float tot0 = __shfl_sync(0xffffffffu, incl, 15);          // G_m: the first half's total
-          const float tot1 = __shfl_sync(0xffffffffu, incl, 31) - tot0;   // G_C - G_m
-          const float d2 = (incl - tot0) * LOG2E;
-          const float e1 = ex2f(d2), e2 = ex2f(-d2);
-          e1c_s[slot] = e1 * kTruncComp;
-          e2_s[slot] = e2;
-          bte1_s[slot] = beta_s[slot] * e1;
-          out_of_range = !(fabsf(tot0) <= kMaxHalfDecay) || !(fabsf(tot1) <= kMaxHalfDecay);   // also true for NaN
-          // state factor from where the previous chunk left the state to this chunk's midpoint, and the factor owed after
-          // it; scalars here, written for every channel so that the chain warps read them as they do for KDA
-          const float f = ex2f((post_prev + tot0) * LOG2E);
-          post_prev = tot1;
-          *reinterpret_cast<float4 *>(fac_s + par * D + lane * 4) = make_float4(f, f, f, f);
-          *reinterpret_cast<float4 *>(post_s + par * D + lane * 4) = make_float4(tot1, tot1, tot1, tot1);
-        }
-        arrive_warp(&misc->rdy_fac[par], lane);
-        asm volatile("bar.sync 2, 128;" ::: "memory");   // the factors are visible to all producer warps
-      }
       wait_bar(&misc->kq_full, par, misc);
       if (KDA) wait_bar(&misc->g_full, par, misc);
       const uint64_t l2e2 = pack2(LOG2E, LOG2E), comp2 = pack2(kLog2TruncComp, kLog2TruncComp);
@@ -758,10 +759,11 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         }
       }
       // the exponents of this chunk may have overflowed: the unit will not be written back
-      if (out_of_range && (KDA ? tg == 0 : lane == 0)) misc->domain_flag = 1;
+      if (KDA && out_of_range && tg == 0) misc->domain_flag = 1;
       fence_smem_to_async();
       arrive_warp(&misc->rdy_prep, lane);  // -> MMA1
       if (ch + 1 < n_chunks) {
+        if (pw == 0) scalars(ch + 1);
         // The next raw k, q (KDA) land once MMA5 of the previous chunk has read the Kh tile of that parity; the next
         // log-decay (KDA) or k, q (GDN) once MMA1 of this chunk has read the tile they go to.
         if (KDA) {
