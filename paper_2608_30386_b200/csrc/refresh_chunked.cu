@@ -58,7 +58,7 @@ constexpr uint32_t OFF_KHT = OFF_KQ + 4 * 64 * 128;     // [2][4][32 rows][128 B
 constexpr uint32_t OFF_KH = OFF_KHT + 2 * 128 * 128;    // [4][32 rows][128 B]  Kh[t][c]
 constexpr uint32_t OFF_TM = OFF_KH + 4 * 32 * 128;      // [1][32 rows][128 B]  T[t][i]; TM|PM later the bf16 O tile
 constexpr uint32_t OFF_PM = OFF_TM + 32 * 128;          // [1][32 rows][128 B]  P[t][i]
-constexpr uint32_t OFF_V = OFF_PM + 32 * 128;           // [32][128] bf16 v
+constexpr uint32_t OFF_V = OFF_PM + 32 * 128;           // [2][32 rows][128 B] V[t][v] bf16
 constexpr uint32_t OFF_L = OFF_V + C * D * 2;           // [32][LDX] fp32 A^T (entries on and above A's diagonal are not used)
 constexpr uint32_t OFF_X = OFF_L + C * LDX * 4;         // [32][LDX] fp32 X = (I + A)^-1
 constexpr uint32_t OFF_FAC = OFF_X + C * LDX * 4;       // [2][128] fp32 state factor per channel, by chunk parity
@@ -109,6 +109,8 @@ struct Misc {
   uint64_t drain;
   // TMA -> producer warps: the log-decay of a chunk has landed in the Kh tile (KDA); its raw k, q have landed
   uint64_t g_full, kq_full;
+  // TMA -> chain warps: V of a chunk has landed
+  uint64_t v_full;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;   // a bounded wait ran out: every later wait of this CTA returns at once
   volatile uint32_t domain_flag;  // a half-chunk decay sum left the range the midpoint factors can carry
@@ -119,11 +121,6 @@ __device__ __forceinline__ float ex2f(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-__device__ __forceinline__ void cp_async16_zfill(uint32_t smem, const void *gmem, bool valid) {
-  const uint32_t n = valid ? 16u : 0u;
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem), "l"(gmem), "r"(n) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
@@ -238,6 +235,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -299,6 +301,7 @@ __device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
 template <bool KDA, typename OT, bool WITH_O>
 __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
                                                                 const __grid_constant__ CUtensorMap tmap_k,
+                                                                const __grid_constant__ CUtensorMap tmap_v,
                                                                 const __grid_constant__ CUtensorMap tmap_g) {
   // The base is a link-time constant (there is no static shared memory), so every operand descriptor is an immediate.
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -357,6 +360,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     mbar_init(&misc->tp_free, NCH / 32);
     mbar_init(&misc->drain, 1);
     mbar_init(&misc->g_full, NP / 32);
+    mbar_init(&misc->v_full, 2);
     mbar_init(&misc->kq_full, WITH_O ? NP / 32 : NP / 64);
     misc->abort_flag = 0;
     misc->domain_flag = 0;
@@ -788,22 +792,17 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     const int vrow = quad * 32 + lane;                                     // the TMEM lane this thread owns
 
     const int g = lane >> 2, tig = lane & 3;
-    // V arrives by cp.async, zeros past the request's last token; 16-byte vector j of token t sits at j ^ (t & 7) (no bank
-    // conflicts for the 8 x 8 blocks it is read in)
-    const __nv_bfloat16 *gv = static_cast<const __nv_bfloat16 *>(a.v) + (tok0 * a.H_v + h) * D;
+    // V arrives by TMA a chunk ahead: two boxes of 32 tokens x 64 values with the 128-byte swizzle (no bank conflicts for the
+    // 8 x 8 blocks it is read in), started by one lane of the first two warps each.
+    int v_issued = 0;
     auto stage_v = [&](int ch) {
-      const int t0 = ch * C, ntok = min(C, n_tok - t0);
-      for (int i = tid; i < C * 16; i += NCH) {
-        const int t = i >> 4, j = i & 15;
-        const bool valid = t < ntok;
-        cp_async16_zfill(sbase + OFF_V + t * 256 + ((j ^ (t & 7)) << 4),
-                         reinterpret_cast<const char *>(gv + (t0 + (valid ? t : 0)) * v_stride) + j * 16, valid);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
+      mbar_expect_tx(&misc->v_full, C * 128);
+      tma_load_3d(sbase + OFF_V + warp * (C * 128), &tmap_v, warp * 64, h, static_cast<int32_t>(tok0 + ch * C), &misc->v_full);
+      ++v_issued;
     };
 
     if (n_chunks > 0) {
-      stage_v(0);
+      if (warp < 2 && lane == 0) stage_v(0);
       // the start state goes into TMEM as it is; the first chunk's state pass scales it like any other
 #pragma unroll 1
       for (int c0 = colh * 64; c0 < colh * 64 + 64; c0 += 32) {
@@ -858,16 +857,17 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       // ---- (3) P = lower_incl_diag(Qt Kh^T) out of TMEM (rows 0-15, 16-31 are in the third and fourth quadrant) straight to
       //          its operand tile.  GDN: the raw q_t . k_j gets its column factor e2_j here, the row factor e1_t is applied
       //          to the outputs ----
-      if (WITH_O && colh == 0 && quad >= 2) {
+      if (WITH_O && quad >= 2) {
         wait_bar(&misc->bar_ap, par, misc);
         tc_fence_after_sync();
-        uint32_t x[16];
-        tmem_ld_16x256b(tlane + COL_AP, x);
+        uint32_t x[8];
+        tmem_ld_16x256b(tlane + COL_AP + colh * 16, x);
+        if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc);  // the previous chunk's outputs have left this storage
         tmem_ld_wait();
         const int t = (quad - 2) * 16 + g;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int j = 8 * i + 2 * tig;
+        for (int i = 0; i < 2; ++i) {
+          const int j = colh * 16 + 8 * i + 2 * tig;
           float2 e = make_float2(kInvTruncComp, kInvTruncComp);
           if constexpr (!KDA) {
             const float2 e2 = *reinterpret_cast<const float2 *>(e2_s + (ch & 3) * C + j);
@@ -886,9 +886,10 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       // ---- (4) RHS^T = beta (V - R)^T as a tf32 pair: high over R^T, low in the consumed A|P columns ----
       wait_bar(&misc->bar_ro, par, misc);
       tc_fence_after_sync();
-      asm volatile("cp.async.wait_all;" ::: "memory");  // V of this chunk
-      wait_bar(&misc->a_taken, par, misc);         // the A|P columns are about to be overwritten
-      sync_chain();
+      // A's and P's columns are about to be overwritten: A's by warps that wait for its readers (the issuing warp read its rows
+      // before it issued MMA2), P's by the warps that read them
+      wait_bar(&misc->a_taken, par, misc);
+      wait_bar(&misc->v_full, par, misc);
       {
         const int tb = colh * 16;
         // blocks of one ldmatrix: tokens 0-7 of the half with values 0-7, 8-15, tokens 8-15 with the same
@@ -897,22 +898,33 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         for (uint32_t hh = 0; hh < 2; ++hh) {
           uint32_t x[8], lo[8], vv[4];
           tmem_ld_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
-          ldmatrix_x4_trans(vv, sbase + OFF_V + vt * 256 + (((quad * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (vt & 7)) << 4));
+          ldmatrix_x4_trans(vv, sbase + OFF_V + (quad >> 1) * (C * 128) + vt * 128 +
+                                    ((((quad & 1) * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (vt & 7)) << 4));
+          if (ntok < C) {
+            // the boxes reached past the request's last token: those values are other tokens' (zeros past the end of the stream)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int t = tb + (i >> 1) * 8 + 2 * tig;
+              if (t >= ntok) vv[i] = 0u;
+              else if (t + 1 >= ntok) vv[i] &= 0xFFFFu;
+            }
+          }
           tmem_ld_wait();
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int t = tb + (i >> 1) * 8 + 2 * tig;
-            const float2 b2 = *reinterpret_cast<const float2 *>(beta_c + t);
-            float2 e = make_float2(1.f, 1.f);
+            uint64_t r = pack2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
             // GDN: the product is k_t S' on the raw keys; its row factor e1_t (with the truncation compensation) comes here
-            if constexpr (!KDA) e = *reinterpret_cast<const float2 *>(e1c_s + (ch & 3) * C + t);
-            const float r0 = b2.x * (bf16lo(vv[i]) - e.x * __uint_as_float(x[2 * i]));
-            const float r1 = b2.y * (bf16hi(vv[i]) - e.y * __uint_as_float(x[2 * i + 1]));
+            if constexpr (!KDA) r = mul2(*reinterpret_cast<const uint64_t *>(e1c_s + (ch & 3) * C + t), r);
+            r = mul2(*reinterpret_cast<const uint64_t *>(beta_c + t), sub2(pack2(bf16lo(vv[i]), bf16hi(vv[i])), r));
             // the high part is the value itself, which the tensor core truncates on reading; the low part the exact rest
+            float r0, r1;
+            unpack2(r, r0, r1);
             x[2 * i] = __float_as_uint(r0);
             x[2 * i + 1] = __float_as_uint(r1);
-            lo[2 * i] = tf32_pre(r0 - __uint_as_float(x[2 * i] & 0xFFFFE000u));
-            lo[2 * i + 1] = tf32_pre(r1 - __uint_as_float(x[2 * i + 1] & 0xFFFFE000u));
+            unpack2(sub2(r, pack2(__uint_as_float(x[2 * i] & 0xFFFFE000u), __uint_as_float(x[2 * i + 1] & 0xFFFFE000u))), r0, r1);
+            lo[2 * i] = tf32_pre(r0);
+            lo[2 * i + 1] = tf32_pre(r1);
           }
           tmem_st_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
           tmem_st_16x256b(tlane + (hh << 20) + COL_AP + tb, lo);
@@ -921,8 +933,10 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
       tc_fence_before_sync();
       arrive_warp(&misc->rdy_rhs, lane);  // -> MMA3 (T tile and RHS^T are ready)
-      sync_chain();                 // everyone is done with V: the next chunk's V may land
-      if (more) stage_v(ch + 1);
+      if (warp < 2 && more) {  // V has been read by everyone: the next chunk's may land
+        wait_bar(&misc->rdy_rhs, par, misc);
+        if (lane == 0 && !misc->abort_flag) stage_v(ch + 1);
+      }
 
       // ---- (5) the part of U^T the tensor core drops when it reads it (the low 13 mantissa bits), written over
       //          the consumed RHS^T: U = U_hi + U_lo exactly ----
@@ -991,8 +1005,9 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
       tc_fence_before_sync();
       arrive_warp(&misc->tp_free, lane);  // this thread is done with the T|P|O tile region
-      sync_chain();  // every chain thread is done with this chunk's P and O tiles before they are rewritten
     }
+    // after a time-out the last copies of V may not have been waited for: they must have landed before the CTA leaves
+    if (misc->abort_flag && v_issued > 0) mbar_wait_bounded(&misc->v_full, (v_issued - 1) & 1, kMaxPolls);
 
     // ---- final state: the factor still owed, then write back ----
     if (n_chunks > 0) {
@@ -1106,7 +1121,7 @@ int launch(DascRefreshArgs a, void *stream) {
   if (prep != 0) return prep;
   // tensor maps of the token streams [Lc*T tokens][heads][128]: boxes of 32 tokens x one head x 128 bytes of channels with
   // the 128-byte swizzle, which is the layout of one block of an operand tile
-  CUtensorMap tmap_q{}, tmap_k{}, tmap_g{};
+  CUtensorMap tmap_q{}, tmap_k{}, tmap_v{}, tmap_g{};
   const EncodeTiledFn encode = encode_tiled_fn();
   if (!encode) return static_cast<int>(cudaErrorNotSupported);
   auto make_map = [&](CUtensorMap *m, CUtensorMapDataType type, const void *base, int heads, cuuint64_t esz) {
@@ -1118,11 +1133,11 @@ int launch(DascRefreshArgs a, void *stream) {
     return encode(m, type, 3, const_cast<void *>(base), dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   };
-  if (!make_map(&tmap_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.k, a.H_k, 2) ||
+  if (!make_map(&tmap_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.k, a.H_k, 2) || !make_map(&tmap_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.v, a.H_v, 2) ||
       (WITH_O && !make_map(&tmap_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.q, a.H_k, 2)) ||
       (KDA && !make_map(&tmap_g, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.g, a.H_v, 4)))
     return static_cast<int>(cudaErrorInvalidValue);
-  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(n_units)), dim3(NT), SMEM_ALLOC, stream, a, tmap_q, tmap_k, tmap_g));
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(n_units)), dim3(NT), SMEM_ALLOC, stream, a, tmap_q, tmap_k, tmap_v, tmap_g));
 }
 
 }  // namespace
