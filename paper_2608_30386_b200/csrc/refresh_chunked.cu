@@ -962,11 +962,13 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       if (WITH_O) {
         const int tb = colh * 16;
         const int ot = tb + (lane >> 4) * 8 + (lane & 7);  // blocks of one stmatrix: as for V
+        uint32_t xx[2][8];
+        tmem_ld_16x256b(tlane + COL_RO + 32 + tb, xx[0]);
+        tmem_ld_16x256b(tlane + (1u << 20) + COL_RO + 32 + tb, xx[1]);
+        tmem_ld_wait();
 #pragma unroll
         for (uint32_t hh = 0; hh < 2; ++hh) {
-          uint32_t x[8];
-          tmem_ld_16x256b(tlane + (hh << 20) + COL_RO + 32 + tb, x);
-          tmem_ld_wait();
+          uint32_t(&x)[8] = xx[hh];
           if constexpr (!KDA) {
             // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
             // the truncation compensation
@@ -996,10 +998,13 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         if constexpr (sizeof(OT) == 2) {
           // through shared memory (the T and P tiles are free now) so that global stores are 16 bytes wide
           sync_chain();
-          for (int i = tid; i < ntok * 16; i += NCH) {
-            const int t = i >> 4, j = i & 15;
-            *reinterpret_cast<uint4 *>(reinterpret_cast<char *>(go + (t0 + t) * v_stride) + j * 16) =
-                *reinterpret_cast<const uint4 *>(smem + OFF_TM + t * 256 + ((j ^ (t & 7)) << 4));
+          const int j = tid & 15;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int t = (tid >> 4) + 16 * i;
+            if (t < ntok)
+              *reinterpret_cast<uint4 *>(reinterpret_cast<char *>(go + (t0 + t) * v_stride) + j * 16) =
+                  *reinterpret_cast<const uint4 *>(smem + OFF_TM + t * 256 + ((j ^ (t & 7)) << 4));
           }
         }
       }
