@@ -14,13 +14,20 @@
 // temporal state (Section 4.1, B_conv of Eq. 6).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "dasc_internal.h"
 #include "launch.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;  // threads per block and loads in flight per thread: the best of a measured sweep
-constexpr int kUnroll = 4;     // over {128..1024} x {2..16}
+constexpr int kUnroll = 4;     // over {128..1024} x {1..16}
+// Loads in flight per thread when `blocks` (of kUnroll loads per thread) are few: eight blocks are resident on an SM, and a grid
+// that leaves most of that unused moves its bytes faster with more threads and fewer loads each.  B200, one checkpoint of
+// 24 layers x 8 heads: store (312 blocks) 4.9 / 3.8 / 3.1 us with 4 / 2 / 1, load (768 blocks) 5.8 / 4.8 / 5.1 us; 32 heads: store
+// (1176 blocks) 6.9 / 7.9 / 8.2 us.
+int unroll_for(uint64_t blocks) { return blocks <= 4 * 148 ? 1 : blocks <= 6 * 148 ? 2 : kUnroll; }
 
 enum class Layout { Ragged, Padded, TpBalanced };
 
@@ -60,11 +67,11 @@ __device__ __forceinline__ uint4 *tp_address(const TpPools &tp, int64_t slot, in
   return tp.base[owner] + slot * slot_stride4 + static_cast<int64_t>(local) * tp.unit_vecs + in_unit;
 }
 
-// grid = (ceil(R_max * vecs_per_unit / (kThreads*kUnroll)), n_layers, pairs).  A "vec" is 16 bytes of a row.  One
+// grid = (ceil(R_max * vecs_per_unit / (kThreads*UNROLL)), n_layers, pairs).  A "vec" is 16 bytes of a row.  One
 // layer per block row: the layer's first packed row and its count are per-block constants, the source address
 // needs the dense row only, and a block past its layer's count leaves at once.
 // pool_stride4: vectors between slots (Ragged, TpBalanced) or between (layer, slot) entries (Padded).
-template <Layout LAYOUT>
+template <Layout LAYOUT, int UNROLL>
 __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restrict__ state, int64_t layer_stride4,
                                                            int64_t req_stride4, const int32_t *__restrict__ src_req,
                                                            uint4 *__restrict__ pool, int64_t pool_stride4,
@@ -74,11 +81,11 @@ __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restri
                                                            uint32_t vecs_per_row, int32_t n_pairs,
                                                            const __grid_constant__ TpPools tp) {
   stream_order_begin();
-  const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
+  const uint32_t base = blockIdx.x * (kThreads * UNROLL) + threadIdx.x;
   const int32_t layer = blockIdx.y;
   const uint32_t first = static_cast<uint32_t>(__ldg(layer_row_off + layer));
   const uint32_t layer_vecs = (static_cast<uint32_t>(__ldg(layer_row_off + layer + 1)) - first) * vecs_per_row;
-  if (blockIdx.x * (kThreads * kUnroll) >= layer_vecs) return;
+  if (blockIdx.x * (kThreads * UNROLL) >= layer_vecs) return;
   const int2 *src_l = reinterpret_cast<const int2 *>(row_src) + first;  // {layer, dense row} of the layer's packed rows
   for (int32_t pair = blockIdx.z; pair < n_pairs; pair += gridDim.z) {
     const uint4 *src_base = state + static_cast<int64_t>(__ldg(src_req + pair)) * req_stride4 + layer * layer_stride4;
@@ -86,9 +93,9 @@ __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restri
     uint4 *dst_base = nullptr;
     if (LAYOUT == Layout::Ragged) dst_base = pool + slot * pool_stride4 + static_cast<int64_t>(first) * vecs_per_row;
     if (LAYOUT == Layout::Padded) dst_base = pool + (layer * n_slots + slot) * pool_stride4;
-    uint4 val[kUnroll];
+    uint4 val[UNROLL];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
+    for (int u = 0; u < UNROLL; ++u) {
       const uint32_t i = base + u * kThreads;
       if (i < layer_vecs) {
         const uint32_t row = i / vecs_per_row;
@@ -97,7 +104,7 @@ __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restri
       }
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
+    for (int u = 0; u < UNROLL; ++u) {
       const uint32_t i = base + u * kThreads;
       if (i < layer_vecs) {
         if (LAYOUT == Layout::TpBalanced)
@@ -109,8 +116,8 @@ __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restri
   }
 }
 
-// grid = (ceil(layer_vecs / (kThreads*kUnroll)), n_layers, pairs).
-template <Layout LAYOUT>
+// grid = (ceil(layer_vecs / (kThreads*UNROLL)), n_layers, pairs).
+template <Layout LAYOUT, int UNROLL>
 __global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restrict__ pool, int64_t pool_stride4,
                                                            int64_t n_slots, const int32_t *__restrict__ src_slot,
                                                            uint4 *__restrict__ state, int64_t layer_stride4,
@@ -121,7 +128,7 @@ __global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restri
                                                            uint32_t vecs_per_row, int32_t n_pairs,
                                                            const __grid_constant__ TpPools tp) {
   stream_order_begin();
-  const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
+  const uint32_t base = blockIdx.x * (kThreads * UNROLL) + threadIdx.x;
   const int32_t layer = blockIdx.y;
   const int32_t *pos_l = row_pos + static_cast<int64_t>(layer) * rows_per_layer;
   // Padded: packed row of the layer's first retained row (positions inside an entry count from it)
@@ -132,9 +139,9 @@ __global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restri
     if (LAYOUT == Layout::Ragged) src_base = pool + slot * pool_stride4;
     if (LAYOUT == Layout::Padded) src_base = pool + (layer * n_slots + slot) * pool_stride4;
     uint4 *dst_base = state + static_cast<int64_t>(__ldg(dst_req + pair)) * req_stride4 + layer * layer_stride4;
-    uint4 val[kUnroll];
+    uint4 val[UNROLL];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
+    for (int u = 0; u < UNROLL; ++u) {
       const uint32_t i = base + u * kThreads;
       val[u] = make_uint4(0u, 0u, 0u, 0u);  // omitted rows: +0.0f
       if (i < layer_vecs) {
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restri
       }
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
+    for (int u = 0; u < UNROLL; ++u) {
       const uint32_t i = base + u * kThreads;
       if (i < layer_vecs) st_stream(dst_base + i, val[u]);
     }
@@ -204,10 +211,22 @@ TpPools make_tp(const DascTpPlacement *p, int64_t unit_floats) {
   return tp;
 }
 
-dim3 copy_grid(uint64_t vecs_per_layer, const dasc_plan_s *plan, int32_t n_pairs) {
-  const uint32_t per_block = kThreads * kUnroll;
+dim3 copy_grid(uint64_t vecs_per_layer, const dasc_plan_s *plan, int32_t n_pairs, int *unroll) {
+  const uint64_t rows = static_cast<uint64_t>(plan->info.n_layers) * (n_pairs < 65535 ? n_pairs : 65535);
+  *unroll = unroll_for((vecs_per_layer + kThreads * kUnroll - 1) / (kThreads * kUnroll) * rows);
+  const uint32_t per_block = kThreads * *unroll;
   return dim3(static_cast<uint32_t>((vecs_per_layer + per_block - 1) / per_block), static_cast<uint32_t>(plan->info.n_layers),
               static_cast<uint32_t>(n_pairs < 65535 ? n_pairs : 65535));
+}
+
+// f(std::integral_constant) of the number of loads in flight
+template <typename F>
+cudaError_t with_unroll(int unroll, F &&f) {
+  switch (unroll) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    default: return f(std::integral_constant<int, kUnroll>{});
+  }
 }
 
 }  // namespace
@@ -221,7 +240,8 @@ int dasc_launch_pack(const dasc_plan_s *plan, const float *state, int64_t layer_
   if (plan->packed_rows == 0 || n_pairs == 0) return cudaSuccess;
   const int64_t rows_per_unit = plan->info.unit_floats / plan->info.d_v;
   const int64_t entry_stride4 = plan->info.r_max * rows_per_unit * vpr;  // vectors of the fullest layer
-  const dim3 grid = copy_grid(static_cast<uint64_t>(entry_stride4), plan, n_pairs);
+  int unroll;
+  const dim3 grid = copy_grid(static_cast<uint64_t>(entry_stride4), plan, n_pairs, &unroll);
   const TpPools tp = make_tp(placement, plan->info.unit_floats);
   const uint4 *st = reinterpret_cast<const uint4 *>(state);
   uint4 *pl = reinterpret_cast<uint4 *>(pool);
@@ -229,14 +249,12 @@ int dasc_launch_pack(const dasc_plan_s *plan, const float *state, int64_t layer_
     return launch_in_order(kernel, grid, dim3(kThreads), 0, stream, st, layer_stride / 4, req_stride / 4, src_req, dst, dst_stride4,
                            slots, dst_slot, plan->d_row_src, plan->d_layer_row_off, vpr, n_pairs, tp);
   };
-  cudaError_t e;
-  if (layout == 0)
-    e = launch(pack_kernel<Layout::Ragged>, pl, pool_stride / 4, 0);
-  else if (layout == 1)
-    e = launch(pack_kernel<Layout::Padded>, pl, entry_stride4, n_slots);
-  else
-    e = launch(pack_kernel<Layout::TpBalanced>, nullptr, pool_stride / 4, 0);
-  return static_cast<int>(e);
+  return static_cast<int>(with_unroll(unroll, [&](auto u) {
+    constexpr int U = decltype(u)::value;
+    if (layout == 0) return launch(pack_kernel<Layout::Ragged, U>, pl, pool_stride / 4, 0);
+    if (layout == 1) return launch(pack_kernel<Layout::Padded, U>, pl, entry_stride4, n_slots);
+    return launch(pack_kernel<Layout::TpBalanced, U>, nullptr, pool_stride / 4, 0);
+  }));
 }
 
 int dasc_launch_restore(const dasc_plan_s *plan, const float *pool, int64_t pool_stride, int64_t n_slots,
@@ -248,7 +266,8 @@ int dasc_launch_restore(const dasc_plan_s *plan, const float *pool, int64_t pool
   if (n_pairs == 0) return cudaSuccess;
   const int64_t rows_per_unit = plan->info.unit_floats / plan->info.d_v;
   const int64_t entry_stride4 = plan->info.r_max * rows_per_unit * vpr;
-  const dim3 grid = copy_grid(layer_vecs, plan, n_pairs);
+  int unroll;
+  const dim3 grid = copy_grid(layer_vecs, plan, n_pairs, &unroll);
   const TpPools tp = make_tp(placement, plan->info.unit_floats);
   const uint4 *pl = reinterpret_cast<const uint4 *>(pool);
   uint4 *st = reinterpret_cast<uint4 *>(state);
@@ -257,14 +276,12 @@ int dasc_launch_restore(const dasc_plan_s *plan, const float *pool, int64_t pool
     return launch_in_order(kernel, grid, dim3(kThreads), 0, stream, src, src_stride4, slots, src_slot, st, layer_stride / 4, req_stride / 4,
                            dst_req, plan->d_row_pos, plan->d_layer_row_off, lv, rpl, vpr, n_pairs, tp);
   };
-  cudaError_t e;
-  if (layout == 0)
-    e = launch(restore_kernel<Layout::Ragged>, pl, pool_stride / 4, 0);
-  else if (layout == 1)
-    e = launch(restore_kernel<Layout::Padded>, pl, entry_stride4, n_slots);
-  else
-    e = launch(restore_kernel<Layout::TpBalanced>, nullptr, pool_stride / 4, 0);
-  return static_cast<int>(e);
+  return static_cast<int>(with_unroll(unroll, [&](auto u) {
+    constexpr int U = decltype(u)::value;
+    if (layout == 0) return launch(restore_kernel<Layout::Ragged, U>, pl, pool_stride / 4, 0);
+    if (layout == 1) return launch(restore_kernel<Layout::Padded, U>, pl, entry_stride4, n_slots);
+    return launch(restore_kernel<Layout::TpBalanced, U>, nullptr, pool_stride / 4, 0);
+  }));
 }
 
 int dasc_launch_blob_copy(const void *src, int64_t src_stride_bytes, const int32_t *src_idx, void *dst,
