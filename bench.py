@@ -40,8 +40,8 @@ import torch  # noqa: E402
 D = 128
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 TF32_OVER_BF16 = 0.489        # nominal dense 1.1 : 2.25
-CHUNKED_FLOPS_PER_TOKEN_HEAD = 196608   # tf32 flops the chunked kernel issues per (token, head): 32-token chunks,
-                                        # MMA1 padded to M = 128, hi/lo pairs in MMA3, MMA4 and MMA5
+CHUNKED_FLOPS_PER_TOKEN_HEAD = 180224   # tf32 flops the chunked kernel issues per (token, head): 32-token chunks,
+                                        # hi/lo pairs in MMA3, MMA4 and MMA5
 
 # Traffic of a launch over its algorithmic bytes, from one ncu capture of the KDA serving workload at 8 requests and a
 # 128-token suffix (a full-size launch is too large to capture; every request and token moves the same bytes, so traffic
@@ -639,9 +639,9 @@ def main():
         "window_refresh_state_only": {"ms": t_window, "tokens_per_s": world * N_REQ * SUFFIX / (t_window * 1e-3),
                                       "token_heads_per_s": world * token_heads / (t_window * 1e-3)},
         "roofline": roofline, "roofline_by_kernel": rl, "clocks": clocks,
-        # per step: pack, restore, and per layer group the tensor-core refresh kernel + the exact kernel's pass over
-        # the units handed to it (AUTO); a single refresh kernel per group when an algorithm is forced
-        "gpu_launches": (2 + n_groups * (2 if args.algo == "auto" else 1)) * args.steps,
+        # per step: pack, restore, and per layer group the refresh kernel, in front of the tensor-core one a small kernel
+        # that readies its workspace, and under AUTO the exact kernel's pass over the units handed to it
+        "gpu_launches": (2 + n_groups * {"auto": 3, "chunked": 2, "sequential": 1}[args.algo]) * args.steps,
     }
     if tp:
         line["tp_placement"] = tp
@@ -727,7 +727,7 @@ def run_mixed_trace(args, c):
         for gi in range(L // group):       # the streams hold t_max tokens per layer; the call sees this round's first T
             dasc.dasc_refresh(plan, active, ls, rs, ids[:n], q, k, v, g, beta, cu, t_max, longest,
                               layer_begin=gi * group, layer_end=(gi + 1) * group, o=o, workspace=ws, stream=s_load)
-            launches += 2
+            launches += 3
 
     def replay(overlap):
         ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)

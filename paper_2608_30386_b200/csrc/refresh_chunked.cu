@@ -11,22 +11,30 @@
 //   S_C  = Diag(exp(G_C - G_m)) (S' + Kh^T U)
 //
 // Roles.  The operand tiles Kt, Qt, Kh depend on the token inputs only, not on the state, so they
-// are built one chunk ahead by four PRODUCER warps; their inputs land in the tiles they become (the
-// KDA log-decay by TMA, k and q by cp.async), off the critical path.  One TRIANGULAR warp forms
-// T = (I + A)^-1, also state-independent.  Eight CHAIN warps carry the state-dependent sequence:
-// state rescale -> right-hand side -> deltas -> outputs.  One warp issues all tensor-core work.
-// The groups meet only at mbarriers.  GDN (one scalar log-decay per token) keeps the decay out of
-// the products: MMA1 and MMA2 run on the raw k, q and the per-token factors are applied where A, P,
-// k S' and the outputs leave tensor memory.
-//   MMA1  [Kt;Qt] Kh^T            -> A (lanes 0-31) and P (lanes 32-63)         smem x smem
+// are built by four PRODUCER warps while the chunk before is in flight; their inputs come by TMA into the
+// tiles they become.  One TRIANGULAR warp forms T = (I + A)^-1, also state-independent.  Eight CHAIN warps
+// carry the state-dependent sequence: state rescale -> right-hand side -> deltas -> outputs.  One warp
+// issues all tensor-core work.  The groups meet only at mbarriers.  GDN (one scalar log-decay per token)
+// keeps the decay out of the products: MMA1 and MMA2 run on the raw k, q and the per-token factors are
+// applied where A, P, k S' and the outputs leave tensor memory.
+//   MMA1  [Kt;Qt] Kh^T            -> A (first two TMEM quadrants, 16 rows each), P (last two)   smem x smem, M = 64
 //   MMA2  S'^T [Kt;Qt]^T          -> R^T | (Qt S')^T                            tmem x smem
 //   MMA3  RHS^T T^T               -> U^T      (RHS as a tf32 high/low pair)     tmem x smem
 //   MMA4  (Qt S')^T += U^T P^T    -> O^T                                         tmem x smem
 //   MMA5  S'^T      += U^T Kh     -> state    (U as a tf32 high/low pair)       tmem x smem
-// Buffers: the Kt/Qt and Kh tiles of chunk n+1 may be written once MMA2 of chunk n has completed
-// (MMA1 and MMA2 are their only readers); MMA5 contracts over the tokens and reads Kh as an MN-major
-// operand from a second tile (tf32 MN-major operands have a swizzle of their own), which, read last,
-// is double-buffered by chunk parity.
+// Buffers: the Kt/Qt tile of chunk n+1 may be written once MMA2 of chunk n has completed, the Kh tile once its
+// MMA1 has; MMA5 contracts over the tokens and reads Kh as an MN-major operand from a second tile (tf32
+// MN-major operands have a swizzle of their own), which, read last, is double-buffered by chunk parity.
+//
+// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1090 us = 1.92 G token-heads/s = 60 % of the
+// floor set by its bytes, GDN 885 us = 2.37 G (46 %); 1685 and 1630 us in the form this one grew from.  No unit of the SM is at
+// its limit: per chunk and SM 4.7 k cycles, of which the shared-memory data pipe (load/store units and the tensor core's
+// operand reads together) is busy 70 %, the issue slots 48 %, the tensor pipe 33 %.  A CTA alone on its SM takes as long per
+// chunk as two CTAs take for one each: by itself it is bound by its chain of hand-offs, two of them by sharing the above.
+// What it was before, in the order in which it was found: 103 cycles of issue per tensor-core instruction (behind
+// `lane == 0` instead of an elected lane), 119 KB of code in the instruction caches (now 56 KB), and 85 % of the
+// shared-memory pipe (8-byte accesses in 16-byte places, A padded to 128 rows, V and O value by value).
+// Under sustained load the part is at its 1000 W limit and runs this kernel at 1.7 instead of 1.965 GHz.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
