@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     auto scalars = [&](int ch) {
       const int slot = (ch & 3) * C + lane;
       const float beta = beta_next;
-      beta_s[slot] = KDA ? beta * kTruncComp : beta;  // KDA: see Kh below
+      beta_s[slot] = beta;
       if constexpr (!KDA) {
         // ---- GDN: one scalar log-decay per token: the running sums and the per-token factors are formed here; nothing per
         // channel needs an exponential, and k, q stay exactly their bf16 values:
@@ -659,7 +659,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       bool out_of_range = false;
       wait_bar(&misc->kq_full, par, misc);
       if (KDA) wait_bar(&misc->g_full, par, misc);
-      const uint64_t l2e2 = pack2(LOG2E, LOG2E);
+      const uint64_t l2e2 = pack2(LOG2E, LOG2E), comp2 = pack2(kLog2TruncComp, kLog2TruncComp);
+      const uint64_t qs2 = pack2(a.q_scale, a.q_scale);
 #pragma unroll 1
       for (int half = 0; half < 2; ++half) {
         const int tr = half * 16 + tg * 4;
@@ -708,10 +709,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
             tot[i] = __shfl_sync(0xffffffffu, incl, cq + 24);    // the half's total
             out_of_range |= !(fabsf(tot[i]) <= kMaxHalfDecay);   // also true for NaN
           }
-          // Minus the midpoint reference, in log2 units, and the truncation compensation of Kt and Qt.  With one exponent for both
-          // signs Kh comes out smaller by the same factor; beta, and with it U, is larger by it, so Kh^T U is not touched, and A
-          // and P are scaled back where they leave tensor memory.
-          uint64_t ref01 = pack2(kLog2TruncComp, kLog2TruncComp), ref23 = ref01;
+          uint64_t ref01 = 0ull, ref23 = 0ull;  // minus the midpoint reference, in log2 units
           if (half == 0) {
             // The factor that takes the state from where the previous chunk left it to this chunk's midpoint needs
             // the first half's sums only: it is handed to the chain warps before the tiles are built.
@@ -722,8 +720,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
                               ex2f((pp.w + tot[3]) * LOG2E));
             }
             arrive_warp(&misc->rdy_fac[par], lane);
-            ref01 = pack2(fmaf(-tot[0], LOG2E, kLog2TruncComp), fmaf(-tot[1], LOG2E, kLog2TruncComp));
-            ref23 = pack2(fmaf(-tot[2], LOG2E, kLog2TruncComp), fmaf(-tot[3], LOG2E, kLog2TruncComp));
+            ref01 = pack2(-tot[0] * LOG2E, -tot[1] * LOG2E);
+            ref23 = pack2(-tot[2] * LOG2E, -tot[3] * LOG2E);
           } else if (tg == 0) {
             *reinterpret_cast<float4 *>(post_s + par * D + c0) = make_float4(tot[0], tot[1], tot[2], tot[3]);  // G_C - G_m
           }
@@ -737,10 +735,12 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
             run01 = add2(run01, pack2(g4[j].x, g4[j].y));
             run23 = add2(run23, pack2(g4[j].z, g4[j].w));
             const uint64_t d01 = fma2(run01, l2e2, ref01), d23 = fma2(run23, l2e2, ref23);  // (G_t - G_m) log2(e)
-            float d[4];
+            float d[4], dc[4];
             unpack2(d01, d[0], d[1]);
             unpack2(d23, d[2], d[3]);
-            const uint64_t e1_01 = pack2(ex2f(d[0]), ex2f(d[1])), e1_23 = pack2(ex2f(d[2]), ex2f(d[3]));
+            unpack2(add2(d01, comp2), dc[0], dc[1]);
+            unpack2(add2(d23, comp2), dc[2], dc[3]);
+            const uint64_t e1_01 = pack2(ex2f(dc[0]), ex2f(dc[1])), e1_23 = pack2(ex2f(dc[2]), ex2f(dc[3]));
             const uint64_t e2_01 = pack2(ex2f(-d[0]), ex2f(-d[1])), e2_23 = pack2(ex2f(-d[2]), ex2f(-d[3]));
             float kt[4], kh[4];
             unpack2(mul2(k01, e1_01), kt[0], kt[1]);
@@ -751,8 +751,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
             if (WITH_O) {
               const uint64_t q01 = pack2(bf16lo(qw[j].x), bf16hi(qw[j].x)), q23 = pack2(bf16lo(qw[j].y), bf16hi(qw[j].y));
               float qt[4];
-              unpack2(mul2(q01, e1_01), qt[0], qt[1]);
-              unpack2(mul2(q23, e1_23), qt[2], qt[3]);
+              unpack2(mul2(q01, mul2(e1_01, qs2)), qt[0], qt[1]);
+              unpack2(mul2(q23, mul2(e1_23, qs2)), qt[2], qt[3]);
               *reinterpret_cast<uint4 *>(pk + 32 * 128) = make_uint4(tf32_pre(qt[0]), tf32_pre(qt[1]), tf32_pre(qt[2]), tf32_pre(qt[3]));
             }
             *reinterpret_cast<uint4 *>(pk) = make_uint4(tf32_pre(kt[0]), tf32_pre(kt[1]), tf32_pre(kt[2]), tf32_pre(kt[3]));
@@ -986,13 +986,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 #pragma unroll
         for (uint32_t hh = 0; hh < 2; ++hh) {
           uint32_t(&x)[8] = xx[hh];
-          if constexpr (KDA) {
-            if (a.q_scale != 1.f) {
-              const uint64_t f = pack2(a.q_scale, a.q_scale);
-#pragma unroll
-              for (int i = 0; i < 8; i += 2) scale2(x[i], x[i + 1], f);
-            }
-          } else {
+          if constexpr (!KDA) {
             // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
             // the truncation compensation
 #pragma unroll
