@@ -26,8 +26,8 @@
 // MMA1 has; MMA5 contracts over the tokens and reads Kh as an MN-major operand from a second tile (tf32
 // MN-major operands have a swizzle of their own), which, read last, is double-buffered by chunk parity.
 //
-// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1086 us = 1.93 G token-heads/s = 61 % of the
-// floor set by its bytes, GDN 839 us = 2.50 G (49 %); 1685 and 1630 us in the form this one grew from.  No unit of the SM is at
+// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1090 us = 1.92 G token-heads/s = 60 % of the
+// floor set by its bytes, GDN 885 us = 2.37 G (46 %); 1685 and 1630 us in the form this one grew from.  No unit of the SM is at
 // its limit: per chunk and SM 4.7 k cycles, of which the shared-memory data pipe (load/store units and the tensor core's
 // operand reads together) is busy 70 %, the issue slots 48 %, the tensor pipe 33 %.  A CTA alone on its SM takes as long per
 // chunk as two CTAs take for one each: by itself it is bound by its chain of hand-offs, two of them by sharing the above.
@@ -85,18 +85,15 @@ static_assert(SMEM_ALLOC <= 113 * 1024, "two CTAs per SM");
 
 constexpr uint32_t kMaxPolls = 1u << 22;
 
-// Largest |sum of the log-decay over half a chunk| per channel for which every factor formed relative to the chunk
-// midpoint stays a normal fp32 number with room for the products that follow.
-constexpr float kMaxHalfDecay = 80.f;
-
-// GDN: largest |log| by which the state in tensor memory may differ from the true one inside a chunk (scalars() below).
-constexpr float kKeepScale = 40.f;
-
 // The tensor core reads the fp32 state as tf32 by dropping its low 13 mantissa bits, i.e. rounding
 // towards zero: on average the operand is 2^-11 * E[1/m] = 3.52e-4 too small in magnitude (m the
 // significand, log-uniform in [1, 2)).  The rows of Kt and Qt, the only partners of that operand,
 // are scaled up by this factor to cancel the bias; A and P, which also come from those rows, are
 // scaled back down when they are taken out of TMEM.
+// Largest |sum of the log-decay over half a chunk| per channel for which every factor formed relative to the chunk
+// midpoint stays a normal fp32 number with room for the products that follow.
+constexpr float kMaxHalfDecay = 80.f;
+
 constexpr float kTruncComp = 1.000352f;
 constexpr float kInvTruncComp = 1.0f / kTruncComp;
 constexpr float kLog2TruncComp = 5.0774e-4f;  // log2(kTruncComp)
@@ -612,7 +609,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       if constexpr (!KDA) {
         // ---- GDN: one scalar log-decay per token: the running sums and the per-token factors are formed here; nothing per
         // channel needs an exponential, and k, q stay exactly their bf16 values:
-        //   e1_t = exp(G_t - G_ref), e2_t = exp(G_ref - G_t), the reference the end of the first half or one kept from before;
+        //   e1_t = exp(G_t - G_m), e2_t = exp(G_m - G_t) with m the end of the first half;
         //   MMA1 works on raw k, q (bf16 tile), MMA2 on raw k, q widened to tf32 containers, MMA5 on k_t e2_t;
         //   e1_t goes onto the rows of A, R and the outputs where they leave tensor memory, e2_j onto the columns of A, P.
         float incl = gsc_next;
@@ -623,13 +620,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         }
         const float tot0 = __shfl_sync(0xffffffffu, incl, 15);          // G_m: the first half's total
         const float tot1 = __shfl_sync(0xffffffffu, incl, 31) - tot0;   // G_C - G_m
-        // The state in tensor memory is the true one times exp(-post_prev).  As long as the exponents relative to that scale stay
-        // small it is kept, and the chain warps skip their state pass; else the scale moves to this chunk's midpoint.  Half of the
-        // decay profiles in use lose less than e^-1 per chunk, so the pass is rare (887 -> 839 us on B200 for
-        // 64 requests x 256 tokens x 4 layers).
-        const float end = post_prev + tot0 + tot1;
-        const bool keep_scale = fabsf(post_prev) <= kKeepScale && fabsf(post_prev + tot0) <= kKeepScale && fabsf(end) <= kKeepScale;
-        const float d2 = (incl + (keep_scale ? post_prev : -tot0)) * LOG2E;
+        const float d2 = (incl - tot0) * LOG2E;
         const float e1 = ex2f(d2), e2 = ex2f(-d2);
         e1c_s[slot] = e1 * kTruncComp;
         e2_s[slot] = e2;
@@ -637,10 +628,10 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         if (lane == 0 && (!(fabsf(tot0) <= kMaxHalfDecay) || !(fabsf(tot1) <= kMaxHalfDecay))) misc->domain_flag = 1;  // also true for NaN
         // state factor from where the previous chunk left the state to this chunk's midpoint, and the factor owed after
         // it; scalars here, written for every channel so that the chain warps read them as they do for KDA
-        const float f = keep_scale ? 1.f : ex2f((post_prev + tot0) * LOG2E);
-        post_prev = keep_scale ? end : tot1;
+        const float f = ex2f((post_prev + tot0) * LOG2E);
+        post_prev = tot1;
         *reinterpret_cast<float4 *>(fac_s + (ch & 1) * D + lane * 4) = make_float4(f, f, f, f);
-        *reinterpret_cast<float4 *>(post_s + (ch & 1) * D + lane * 4) = make_float4(post_prev, post_prev, post_prev, post_prev);
+        *reinterpret_cast<float4 *>(post_s + (ch & 1) * D + lane * 4) = make_float4(tot1, tot1, tot1, tot1);
         arrive_warp(&misc->rdy_fac[ch & 1], lane);
       }
       const bool v1 = lane < n_tok - (ch + 1) * C;
@@ -849,7 +840,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       tc_fence_after_sync();
 
       // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
-      if (KDA || fac_c[0] != 1.f) {  // GDN: one factor for all channels, 1 where the scale is kept
+      {
         uint64_t f[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const uint64_t *>(fac_c + colh * 64 + 8 * i + 2 * tig);
