@@ -29,8 +29,8 @@
 // Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1090 us = 1.92 G token-heads/s = 60 % of the
 // floor set by its bytes, GDN 885 us = 2.37 G (46 %); 1685 and 1630 us in the form this one grew from.  No unit of the SM is at
 // its limit: per chunk and SM 4.7 k cycles, of which the shared-memory data pipe (load/store units and the tensor core's
-// operand reads together) is busy 70 %, the issue slots 48 %, the tensor pipe 33 %.  A CTA alone on its SM takes as long per
-// chunk as two CTAs take for one each: by itself it is bound by its chain of hand-offs, two of them by sharing the above.
+// operand reads together) is busy 70 %, the issue slots 48 %, the tensor pipe 33 %.  A CTA alone on its SM also
+// completes a chunk every 4.8 k cycles: by itself it is bound by its chain of hand-offs, two of them by sharing the above.
 // What it was before, in the order in which it was found: 103 cycles of issue per tensor-core instruction (behind
 // `lane == 0` instead of an elected lane), 119 KB of code in the instruction caches (now 56 KB), and 85 % of the
 // shared-memory pipe (8-byte accesses in 16-byte places, A padded to 128 rows, V and O value by value).
