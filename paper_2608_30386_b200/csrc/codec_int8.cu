@@ -34,9 +34,10 @@ constexpr int kThreads = DASC_INT8_THREADS;          // tuning knobs; defaults =
 constexpr int kUnroll = DASC_INT8_PACK_UNROLL;       // rows (pack) / vectors (restore) in flight per thread
 constexpr int kRUnroll = DASC_INT8_RESTORE_UNROLL;
 
+// Not the non-coherent path: see launch.cuh.
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
@@ -48,7 +49,7 @@ __device__ __forceinline__ void st_stream(uint4 *p, const uint4 &v) {
 }
 __device__ __forceinline__ uint32_t ld_stream32(const uint32_t *p) {
   uint32_t v;
-  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
 __device__ __forceinline__ void st_stream32(uint32_t *p, uint32_t v) {
@@ -115,10 +116,10 @@ __device__ __forceinline__ float absmax4(const uint4 &v) {
 // a row is held by `lanes_per_row` = d_v/4 consecutive lanes of one warp (a power of two <= 32).
 // FULL_WARP_ROWS: d_v = 128, a row is exactly one warp and the abs-max is one warp reduction.
 template <bool FULL_WARP_ROWS>
-__global__ void __launch_bounds__(kThreads, DASC_INT8_PACK_MIN_BLOCKS) pack_int8_kernel(const uint4 *__restrict__ state, int64_t layer_stride4,
-                                                             int64_t req_stride4, const int32_t *__restrict__ src_req,
-                                                             uint8_t *__restrict__ pool, int64_t slot_stride_bytes,
-                                                             const int32_t *__restrict__ dst_slot,
+__global__ void __launch_bounds__(kThreads, DASC_INT8_PACK_MIN_BLOCKS) pack_int8_kernel(const uint4 *state, int64_t layer_stride4,
+                                                             int64_t req_stride4, const int32_t *src_req,
+                                                             uint8_t *pool, int64_t slot_stride_bytes,
+                                                             const int32_t *dst_slot,
                                                              const DascRowSrc *__restrict__ row_src,
                                                              uint32_t packed_vecs, uint32_t packed_rows,
                                                              uint32_t lanes_per_row_arg, int32_t n_pairs) {
@@ -126,8 +127,8 @@ __global__ void __launch_bounds__(kThreads, DASC_INT8_PACK_MIN_BLOCKS) pack_int8
   const uint32_t lanes_per_row = FULL_WARP_ROWS ? 32u : lanes_per_row_arg;
   const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
   for (int32_t pair = blockIdx.y; pair < n_pairs; pair += gridDim.y) {
-    const uint4 *src_base = state + static_cast<int64_t>(__ldg(src_req + pair)) * req_stride4;
-    uint8_t *slot = pool + static_cast<int64_t>(__ldg(dst_slot + pair)) * slot_stride_bytes;
+    const uint4 *src_base = state + static_cast<int64_t>(src_req[pair]) * req_stride4;
+    uint8_t *slot = pool + static_cast<int64_t>(dst_slot[pair]) * slot_stride_bytes;
     uint32_t *codes = reinterpret_cast<uint32_t *>(slot);
     float *scales = reinterpret_cast<float *>(slot + static_cast<size_t>(packed_rows) * lanes_per_row * 4u);
     uint4 val[kUnroll];
@@ -208,11 +209,11 @@ __device__ __forceinline__ uint4 dequant4(uint32_t word, float s) {
 
 // grid = (ceil(layer_vecs / (kThreads*kRUnroll)), n_layers, pairs).
 template <bool FULL_WARP_ROWS>
-__global__ void __launch_bounds__(kThreads, DASC_INT8_RESTORE_MIN_BLOCKS) restore_int8_kernel(const uint8_t *__restrict__ pool,
+__global__ void __launch_bounds__(kThreads, DASC_INT8_RESTORE_MIN_BLOCKS) restore_int8_kernel(const uint8_t *pool,
                                                                 int64_t slot_stride_bytes,
-                                                                const int32_t *__restrict__ src_slot,
-                                                                uint4 *__restrict__ state, int64_t layer_stride4,
-                                                                int64_t req_stride4, const int32_t *__restrict__ dst_req,
+                                                                const int32_t *src_slot,
+                                                                uint4 *state, int64_t layer_stride4,
+                                                                int64_t req_stride4, const int32_t *dst_req,
                                                                 const int32_t *__restrict__ row_pos, uint32_t layer_vecs,
                                                                 uint32_t rows_per_layer, uint32_t packed_rows,
                                                                 uint32_t lanes_per_row_arg, int32_t n_pairs) {
@@ -222,10 +223,10 @@ __global__ void __launch_bounds__(kThreads, DASC_INT8_RESTORE_MIN_BLOCKS) restor
   const int32_t layer = blockIdx.y;
   const int32_t *pos_l = row_pos + static_cast<int64_t>(layer) * rows_per_layer;
   for (int32_t pair = blockIdx.z; pair < n_pairs; pair += gridDim.z) {
-    const uint8_t *slot = pool + static_cast<int64_t>(__ldg(src_slot + pair)) * slot_stride_bytes;
+    const uint8_t *slot = pool + static_cast<int64_t>(src_slot[pair]) * slot_stride_bytes;
     const uint32_t *codes = reinterpret_cast<const uint32_t *>(slot);
     const float *scales = reinterpret_cast<const float *>(slot + static_cast<size_t>(packed_rows) * lanes_per_row * 4u);
-    uint4 *dst_base = state + static_cast<int64_t>(__ldg(dst_req + pair)) * req_stride4 + layer * layer_stride4;
+    uint4 *dst_base = state + static_cast<int64_t>(dst_req[pair]) * req_stride4 + layer * layer_stride4;
     uint32_t word[kRUnroll];
     float scale[kRUnroll];  // 0 marks an omitted row: a stored scale is at least 1e-8/127
 #pragma unroll
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kThreads, DASC_INT8_RESTORE_MIN_BLOCKS) restor
         const int32_t pos = __ldg(pos_l + row);
         if (pos >= 0) {
           word[u] = ld_stream32(codes + static_cast<uint32_t>(pos) * lanes_per_row + vec);
-          scale[u] = __ldg(scales + pos);
+          scale[u] = scales[pos];
         }
       }
     }

@@ -41,9 +41,10 @@ struct TpPools {
   uint32_t width_shift;
 };
 
+// Not the non-coherent path: see launch.cuh.
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
@@ -72,10 +73,10 @@ __device__ __forceinline__ uint4 *tp_address(const TpPools &tp, int64_t slot, in
 // needs the dense row only, and a block past its layer's count leaves at once.
 // pool_stride4: vectors between slots (Ragged, TpBalanced) or between (layer, slot) entries (Padded).
 template <Layout LAYOUT, int UNROLL>
-__global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restrict__ state, int64_t layer_stride4,
-                                                           int64_t req_stride4, const int32_t *__restrict__ src_req,
-                                                           uint4 *__restrict__ pool, int64_t pool_stride4,
-                                                           int64_t n_slots, const int32_t *__restrict__ dst_slot,
+__global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *state, int64_t layer_stride4,
+                                                           int64_t req_stride4, const int32_t *src_req,
+                                                           uint4 *pool, int64_t pool_stride4,
+                                                           int64_t n_slots, const int32_t *dst_slot,
                                                            const DascRowSrc *__restrict__ row_src,
                                                            const int32_t *__restrict__ layer_row_off,
                                                            uint32_t vecs_per_row, int32_t n_pairs,
@@ -88,8 +89,8 @@ __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restri
   if (blockIdx.x * (kThreads * UNROLL) >= layer_vecs) return;
   const int2 *src_l = reinterpret_cast<const int2 *>(row_src) + first;  // {layer, dense row} of the layer's packed rows
   for (int32_t pair = blockIdx.z; pair < n_pairs; pair += gridDim.z) {
-    const uint4 *src_base = state + static_cast<int64_t>(__ldg(src_req + pair)) * req_stride4 + layer * layer_stride4;
-    const int64_t slot = __ldg(dst_slot + pair);
+    const uint4 *src_base = state + static_cast<int64_t>(src_req[pair]) * req_stride4 + layer * layer_stride4;
+    const int64_t slot = dst_slot[pair];
     uint4 *dst_base = nullptr;
     if (LAYOUT == Layout::Ragged) dst_base = pool + slot * pool_stride4 + static_cast<int64_t>(first) * vecs_per_row;
     if (LAYOUT == Layout::Padded) dst_base = pool + (layer * n_slots + slot) * pool_stride4;
@@ -118,10 +119,10 @@ __global__ void __launch_bounds__(kThreads, 8) pack_kernel(const uint4 *__restri
 
 // grid = (ceil(layer_vecs / (kThreads*UNROLL)), n_layers, pairs).
 template <Layout LAYOUT, int UNROLL>
-__global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restrict__ pool, int64_t pool_stride4,
-                                                           int64_t n_slots, const int32_t *__restrict__ src_slot,
-                                                           uint4 *__restrict__ state, int64_t layer_stride4,
-                                                           int64_t req_stride4, const int32_t *__restrict__ dst_req,
+__global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *pool, int64_t pool_stride4,
+                                                           int64_t n_slots, const int32_t *src_slot,
+                                                           uint4 *state, int64_t layer_stride4,
+                                                           int64_t req_stride4, const int32_t *dst_req,
                                                            const int32_t *__restrict__ row_pos,
                                                            const int32_t *__restrict__ layer_row_off,
                                                            uint32_t layer_vecs, uint32_t rows_per_layer,
@@ -134,11 +135,11 @@ __global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restri
   // Padded: packed row of the layer's first retained row (positions inside an entry count from it)
   const int32_t first = LAYOUT == Layout::Padded ? __ldg(layer_row_off + layer) : 0;
   for (int32_t pair = blockIdx.z; pair < n_pairs; pair += gridDim.z) {
-    const int64_t slot = __ldg(src_slot + pair);
+    const int64_t slot = src_slot[pair];
     const uint4 *src_base = nullptr;
     if (LAYOUT == Layout::Ragged) src_base = pool + slot * pool_stride4;
     if (LAYOUT == Layout::Padded) src_base = pool + (layer * n_slots + slot) * pool_stride4;
-    uint4 *dst_base = state + static_cast<int64_t>(__ldg(dst_req + pair)) * req_stride4 + layer * layer_stride4;
+    uint4 *dst_base = state + static_cast<int64_t>(dst_req[pair]) * req_stride4 + layer * layer_stride4;
     uint4 val[UNROLL];
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
@@ -165,16 +166,16 @@ __global__ void __launch_bounds__(kThreads) restore_kernel(const uint4 *__restri
 }
 
 // dst[dst_idx[i]] = src[src_idx[i]] for blobs of `vecs` 16-byte vectors; grid = (ceil(vecs / (kThreads*kUnroll)), pairs).
-__global__ void __launch_bounds__(kThreads) blob_copy_kernel(const uint4 *__restrict__ src, int64_t src_stride4,
-                                                             const int32_t *__restrict__ src_idx,
-                                                             uint4 *__restrict__ dst, int64_t dst_stride4,
-                                                             const int32_t *__restrict__ dst_idx, uint32_t vecs,
+__global__ void __launch_bounds__(kThreads) blob_copy_kernel(const uint4 *src, int64_t src_stride4,
+                                                             const int32_t *src_idx,
+                                                             uint4 *dst, int64_t dst_stride4,
+                                                             const int32_t *dst_idx, uint32_t vecs,
                                                              int32_t n_pairs) {
   stream_order_begin();
   const uint32_t base = blockIdx.x * (kThreads * kUnroll) + threadIdx.x;
   for (int32_t pair = blockIdx.y; pair < n_pairs; pair += gridDim.y) {
-    const uint4 *s = src + static_cast<int64_t>(__ldg(src_idx + pair)) * src_stride4;
-    uint4 *d = dst + static_cast<int64_t>(__ldg(dst_idx + pair)) * dst_stride4;
+    const uint4 *s = src + static_cast<int64_t>(src_idx[pair]) * src_stride4;
+    uint4 *d = dst + static_cast<int64_t>(dst_idx[pair]) * dst_stride4;
     uint4 val[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
