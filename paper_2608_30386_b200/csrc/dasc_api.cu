@@ -59,9 +59,9 @@ void free_device_tables(dasc_plan_s *p) {
   p->d_row_keep = nullptr;
 }
 
-// The plan's index tables live on plan->info.device; a launch from another current device would hand the kernel
-// pointers of a GPU it may not be able to reach.
-// Upload the index tables of a host plan to `device` (the only device allocation this library makes).
+// Upload the index tables of a host plan to `device` (the only device allocation this library makes).  They are on the
+// device when this returns: a copy from pageable memory may return while its last part is still on the way, and the plan's
+// first launch can be on a stream that does not wait for the legacy stream the copies are on.
 dasc_status_t attach_device(dasc_plan_s *p, int device) {
   DeviceGuard guard(device);
   if (!guard.ok) return DASC_ERR_CUDA;
@@ -76,6 +76,7 @@ dasc_status_t attach_device(dasc_plan_s *p, int device) {
   std::vector<int32_t> row_off(p->layer_offset.size());
   for (size_t l = 0; l < row_off.size(); ++l) row_off[l] = static_cast<int32_t>(p->layer_offset[l] * rows_per_unit);
   if (e == cudaSuccess) e = upload(&p->d_layer_row_off, row_off.data(), row_off.size());
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) {
     free_device_tables(p);
     p->info.device = -1;
@@ -84,6 +85,8 @@ dasc_status_t attach_device(dasc_plan_s *p, int device) {
   return DASC_OK;
 }
 
+// The plan's index tables live on plan->info.device; a launch from another current device would hand the kernel
+// pointers of a GPU it may not be able to reach.
 dasc_status_t check_device(const dasc_plan_t *plan) {
   if (!plan || plan->info.device < 0) return DASC_ERR_INVALID_ARG;
   int dev = -1;

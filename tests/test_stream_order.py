@@ -32,3 +32,9 @@ def test_only_plan_tables_take_the_non_coherent_path(name):
         assert first in PLAN_TABLES, f"__ldg({arg[:40]}"
     for param in re.findall(r"__restrict__\s+(\w+)", code):
         assert param in PLAN_TABLES, param
+
+
+def test_plan_tables_are_on_the_device_when_the_plan_is_returned():
+    body = re.search(r"dasc_status_t attach_device\(.*?\n}\n", _code("dasc_api.cu"), flags=re.S).group(0)
+    last_copy = max(m.start() for m in re.finditer(r"upload\(", body))
+    assert re.search(r"cuda(Stream|Device)Synchronize\(", body[last_copy:])
