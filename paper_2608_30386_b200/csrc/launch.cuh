@@ -13,7 +13,12 @@
 
 __device__ __forceinline__ void stream_order_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void stream_order_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// The next kernel's blocks cannot be placed before every block of this one has been, so releasing it at once delays nothing.
+// Once every block of a kernel has released or ended, the next kernel's blocks are placed wherever there is room, and hold their
+// registers, shared memory and threads there while they wait: on this stream that delays nothing, but work of OTHER streams
+// cannot have that room meanwhile.  So only kernels that end soon after their last block has started release at once (the
+// copies, the kernel in front of a refresh).  The refresh kernels, which can run for milliseconds on a few SMs, wait first
+// and release a few microseconds before they end, enough to hide the launch.  With a release at once, a Store beside a
+// refresh of one long request (2 of 148 SMs) ended behind it.
 __device__ __forceinline__ void stream_order_begin() {
   stream_order_release();
   stream_order_wait();

@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   const int tid = threadIdx.x, warp = uni(tid >> 5), lane = tid & 31;
   const int h = blockIdx.x % a.H_v;
   const int lc = (blockIdx.x / a.H_v) % a.n_layers_in_call;
-  stream_order_begin();
+  stream_order_wait();
   int r = blockIdx.x / (a.H_v * a.n_layers_in_call);
   if (a.ordered) r = uni(static_cast<const uint8_t *>(a.workspace)[kRefreshWsOrder + r]);
   const int unit = (r * a.n_layers_in_call + lc) * a.H_v + h;
@@ -833,6 +833,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       const bool more = ch + 1 < n_chunks;
       const float *beta_c = beta_s + (ch & 3) * C;
       const float *fac_c = fac_s + par * D;
+      if (!more && tid == 0) stream_order_release();  // one chunk (2.5 us) before the end: see launch.cuh
 
       // ---- (1) the previous chunk's state update is complete; this chunk's factors and tiles are ready ----
       if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);

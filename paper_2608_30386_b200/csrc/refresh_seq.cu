@@ -310,6 +310,8 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
   if (AHEAD) __syncthreads();
   for (int grp = 0; grp < n_grp; ++grp) {
     const int cnt = min(TB, n_tok - grp * TB);
+    // one token group (about 2 us) before the end: see launch.cuh; a list has more units to come
+    if (grp + 1 == n_grp && !a.from_list) stream_order_release();
     if constexpr (AHEAD) {
       // extra warps: the group before goes out, the next one is converted, the one after that is fetched
       if (helper) {
@@ -437,7 +439,7 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
 template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
 __global__ void __launch_bounds__(NCOL / COLS *SL + NHELP) refresh_seq_kernel(DascRefreshArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  stream_order_begin();
+  stream_order_wait();
   constexpr int PARTS = DV / NCOL;
   if (!a.from_list) {
     seq_unit<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x) / PARTS, static_cast<int>(blockIdx.x) % PARTS, smem_raw);
