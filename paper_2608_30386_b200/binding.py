@@ -307,14 +307,14 @@ def dasc_padded_pool_floats(plan: Plan, n_slots: int) -> int:
 def dasc_pack_padded(plan: Plan, state: torch.Tensor, layer_stride: int, req_stride: int, src_req: torch.Tensor,
                      pool: torch.Tensor, n_slots: int, dst_slot: torch.Tensor, stream=None):
     """``dasc_pack`` into the padded pool; padding entries are not written."""
-    _check((_native or _call()).pack_padded(plan.handle, state, layer_stride, req_stride, src_req, pool, n_slots, dst_slot, stream),
+    _check((_native or _call()).pack_padded(plan.handle, state, layer_stride, req_stride, src_req, pool, int(n_slots), dst_slot, stream),
            "dasc_pack_padded")
 
 
 def dasc_restore_padded(plan: Plan, pool: torch.Tensor, n_slots: int, src_slot: torch.Tensor, state: torch.Tensor,
                         layer_stride: int, req_stride: int, dst_req: torch.Tensor, stream=None):
     """``dasc_restore`` from the padded pool."""
-    _check((_native or _call()).restore_padded(plan.handle, pool, n_slots, src_slot, state, layer_stride, req_stride, dst_req, stream),
+    _check((_native or _call()).restore_padded(plan.handle, pool, int(n_slots), src_slot, state, layer_stride, req_stride, dst_req, stream),
            "dasc_restore_padded")
 
 

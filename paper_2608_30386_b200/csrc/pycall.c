@@ -35,7 +35,21 @@ static int as_ptr(PyObject *o, void **out) {
   return *out == NULL && PyErr_Occurred() ? -1 : 0;
 }
 
-static int as_i64(PyObject *o, int64_t *out) {
+/* A stride, a layer, an enumerator: whole numbers only, a float is an error and not cut off. */
+static int as_index(PyObject *o, int64_t *out) {
+  if (PyLong_Check(o)) {
+    *out = PyLong_AsLongLong(o);
+  } else {
+    PyObject *v = PyNumber_Index(o);
+    if (!v) return -1;
+    *out = PyLong_AsLongLong(v);
+    Py_DECREF(v);
+  }
+  return *out == -1 && PyErr_Occurred() ? -1 : 0;
+}
+
+/* A token count: whatever int() takes. */
+static int as_count(PyObject *o, int64_t *out) {
   if (PyLong_Check(o)) {
     *out = PyLong_AsLongLong(o);
   } else {
@@ -50,7 +64,7 @@ static int as_i64(PyObject *o, int64_t *out) {
 static int method_i64(PyObject *o, PyObject *name, int64_t *out) {
   PyObject *v = PyObject_CallMethodNoArgs(o, name);
   if (!v) return -1;
-  const int r = as_i64(v, out);
+  const int r = as_index(v, out);
   Py_DECREF(v);
   return r;
 }
@@ -113,8 +127,8 @@ typedef dasc_status_t (*store_fn)(const dasc_plan_t *, const float *, int64_t, i
 static PyObject *store_call(store_fn fn, PyObject *const *a, Py_ssize_t n) {
   void *plan, *state, *src, *pool, *dst, *stream;
   int64_t ls, rs, arg, pairs;
-  if (arg_count(n, 9) || as_ptr(a[0], &plan) || as_ptr(a[1], &state) || as_i64(a[2], &ls) || as_i64(a[3], &rs) ||
-      as_ptr(a[4], &src) || as_ptr(a[5], &pool) || as_i64(a[6], &arg) || as_ptr(a[7], &dst) ||
+  if (arg_count(n, 9) || as_ptr(a[0], &plan) || as_ptr(a[1], &state) || as_index(a[2], &ls) || as_index(a[3], &rs) ||
+      as_ptr(a[4], &src) || as_ptr(a[5], &pool) || as_index(a[6], &arg) || as_ptr(a[7], &dst) ||
       method_i64(a[4], s_numel, &pairs) || as_stream(a[8], &stream))
     return NULL;
   dasc_status_t st;
@@ -130,8 +144,8 @@ typedef dasc_status_t (*load_fn)(const dasc_plan_t *, const void *, int64_t, con
 static PyObject *load_call(load_fn fn, PyObject *const *a, Py_ssize_t n) {
   void *plan, *state, *src, *pool, *dst, *stream;
   int64_t ls, rs, arg, pairs;
-  if (arg_count(n, 9) || as_ptr(a[0], &plan) || as_ptr(a[1], &pool) || as_i64(a[2], &arg) || as_ptr(a[3], &src) ||
-      as_ptr(a[4], &state) || as_i64(a[5], &ls) || as_i64(a[6], &rs) || as_ptr(a[7], &dst) ||
+  if (arg_count(n, 9) || as_ptr(a[0], &plan) || as_ptr(a[1], &pool) || as_index(a[2], &arg) || as_ptr(a[3], &src) ||
+      as_ptr(a[4], &state) || as_index(a[5], &ls) || as_index(a[6], &rs) || as_ptr(a[7], &dst) ||
       method_i64(a[3], s_numel, &pairs) || as_stream(a[8], &stream))
     return NULL;
   dasc_status_t st;
@@ -160,16 +174,17 @@ struct refresh_args {
   size_t ws_bytes;
 };
 static int refresh_parse(struct refresh_args *r, PyObject *const *a, PyObject *io_from) {
-  if (as_ptr(a[0], &r->plan) || as_ptr(a[1], &r->state) || as_i64(a[2], &r->ls) || as_i64(a[3], &r->rs) ||
+  if (as_ptr(a[0], &r->plan) || as_ptr(a[1], &r->state) || as_index(a[2], &r->ls) || as_index(a[3], &r->rs) ||
       as_ptr(a[4], &r->req) || as_ptr(a[5], &r->q) || as_ptr(a[6], &r->k) || as_ptr(a[7], &r->v) || as_ptr(a[8], &r->g) ||
-      as_ptr(a[9], &r->beta) || as_ptr(a[10], &r->cu) || method_i64(a[10], s_numel, &r->n_cu) || as_i64(a[11], &r->total) ||
-      as_i64(a[12], &r->bound) || as_i64(a[13], &r->lb) || as_i64(a[14], &r->le) || as_ptr(a[16], &r->o) ||
-      as_i64(a[17], &r->algo) || as_ptr(a[18], &r->ws) || nbytes(a[18], &r->ws_bytes) || as_stream(a[19], &r->stream) ||
+      as_ptr(a[9], &r->beta) || as_ptr(a[10], &r->cu) || method_i64(a[10], s_numel, &r->n_cu) || as_count(a[11], &r->total) ||
+      as_count(a[12], &r->bound) || as_index(a[13], &r->lb) || as_index(a[14], &r->le) || as_ptr(a[16], &r->o) ||
+      as_index(a[17], &r->algo) || as_ptr(a[18], &r->ws) || nbytes(a[18], &r->ws_bytes) || as_stream(a[19], &r->stream) ||
       as_io(io_from, &r->io) || as_io(a[16], &r->o_io))
     return -1;
-  const double s = PyFloat_AsDouble(a[15]);
-  if (s == -1.0 && PyErr_Occurred()) return -1;
-  r->q_scale = (float)s;
+  PyObject *s = PyNumber_Float(a[15]);
+  if (!s) return -1;
+  r->q_scale = (float)PyFloat_AS_DOUBLE(s);
+  Py_DECREF(s);
   return 0;
 }
 
@@ -177,7 +192,7 @@ static int refresh_parse(struct refresh_args *r, PyObject *const *a, PyObject *i
 static PyObject *py_refresh(PyObject *self, PyObject *const *a, Py_ssize_t n) {
   struct refresh_args r;
   int64_t mode;
-  if (arg_count(n, 21) || refresh_parse(&r, a, a[5]) || as_i64(a[20], &mode)) return NULL;
+  if (arg_count(n, 21) || refresh_parse(&r, a, a[5]) || as_index(a[20], &mode)) return NULL;
   dasc_status_t st;
   Py_BEGIN_ALLOW_THREADS
   st = dasc_refresh(r.plan, r.state, r.ls, r.rs, r.req, r.q, r.k, r.v, r.io, r.g, r.beta, r.cu, (int32_t)(r.n_cu - 1), r.total,
