@@ -77,3 +77,17 @@ def test_whole_numbers_of_a_refresh(call, plan):
         _reaches_the_library(call, plan, q_scale=scale)
     with pytest.raises(TypeError):
         call(plan, q_scale=None)
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_the_current_stream_without_private_entries_of_torch(missing, monkeypatch):
+    monkeypatch.setattr(torch.cuda, "is_available", lambda: True)
+    monkeypatch.setattr(torch.cuda, "init", lambda: None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: type("S", (), {"cuda_stream": 77})())
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.setattr(torch._C, name, lambda *_: 1, raising=False)
+    raw_stream, device = binding._stream_lookup()
+    assert raw_stream(device()) == 1
+    monkeypatch.delattr(torch._C, missing)
+    raw_stream, device = binding._stream_lookup()
+    assert raw_stream(device()) == 77
