@@ -13,12 +13,14 @@ LIB = os.path.join(HERE, "libdasc.so")
 CALL = os.path.join(HERE, "_dasccall.so")   # CPython entry to the library's device calls
 CALL_SOURCE = "pycall.c"
 SOURCES = ["dasc_api.cu", "plan_host.cpp", "pack_restore.cu", "codec_int8.cu", "refresh_seq.cu", "refresh_chunked.cu"]
+# sources compiled several times, side by side: object name and define of each translation unit
+UNITS = {"refresh_seq.cu": [(f"refresh_seq_{d}", f"-DDASC_SEQ_DIM={d}") for d in (128, 64, 32)]}
 HEADERS = [os.path.join(ROOT, "include", "dasc.h"), os.path.join(CSRC, "dasc_internal.h"),
            os.path.join(CSRC, "tcgen05_util.cuh"), os.path.join(CSRC, "launch.cuh")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "-Xcompiler", "-fPIC",
+    "-Xcompiler", "-fPIC", "-Xfatbin=-compress-all",
 ]
 
 
@@ -44,10 +46,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(objdir, exist_ok=True)
     objs = []
     procs = []
-    for s in SOURCES:
-        obj = os.path.join(objdir, os.path.splitext(s)[0] + ".o")
+    for s, name, *define in ((s, *u) for s in SOURCES for u in UNITS.get(s, [(os.path.splitext(s)[0],)])):
+        obj = os.path.join(objdir, name + ".o")
         objs.append(obj)
-        cmd = [_nvcc(), *NVCC_FLAGS, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-x", "cu", "-c",
+        cmd = [_nvcc(), *NVCC_FLAGS, *define, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-x", "cu", "-c",
                os.path.join(CSRC, s), "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")

@@ -121,6 +121,17 @@ dasc_status_t check_copy_args(const dasc_plan_t *plan, const void *state, int64_
 
 }  // namespace
 
+// Returns a cudaError_t as int, or -1 if the shape has no instantiation.
+int dasc_launch_refresh_seq(const DascRefreshArgs &a, void *stream) {
+  if (a.d_k != a.d_v) return -1;
+  switch (a.d_k) {
+    case 128: return dasc_launch_refresh_seq_dim<128>(a, stream);
+    case 64: return dasc_launch_refresh_seq_dim<64>(a, stream);
+    case 32: return dasc_launch_refresh_seq_dim<32>(a, stream);
+  }
+  return -1;
+}
+
 extern "C" {
 
 dasc_status_t dasc_plan(const dasc_plan_desc_t *desc, int32_t device, dasc_plan_t **out) {

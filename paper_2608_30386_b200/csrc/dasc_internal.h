@@ -117,7 +117,9 @@ struct DascRefreshArgs {
 // What has to be on the device before a refresh kernel: tok_begin (window > 0), cleared header words and the request order
 // (workspace).
 int dasc_launch_refresh_prep(const DascRefreshArgs &a, void *stream);
-int dasc_launch_refresh_seq(const DascRefreshArgs &a, void *stream);
+template <int D>
+int dasc_launch_refresh_seq_dim(const DascRefreshArgs &a, void *stream);  // d_k = d_v = D; one translation unit each
+int dasc_launch_refresh_seq(const DascRefreshArgs &a, void *stream);      // dasc_api.cu: picks one of those
 int dasc_launch_refresh_chunked(const DascRefreshArgs &a, void *stream);
 size_t dasc_refresh_chunked_workspace_bytes(int32_t n_req, int32_t n_layers_in_call, int32_t H_v);
 // Test hook (see dasc_debug_set_refresh_poll_limit in dasc.h).
