@@ -63,14 +63,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst_smem, const void *tmap,
       "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
       : "memory");
 }
-__device__ __forceinline__ void tma_load_4d(uint32_t dst_smem, const void *tmap, int32_t x, int32_t y, int32_t z, int32_t w,
-                                            uint64_t *bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(
-          dst_smem),
-      "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
-      : "memory");
-}
 
 // One lane of a converged warp.  The compiler knows that a branch on this predicate runs with a single active thread, so the
 // tcgen05 instructions below it take their descriptors straight from uniform registers; behind `lane == 0` it has to allow
@@ -197,8 +189,6 @@ __device__ __forceinline__ void tmem_st_16x256b(uint32_t taddr, const uint32_t (
 // cost an order of magnitude more issue time on this part.
 // tf32_pre(x): container whose truncation is the rounded value (for operands only tensor cores read).
 __device__ __forceinline__ uint32_t tf32_pre(float x) { return __float_as_uint(x) + 0x1000u; }
-// to_tf32(x): the rounded value itself, low 13 bits cleared.
-__device__ __forceinline__ uint32_t to_tf32(float x) { return (__float_as_uint(x) + 0x1000u) & 0xFFFFE000u; }
 
 // Shared-memory operand tiles use the 128-byte-swizzle canonical layout.  A tile of R rows
 // and 32*NB tf32 columns is stored as NB blocks of [R rows][128 bytes]; inside a block the
