@@ -1,7 +1,7 @@
 // Kernel launch with programmatic stream serialisation: the grid may be set up while the last blocks of the kernel before
-// it in the stream still run.  Every kernel launched this way begins with stream_order_begin(): the wait holds until
-// all earlier work of the stream has completed and its writes are visible, so the order on the stream is the usual one, and
-// only launch latency (1 to 2 us on B200, a quarter of the smallest calls) overlaps.
+// it in the stream still run.  Every kernel launched this way begins with stream_order_begin() or stream_order_wait(), before it
+// touches any memory: the wait holds until all earlier work of the stream has completed and its writes are visible, so the
+// order on the stream is the usual one, and only launch latency (1 to 2 us on B200, a quarter of the smallest calls) overlaps.
 //
 // A kernel launched this way is on the GPU while the one before it still writes, so what that one may write (states, pools,
 // streams, index arrays) is not read-only for the kernel's lifetime, which is what the non-coherent path (ld.global.nc, __ldg,

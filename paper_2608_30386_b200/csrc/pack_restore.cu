@@ -1,6 +1,6 @@
 // Store / Load copy kernels: pack (gather retained rows into a checkpoint pool) and restore
 // (scatter back with the zero-fill fused, every dense byte written once).  Pure HBM-bandwidth
-// work: 128-bit streaming loads and stores, four independent loads in flight per thread, index
+// work: 128-bit streaming loads and stores, four independent loads in flight per thread (fewer in small grids), index
 // tables small enough to live in L2.
 //
 // One pair of kernels serves three pool layouts; only the pool address of a packed row differs:
@@ -24,9 +24,12 @@ namespace {
 constexpr int kThreads = 256;  // threads per block and loads in flight per thread: the best of a measured sweep
 constexpr int kUnroll = 4;     // over {128..1024} x {1..16}
 // Loads in flight per thread when `blocks` (of kUnroll loads per thread) are few: eight blocks are resident on an SM, and a grid
-// that leaves most of that unused moves its bytes faster with more threads and fewer loads each.  B200, one checkpoint of
-// 24 layers x 8 heads: store (312 blocks) 4.9 / 3.8 / 3.1 us with 4 / 2 / 1, load (768 blocks) 5.8 / 4.8 / 5.1 us; 32 heads: store
-// (1176 blocks) 6.9 / 7.9 / 8.2 us.
+// that leaves most of that unused moves its bytes faster with more threads and fewer loads each.  B200, one checkpoint of 24
+// layers of 2 .. 48 heads, microseconds with 4 / 2 / 1 loads at so many blocks:
+//   store  312: 4.9 3.5 3.5   600: 6.0 5.2 5.4   744: 6.5 6.3 6.3   816: 6.8 6.7 6.7   888: 7.0 7.0 7.1   1176: 8.4 8.5 8.8
+//   load   480: 5.1 4.0 3.8   672: 5.9 5.4 5.0   768: 5.8 5.8 5.4   864: 6.0 6.1 5.8   960: 6.3 6.5 6.3   1152: 6.9 7.2 7.1
+// Both kernels gain nothing from fewer loads from about 888 blocks on; below that a load would do a little better with 1 than
+// with 2.
 int unroll_for(uint64_t blocks) { return blocks <= 4 * 148 ? 1 : blocks <= 6 * 148 ? 2 : kUnroll; }
 
 enum class Layout { Ragged, Padded, TpBalanced };

@@ -1,6 +1,6 @@
 /* CPython entry to the device calls of libdasc that sit on a serving engine's path: argument marshalling only, like
  * binding.py, which uses it for these calls.  A ctypes call with ten to twenty-six arguments costs 4 to 8 us of interpreter
- * time on this GPU machine's host, more than the GPU needs for the smallest calls; here it is under 1 us.
+ * time on the host of a B200, more than the GPU needs for the smallest calls; here it is under 1 us.
  *
  * Tensors are taken as they are: None is a null pointer, an int an address, anything with a data_ptr() that; what an address
  * is for other objects binding.py says.  `stream` is None (torch's current stream) or has a cuda_stream attribute.  Every function

@@ -27,10 +27,12 @@
 // MN-major operands have a swizzle of their own), which, read last, is double-buffered by chunk parity.
 //
 // Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1090 us = 1.92 G token-heads/s = 60 % of the
-// floor set by its bytes, GDN 885 us = 2.37 G (46 %); 1685 and 1630 us in the form this one grew from.  No unit of the SM is at
-// its limit: per chunk and SM 4.7 k cycles, of which the shared-memory data pipe (load/store units and the tensor core's
-// operand reads together) is busy 70 %, the issue slots 48 %, the tensor pipe 33 %.  A CTA alone on its SM also
-// completes a chunk every 4.8 k cycles: by itself it is bound by its chain of hand-offs, two of them by sharing the above.
+// rate at which HBM could bring its bytes (657 us), GDN 885 us = 2.37 G (46 %); 1685 and 1630 us in the form this one grew from.
+// No unit of the SM is at its limit: per chunk and SM (two CTAs) KDA takes 4.5 k cycles, of which the shared-memory data pipe
+// (load/store units and the tensor core's operand reads together) is busy 74 %, the issue slots 50 %, the tensor pipe 35 %; GDN
+// 3.7 k, 82 %, 47 %, 39 %; the state-only form 4.8 k at 2 to 4 chunks per unit, 59 %, 46 %, 24 %.  A CTA alone on its SM
+// completes a chunk every 4.8 k cycles (GDN 4.5 k), bound by its chain of hand-offs; the second CTA hides some of that
+// and the starts and ends of units.
 // What it was before, in the order in which it was found: 103 cycles of issue per tensor-core instruction (behind
 // `lane == 0` instead of an elected lane), 119 KB of code in the instruction caches (now 56 KB), and 85 % of the
 // shared-memory pipe (8-byte accesses in 16-byte places, A padded to 128 rows, V and O value by value).
@@ -85,39 +87,42 @@ static_assert(SMEM_ALLOC <= 113 * 1024, "two CTAs per SM");
 
 constexpr uint32_t kMaxPolls = 1u << 22;
 
+// Largest |sum of the log-decay over half a chunk| per channel for which every factor formed relative to the chunk
+// midpoint stays a normal fp32 number with room for the products that follow.
+constexpr float kMaxHalfDecay = 80.f;
+
 // The tensor core reads the fp32 state as tf32 by dropping its low 13 mantissa bits, i.e. rounding
 // towards zero: on average the operand is 2^-11 * E[1/m] = 3.52e-4 too small in magnitude (m the
 // significand, log-uniform in [1, 2)).  The rows of Kt and Qt, the only partners of that operand,
 // are scaled up by this factor to cancel the bias; A and P, which also come from those rows, are
 // scaled back down when they are taken out of TMEM.
-// Largest |sum of the log-decay over half a chunk| per channel for which every factor formed relative to the chunk
-// midpoint stays a normal fp32 number with room for the products that follow.
-constexpr float kMaxHalfDecay = 80.f;
-
 constexpr float kTruncComp = 1.000352f;
 constexpr float kInvTruncComp = 1.0f / kTruncComp;
 constexpr float kLog2TruncComp = 5.0774e-4f;  // log2(kTruncComp)
 
 struct Misc {
-  // tensor core -> chain warps (one tcgen05.commit each per chunk); bar_ro also releases the producer
+  // Each barrier completes one phase per chunk.  Where the arrivals are "per warp", a warp's first lane arrives for it.
+  // tensor core -> chain warps (one tcgen05.commit each); bar_ap also releases the triangular and the issuing warp and the
+  // next log-decay (KDA) or k, q (GDN), bar_ro the Kt/Qt tile, bar_s the Kh tile of its parity (KDA)
   uint64_t bar_ap, bar_ro, bar_u, bar_o, bar_s;
-  // producer -> issuing warp and chain warps (128 arrivals per chunk)
+  // producer -> issuing warp and chain warps (per warp: 4 arrivals)
   uint64_t rdy_prep;
-  // producer -> chain warps: the state factors of a chunk are ready (128 arrivals per chunk)
+  // producer -> chain warps: the state factors of a chunk are ready (KDA per warp: 4 arrivals; GDN the first warp only: 1)
   // One barrier per chunk parity: the producer may hand over the factors of chunk n+1 before the chain warps
   // have waited for those of chunk n, and a single barrier cannot tell phases two apart.
   uint64_t rdy_fac[2];
-  // chain warps -> issuing warp (256 arrivals each per chunk)
+  // chain warps -> issuing warp (per warp: 8 arrivals each)
   uint64_t rdy_state, rdy_rhs, rdy_u;
-  // triangular warp -> chain warps (A has left TMEM: 32 arrivals) and -> issuing warp (T tile ready: 32 arrivals)
+  // triangular warp -> chain warps (A has left TMEM: 1 arrival) and -> issuing warp (T tile ready: 1 arrival)
   uint64_t a_taken, rdy_t;
-  // chain warps -> triangular warp: the T|P tile region is free again (256 arrivals per chunk)
+  // chain warps -> triangular warp and one another: the T|P tile region is free again (per warp: 8 arrivals)
   uint64_t tp_free;
   // issuing thread, only after a wait has run out: arrives once every tensor-core product issued so far has completed
   uint64_t drain;
-  // TMA -> producer warps: the log-decay of a chunk has landed in the Kh tile (KDA); its raw k, q have landed
+  // TMA -> producer warps: the log-decay of a chunk has landed in the Kh tile (KDA: 4 copies, one arrival with each); its raw
+  // k, q have landed (4 copies, 2 without outputs)
   uint64_t g_full, kq_full;
-  // TMA -> chain warps: V of a chunk has landed
+  // TMA -> chain warps: V of a chunk has landed (2 copies)
   uint64_t v_full;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;   // a bounded wait ran out: every later wait of this CTA returns at once
@@ -1065,9 +1070,9 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
 }
 
 // Blocks are placed in index order, so the requests are taken longest first: a long one started last would run on while
-// the rest of the GPU is idle.  64 requests of 1 .. 1023 tokens x 32 heads (2048 units, 296 resident): 635 -> 610 us on B200.
-// Ties keep their order; up to 240 requests (the table lives in the workspace header), beyond which the units far outnumber
-// the resident ones.
+// the rest of the GPU is idle.  Requests of 1 .. 1023 tokens on B200 (296 units resident): 64 x 32 heads 618 -> 528 us, 240 x 4 heads
+// 335 -> 264 us.  Ties keep their order.  The limit of 240 requests is what fits the spare bytes of the workspace header, not
+// where the order stops to pay: 241 x 4 heads take 354 us, and 265 us where the caller lists them longest first.
 bool ordered(const DascRefreshArgs &a) { return a.n_req > 1 && a.n_req <= kRefreshOrderMax; }
 
 constexpr int kPrepThreads = 256;

@@ -16,8 +16,8 @@
 // serial chain (a dot product and its shuffles per token; the next token's is started before this token's update, see
 // below), else instruction issue and the registers' share of the shared-memory bandwidth (128 bytes per cycle whatever is
 // broadcast, hence 4 columns per lane in the wide variants).
-// Measured on B200 (the form before: one column per thread and row half, a block barrier per token): 4 units of 64 x 64, 64 fp32
-// tokens 26.7 -> 15.8 us; 4 of 128 x 128 54 -> 18.5 us; 256 of 128 x 128, 256 tokens 407 -> 345 us; 8192 of them 11.2 -> 9.5 ms.
+// Measured on B200, fp32 (the form before: one column per thread and row half, a block barrier per token): 4 units of 64 x 64, 64
+// tokens 26.7 -> 12.6 us; 4 of 128 x 128 54 -> 17.4 us; 256 of 128 x 128, 256 tokens 407 -> 345 us; 8192 of them 11.2 -> 9.6 ms.
 // Token inputs are staged TB tokens at a time: raw rows by cp.async into a double
 // buffer, then converted once (bf16 -> fp32, alpha = exp(g)); outputs leave a group later, 16 bytes per store.  With NHELP > 0
 // that many extra threads do both, a group ahead of and a group behind the tokens being replayed.
@@ -475,8 +475,10 @@ int launch(const DascRefreshArgs &a, void *stream) {
 // Columns do not interact, so units that leave SMs idle are split by columns: parts of 8 (16 at d = 32) with 16 (8) lanes per
 // column and warps of their own for the conversions while that gives at most two CTAs per SM (beyond, the conversions, which
 // every part repeats, cost more than the shorter chain saves); at d = 128 halves while those fit one CTA per SM.
-// B200, 128 tokens, split / whole: d = 64, 16 units 25 / 49 us, 32 units 33 / 43 us, 64 units 62 / 43 us; d = 128, 16 units
-// 60 / 90 us, 32 units 115 / 90 us (halves 64 us).
+// B200, 128 fp32 tokens, microseconds split / whole on both sides of each line (KDA; GDN the same within 2 us where not given):
+//   d = 32   148 units 27 / 31, 149 units 45 / 35
+//   d = 64    37 units 29 / 42,  38 units 48 / 42 (GDN 37 / 41: its line would lie at 48 units)
+//   d = 128   18 units 60 / 89 (halves 59; GDN split 36, halves 58), 19 units 88 / 89 (59); halves 74 units 60 / 89, 75 units 116 / 91
 constexpr int64_t kSplitCtas = 296, kHalfCtas = 148;
 
 template <int D, typename IO, typename OT, bool KDA>
