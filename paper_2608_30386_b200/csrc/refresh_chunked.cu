@@ -1029,6 +1029,15 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     if (misc->abort_flag && v_issued > 0) mbar_wait_bounded(&misc->v_full, (v_issued - 1) & 1, kMaxPolls);
 
     // ---- final state: the factor still owed, then write back ----
+    // Which of this warp's rows are written, a bit each, fetched before the waits: looked up row by row beside the stores, the
+    // 64 loads came one behind the other and the write-back of a unit in the merge mode took 7.1 k cycles (2.6 k where all rows
+    // are written); 32 requests of 1 .. 128 tokens x 4 layers x 32 heads, state only: 277 -> 262 us.
+    uint32_t rows[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * D;
+      rows[i] = __ballot_sync(0xffffffffu, a.mode == DASC_REFRESH_CONTINUE || !keep[colh * 64 + i * 32 + lane]);
+    }
     if (n_chunks > 0) {
       wait_bar(&misc->rdy_prep, (n_chunks - 1) & 1, misc);  // the last chunk's post_s
       wait_bar(&misc->bar_s, (n_chunks - 1) & 1, misc);
@@ -1043,10 +1052,10 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     if (bad) {
       if (tid == 0 && misc->abort_flag == 0) hand_over(a, unit, true);
     } else {
-      const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * D;
-      const bool merge = a.mode != DASC_REFRESH_CONTINUE;
 #pragma unroll 1
-      for (int c0 = colh * 64; c0 < colh * 64 + 64; c0 += 32) {
+      for (int i = 0; i < 2; ++i) {
+        const int c0 = colh * 64 + i * 32;
+        const uint32_t write = i == 0 ? rows[0] : rows[1];
         uint32_t s[32];
         if (n_chunks > 0) {
           tmem_ld32(tlane + COL_S + c0, s);
@@ -1056,10 +1065,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
           for (int j = 0; j < 32; ++j) s[j] = 0u;  // scratch mode with an empty suffix
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int c = c0 + j;
-          if (!merge || !keep[c]) st[c * D + vrow] = __uint_as_float(s[j]) * fac_s[c];
-        }
+        for (int j = 0; j < 32; ++j)
+          if (write >> j & 1u) st[(c0 + j) * D + vrow] = __uint_as_float(s[j]) * fac_s[c0 + j];
       }
     }
   }
