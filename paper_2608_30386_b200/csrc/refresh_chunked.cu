@@ -122,7 +122,7 @@ struct Misc {
   // TMA -> producer warps: the log-decay of a chunk has landed in the Kh tile (KDA: 4 copies, one arrival with each); its raw
   // k, q have landed (4 copies, 2 without outputs)
   uint64_t g_full, kq_full;
-  // TMA -> chain warps: V of a chunk has landed (2 copies)
+  // TMA -> chain warps: V of a chunk has landed (2 copies, started by the triangular warp)
   uint64_t v_full;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;   // a bounded wait ran out: every later wait of this CTA returns at once
@@ -502,6 +502,19 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     // T = (I + A)^-1 depends on the token inputs only, so it is formed off the chain: rows 0-15 of A out of TMEM (this
     // warp's quadrant; the issuing warp brings rows 16-31), 16x16 diagonal blocks by fp32 substitution, the off-diagonal
     // block by mma.sync products.
+    // This warp also starts the copies of V, a chunk ahead: two boxes of 32 tokens x 64 values with the 128-byte swizzle (no bank
+    // conflicts for the 8 x 8 blocks it is read in).  Started by two of the chain warps they held those up for 280 cycles of every
+    // chunk; here they fall into the wait for the next A (0.3 to 1 % of a launch).
+    int v_issued = 0;
+    auto stage_v = [&](int ch) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        mbar_expect_tx(&misc->v_full, C * 128);
+        tma_load_3d(sbase + OFF_V + i * (C * 128), &tmap_v, i * 64, h, static_cast<int32_t>(tok0 + ch * C), &misc->v_full);
+      }
+      ++v_issued;
+    };
+    if (lane == 0 && n_chunks > 0) stage_v(0);
     for (int ch = 0; ch < n_chunks; ++ch) {
       const uint32_t par = ch & 1;
       wait_bar(&misc->bar_ap, par, misc);
@@ -560,8 +573,14 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
       fence_smem_to_async();
       arrive_warp(&misc->rdy_t, lane);  // -> MMA3
+      if (ch + 1 < n_chunks) {  // once V has been read by every chain warp the next chunk's may land
+        wait_bar(&misc->rdy_rhs, par, misc);
+        if (lane == 0 && !misc->abort_flag) stage_v(ch + 1);
+      }
       __syncwarp();
     }
+    // after a time-out the last copies of V may not have been waited for: they must have landed before the CTA leaves
+    if (lane == 0 && misc->abort_flag && v_issued > 0) mbar_wait_bounded(&misc->v_full, (v_issued - 1) & 1, kMaxPolls);
   } else if (warp >= 8) {
     // =============================== producer warps ===============================
     // warp = block of 32 channels; per half of the chunk, lane = (4 adjacent channels, 4 consecutive tokens), a 4 x 4
@@ -805,17 +824,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     const int vrow = quad * 32 + lane;                                     // the TMEM lane this thread owns
 
     const int g = lane >> 2, tig = lane & 3;
-    // V arrives by TMA a chunk ahead: two boxes of 32 tokens x 64 values with the 128-byte swizzle (no bank conflicts for the
-    // 8 x 8 blocks it is read in), started by one lane of the first two warps each.
-    int v_issued = 0;
-    auto stage_v = [&](int ch) {
-      mbar_expect_tx(&misc->v_full, C * 128);
-      tma_load_3d(sbase + OFF_V + warp * (C * 128), &tmap_v, warp * 64, h, static_cast<int32_t>(tok0 + ch * C), &misc->v_full);
-      ++v_issued;
-    };
-
     if (n_chunks > 0) {
-      if (warp < 2 && lane == 0) stage_v(0);
       // the start state goes into TMEM as it is; the first chunk's state pass scales it like any other
 #pragma unroll 1
       for (int c0 = colh * 64; c0 < colh * 64 + 64; c0 += 32) {
@@ -835,10 +844,9 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       const uint32_t par = ch & 1;
       const int t0 = ch * C;
       const int ntok = min(C, n_tok - t0);
-      const bool more = ch + 1 < n_chunks;
       const float *beta_c = beta_s + (ch & 3) * C;
       const float *fac_c = fac_s + par * D;
-      if (!more && tid == 0) stream_order_release();  // one chunk (2.5 us) before the end: see launch.cuh
+      if (ch + 1 == n_chunks && tid == 0) stream_order_release();  // one chunk (2.5 us) before the end: see launch.cuh
 
       // ---- (1) the previous chunk's state update is complete; this chunk's factors and tiles are ready ----
       if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
@@ -947,10 +955,6 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
       tc_fence_before_sync();
       arrive_warp(&misc->rdy_rhs, lane);  // -> MMA3 (T tile and RHS^T are ready)
-      if (warp < 2 && more) {  // V has been read by everyone: the next chunk's may land
-        wait_bar(&misc->rdy_rhs, par, misc);
-        if (lane == 0 && !misc->abort_flag) stage_v(ch + 1);
-      }
 
       // ---- (5) the part of U^T the tensor core drops when it reads it (the low 13 mantissa bits), written over
       //          the consumed RHS^T: U = U_hi + U_lo exactly ----
@@ -1025,9 +1029,6 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       tc_fence_before_sync();
       arrive_warp(&misc->tp_free, lane);  // this thread is done with the T|P|O tile region
     }
-    // after a time-out the last copies of V may not have been waited for: they must have landed before the CTA leaves
-    if (misc->abort_flag && v_issued > 0) mbar_wait_bounded(&misc->v_full, (v_issued - 1) & 1, kMaxPolls);
-
     // ---- final state: the factor still owed, then write back ----
     // Which of this warp's rows are written, a bit each, fetched before the waits: looked up row by row beside the stores, the
     // 64 loads came one behind the other and the write-back of a unit in the merge mode took 7.1 k cycles (2.6 k where all rows
