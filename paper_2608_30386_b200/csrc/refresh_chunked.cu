@@ -1,5 +1,5 @@
 // Suffix refresh, chunked form, on the Blackwell tensor cores (tcgen05 + TMEM), warp-specialised:
-// 32-token chunks, two CTAs resident per SM, four roles per CTA.
+// 32-token chunks, two CTAs resident per SM, four roles per CTA, several units (request, layer, value head) per CTA one after another.
 //
 // Eq. 1 (transposed orientation) over a chunk of C = 32 tokens starting from S_0, with
 // G_t the running sum of the log-decay inside the chunk and m the chunk midpoint:
@@ -41,6 +41,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "dasc_internal.h"
 #include "launch.cuh"
 #include "tcgen05_util.cuh"
@@ -72,16 +74,18 @@ constexpr uint32_t OFF_V = OFF_PM + 32 * 128;           // [2][32 rows][128 B] V
 constexpr uint32_t OFF_L = OFF_V + C * D * 2;           // [32][LDX] fp32 A^T (entries on and above A's diagonal are not used)
 constexpr uint32_t OFF_X = OFF_L + C * LDX * 4;         // [32][LDX] fp32 X = (I + A)^-1
 constexpr uint32_t OFF_FAC = OFF_X + C * LDX * 4;       // [2][128] fp32 state factor per channel, by chunk parity
-constexpr uint32_t OFF_POST = OFF_FAC + 2 * D * 4;      // [2][128] fp32 log-factor owed after a chunk, by chunk parity
+constexpr uint32_t OFF_POST = OFF_FAC + 2 * D * 4;      // log-factor owed after a chunk: KDA [2][128] fp32 by chunk parity, GDN [4] by chunk index mod 4
 constexpr uint32_t OFF_BETA = OFF_POST + 2 * D * 4;     // [4][32] fp32, by chunk index mod 4 (written well ahead)
 // GDN only, same ring as beta: per-token factors of the scalar decay, e1 = exp(G_t - G_m), e2 = exp(G_m - G_t)
 constexpr uint32_t OFF_E1C = OFF_BETA + 4 * C * 4;      // [4][32] fp32 e1 * (truncation compensation)
 constexpr uint32_t OFF_E2 = OFF_E1C + 4 * C * 4;        // [4][32] fp32 e2
 constexpr uint32_t OFF_BTE1 = OFF_E2 + 4 * C * 4;       // [4][32] fp32 beta * e1
-constexpr uint32_t OFF_MISC = OFF_BTE1 + 4 * C * 4;     // barriers, tmem base, abort flag
+constexpr uint32_t OFF_FIN = OFF_BTE1 + 4 * C * 4;      // [128] fp32 state factor per channel behind the last chunk of a unit
+constexpr uint32_t OFF_UNIT = OFF_FIN + D * 4;          // the CTA's units
+constexpr uint32_t OFF_MISC = OFF_UNIT + 16 * 48;       // barriers, tmem base, flags
 // GDN only: raw k (rows 0-31) and q (rows 32-63) as bf16, [2][64 rows][128 B], in the place of the K-major Kh tile
 constexpr uint32_t OFF_KQ16 = OFF_KH;
-constexpr uint32_t SMEM_BYTES = OFF_MISC + 192;
+constexpr uint32_t SMEM_BYTES = OFF_MISC + 224;
 constexpr uint32_t SMEM_ALLOC = SMEM_BYTES;
 static_assert(SMEM_ALLOC <= 113 * 1024, "two CTAs per SM");
 
@@ -105,7 +109,7 @@ struct Misc {
   // tensor core -> chain warps (one tcgen05.commit each); bar_ap also releases the triangular and the issuing warp and the
   // next log-decay (KDA) or k, q (GDN), bar_ro the Kt/Qt tile, bar_s the Kh tile of its parity (KDA)
   uint64_t bar_ap, bar_ro, bar_u, bar_o, bar_s;
-  // producer -> issuing warp and chain warps (per warp: 4 arrivals)
+  // producer -> issuing warp: the tiles of a chunk are ready (per warp: 4 arrivals; KDA one more from the triangular warp, for beta)
   uint64_t rdy_prep;
   // producer -> chain warps: the state factors of a chunk are ready (KDA per warp: 4 arrivals; GDN the first warp only: 1)
   // One barrier per chunk parity: the producer may hand over the factors of chunk n+1 before the chain warps
@@ -126,9 +130,18 @@ struct Misc {
   uint64_t v_full;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;   // a bounded wait ran out: every later wait of this CTA returns at once
-  volatile uint32_t domain_flag;  // a half-chunk decay sum left the range the midpoint factors can carry
+  int32_t n_units, all_chunks;    // this CTA's units (those that have tokens listed first) and the chunks of all of them
+  volatile uint32_t domain_flag[4];  // a half-chunk decay sum left the range the midpoint factors can carry; by unit index mod 4
 };
-static_assert(sizeof(Misc) <= 192, "Misc outgrew its shared-memory slot");
+static_assert(sizeof(Misc) <= 224, "Misc outgrew its shared-memory slot");
+
+// One of a CTA's units, as all roles read it from shared memory.
+constexpr int kMaxWalk = 16;
+struct alignas(16) Unit {
+  int64_t state;  // offset of its state, in floats
+  int64_t tok0;   // its first token in the streams of the call
+  int32_t n_tok, head, k_head, index, keep_row;
+};
 
 __device__ __forceinline__ float ex2f(float x) {
   float y;
@@ -152,23 +165,20 @@ __device__ __forceinline__ void sync_chain() { asm volatile("bar.sync 1, 256;" :
 // What comes out of a broadcast shuffle the compiler may keep in uniform registers.
 __device__ __forceinline__ int uni(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
-// Bounded wait; after one time-out no wait of this CTA lasts longer than 8 polls.  Inlined at some thirty places, so it is
-// written as the smallest loop there is: the roles' code together has to stay within reach of the instruction caches.
+// Bounded wait; after one time-out no wait of this CTA lasts longer than one poll (which itself waits for a while).  Inlined at some
+// thirty places, so it is written as the smallest loop there is: the roles' code together has to stay within reach of the
+// instruction caches.
 __device__ __forceinline__ void wait_bar(uint64_t *bar, uint32_t parity, Misc *misc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b32 n, f;\n\t"
+      "{\n\t.reg .pred p, q;\n\t.reg .b32 n, f;\n\t"
       "mov.b32 n, 0;\n"
       "POLL:\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n\t"
       "@p bra DONE;\n\t"
-      "add.u32 n, n, 1;\n\t"
-      "and.b32 f, n, 7;\n\t"
-      "setp.ne.b32 p, f, 0;\n\t"
-      "@p bra POLL;\n\t"
       "ld.volatile.shared.b32 f, [%2];\n\t"
-      "setp.ne.b32 p, f, 0;\n\t"
-      "@p bra DONE;\n\t"
-      "setp.ne.b32 p, n, %3;\n\t"
+      "add.u32 n, n, 1;\n\t"
+      "setp.ne.b32 q, n, %3;\n\t"
+      "setp.eq.and.b32 p, f, 0, q;\n\t"
       "@p bra POLL;\n\t"
       "st.volatile.shared.b32 [%2], 1;\n"
       "DONE:\n\t}" ::"r"(smem_u32(bar)),
@@ -312,7 +322,7 @@ __device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
 // WITH_O = false is the state-only variant (no outputs wanted): q is never read, the Qt rows, P and the
 // output product are left out.
 template <bool KDA, typename OT, bool WITH_O>
-__global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
+__global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_constant__ DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
                                                                 const __grid_constant__ CUtensorMap tmap_k,
                                                                 const __grid_constant__ CUtensorMap tmap_v,
                                                                 const __grid_constant__ CUtensorMap tmap_g) {
@@ -327,33 +337,12 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   float *e1c_s = reinterpret_cast<float *>(smem + OFF_E1C);
   float *e2_s = reinterpret_cast<float *>(smem + OFF_E2);
   float *bte1_s = reinterpret_cast<float *>(smem + OFF_BTE1);
+  float *fin_s = reinterpret_cast<float *>(smem + OFF_FIN);
+  Unit *const units = reinterpret_cast<Unit *>(smem + OFF_UNIT);
   Misc *misc = reinterpret_cast<Misc *>(smem + OFF_MISC);
 
   const int tid = threadIdx.x, warp = uni(tid >> 5), lane = tid & 31;
-  const int h = blockIdx.x % a.H_v;
-  const int lc = (blockIdx.x / a.H_v) % a.n_layers_in_call;
-  stream_order_wait();
-  int r = blockIdx.x / (a.H_v * a.n_layers_in_call);
-  if (a.ordered) r = uni(static_cast<const uint8_t *>(a.workspace)[kRefreshWsOrder + r]);
-  const int unit = (r * a.n_layers_in_call + lc) * a.H_v + h;
-  const int hk = h / (a.H_v / a.H_k);
-  const int layer = a.layer_begin + lc;
-  const int t_begin = uni(a.tok_begin ? a.tok_begin[r] : a.cu_seqlens[r]);
-  const int n_tok = uni(a.cu_seqlens[r + 1] - t_begin);
-  if (n_tok <= 0 && a.mode == DASC_REFRESH_CONTINUE) return;
-  if (n_tok <= a.short_thr) {  // left to the exact kernel (short_thr = -1: never)
-    if (tid == 0) hand_over(a, unit, false);
-    return;
-  }
-
-  float *st = a.state + static_cast<int64_t>(uni(a.req_idx[r])) * a.req_stride + static_cast<int64_t>(layer) * a.layer_stride +
-              static_cast<int64_t>(h) * D * D;
-  const int64_t tok0 = static_cast<int64_t>(lc) * a.total_tokens + t_begin;
-  const float *gg = a.g + (tok0 * a.H_v + h) * (KDA ? D : 1);
-  const float *gb = a.beta + tok0 * a.H_v + h;
-  OT *const go = WITH_O ? static_cast<OT *>(a.o) + (tok0 * a.H_v + h) * D : nullptr;
   const int64_t v_stride = static_cast<int64_t>(a.H_v) * D;
-  const int64_t g_stride = static_cast<int64_t>(a.H_v) * (KDA ? D : 1), b_stride = a.H_v;
 
   // ---- set-up: barriers and tensor memory ----
   if (tid == 0) {
@@ -362,7 +351,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     mbar_init(&misc->bar_u, 1);
     mbar_init(&misc->bar_o, 1);
     mbar_init(&misc->bar_s, 1);
-    mbar_init(&misc->rdy_prep, NP / 32);
+    mbar_init(&misc->rdy_prep, NP / 32 + (KDA ? 1 : 0));
     mbar_init(&misc->rdy_fac[0], KDA ? NP / 32 : 1);
     mbar_init(&misc->rdy_fac[1], KDA ? NP / 32 : 1);
     mbar_init(&misc->rdy_state, NCH / 32);
@@ -376,18 +365,57 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     mbar_init(&misc->v_full, 2);
     mbar_init(&misc->kq_full, WITH_O ? NP / 32 : NP / 64);
     misc->abort_flag = 0;
-    misc->domain_flag = 0;
+    for (int i = 0; i < 4; ++i) misc->domain_flag[i] = 0;
     fence_mbar_init();
   }
   if (warp == WARP_MMA) {
     tmem_alloc(&misc->tmem_base, TMEM_COLS);
     tmem_relinquish();
   }
+  // This CTA's units, a lane of one warp each: every gridDim.x-th, there and back (see grid_for).  Which they are is worked out
+  // before the wait for earlier work, their tokens and state are looked up behind it.
+  if (warp == WARP_T) {
+    const int64_t idx = static_cast<int64_t>(lane) * gridDim.x + ((lane & 1) ? gridDim.x - 1u - blockIdx.x : blockIdx.x);
+    bool here = lane < kMaxWalk && idx < static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
+    const uint32_t row = static_cast<uint32_t>(idx) / a.H_v;  // (the host sees to it that units fit 31 bits)
+    Unit x;
+    x.head = static_cast<int32_t>(static_cast<uint32_t>(idx) - row * a.H_v);
+    x.k_head = KDA && a.H_k == a.H_v ? x.head : x.head / (a.H_v / a.H_k);
+    int r = static_cast<int>(row / a.n_layers_in_call);
+    const int lc = static_cast<int>(row) - r * a.n_layers_in_call;
+    x.keep_row = (a.layer_begin + lc) * static_cast<int32_t>(a.rows_per_layer) + x.head * D;
+    x.n_tok = 0;
+    stream_order_wait();
+    if (here) {
+      if (a.ordered) r = static_cast<const uint8_t *>(a.workspace)[kRefreshWsOrder + r];
+      const int t_begin = a.tok_begin ? a.tok_begin[r] : a.cu_seqlens[r];
+      x.n_tok = max(a.cu_seqlens[r + 1] - t_begin, 0);
+      x.tok0 = static_cast<int64_t>(lc) * a.total_tokens + t_begin;
+      x.state = a.req_idx[r] * a.req_stride + (a.layer_begin + lc) * a.layer_stride + x.head * (D * D);
+      x.index = (r * a.n_layers_in_call + lc) * a.H_v + x.head;
+      if (x.n_tok == 0 && a.mode == DASC_REFRESH_CONTINUE) {
+        here = false;
+      } else if (x.n_tok <= a.short_thr) {  // left to the exact kernel (short_thr = -1: never)
+        hand_over(a, x.index, false);
+        here = false;
+      }
+    }
+    const uint32_t with = __ballot_sync(0xffffffffu, here && x.n_tok > 0), without = __ballot_sync(0xffffffffu, here && x.n_tok == 0);
+    const uint32_t before = (1u << lane) - 1u;
+    if (here) units[x.n_tok > 0 ? __popc(with & before) : __popc(with) + __popc(without & before)] = x;  // those without tokens last
+    const int chunks = __reduce_add_sync(0xffffffffu, here ? (x.n_tok + C - 1) / C : 0);
+    if (lane == 0) {
+      misc->n_units = __popc(with | without);
+      misc->all_chunks = chunks;
+    }
+  } else {
+    stream_order_wait();
+  }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tm = static_cast<uint32_t>(uni(static_cast<int>(misc->tmem_base)));
-  const int n_chunks = (n_tok + C - 1) / C;
+  const int all_chunks = uni(misc->all_chunks);  // of all the CTA's units: buffers and barrier phases go by the index among these
   constexpr float LOG2E = 1.4426950408889634f;
 
   constexpr uint32_t ID_N32 = idesc_tf32(128, 32, false, false);
@@ -398,10 +426,10 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
   if (warp == WARP_MMA) {
     // =========================== tensor-core issue warp ===========================
     // The whole warp walks the chunks and waits; an elected lane issues.
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      const uint32_t par = ch & 1;
+    for (int n = 0; n < all_chunks; ++n) {
+      const uint32_t par = n & 1;
       // MMA1: [Kt;Qt] Kh^T, M = 64: 16 rows in each TMEM quadrant, A's in the first two, P's in the last two.
-      if (ch == 0 && a.poll_limit_first_wait)
+      if (n == 0 && a.poll_limit_first_wait)
         wait_bar_short(&misc->rdy_prep, par, misc, a.poll_limit_first_wait);
       else
         wait_bar(&misc->rdy_prep, par, misc);
@@ -428,16 +456,19 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       // rows 16-31 of A are in this warp's quadrant: hand them to the triangular warp
       wait_bar(&misc->bar_ap, par, misc);
       tc_fence_after_sync();
-      take_a_rows<KDA>(tm + (32u << 16) + COL_AP, 16, (KDA ? beta_s : bte1_s) + (ch & 3) * C, e2_s + (ch & 3) * C, LT, lane);
+      take_a_rows<KDA>(tm + (32u << 16) + COL_AP, 16, (KDA ? beta_s : bte1_s) + (n & 3) * C, e2_s + (n & 3) * C, LT, lane);
       asm volatile("bar.arrive 3, 64;" ::: "memory");
       // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
       wait_bar(&misc->rdy_state, par, misc);
       tc_fence_after_sync();
       if (elect_one()) {
+#pragma unroll 1
+        for (int kb = 0; kb < 4; ++kb) {
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk)
-          mma_ts(tm + COL_RO, tm + COL_S + kk * 8, desc_kmajor(sbase + OFF_KQ + (kk >> 2) * (64 * 128) + (kk & 3) * 32),
-                 WITH_O ? ID_N64 : ID_N32, kk != 0);  // without outputs only the Kt rows are needed
+          for (int kk = 0; kk < 4; ++kk)
+            mma_ts(tm + COL_RO, tm + COL_S + kb * 32 + kk * 8, desc_kmajor(sbase + OFF_KQ + kk * 32) + kb * (64 * 128 / 16),
+                   WITH_O ? ID_N64 : ID_N32, (kb | kk) != 0);  // without outputs only the Kt rows are needed
+        }
         mma_commit(&misc->bar_ro);
       }
       __syncwarp();
@@ -505,21 +536,45 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     // This warp also starts the copies of V, a chunk ahead: two boxes of 32 tokens x 64 values with the 128-byte swizzle (no bank
     // conflicts for the 8 x 8 blocks it is read in).  Started by two of the chain warps they held those up for 280 cycles of every
     // chunk; here they fall into the wait for the next A (0.3 to 1 % of a launch).
-    int v_issued = 0;
-    auto stage_v = [&](int ch) {
+    int v_issued = 0, v_unit = 0, v_tok = 0;  // copies started; the next one's unit and first token in it
+    auto stage_v = [&]() {  // (the copies by the first lane)
+      const Unit &x = units[v_unit];
+      if (lane == 0 && !misc->abort_flag) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        mbar_expect_tx(&misc->v_full, C * 128);
-        tma_load_3d(sbase + OFF_V + i * (C * 128), &tmap_v, i * 64, h, static_cast<int32_t>(tok0 + ch * C), &misc->v_full);
+        for (int i = 0; i < 2; ++i) {
+          mbar_expect_tx(&misc->v_full, C * 128);
+          tma_load_3d(sbase + OFF_V + i * (C * 128), &tmap_v, i * 64, x.head, static_cast<int32_t>(x.tok0 + v_tok), &misc->v_full);
+        }
+        // the state that the unit starts from, 64 KB in one piece, is brought into L2 meanwhile
+        if (v_tok == 0 && v_issued > 0 && a.mode == DASC_REFRESH_CONTINUE)
+          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.state + x.state), "n"(D * D * 4) : "memory");
+        ++v_issued;
       }
-      ++v_issued;
+      v_tok += C;
+      if (v_tok >= x.n_tok) {
+        v_tok = 0;
+        ++v_unit;
+      }
     };
-    if (lane == 0 && n_chunks > 0) stage_v(0);
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      const uint32_t par = ch & 1;
+    // KDA: it also brings in beta, a chunk ahead (GDN: the producer warps, whose per-token factors contain it), and arrives on rdy_prep.
+    auto fetch_beta = [&]() {  // of the chunk whose copy comes next, lane = token
+      const Unit &x = units[v_unit];
+      return lane < x.n_tok - v_tok ? a.beta[(x.tok0 + v_tok + lane) * a.H_v + x.head] : 0.f;
+    };
+    if (all_chunks > 0) {
+      if (KDA) {
+        beta_s[lane] = fetch_beta();
+        arrive_warp(&misc->rdy_prep, lane);
+      }
+      stage_v();
+    }
+    for (int n = 0; n < all_chunks; ++n) {
+      const uint32_t par = n & 1;
+      float beta_next = 0.f;
+      if (KDA && n + 1 < all_chunks) beta_next = fetch_beta();
       wait_bar(&misc->bar_ap, par, misc);
       tc_fence_after_sync();
-      take_a_rows<KDA>(tm + COL_AP, 0, (KDA ? beta_s : bte1_s) + (ch & 3) * C, e2_s + (ch & 3) * C, LT, lane);
+      take_a_rows<KDA>(tm + COL_AP, 0, (KDA ? beta_s : bte1_s) + (n & 3) * C, e2_s + (n & 3) * C, LT, lane);
       tc_fence_before_sync();
       asm volatile("bar.sync 3, 64;" ::: "memory");
       arrive_warp(&misc->a_taken, lane);  // the chain warps may reuse the A|P columns
@@ -551,7 +606,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         warp_mm_store(Xm + 16, acc, 1.f, lane);
         // T -> tf32 operand tile, straight from the registers.  Its storage (shared with the P tile and the chain warps'
         // output tile) is free once the chain warps have copied the previous chunk's outputs out.
-        if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
+        if (n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
 #pragma unroll
         for (int rr = 0; rr < 16; ++rr)
           *reinterpret_cast<uint32_t *>(smem + OFF_TM + sw128_offset(32, b * 16 + rr, b * 16 + cc)) = tf32_pre(xs[rr]);
@@ -573,9 +628,13 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
       }
       fence_smem_to_async();
       arrive_warp(&misc->rdy_t, lane);  // -> MMA3
-      if (ch + 1 < n_chunks) {  // once V has been read by every chain warp the next chunk's may land
+      if (n + 1 < all_chunks) {  // once V has been read by every chain warp the next chunk's may land
+        if (KDA) {
+          beta_s[((n + 1) & 3) * C + lane] = beta_next;
+          arrive_warp(&misc->rdy_prep, lane);
+        }
         wait_bar(&misc->rdy_rhs, par, misc);
-        if (lane == 0 && !misc->abort_flag) stage_v(ch + 1);
+        stage_v();
       }
       __syncwarp();
     }
@@ -586,7 +645,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     // warp = block of 32 channels; per half of the chunk, lane = (4 adjacent channels, 4 consecutive tokens), a 4 x 4
     // tile.  The midpoint is the end of the first half: first-half exponents are (local sum - the half's total),
     // second-half exponents the local sums themselves, so the halves are independent of one another.
-    const int pw = warp - 8, ptid = tid - NCH;
+    const int pw = warp - 8;
     const int cq = lane & 7, tg = lane >> 3;
     const int c0 = pw * 32 + cq * 4;
     // Inputs come by TMA a chunk ahead into tiles they will be overwritten with (KDA) or that are
@@ -600,74 +659,89 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     int g_issued = 0, kq_issued = 0;
     // Each warp's first lane starts one box of each stream: a copy takes its issuing thread 200 to 300 cycles, and the warp that
     // issued all of them arrived 800 cycles behind the others.
-    auto stage_kq = [&](int ch) {
+    // token coordinate, head and key head of a chunk's copies, read ahead of the waits that the copies stand behind
+    int32_t cp_tok = 0, cp_head = 0, cp_k_head = 0;
+    auto next_copies = [&](const Unit &x, int t0) {
+      cp_tok = static_cast<int32_t>(x.tok0 + t0);
+      cp_head = x.head;
+      cp_k_head = x.k_head;
+    };
+    auto stage_kq = [&](int n) {
       if (!WITH_O && pw >= 2) return;
-      const uint32_t dst = sbase + (KDA ? OFF_KHT + (ch & 1) * (128 * 128) : OFF_KQ16) + (pw & 1) * (RAW_ROWS * 128);
-      const int32_t z = static_cast<int32_t>(tok0 + ch * C);
+      const uint32_t dst = sbase + (KDA ? OFF_KHT + (n & 1) * (128 * 128) : OFF_KQ16) + (pw & 1) * (RAW_ROWS * 128);
       mbar_expect_tx(&misc->kq_full, C * 128);
       if (pw < 2)
-        tma_load_3d(dst, &tmap_k, pw * 64, hk, z, &misc->kq_full);
+        tma_load_3d(dst, &tmap_k, pw * 64, cp_k_head, cp_tok, &misc->kq_full);
       else
-        tma_load_3d(dst + OFF_RAW_Q, &tmap_q, (pw & 1) * 64, hk, z, &misc->kq_full);
+        tma_load_3d(dst + OFF_RAW_Q, &tmap_q, (pw & 1) * 64, cp_k_head, cp_tok, &misc->kq_full);
       ++kq_issued;
     };
-    auto stage_g = [&](int ch) {
+    auto stage_g = [&]() {
       mbar_expect_tx(&misc->g_full, C * 128);
-      tma_load_3d(sbase + OFF_KH + pw * (C * 128), &tmap_g, pw * 32, h, static_cast<int32_t>(tok0 + ch * C), &misc->g_full);
+      tma_load_3d(sbase + OFF_KH + pw * (C * 128), &tmap_g, pw * 32, cp_head, cp_tok, &misc->g_full);
       ++g_issued;
     };
-    if (lane == 0 && n_chunks > 0) {
-      if (KDA) stage_g(0);
+    if (lane == 0 && all_chunks > 0) {
+      next_copies(units[0], 0);
+      if (KDA) stage_g();
       stage_kq(0);
     }
-    // Per-token scalars, by the first warp (lane = token): a chunk's go to their ring slots (the chain warps are at most two
+    // GDN, per-token scalars, by the first warp (lane = token): a chunk's go to their ring slots (the chain warps are at most two
     // chunks behind) while MMA1 of the chunk before runs; the next chunk's are fetched then and stored one chunk later.
-    const float *gbp = gb + static_cast<int64_t>(lane) * b_stride, *ggp = gg + static_cast<int64_t>(lane) * g_stride;
-    float beta_next = (n_chunks > 0 && ptid < min(C, n_tok)) ? *gbp : 0.f;
-    float gsc_next = (!KDA && n_chunks > 0 && ptid < min(C, n_tok)) ? *ggp : 0.f;
-    float post_prev = 0.f;  // GDN: the factor owed by the previous chunk
-    auto scalars = [&](int ch) {
-      const int slot = (ch & 3) * C + lane;
+    float beta_next = 0.f, gsc_next = 0.f;
+    auto fetch_scalars = [&](const Unit &x, int t0) {
+      const bool here = lane < x.n_tok - t0;
+      const int64_t off = (x.tok0 + t0 + lane) * a.H_v + x.head;
+      beta_next = here ? a.beta[off] : 0.f;
+      gsc_next = here ? a.g[off] : 0.f;
+    };
+    float post_prev = 0.f;  // the factor owed by the previous chunk
+    // One scalar log-decay per token: the running sums and the per-token factors are formed here; nothing per
+    // channel needs an exponential, and k, q stay exactly their bf16 values:
+    //   e1_t = exp(G_t - G_m), e2_t = exp(G_m - G_t) with m the end of the first half;
+    //   MMA1 works on raw k, q (bf16 tile), MMA2 on raw k, q widened to tf32 containers, MMA5 on k_t e2_t;
+    //   e1_t goes onto the rows of A, R and the outputs where they leave tensor memory, e2_j onto the columns of A, P.
+    auto scalars = [&](int n, int u, int t0) {  // chunk n of the CTA: the tokens of unit u from t0 on
+      const int slot = (n & 3) * C + lane;
       const float beta = beta_next;
       beta_s[slot] = beta;
-      if constexpr (!KDA) {
-        // ---- GDN: one scalar log-decay per token: the running sums and the per-token factors are formed here; nothing per
-        // channel needs an exponential, and k, q stay exactly their bf16 values:
-        //   e1_t = exp(G_t - G_m), e2_t = exp(G_m - G_t) with m the end of the first half;
-        //   MMA1 works on raw k, q (bf16 tile), MMA2 on raw k, q widened to tf32 containers, MMA5 on k_t e2_t;
-        //   e1_t goes onto the rows of A, R and the outputs where they leave tensor memory, e2_j onto the columns of A, P.
-        float incl = gsc_next;
+      float incl = gsc_next;
 #pragma unroll
-        for (int dlt = 1; dlt < 32; dlt <<= 1) {
-          const float x = __shfl_up_sync(0xffffffffu, incl, dlt);
-          if (lane >= dlt) incl += x;
-        }
-        const float tot0 = __shfl_sync(0xffffffffu, incl, 15);          // G_m: the first half's total
-        const float tot1 = __shfl_sync(0xffffffffu, incl, 31) - tot0;   // G_C - G_m
-        const float d2 = (incl - tot0) * LOG2E;
-        const float e1 = ex2f(d2), e2 = ex2f(-d2);
-        e1c_s[slot] = e1 * kTruncComp;
-        e2_s[slot] = e2;
-        bte1_s[slot] = beta * e1;
-        if (lane == 0 && (!(fabsf(tot0) <= kMaxHalfDecay) || !(fabsf(tot1) <= kMaxHalfDecay))) misc->domain_flag = 1;  // also true for NaN
-        // state factor from where the previous chunk left the state to this chunk's midpoint, and the factor owed after
-        // it; scalars here, written for every channel so that the chain warps read them as they do for KDA
-        const float f = ex2f((post_prev + tot0) * LOG2E);
-        post_prev = tot1;
-        *reinterpret_cast<float4 *>(fac_s + (ch & 1) * D + lane * 4) = make_float4(f, f, f, f);
-        *reinterpret_cast<float4 *>(post_s + (ch & 1) * D + lane * 4) = make_float4(tot1, tot1, tot1, tot1);
-        arrive_warp(&misc->rdy_fac[ch & 1], lane);
+      for (int dlt = 1; dlt < 32; dlt <<= 1) {
+        const float x = __shfl_up_sync(0xffffffffu, incl, dlt);
+        if (lane >= dlt) incl += x;
       }
-      const bool v1 = lane < n_tok - (ch + 1) * C;
-      gbp += C * b_stride;
-      ggp += C * g_stride;
-      beta_next = v1 ? *gbp : 0.f;
-      if (!KDA) gsc_next = v1 ? *ggp : 0.f;
+      const float tot0 = __shfl_sync(0xffffffffu, incl, 15);          // G_m: the first half's total
+      const float tot1 = __shfl_sync(0xffffffffu, incl, 31) - tot0;   // G_C - G_m
+      const float d2 = (incl - tot0) * LOG2E;
+      const float e1 = ex2f(d2), e2 = ex2f(-d2);
+      e1c_s[slot] = e1 * kTruncComp;
+      e2_s[slot] = e2;
+      bte1_s[slot] = beta * e1;
+      if (lane == 0 && (!(fabsf(tot0) <= kMaxHalfDecay) || !(fabsf(tot1) <= kMaxHalfDecay))) misc->domain_flag[u & 3] = 1;  // also true for NaN
+      // state factor from where the previous chunk left the state to this chunk's midpoint, and the factor owed after
+      // it; scalars here, written for every channel so that the chain warps read them as they do for KDA
+      if (t0 == 0) post_prev = 0.f;
+      const float f = ex2f((post_prev + tot0) * LOG2E);
+      post_prev = tot1;
+      *reinterpret_cast<float4 *>(fac_s + (n & 1) * D + lane * 4) = make_float4(f, f, f, f);
+      if (lane == 0) post_s[n & 3] = tot1;
+      arrive_warp(&misc->rdy_fac[n & 1], lane);
+      t0 += C;
+      if (t0 >= units[u].n_tok) {
+        t0 = 0;
+        ++u;
+      }
+      if (n + 1 < all_chunks) fetch_scalars(units[u], t0);
     };
-    if (pw == 0 && n_chunks > 0) scalars(0);
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      const uint32_t par = ch & 1;
-      const int t0 = ch * C, ntok = min(C, n_tok - t0);
+    if (!KDA && pw == 0 && all_chunks > 0) {
+      fetch_scalars(units[0], 0);
+      scalars(0, 0, 0);
+    }
+    int n_tok = units[0].n_tok;
+    for (int n = 0, u = 0, t0 = 0; n < all_chunks; ++n) {
+      const uint32_t par = n & 1;
+      const int ntok = min(C, n_tok - t0);
       unsigned char *kht_tile = smem + OFF_KHT + par * (128 * 128);
       unsigned char *raw = KDA ? kht_tile : smem + OFF_KQ16;
       if (!KDA) asm volatile("bar.sync 2, 128;" ::: "memory");   // the per-token factors are visible to all producer warps
@@ -729,7 +803,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
             // The factor that takes the state from where the previous chunk left it to this chunk's midpoint needs
             // the first half's sums only: it is handed to the chain warps before the tiles are built.
             if (tg == 0) {
-              const float4 pp = ch > 0 ? *reinterpret_cast<const float4 *>(post_s + (par ^ 1) * D + c0) : make_float4(0.f, 0.f, 0.f, 0.f);
+              const float4 pp = t0 > 0 ? *reinterpret_cast<const float4 *>(post_s + (par ^ 1) * D + c0) : make_float4(0.f, 0.f, 0.f, 0.f);
               *reinterpret_cast<float4 *>(fac_s + par * D + c0) =
                   make_float4(ex2f((pp.x + tot[0]) * LOG2E), ex2f((pp.y + tot[1]) * LOG2E), ex2f((pp.z + tot[2]) * LOG2E),
                               ex2f((pp.w + tot[3]) * LOG2E));
@@ -742,7 +816,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
           }
           asm volatile("bar.sync 2, 128;" ::: "memory");  // this half's raw k, q have been read: Kh may take their place
           // the Kt/Qt tile is free once MMA2 of the previous chunk has completed
-          if (ch > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
+          if (n > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
           uint64_t run01 = pack2(run0[0], run0[1]), run23 = pack2(run0[2], run0[3]);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -779,7 +853,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
             *reinterpret_cast<uint4 *>(kht_tile + (om0 ^ (j << 5)) + j * 128) = khv;
           }
         } else {
-          if (ch > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
+          if (n > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             unsigned char *pk = smem + OFF_KQ + (ok0 ^ (j << 4)) + j * 128;
@@ -787,7 +861,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
             *reinterpret_cast<uint4 *>(pk) = kf;
             if (WITH_O)
               *reinterpret_cast<uint4 *>(pk + 32 * 128) = make_uint4(qw[j].x << 16, qw[j].x & 0xFFFF0000u, qw[j].y << 16, qw[j].y & 0xFFFF0000u);
-            const float e2 = e2_s[(ch & 3) * C + tr + j];
+            const float e2 = e2_s[(n & 3) * C + tr + j];
             *reinterpret_cast<uint4 *>(kht_tile + (om0 ^ (j << 5)) + j * 128) =
                 make_uint4(tf32_pre(__uint_as_float(kf.x) * e2), tf32_pre(__uint_as_float(kf.y) * e2),
                            tf32_pre(__uint_as_float(kf.z) * e2), tf32_pre(__uint_as_float(kf.w) * e2));
@@ -795,20 +869,27 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
         }
       }
       // the exponents of this chunk may have overflowed: the unit will not be written back
-      if (KDA && out_of_range && tg == 0) misc->domain_flag = 1;
+      if (KDA && out_of_range && tg == 0) misc->domain_flag[u & 3] = 1;
       fence_smem_to_async();
       arrive_warp(&misc->rdy_prep, lane);  // -> MMA1
-      if (ch + 1 < n_chunks) {
-        if (pw == 0) scalars(ch + 1);
+      t0 += C;
+      if (t0 >= n_tok) {
+        t0 = 0;
+        ++u;
+      }
+      if (n + 1 < all_chunks) {
+        next_copies(units[u], t0);
+        n_tok = units[u].n_tok;
+        if (!KDA && pw == 0) scalars(n + 1, u, t0);
         // The next raw k, q (KDA) land once MMA5 of the previous chunk has read the Kh tile of that parity; the next
         // log-decay (KDA) or k, q (GDN) once MMA1 of this chunk has read the tile they go to.
         if (KDA) {
-          if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
-          if (lane == 0 && !misc->abort_flag) stage_kq(ch + 1);
+          if (n > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
+          if (lane == 0 && !misc->abort_flag) stage_kq(n + 1);
         }
         wait_bar(&misc->bar_ap, par, misc);
         if (lane == 0 && !misc->abort_flag) {
-          if (KDA) stage_g(ch + 1); else stage_kq(ch + 1);
+          if (KDA) stage_g(); else stage_kq(n + 1);
         }
       }
     }
@@ -824,250 +905,264 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(DascRefreshArgs 
     const int vrow = quad * 32 + lane;                                     // the TMEM lane this thread owns
 
     const int g = lane >> 2, tig = lane & 3;
-    if (n_chunks > 0) {
-      // the start state goes into TMEM as it is; the first chunk's state pass scales it like any other
+    int n = 0;  // index among the CTA's chunks
 #pragma unroll 1
-      for (int c0 = colh * 64; c0 < colh * 64 + 64; c0 += 32) {
-        uint32_t s[32];
-        if (a.mode == DASC_REFRESH_CONTINUE) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) s[j] = __float_as_uint(st[(c0 + j) * D + vrow]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) s[j] = 0u;
-        }
-        tmem_st32(tlane + COL_S + c0, s);
-      }
-      tmem_st_wait();
-    }
-    for (int ch = 0; ch < n_chunks; ++ch) {
-      const uint32_t par = ch & 1;
-      const int t0 = ch * C;
-      const int ntok = min(C, n_tok - t0);
-      const float *beta_c = beta_s + (ch & 3) * C;
-      const float *fac_c = fac_s + par * D;
-      if (ch + 1 == n_chunks && tid == 0) stream_order_release();  // one chunk (2.5 us) before the end: see launch.cuh
-
-      // ---- (1) the previous chunk's state update is complete; this chunk's factors and tiles are ready ----
-      if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
-      wait_bar(&misc->rdy_fac[par], (ch >> 1) & 1, misc);
-      tc_fence_after_sync();
-
-      // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
-      {
-        uint64_t f[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const uint64_t *>(fac_c + colh * 64 + 8 * i + 2 * tig);
+    for (int u = 0; u < uni(misc->n_units); ++u) {
+      const Unit &x = units[u];
+      // where this thread's part of the outputs of a chunk starts (bf16: 16 bytes of every 16th token; fp32: see below)
+      OT *go = WITH_O ? static_cast<OT *>(a.o) + (x.tok0 * a.H_v + x.head) * D : nullptr;
+      if (WITH_O && sizeof(OT) == 2) go += (tid >> 4) * v_stride + (tid & 15) * 8;
+      const int n_tok = uni(x.n_tok), n_chunks = (n_tok + C - 1) / C;
+      if (n_chunks > 0) {
+        // the start state goes into TMEM as it is; the first chunk's state pass scales it like any other.  (The state of the unit
+        // before has been read out by the same threads.)
 #pragma unroll 1
-        for (uint32_t hh = 0; hh < 2; ++hh) {  // lanes 0-15, 16-31 of the quadrant
-          const uint32_t addr = tlane + (hh << 20) + COL_S + colh * 64;
+        for (int c0 = colh * 64; c0 < colh * 64 + 64; c0 += 32) {
+          const float *const st_c = a.state + x.state + (c0 * D + vrow);
           uint32_t s[32];
-          tmem_ld_16x256b(addr, s);
-          tmem_ld_wait();
+          if (a.mode == DASC_REFRESH_CONTINUE) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            scale2(s[4 * i + 0], s[4 * i + 1], f[i]);
-            scale2(s[4 * i + 2], s[4 * i + 3], f[i]);
+            for (int j = 0; j < 32; ++j) s[j] = __float_as_uint(st_c[j * D]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) s[j] = 0u;
           }
-          tmem_st_16x256b(addr, s);
+          tmem_st32(tlane + COL_S + c0, s);
         }
         tmem_st_wait();
       }
-      tc_fence_before_sync();
-      arrive_warp(&misc->rdy_state, lane);  // -> MMA2
+      for (int ch = 0; ch < n_chunks; ++ch, ++n) {
+        const uint32_t par = n & 1;
+        const int ntok = min(C, n_tok - ch * C);
+        const float *beta_c = beta_s + (n & 3) * C;
+        const float *fac_c = fac_s + par * D;
+        if (n + 1 == all_chunks && tid == 0) stream_order_release();  // one chunk (2.5 us) before the end: see launch.cuh
 
-      // ---- (3) P = lower_incl_diag(Qt Kh^T) out of TMEM (rows 0-15, 16-31 are in the third and fourth quadrant) straight to
-      //          its operand tile.  GDN: the raw q_t . k_j gets its column factor e2_j here, the row factor e1_t is applied
-      //          to the outputs ----
-      if (WITH_O && quad >= 2) {
-        wait_bar(&misc->bar_ap, par, misc);
+        // ---- (1) the previous chunk's state update is complete; this chunk's factors and tiles are ready ----
+        if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
+        wait_bar(&misc->rdy_fac[par], (n >> 1) & 1, misc);
         tc_fence_after_sync();
-        uint32_t x[8];
-        tmem_ld_16x256b(tlane + COL_AP + colh * 16, x);
-        if (ch > 0) wait_bar(&misc->tp_free, par ^ 1, misc);  // the previous chunk's outputs have left this storage
-        tmem_ld_wait();
-        const int t = (quad - 2) * 16 + g;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const int j = colh * 16 + 8 * i + 2 * tig;
-          float2 e = make_float2(kInvTruncComp, kInvTruncComp);
-          if constexpr (!KDA) {
-            const float2 e2 = *reinterpret_cast<const float2 *>(e2_s + (ch & 3) * C + j);
-            e.x *= e2.x;
-            e.y *= e2.y;
-          }
-          unsigned char *const p = smem + OFF_PM + sw128_offset(32, t, j);
-          *reinterpret_cast<uint2 *>(p) = make_uint2(j <= t ? tf32_pre(__uint_as_float(x[4 * i]) * e.x) : 0u,
-                                                     j + 1 <= t ? tf32_pre(__uint_as_float(x[4 * i + 1]) * e.y) : 0u);
-          *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(j <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 2]) * e.x) : 0u,
-                                                            j + 1 <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 3]) * e.y) : 0u);
-        }
-        fence_smem_to_async();
-      }
 
-      // ---- (4) RHS^T = beta (V - R)^T as a tf32 pair: high over R^T, low in the consumed A|P columns ----
-      wait_bar(&misc->bar_ro, par, misc);
-      tc_fence_after_sync();
-      // A's and P's columns are about to be overwritten: A's by warps that wait for its readers (the issuing warp read its rows
-      // before it issued MMA2), P's by the warps that read them
-      wait_bar(&misc->a_taken, par, misc);
-      wait_bar(&misc->v_full, par, misc);
-      {
-        const int tb = colh * 16;
-        // blocks of one ldmatrix: tokens 0-7 of the half with values 0-7, 8-15, tokens 8-15 with the same
-        const int vt = tb + (lane >> 4) * 8 + (lane & 7);
+        // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
+        {
+          uint64_t f[8];
 #pragma unroll
-        for (uint32_t hh = 0; hh < 2; ++hh) {
-          uint32_t x[8], lo[8], vv[4];
-          tmem_ld_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
-          ldmatrix_x4_trans(vv, sbase + OFF_V + (quad >> 1) * (C * 128) + vt * 128 +
-                                    ((((quad & 1) * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (vt & 7)) << 4));
-          if (ntok < C) {
-            // the boxes reached past the request's last token: those values are other tokens' (zeros past the end of the stream)
+          for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const uint64_t *>(fac_c + colh * 64 + 8 * i + 2 * tig);
+#pragma unroll 1
+          for (uint32_t hh = 0; hh < 2; ++hh) {  // lanes 0-15, 16-31 of the quadrant
+            const uint32_t addr = tlane + (hh << 20) + COL_S + colh * 64;
+            uint32_t s[32];
+            tmem_ld_16x256b(addr, s);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              scale2(s[4 * i + 0], s[4 * i + 1], f[i]);
+              scale2(s[4 * i + 2], s[4 * i + 3], f[i]);
+            }
+            tmem_st_16x256b(addr, s);
+          }
+          tmem_st_wait();
+        }
+        tc_fence_before_sync();
+        arrive_warp(&misc->rdy_state, lane);  // -> MMA2
+
+        // ---- (3) P = lower_incl_diag(Qt Kh^T) out of TMEM (rows 0-15, 16-31 are in the third and fourth quadrant) straight to
+        //          its operand tile.  GDN: the raw q_t . k_j gets its column factor e2_j here, the row factor e1_t is applied
+        //          to the outputs ----
+        if (WITH_O && quad >= 2) {
+          wait_bar(&misc->bar_ap, par, misc);
+          tc_fence_after_sync();
+          uint32_t x[8];
+          tmem_ld_16x256b(tlane + COL_AP + colh * 16, x);
+          if (n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);  // the previous chunk's outputs have left this storage
+          tmem_ld_wait();
+          const int t = (quad - 2) * 16 + g;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int j = colh * 16 + 8 * i + 2 * tig;
+            float2 e = make_float2(kInvTruncComp, kInvTruncComp);
+            if constexpr (!KDA) {
+              const float2 e2 = *reinterpret_cast<const float2 *>(e2_s + (n & 3) * C + j);
+              e.x *= e2.x;
+              e.y *= e2.y;
+            }
+            unsigned char *const p = smem + OFF_PM + sw128_offset(32, t, j);
+            *reinterpret_cast<uint2 *>(p) = make_uint2(j <= t ? tf32_pre(__uint_as_float(x[4 * i]) * e.x) : 0u,
+                                                       j + 1 <= t ? tf32_pre(__uint_as_float(x[4 * i + 1]) * e.y) : 0u);
+            *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(j <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 2]) * e.x) : 0u,
+                                                              j + 1 <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 3]) * e.y) : 0u);
+          }
+          fence_smem_to_async();
+        }
+
+        // ---- (4) RHS^T = beta (V - R)^T as a tf32 pair: high over R^T, low in the consumed A|P columns ----
+        wait_bar(&misc->bar_ro, par, misc);
+        tc_fence_after_sync();
+        // A's and P's columns are about to be overwritten: A's by warps that wait for its readers (the issuing warp read its rows
+        // before it issued MMA2), P's by the warps that read them
+        wait_bar(&misc->a_taken, par, misc);
+        wait_bar(&misc->v_full, par, misc);
+        {
+          const int tb = colh * 16;
+          // blocks of one ldmatrix: tokens 0-7 of the half with values 0-7, 8-15, tokens 8-15 with the same
+          const int vt = tb + (lane >> 4) * 8 + (lane & 7);
+#pragma unroll
+          for (uint32_t hh = 0; hh < 2; ++hh) {
+            uint32_t x[8], lo[8], vv[4];
+            tmem_ld_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
+            ldmatrix_x4_trans(vv, sbase + OFF_V + (quad >> 1) * (C * 128) + vt * 128 +
+                                      ((((quad & 1) * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (vt & 7)) << 4));
+            if (ntok < C) {
+              // the boxes reached past the request's last token: those values are other tokens' (zeros past the end of the stream)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int t = tb + (i >> 1) * 8 + 2 * tig;
+                if (t >= ntok) vv[i] = 0u;
+                else if (t + 1 >= ntok) vv[i] &= 0xFFFFu;
+              }
+            }
+            tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const int t = tb + (i >> 1) * 8 + 2 * tig;
-              if (t >= ntok) vv[i] = 0u;
-              else if (t + 1 >= ntok) vv[i] &= 0xFFFFu;
+              uint64_t r = pack2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+              // GDN: the product is k_t S' on the raw keys; its row factor e1_t (with the truncation compensation) comes here
+              if constexpr (!KDA) r = mul2(*reinterpret_cast<const uint64_t *>(e1c_s + (n & 3) * C + t), r);
+              r = mul2(*reinterpret_cast<const uint64_t *>(beta_c + t), sub2(pack2(bf16lo(vv[i]), bf16hi(vv[i])), r));
+              // the high part is the value itself, which the tensor core truncates on reading; the low part the exact rest
+              float r0, r1;
+              unpack2(r, r0, r1);
+              x[2 * i] = __float_as_uint(r0);
+              x[2 * i + 1] = __float_as_uint(r1);
+              unpack2(sub2(r, pack2(__uint_as_float(x[2 * i] & 0xFFFFE000u), __uint_as_float(x[2 * i + 1] & 0xFFFFE000u))), r0, r1);
+              lo[2 * i] = tf32_pre(r0);
+              lo[2 * i + 1] = tf32_pre(r1);
             }
+            tmem_st_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
+            tmem_st_16x256b(tlane + (hh << 20) + COL_AP + tb, lo);
           }
+          tmem_st_wait();
+        }
+        tc_fence_before_sync();
+        arrive_warp(&misc->rdy_rhs, lane);  // -> MMA3 (T tile and RHS^T are ready)
+
+        // ---- (5) the part of U^T the tensor core drops when it reads it (the low 13 mantissa bits), written over
+        //          the consumed RHS^T: U = U_hi + U_lo exactly ----
+        wait_bar(&misc->bar_u, par, misc);
+        tc_fence_after_sync();
+        {
+          const int tb = colh * 16;
+          uint32_t x[16];
+          tmem_ld16(tlane + COL_U + tb, x);
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int t = tb + (i >> 1) * 8 + 2 * tig;
-            uint64_t r = pack2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
-            // GDN: the product is k_t S' on the raw keys; its row factor e1_t (with the truncation compensation) comes here
-            if constexpr (!KDA) r = mul2(*reinterpret_cast<const uint64_t *>(e1c_s + (ch & 3) * C + t), r);
-            r = mul2(*reinterpret_cast<const uint64_t *>(beta_c + t), sub2(pack2(bf16lo(vv[i]), bf16hi(vv[i])), r));
-            // the high part is the value itself, which the tensor core truncates on reading; the low part the exact rest
-            float r0, r1;
-            unpack2(r, r0, r1);
-            x[2 * i] = __float_as_uint(r0);
-            x[2 * i + 1] = __float_as_uint(r1);
-            unpack2(sub2(r, pack2(__uint_as_float(x[2 * i] & 0xFFFFE000u), __uint_as_float(x[2 * i + 1] & 0xFFFFE000u))), r0, r1);
-            lo[2 * i] = tf32_pre(r0);
-            lo[2 * i + 1] = tf32_pre(r1);
-          }
-          tmem_st_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
-          tmem_st_16x256b(tlane + (hh << 20) + COL_AP + tb, lo);
+          for (int j = 0; j < 16; ++j)
+            x[j] = tf32_pre(__uint_as_float(x[j]) - __uint_as_float(x[j] & 0xFFFFE000u));
+          tmem_st16(tlane + COL_RO + tb, x);
+          tmem_st_wait();
         }
-        tmem_st_wait();
-      }
-      tc_fence_before_sync();
-      arrive_warp(&misc->rdy_rhs, lane);  // -> MMA3 (T tile and RHS^T are ready)
+        tc_fence_before_sync();
+        arrive_warp(&misc->rdy_u, lane);  // -> MMA4, MMA5
 
-      // ---- (5) the part of U^T the tensor core drops when it reads it (the low 13 mantissa bits), written over
-      //          the consumed RHS^T: U = U_hi + U_lo exactly ----
-      wait_bar(&misc->bar_u, par, misc);
-      tc_fence_after_sync();
-      {
-        const int tb = colh * 16;
-        uint32_t x[16];
-        tmem_ld16(tlane + COL_U + tb, x);
-        tmem_ld_wait();
+        // ---- (6) outputs of this chunk ----
+        wait_bar(&misc->bar_o, par, misc);
+        tc_fence_after_sync();
+        if (WITH_O) {
+          const int tb = colh * 16;
+          const int ot = tb + (lane >> 4) * 8 + (lane & 7);  // blocks of one stmatrix: as for V
+          uint32_t xx[2][8];
+          tmem_ld_16x256b(tlane + COL_RO + 32 + tb, xx[0]);
+          tmem_ld_16x256b(tlane + (1u << 20) + COL_RO + 32 + tb, xx[1]);
+          tmem_ld_wait();
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          x[j] = tf32_pre(__uint_as_float(x[j]) - __uint_as_float(x[j] & 0xFFFFE000u));
-        tmem_st16(tlane + COL_RO + tb, x);
-        tmem_st_wait();
-      }
-      tc_fence_before_sync();
-      arrive_warp(&misc->rdy_u, lane);  // -> MMA4, MMA5
-
-      // ---- (6) outputs of this chunk ----
-      wait_bar(&misc->bar_o, par, misc);
-      tc_fence_after_sync();
-      if (WITH_O) {
-        const int tb = colh * 16;
-        const int ot = tb + (lane >> 4) * 8 + (lane & 7);  // blocks of one stmatrix: as for V
-        uint32_t xx[2][8];
-        tmem_ld_16x256b(tlane + COL_RO + 32 + tb, xx[0]);
-        tmem_ld_16x256b(tlane + (1u << 20) + COL_RO + 32 + tb, xx[1]);
-        tmem_ld_wait();
+          for (uint32_t hh = 0; hh < 2; ++hh) {
+            uint32_t(&x)[8] = xx[hh];
+            if constexpr (!KDA) {
+              // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
+              // the truncation compensation
 #pragma unroll
-        for (uint32_t hh = 0; hh < 2; ++hh) {
-          uint32_t(&x)[8] = xx[hh];
-          if constexpr (!KDA) {
-            // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
-            // the truncation compensation
+              for (int i = 0; i < 2; ++i) {
+                const float2 e = *reinterpret_cast<const float2 *>(e1c_s + (n & 3) * C + tb + 8 * i + 2 * tig);
+                x[4 * i + 0] = __float_as_uint(__uint_as_float(x[4 * i + 0]) * (e.x * a.q_scale));
+                x[4 * i + 1] = __float_as_uint(__uint_as_float(x[4 * i + 1]) * (e.y * a.q_scale));
+                x[4 * i + 2] = __float_as_uint(__uint_as_float(x[4 * i + 2]) * (e.x * a.q_scale));
+                x[4 * i + 3] = __float_as_uint(__uint_as_float(x[4 * i + 3]) * (e.y * a.q_scale));
+              }
+            }
+            if constexpr (sizeof(OT) == 2) {
+              uint32_t w[4];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const float2 e = *reinterpret_cast<const float2 *>(e1c_s + (ch & 3) * C + tb + 8 * i + 2 * tig);
-              x[4 * i + 0] = __float_as_uint(__uint_as_float(x[4 * i + 0]) * (e.x * a.q_scale));
-              x[4 * i + 1] = __float_as_uint(__uint_as_float(x[4 * i + 1]) * (e.y * a.q_scale));
-              x[4 * i + 2] = __float_as_uint(__uint_as_float(x[4 * i + 2]) * (e.x * a.q_scale));
-              x[4 * i + 3] = __float_as_uint(__uint_as_float(x[4 * i + 3]) * (e.y * a.q_scale));
+              for (int i = 0; i < 4; ++i) w[i] = pack_bf16x2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+              stmatrix_x4_trans(sbase + OFF_TM + ot * 256 + (((quad * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (ot & 7)) << 4), w[0], w[1], w[2], w[3]);
+            } else {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int t = tb + (i >> 1) * 8 + 2 * tig, v = quad * 32 + hh * 16 + (i & 1) * 8 + g;
+                if (t < ntok) go[t * v_stride + v] = __uint_as_float(x[2 * i]);
+                if (t + 1 < ntok) go[(t + 1) * v_stride + v] = __uint_as_float(x[2 * i + 1]);
+              }
             }
           }
           if constexpr (sizeof(OT) == 2) {
-            uint32_t w[4];
+            // through shared memory (the T and P tiles are free now) so that global stores are 16 bytes wide
+            sync_chain();
+            const int j = tid & 15;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) w[i] = pack_bf16x2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
-            stmatrix_x4_trans(sbase + OFF_TM + ot * 256 + (((quad * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (ot & 7)) << 4), w[0], w[1], w[2], w[3]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int t = tb + (i >> 1) * 8 + 2 * tig, v = quad * 32 + hh * 16 + (i & 1) * 8 + g;
-              if (t < ntok) go[(t0 + t) * v_stride + v] = __uint_as_float(x[2 * i]);
-              if (t + 1 < ntok) go[(t0 + t + 1) * v_stride + v] = __uint_as_float(x[2 * i + 1]);
+            for (int i = 0; i < 2; ++i) {
+              const int t = (tid >> 4) + 16 * i;
+              if (t < ntok)
+                *reinterpret_cast<uint4 *>(go + i * 16 * v_stride) =
+                    *reinterpret_cast<const uint4 *>(smem + OFF_TM + t * 256 + ((j ^ (t & 7)) << 4));
             }
           }
+          go += C * v_stride;
         }
-        if constexpr (sizeof(OT) == 2) {
-          // through shared memory (the T and P tiles are free now) so that global stores are 16 bytes wide
-          sync_chain();
-          const int j = tid & 15;
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int t = (tid >> 4) + 16 * i;
-            if (t < ntok)
-              *reinterpret_cast<uint4 *>(reinterpret_cast<char *>(go + (t0 + t) * v_stride) + j * 16) =
-                  *reinterpret_cast<const uint4 *>(smem + OFF_TM + t * 256 + ((j ^ (t & 7)) << 4));
-          }
-        }
+        tc_fence_before_sync();
+        arrive_warp(&misc->tp_free, lane);  // this thread is done with the T|P|O tile region
       }
-      tc_fence_before_sync();
-      arrive_warp(&misc->tp_free, lane);  // this thread is done with the T|P|O tile region
-    }
-    // ---- final state: the factor still owed, then write back ----
-    // Which of this warp's rows are written, a bit each, fetched before the waits: looked up row by row beside the stores, the
-    // 64 loads came one behind the other and the write-back of a unit in the merge mode took 7.1 k cycles (2.6 k where all rows
-    // are written); 32 requests of 1 .. 128 tokens x 4 layers x 32 heads, state only: 277 -> 262 us.
-    uint32_t rows[2];
+      // ---- final state: the factor still owed, then write back ----
+      // Which of this warp's rows are written, a bit each, fetched before the waits: looked up row by row beside the stores, the
+      // 64 loads came one behind the other and the write-back of a unit in the merge mode took 7.1 k cycles (2.6 k where all rows
+      // are written); 32 requests of 1 .. 128 tokens x 4 layers x 32 heads, state only: 277 -> 262 us.
+      uint32_t rows[2];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * D;
-      rows[i] = __ballot_sync(0xffffffffu, a.mode == DASC_REFRESH_CONTINUE || !keep[colh * 64 + i * 32 + lane]);
-    }
-    if (n_chunks > 0) {
-      wait_bar(&misc->rdy_prep, (n_chunks - 1) & 1, misc);  // the last chunk's post_s
-      wait_bar(&misc->bar_s, (n_chunks - 1) & 1, misc);
-    }
-    // fac_s is free: the producer has finished (its last arrival was waited for above)
-    if (tid < D) fac_s[tid] = n_chunks > 0 ? ex2f(post_s[((n_chunks - 1) & 1) * D + tid] * LOG2E) : 1.f;
-    sync_chain();
-    tc_fence_after_sync();
-    // A unit whose decay left the range, or whose CTA gave up on a wait, is NOT written back: its stored state keeps
-    // the bits it had before the call, so that it can be replayed by the exact kernel (or by the caller).
-    const bool bad = misc->abort_flag != 0 || misc->domain_flag != 0;
-    if (bad) {
-      if (tid == 0 && misc->abort_flag == 0) hand_over(a, unit, true);
-    } else {
-#pragma unroll 1
       for (int i = 0; i < 2; ++i) {
-        const int c0 = colh * 64 + i * 32;
-        const uint32_t write = i == 0 ? rows[0] : rows[1];
-        uint32_t s[32];
-        if (n_chunks > 0) {
-          tmem_ld32(tlane + COL_S + c0, s);
-          tmem_ld_wait();
-        } else {
+        const uint8_t *keep = a.row_keep + x.keep_row;
+        rows[i] = __ballot_sync(0xffffffffu, a.mode == DASC_REFRESH_CONTINUE || !keep[colh * 64 + i * 32 + lane]);
+      }
+      // post_s of the last chunk is visible: its writers arrived on rdy_prep, which the issuing warp waited for before it met the
+      // triangular warp, which arrived on a_taken, which these warps have waited for.  (Waiting for rdy_prep itself here could wait for
+      // the wrong phase: the next unit's tiles can be complete by now.)
+      if (n_chunks > 0) wait_bar(&misc->bar_s, (n - 1) & 1, misc);
+      if (tid < D) fin_s[tid] = n_chunks > 0 ? ex2f(post_s[KDA ? ((n - 1) & 1) * D + tid : (n - 1) & 3] * LOG2E) : 1.f;
+      sync_chain();
+      tc_fence_after_sync();
+      // A unit whose decay left the range, or whose CTA gave up on a wait, is NOT written back: its stored state keeps
+      // the bits it had before the call, so that it can be replayed by the exact kernel (or by the caller).
+      const bool bad = misc->abort_flag != 0 || misc->domain_flag[u & 3] != 0;
+      // The flag of unit u - 1, which everyone has looked at, becomes that of unit u + 3, which the producer warps cannot have reached.
+      if (tid == 0) misc->domain_flag[(u + 3) & 3] = 0;
+      if (bad) {
+        if (tid == 0 && misc->abort_flag == 0) hand_over(a, x.index, true);
+      } else {
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          const int c0 = colh * 64 + i * 32;
+          const uint32_t write = i == 0 ? rows[0] : rows[1];
+          float *const st_c = a.state + x.state + (c0 * D + vrow);
+          const float *const fin_c = fin_s + c0;
+          uint32_t s[32];
+          if (n_chunks > 0) {
+            tmem_ld32(tlane + COL_S + c0, s);
+            tmem_ld_wait();
+          } else {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) s[j] = 0u;  // scratch mode with an empty suffix
+            for (int j = 0; j < 32; ++j) s[j] = 0u;  // scratch mode with an empty suffix
+          }
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (write >> j & 1u) st_c[j * D] = __uint_as_float(s[j]) * fin_c[j];
         }
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (write >> j & 1u) st[(c0 + j) * D + vrow] = __uint_as_float(s[j]) * fac_s[c0 + j];
       }
     }
   }
@@ -1135,6 +1230,33 @@ EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
+// CTAs of a launch.  A CTA replays its units one behind the other, and the roles that need no state (tiles, A, T) run into the next
+// unit's first chunk while the chain warps write the last one's state back: a unit of its own costs a CTA about 16 k cycles
+// of start and end beside 7.5 k per chunk.  With a grid of G, CTA b takes units b, 2G - 1 - b, 2G + b, ... (there and back): as
+// requests come longest first, each gets long and short ones, and adjacent heads still run side by side.  The grid is a
+// multiple of the CTAs that are resident at once, so that no last wave is nearly empty.
+// Measured, us, a CTA per unit / this rule (KDA unless GDN): 4096 units of 1 .. 128 tokens, state only 253 / 223; 8192 of 64 tokens, state
+// only 379 / 309; 7680 of 16 tokens, state only 255 / 182; 8192 of 256 tokens 1128 / 1090 (GDN 1007 / 956).
+// Where the lines lie:
+//  - at most kWalkChunks chunks per CTA (a quarter of a millisecond): work of other streams is placed when CTAs end.  One grid of
+//    resident CTAs, whatever they have to do, gains nothing more where there are more chunks than that (1365, GDN 1101).
+//  - no request longer than half of a CTA's share by the caller's bound, since here a CTA's units are fixed beforehand, while blocks of
+//    a unit each go to whichever CTA ends first: 2048 units of 1 .. 1023 tokens take 669 / 658 walked, 1600 of 1 .. 1199 596 / 601: little
+//    to gain where units are long.
+//  - requests that are not in order of length (more than kRefreshOrderMax): only if they are about equally long.
+constexpr int64_t kResident = 2 * 148, kWalkChunks = 64;
+int64_t grid_for(const DascRefreshArgs &a, int64_t n_units) {
+  const int64_t tokens = a.window > 0 ? std::min<int64_t>(a.total_tokens, static_cast<int64_t>(a.n_req) * a.window) : a.total_tokens;
+  const int64_t longest = (std::max(a.max_seqlen, 1) + C - 1) / C;
+  const int64_t per_head = tokens / C + a.n_req / 2;  // chunks, about: half a one more per request
+  const int64_t chunks = per_head * a.n_layers_in_call * a.H_v;
+  int64_t g = kResident * std::max<int64_t>((chunks + kResident * kWalkChunks - 1) / (kResident * kWalkChunks),
+                                            (n_units + kResident * kMaxWalk - 1) / (kResident * kMaxWalk));
+  const bool in_order = a.ordered || a.n_req == 1;
+  const bool even = in_order ? longest * 2 * g <= chunks : longest * a.n_req * 9 <= per_head * 10;
+  return even && g < n_units ? g : n_units;
+}
+
 template <bool KDA, typename OT, bool WITH_O>
 int launch(DascRefreshArgs a, void *stream) {
   auto kern = refresh_chunked_kernel<KDA, OT, WITH_O>;
@@ -1164,7 +1286,7 @@ int launch(DascRefreshArgs a, void *stream) {
       (WITH_O && !make_map(&tmap_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.q, a.H_k, 2)) ||
       (KDA && !make_map(&tmap_g, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.g, a.H_v, 4)))
     return static_cast<int>(cudaErrorInvalidValue);
-  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(n_units)), dim3(NT), SMEM_ALLOC, stream, a, tmap_q, tmap_k, tmap_v, tmap_g));
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(grid_for(a, n_units))), dim3(NT), SMEM_ALLOC, stream, a, tmap_q, tmap_k, tmap_v, tmap_g));
 }
 
 }  // namespace

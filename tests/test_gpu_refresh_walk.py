@@ -1,0 +1,55 @@
+"""The chunked kernel's CTAs replay several units one behind the other where a launch has enough of them and no request is much
+longer than a CTA's share; the caller's bound on the longest request is part of that rule, so a loose bound gives every unit a
+CTA of its own.  Both have to give the same bits, and the oracle's results."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2608_30386_b200 as dasc
+from helpers import assert_refresh_close, make_refresh_case, run_refresh_oracle
+
+pytestmark = pytest.mark.gpu
+
+LOOSE = 1 << 30  # tokens: no request can be that long
+
+
+def replay(case, bound, mode, o_dtype, algo=dasc.ALGO_AUTO):
+    dev, n = case.state0.device, case.cu.numel() - 1
+    dense = case.H_v * 128 * 128
+    s, state, T = case.streams, case.state0.clone(), int(case.cu[-1])
+    o = None if o_dtype is None else torch.full((case.L, T, case.H_v, 128), float("nan"), device=dev, dtype=o_dtype)
+    ws = torch.zeros(dasc.dasc_refresh_workspace_bytes(case.plan, n, case.L, algo), dtype=torch.uint8, device=dev)
+    dasc.dasc_refresh(case.plan, state, dense, case.L * dense, torch.arange(n, dtype=torch.int32, device=dev), s.q, s.k, s.v, s.g,
+                      s.beta, case.cu.to(dev), T, bound, o=o, mode=mode, algo=algo, workspace=ws)
+    torch.cuda.synchronize()
+    assert dasc.dasc_refresh_status(ws) == 0
+    return state, o, dasc.dasc_refresh_counters(ws)
+
+
+# units and lengths around what changes a walk: 2 and 3 units of 2 chunks each; single chunks, 16 units to a CTA and the step to a
+# larger grid behind it (296 x 16 = 4736 units); ragged with empty requests, requests of at most 8 tokens (handed over
+# from the middle of a walk) and full chunks; more requests than are put in order; outputs in both types and none
+@pytest.mark.parametrize("kind,L,H,lens,mode,o_dtype", [
+    (dasc.KDA, 1, 8, [64] * 60, dasc.REFRESH_CONTINUE, torch.bfloat16),
+    (dasc.GDN, 1, 8, [50] * 111, dasc.REFRESH_CONTINUE, torch.float32),
+    (dasc.KDA, 1, 32, [32] * 148, dasc.REFRESH_SCRATCH_MERGE_LOCAL, None),
+    (dasc.GDN, 1, 32, [9] * 149, dasc.REFRESH_SCRATCH_MERGE_LOCAL, None),
+    (dasc.KDA, 2, 8, [1, 96, 0, 33, 8, 64, 9, 31] * 12, dasc.REFRESH_CONTINUE, torch.float32),
+    (dasc.KDA, 2, 8, [1, 96, 0, 33, 8, 64, 9, 31] * 12, dasc.REFRESH_SCRATCH_MERGE_LOCAL, None),
+    (dasc.GDN, 2, 8, [96, 32, 0, 95, 65, 97, 2] * 14, dasc.REFRESH_CONTINUE, torch.bfloat16),
+    (dasc.KDA, 1, 4, [64] * 250, dasc.REFRESH_CONTINUE, torch.bfloat16),
+])
+def test_walked_units_match_units_of_their_own(kind, L, H, lens, mode, o_dtype):
+    case = make_refresh_case(61, kind, L, H, H if kind == dasc.KDA else H // 2, 128, 128, lens, scope=dasc.SCOPE_LAYER, keep_ratio=0.4)
+    if kind == dasc.KDA and L > 1:  # a unit in the middle leaves the kernel's log-decay range and is replayed exactly
+        case.streams.g[1, int(case.cu[9]):int(case.cu[10]), 3, 7] = -7.0
+    walked, alone = replay(case, max(lens), mode, o_dtype), replay(case, LOOSE, mode, o_dtype)
+    assert walked[2] == alone[2]
+    assert torch.equal(walked[0].view(torch.int32), alone[0].view(torch.int32))
+    if o_dtype is not None:
+        assert torch.equal(walked[1], alone[1])
+    if len(lens) * L * H <= 1600 and o_dtype != torch.bfloat16:
+        merge = mode != dasc.REFRESH_CONTINUE
+        ref_s, ref_o = run_refresh_oracle(case, mode=oracle.MODE_SCRATCH_MERGE_LOCAL if merge else oracle.MODE_CONTINUE, want_o=not merge)
+        assert_refresh_close(case, walked[0].cpu().numpy(), None if merge else walked[1].cpu().numpy(), ref_s, ref_o, 1e-3)
