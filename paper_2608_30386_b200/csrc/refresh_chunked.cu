@@ -54,15 +54,31 @@ using namespace tc5;
 constexpr int C = 32;          // chunk length
 constexpr int D = 128;         // d_k = d_v
 constexpr int NCH = 256;       // chain threads (warps 0-7)
-constexpr int NP = 128;        // producer threads (warps 8-11)
-constexpr int WARP_T = 12;     // the warp that inverts the triangular system
-constexpr int WARP_MMA = 13;   // the warp that issues tensor-core work
-constexpr int NT = NCH + NP + 64;
+// Two forms.  SHARED: two CTAs per SM.  ALONE (see kAloneUnits): one, with more warps and second buffers, so that the tiles, MMA1 and T of
+// the next chunk are made while the chain is in this one, and the outputs leave meanwhile.
+template <bool ALONE>
+struct Form {
+  static constexpr int NP = ALONE ? 256 : 128;           // producer threads (from warp 8 on)
+  static constexpr int WARP_T = 8 + NP / 32;             // the warp that inverts the triangular system (in TMEM quadrant 0)
+  // ALONE: MMA1, rows 16-31 of A and the copies of the inputs are a warp's own (in quadrant 1), P and the outputs those of four more
+  // (one per quadrant), so that the issuing warp and the chain warps do the chain's work only.
+  static constexpr int WARP_MMA1 = WARP_T + 1;
+  static constexpr int WARP_O = WARP_T + 2;
+  static constexpr int WARP_MMA = ALONE ? WARP_O + 4 : WARP_T + 1;  // the warp that issues tensor-core work (SHARED: in quadrant 1)
+  static constexpr int NT = (WARP_MMA + 1) * 32;
+  static constexpr int BUF = ALONE ? 2 : 1;              // buffers of what SHARED has one of: Kt/Qt, K-major Kh (GDN: raw k, q), T, A|P, R|O
+  static constexpr int RING = ALONE ? 8 : 4;             // per-token scalars, by chunk index mod RING
+  static constexpr int FAC = ALONE ? 4 : 2;              // state factors, by chunk index mod FAC
+  static constexpr uint32_t TMEM_COLS = ALONE ? 512 : 256;
+};
 constexpr int LDX = 36;        // row pitch (floats) of the fp32 triangular work matrices
-constexpr uint32_t TMEM_COLS = 256;
 
-// TMEM columns
-constexpr uint32_t COL_S = 0, COL_AP = 128, COL_RO = 160, COL_U = 224;  // RO: R^T 160-191 | (Qt S')^T 192-223
+// TMEM columns; RO: R^T 32 columns | (Qt S')^T 32; RL: the right-hand side's low part (SHARED: over the consumed A|P)
+constexpr uint32_t COL_S = 0, COL_AP = 128;
+template <bool ALONE>
+constexpr uint32_t COL_RO = ALONE ? 192 : 160;  // ALONE: AP 128-191, RO 192-383 (three), U 384-415, RL 416-447
+template <bool ALONE>
+constexpr uint32_t COL_U = ALONE ? 384 : 224;
 
 // shared memory map (bytes)
 constexpr uint32_t OFF_KQ = 0;                          // [4][64 rows][128 B]  rows 0-31 Kt, 32-63 Qt
@@ -83,11 +99,19 @@ constexpr uint32_t OFF_BTE1 = OFF_E2 + 4 * C * 4;       // [4][32] fp32 beta * e
 constexpr uint32_t OFF_FIN = OFF_BTE1 + 4 * C * 4;      // [128] fp32 state factor per channel behind the last chunk of a unit
 constexpr uint32_t OFF_UNIT = OFF_FIN + D * 4;          // the CTA's units
 constexpr uint32_t OFF_MISC = OFF_UNIT + 16 * 48;       // barriers, tmem base, flags
-// GDN only: raw k (rows 0-31) and q (rows 32-63) as bf16, [2][64 rows][128 B], in the place of the K-major Kh tile
-constexpr uint32_t OFF_KQ16 = OFF_KH;
-constexpr uint32_t SMEM_BYTES = OFF_MISC + 224;
-constexpr uint32_t SMEM_ALLOC = SMEM_BYTES;
-static_assert(SMEM_ALLOC <= 113 * 1024, "two CTAs per SM");
+// (GDN: the K-major Kh tile's place holds raw k (rows 0-31) and q (rows 32-63) as bf16, [2][64 rows][128 B])
+constexpr uint32_t SMEM_BYTES = OFF_MISC + 320;
+static_assert(SMEM_BYTES <= 113 * 1024, "two CTAs per SM");
+// ALONE: the second buffers and longer rings, behind the map above
+constexpr uint32_t OFF_KQ_2 = (SMEM_BYTES + 1023) / 1024 * 1024;
+constexpr uint32_t OFF_KH_2 = OFF_KQ_2 + 4 * 64 * 128;     // (GDN: raw k, q)
+constexpr uint32_t OFF_TM_2 = OFF_KH_2 + 4 * 32 * 128;
+constexpr uint32_t OFF_OUT_2 = OFF_TM_2 + 32 * 128;        // the bf16 O tile
+constexpr uint32_t OFF_KHT_2 = OFF_OUT_2 + C * D * 2;      // third and fourth MN-major Kh tile
+constexpr uint32_t OFF_RING_2 = OFF_KHT_2 + 2 * 128 * 128;     // beta, e1c, e2, bte1: [8][32] fp32 each
+constexpr uint32_t OFF_FAC_2 = OFF_RING_2 + 4 * 8 * C * 4;     // [4][128] fp32 state factors
+constexpr uint32_t SMEM_ALONE = OFF_FAC_2 + 4 * D * 4;
+static_assert(SMEM_ALONE <= 227 * 1024, "one CTA per SM");
 
 constexpr uint32_t kMaxPolls = 1u << 22;
 
@@ -108,24 +132,25 @@ struct Misc {
   // Each barrier completes one phase per chunk.  Where the arrivals are "per warp", a warp's first lane arrives for it.
   // tensor core -> chain warps (one tcgen05.commit each); bar_ap also releases the triangular and the issuing warp and the
   // next log-decay (KDA) or k, q (GDN), bar_ro the Kt/Qt tile, bar_s the Kh tile of its parity (KDA)
-  uint64_t bar_ap, bar_ro, bar_u, bar_o, bar_s;
+  // (two of each where a phase can complete before all have waited for the one before: ALONE, by chunk parity)
+  uint64_t bar_ap[2], bar_ro[2], bar_s[2], bar_u, bar_o;
   // producer -> issuing warp: the tiles of a chunk are ready (per warp: 4 arrivals; KDA one more from the triangular warp, for beta)
-  uint64_t rdy_prep;
+  uint64_t rdy_prep[2];  // (ALONE: by chunk parity)
   // producer -> chain warps: the state factors of a chunk are ready (KDA per warp: 4 arrivals; GDN the first warp only: 1)
   // One barrier per chunk parity: the producer may hand over the factors of chunk n+1 before the chain warps
   // have waited for those of chunk n, and a single barrier cannot tell phases two apart.
-  uint64_t rdy_fac[2];
+  uint64_t rdy_fac[4];
   // chain warps -> issuing warp (per warp: 8 arrivals each)
-  uint64_t rdy_state, rdy_rhs, rdy_u;
+  uint64_t rdy_state, rdy_half, rdy_rhs, rdy_u;  // (rdy_half, ALONE: the first half of the state's channels)
   // triangular warp -> chain warps (A has left TMEM: 1 arrival) and -> issuing warp (T tile ready: 1 arrival)
   uint64_t a_taken, rdy_t;
   // chain warps -> triangular warp and one another: the T|P tile region is free again (per warp: 8 arrivals)
   uint64_t tp_free;
   // issuing thread, only after a wait has run out: arrives once every tensor-core product issued so far has completed
-  uint64_t drain;
+  uint64_t drain, drain_1;
   // TMA -> producer warps: the log-decay of a chunk has landed in the Kh tile (KDA: 4 copies, one arrival with each); its raw
   // k, q have landed (4 copies, 2 without outputs)
-  uint64_t g_full, kq_full;
+  uint64_t g_full[2], kq_full[2];
   // TMA -> chain warps: V of a chunk has landed (2 copies, started by the triangular warp)
   uint64_t v_full;
   uint32_t tmem_base;
@@ -133,7 +158,7 @@ struct Misc {
   int32_t n_units, all_chunks;    // this CTA's units (those that have tokens listed first) and the chunks of all of them
   volatile uint32_t domain_flag[4];  // a half-chunk decay sum left the range the midpoint factors can carry; by unit index mod 4
 };
-static_assert(sizeof(Misc) <= 224, "Misc outgrew its shared-memory slot");
+static_assert(sizeof(Misc) <= 320, "Misc outgrew its shared-memory slot");
 
 // One of a CTA's units, as all roles read it from shared memory.
 constexpr int kMaxWalk = 16;
@@ -321,22 +346,34 @@ __device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
 
 // WITH_O = false is the state-only variant (no outputs wanted): q is never read, the Qt rows, P and the
 // output product are left out.
-template <bool KDA, typename OT, bool WITH_O>
-__global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_constant__ DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
+template <bool KDA, typename OT, bool WITH_O, bool ALONE>
+__global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunked_kernel(const __grid_constant__ DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
                                                                 const __grid_constant__ CUtensorMap tmap_k,
                                                                 const __grid_constant__ CUtensorMap tmap_v,
                                                                 const __grid_constant__ CUtensorMap tmap_g) {
   // The base is a link-time constant (there is no static shared memory), so every operand descriptor is an immediate.
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t sbase = smem_u32(smem);
+  using F = Form<ALONE>;
+  constexpr int NP = F::NP, WARP_T = F::WARP_T, WARP_MMA = F::WARP_MMA, WARP_O = F::WARP_O, WARP_MMA1 = F::WARP_MMA1, RING = F::RING, FAC = F::FAC;
+  // where chunk n's buffer is, and the barrier and the parity that stand for it
+  auto buf = [](int n) { return static_cast<uint32_t>(ALONE ? n & 1 : 0); };
+  auto phase = [](int n) { return static_cast<uint32_t>(ALONE ? (n >> 1) & 1 : n & 1); };
+  auto off_kq = [&](int n) { return OFF_KQ + buf(n) * (OFF_KQ_2 - OFF_KQ); };
+  auto off_kh = [&](int n) { return OFF_KH + buf(n) * (OFF_KH_2 - OFF_KH); };  // GDN: raw k, q
+  auto off_kht = [&](int n) { return OFF_KHT + (n & 1) * (128 * 128) + (ALONE && (n & 2) ? OFF_KHT_2 - OFF_KHT : 0u); };
+  auto off_t = [&](int n) { return OFF_TM + buf(n) * (OFF_TM_2 - OFF_TM); };
+  auto col_ap = [&](int n) { return COL_AP + buf(n) * 32; };
+  auto col_ro = [&](int n) { return COL_RO<ALONE> + (ALONE ? static_cast<uint32_t>(n) % 3u * 64 : 0u); };
+  constexpr uint32_t COL_RL = ALONE ? 416 : COL_AP, OFF_O = ALONE ? OFF_OUT_2 : OFF_TM;
   float *LT = reinterpret_cast<float *>(smem + OFF_L);
   float *Xm = reinterpret_cast<float *>(smem + OFF_X);
-  float *fac_s = reinterpret_cast<float *>(smem + OFF_FAC);
+  float *fac_s = reinterpret_cast<float *>(smem + (ALONE ? OFF_FAC_2 : OFF_FAC));
   float *post_s = reinterpret_cast<float *>(smem + OFF_POST);
-  float *beta_s = reinterpret_cast<float *>(smem + OFF_BETA);
-  float *e1c_s = reinterpret_cast<float *>(smem + OFF_E1C);
-  float *e2_s = reinterpret_cast<float *>(smem + OFF_E2);
-  float *bte1_s = reinterpret_cast<float *>(smem + OFF_BTE1);
+  float *beta_s = reinterpret_cast<float *>(smem + (ALONE ? OFF_RING_2 + 0 * 8 * C * 4 : OFF_BETA));
+  float *e1c_s = reinterpret_cast<float *>(smem + (ALONE ? OFF_RING_2 + 1 * 8 * C * 4 : OFF_E1C));
+  float *e2_s = reinterpret_cast<float *>(smem + (ALONE ? OFF_RING_2 + 2 * 8 * C * 4 : OFF_E2));
+  float *bte1_s = reinterpret_cast<float *>(smem + (ALONE ? OFF_RING_2 + 3 * 8 * C * 4 : OFF_BTE1));
   float *fin_s = reinterpret_cast<float *>(smem + OFF_FIN);
   Unit *const units = reinterpret_cast<Unit *>(smem + OFF_UNIT);
   Misc *misc = reinterpret_cast<Misc *>(smem + OFF_MISC);
@@ -346,37 +383,41 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
 
   // ---- set-up: barriers and tensor memory ----
   if (tid == 0) {
-    mbar_init(&misc->bar_ap, 1);
-    mbar_init(&misc->bar_ro, 1);
+    for (int i = 0; i < F::BUF; ++i) {
+      mbar_init(&misc->rdy_prep[i], NP / 32 + (KDA && !ALONE ? 1 : 0));
+      mbar_init(&misc->bar_ap[i], 1);
+      mbar_init(&misc->bar_ro[i], 1);
+      mbar_init(&misc->bar_s[i], 1);
+      mbar_init(&misc->g_full[i], 4);
+      mbar_init(&misc->kq_full[i], WITH_O ? 4 : 2);
+    }
+    for (int i = 0; i < FAC; ++i) mbar_init(&misc->rdy_fac[i], KDA ? 4 : 1);
     mbar_init(&misc->bar_u, 1);
     mbar_init(&misc->bar_o, 1);
-    mbar_init(&misc->bar_s, 1);
-    mbar_init(&misc->rdy_prep, NP / 32 + (KDA ? 1 : 0));
-    mbar_init(&misc->rdy_fac[0], KDA ? NP / 32 : 1);
-    mbar_init(&misc->rdy_fac[1], KDA ? NP / 32 : 1);
     mbar_init(&misc->rdy_state, NCH / 32);
-    mbar_init(&misc->rdy_rhs, NCH / 32);
+    mbar_init(&misc->rdy_half, NCH / 32);
+    mbar_init(&misc->rdy_rhs, NCH / 32 + (ALONE ? (WITH_O ? 5 : 1) : 0));
     mbar_init(&misc->rdy_u, NCH / 32);
     mbar_init(&misc->a_taken, 1);
     mbar_init(&misc->rdy_t, 1);
     mbar_init(&misc->tp_free, NCH / 32);
     mbar_init(&misc->drain, 1);
-    mbar_init(&misc->g_full, NP / 32);
+    mbar_init(&misc->drain_1, 1);
+
     mbar_init(&misc->v_full, 2);
-    mbar_init(&misc->kq_full, WITH_O ? NP / 32 : NP / 64);
     misc->abort_flag = 0;
     for (int i = 0; i < 4; ++i) misc->domain_flag[i] = 0;
     fence_mbar_init();
   }
   if (warp == WARP_MMA) {
-    tmem_alloc(&misc->tmem_base, TMEM_COLS);
+    tmem_alloc(&misc->tmem_base, F::TMEM_COLS);
     tmem_relinquish();
   }
   // This CTA's units, a lane of one warp each: every gridDim.x-th, there and back (see grid_for).  Which they are is worked out
   // before the wait for earlier work, their tokens and state are looked up behind it.
   if (warp == WARP_T) {
     const int64_t idx = static_cast<int64_t>(lane) * gridDim.x + ((lane & 1) ? gridDim.x - 1u - blockIdx.x : blockIdx.x);
-    bool here = lane < kMaxWalk && idx < static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
+    bool here = lane < (ALONE ? 1 : kMaxWalk) && idx < static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
     const uint32_t row = static_cast<uint32_t>(idx) / a.H_v;  // (the host sees to it that units fit 31 bits)
     Unit x;
     x.head = static_cast<int32_t>(static_cast<uint32_t>(idx) - row * a.H_v);
@@ -423,63 +464,175 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
   constexpr uint32_t ID_N64 = idesc_tf32(128, 64, false, false);
   constexpr uint32_t ID_N128_MN = idesc_tf32(128, 128, false, true);  // B = Kh[t][c]: the channel index N is the contiguous one
 
+  auto mma1 = [&](int n) {
+    // MMA1: [Kt;Qt] Kh^T, M = 64: 16 rows in each TMEM quadrant, A's in the first two, P's in the last two.
+    if (n == 0 && a.poll_limit_first_wait)
+      wait_bar_short(&misc->rdy_prep[buf(n)], phase(n), misc, a.poll_limit_first_wait);
+    else
+      wait_bar(&misc->rdy_prep[buf(n)], phase(n), misc);
+    tc_fence_after_sync();
+    if (elect_one()) {
+      if constexpr (KDA) {
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk)  // K = 128 in slices of 8: block kk / 4, 32 bytes per slice inside a block
+          mma_ss(tm + col_ap(n), desc_kmajor(sbase + off_kq(n) + (kk >> 2) * (64 * 128) + (kk & 3) * 32),
+                 desc_kmajor(sbase + off_kh(n) + (kk >> 2) * (32 * 128) + (kk & 3) * 32), ID_M64, kk != 0);
+      } else {
+        // GDN: the decay is one scalar per token, so it is applied to A and P after the product, and the product
+        // itself is [k; q] k^T on the raw bf16 inputs: exact operands, K = 16 per instruction.  A and B come from
+        // the same tile (B = its first 32 rows).
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint64_t d = desc_kmajor(sbase + off_kh(n) + (kk >> 2) * (64 * 128) + (kk & 3) * 32);
+          mma_ss_bf16(tm + col_ap(n), d, d, ID_BF16_M64, kk != 0);
+        }
+      }
+      mma_commit(&misc->bar_ap[buf(n)]);
+    }
+    __syncwarp();
+  };
+  auto take_a = [&](int n) {
+    // rows 16-31 of A are in this warp's quadrant: hand them to the triangular warp
+    wait_bar(&misc->bar_ap[buf(n)], phase(n), misc);
+    if (ALONE && n > 0) wait_bar(&misc->rdy_rhs, (n - 1) & 1, misc);  // the triangular warp has read the chunk before's
+    tc_fence_after_sync();
+    take_a_rows<KDA>(tm + (32u << 16) + col_ap(n), 16, (KDA ? beta_s : bte1_s) + (n % RING) * C, e2_s + (n % RING) * C, LT, lane);
+    asm volatile("bar.arrive 3, 64;" ::: "memory");
+  };
+  // where a chunk's raw k, q lie: rows of a 64-channel block, and q behind k
+  constexpr uint32_t RAW_ROWS = KDA ? 32 : 64, OFF_RAW_Q = KDA ? 2 * 32 * 128 : 32 * 128;
+  // ---- the two steps that the chain warps take, or warps of their own ----
+  // P = lower_incl_diag(Qt Kh^T) of chunk n out of TMEM (rows 0-15, 16-31 are in the third and fourth quadrant) straight to its operand
+  // tile, 16 columns.  GDN: the raw q_t . k_j gets its column factor e2_j here, the row factor e1_t is applied to the outputs.
+  const int quad = warp & 3;                                             // TMEM lane quadrant
+  const uint32_t tlane = tm + (static_cast<uint32_t>(quad * 32) << 16);  // this warp's TMEM lanes
+  const int g = lane >> 2, tig = lane & 3;
+  auto take_p = [&](int n, int colh) {
+    wait_bar(&misc->bar_ap[buf(n)], phase(n), misc);
+    tc_fence_after_sync();
+    uint32_t x[8];
+    tmem_ld_16x256b(tlane + col_ap(n) + colh * 16, x);
+    if (!ALONE && n > 0) wait_bar(&misc->tp_free, (n - 1) & 1, misc);  // the previous chunk's outputs have left this storage
+    tmem_ld_wait();
+    const int t = (quad - 2) * 16 + g;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int j = colh * 16 + 8 * i + 2 * tig;
+      float2 e = make_float2(kInvTruncComp, kInvTruncComp);
+      if constexpr (!KDA) {
+        const float2 e2 = *reinterpret_cast<const float2 *>(e2_s + (n % RING) * C + j);
+        e.x *= e2.x;
+        e.y *= e2.y;
+      }
+      unsigned char *const p = smem + OFF_PM + sw128_offset(32, t, j);
+      *reinterpret_cast<uint2 *>(p) = make_uint2(j <= t ? tf32_pre(__uint_as_float(x[4 * i]) * e.x) : 0u,
+                                                 j + 1 <= t ? tf32_pre(__uint_as_float(x[4 * i + 1]) * e.y) : 0u);
+      *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(j <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 2]) * e.x) : 0u,
+                                                        j + 1 <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 3]) * e.y) : 0u);
+    }
+    fence_smem_to_async();
+  };
+  // Outputs of chunk n, of which `ntok` tokens are the request's: one token half (SHARED: the warp's) or both
+  // by this warp, thread ti of those that take them.
+  auto outputs = [&](int n, int ntok, OT *go, int half_0, int ti) {
+    constexpr int NTH = ALONE ? 128 : NCH;
+    wait_bar(&misc->bar_o, n & 1, misc);
+    tc_fence_after_sync();
+    if (WITH_O) {
+#pragma unroll
+      for (int k = 0; k < F::BUF; ++k) {
+        const int tb = (half_0 + k) * 16;
+        const int ot = tb + (lane >> 4) * 8 + (lane & 7);  // blocks of one stmatrix: as for V
+        uint32_t xx[2][8];
+        tmem_ld_16x256b(tlane + col_ro(n) + 32 + tb, xx[0]);
+        tmem_ld_16x256b(tlane + (1u << 20) + col_ro(n) + 32 + tb, xx[1]);
+        tmem_ld_wait();
+#pragma unroll
+        for (uint32_t hh = 0; hh < 2; ++hh) {
+          uint32_t(&x)[8] = xx[hh];
+          if constexpr (!KDA) {
+            // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
+            // the truncation compensation
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const float2 e = *reinterpret_cast<const float2 *>(e1c_s + (n % RING) * C + tb + 8 * i + 2 * tig);
+              x[4 * i + 0] = __float_as_uint(__uint_as_float(x[4 * i + 0]) * (e.x * a.q_scale));
+              x[4 * i + 1] = __float_as_uint(__uint_as_float(x[4 * i + 1]) * (e.y * a.q_scale));
+              x[4 * i + 2] = __float_as_uint(__uint_as_float(x[4 * i + 2]) * (e.x * a.q_scale));
+              x[4 * i + 3] = __float_as_uint(__uint_as_float(x[4 * i + 3]) * (e.y * a.q_scale));
+            }
+          }
+          if constexpr (sizeof(OT) == 2) {
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = pack_bf16x2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+            stmatrix_x4_trans(sbase + OFF_O + ot * 256 + (((quad * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (ot & 7)) << 4), w[0], w[1], w[2], w[3]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int t = tb + (i >> 1) * 8 + 2 * tig, v = quad * 32 + hh * 16 + (i & 1) * 8 + g;
+              if (t < ntok) go[t * v_stride + v] = __uint_as_float(x[2 * i]);
+              if (t + 1 < ntok) go[(t + 1) * v_stride + v] = __uint_as_float(x[2 * i + 1]);
+            }
+          }
+        }
+      }
+      if constexpr (sizeof(OT) == 2) {
+        // through shared memory (SHARED: where the T and P tiles were, which are free now) so that global stores are 16 bytes wide
+        asm volatile("bar.sync %0, %1;" ::"n"(ALONE ? 6 : 1), "n"(NTH) : "memory");
+        const int j = ti & 15;
+#pragma unroll
+        for (int i = 0; i < C / (NTH / 16); ++i) {
+          const int t = (ti >> 4) + NTH / 16 * i;
+          if (t < ntok)
+            *reinterpret_cast<uint4 *>(go + i * (NTH / 16) * v_stride) =
+                *reinterpret_cast<const uint4 *>(smem + OFF_O + t * 256 + ((j ^ (t & 7)) << 4));
+        }
+      }
+    }
+  };
+
   if (warp == WARP_MMA) {
     // =========================== tensor-core issue warp ===========================
     // The whole warp walks the chunks and waits; an elected lane issues.
     for (int n = 0; n < all_chunks; ++n) {
       const uint32_t par = n & 1;
-      // MMA1: [Kt;Qt] Kh^T, M = 64: 16 rows in each TMEM quadrant, A's in the first two, P's in the last two.
-      if (n == 0 && a.poll_limit_first_wait)
-        wait_bar_short(&misc->rdy_prep, par, misc, a.poll_limit_first_wait);
-      else
-        wait_bar(&misc->rdy_prep, par, misc);
-      tc_fence_after_sync();
-      if (elect_one()) {
-        if constexpr (KDA) {
-#pragma unroll
-          for (int kk = 0; kk < 16; ++kk)  // K = 128 in slices of 8: block kk / 4, 32 bytes per slice inside a block
-            mma_ss(tm + COL_AP, desc_kmajor(sbase + OFF_KQ + (kk >> 2) * (64 * 128) + (kk & 3) * 32),
-                   desc_kmajor(sbase + OFF_KH + (kk >> 2) * (32 * 128) + (kk & 3) * 32), ID_M64, kk != 0);
-        } else {
-          // GDN: the decay is one scalar per token, so it is applied to A and P after the product, and the product
-          // itself is [k; q] k^T on the raw bf16 inputs: exact operands, K = 16 per instruction.  A and B come from
-          // the same tile (B = its first 32 rows).
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint64_t d = desc_kmajor(sbase + OFF_KQ16 + (kk >> 2) * (64 * 128) + (kk & 3) * 32);
-            mma_ss_bf16(tm + COL_AP, d, d, ID_BF16_M64, kk != 0);
-          }
-        }
-        mma_commit(&misc->bar_ap);
+      if (!ALONE) {
+        mma1(n);
+        take_a(n);
       }
-      __syncwarp();
-      // rows 16-31 of A are in this warp's quadrant: hand them to the triangular warp
-      wait_bar(&misc->bar_ap, par, misc);
-      tc_fence_after_sync();
-      take_a_rows<KDA>(tm + (32u << 16) + COL_AP, 16, (KDA ? beta_s : bte1_s) + (n & 3) * C, e2_s + (n & 3) * C, LT, lane);
-      asm volatile("bar.arrive 3, 64;" ::: "memory");
       // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
+      auto mma2 = [&](int kb_0, int kb_n) {
+#pragma unroll 1
+        for (int kb = kb_0; kb < kb_n; ++kb) {
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            mma_ts(tm + col_ro(n), tm + COL_S + kb * 32 + kk * 8, desc_kmajor(sbase + off_kq(n) + kk * 32) + kb * (64 * 128 / 16),
+                   WITH_O ? ID_N64 : ID_N32, (kb | kk) != 0);  // without outputs only the Kt rows are needed
+        }
+      };
+      if (ALONE) {
+        wait_bar(&misc->bar_ap[buf(n)], phase(n), misc);  // the tiles of this chunk are there: the warp that issued MMA1 has waited for them
+        wait_bar(&misc->rdy_half, par, misc);
+        tc_fence_after_sync();
+        if (elect_one()) mma2(0, 2);
+        __syncwarp();
+      }
       wait_bar(&misc->rdy_state, par, misc);
       tc_fence_after_sync();
       if (elect_one()) {
-#pragma unroll 1
-        for (int kb = 0; kb < 4; ++kb) {
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_ts(tm + COL_RO, tm + COL_S + kb * 32 + kk * 8, desc_kmajor(sbase + OFF_KQ + kk * 32) + kb * (64 * 128 / 16),
-                   WITH_O ? ID_N64 : ID_N32, (kb | kk) != 0);  // without outputs only the Kt rows are needed
-        }
-        mma_commit(&misc->bar_ro);
+        mma2(ALONE ? 2 : 0, 4);
+        mma_commit(&misc->bar_ro[buf(n)]);
       }
       __syncwarp();
       // MMA3: U^T = RHS^T T^T; RHS^T is a tf32 pair (high part over R^T, low part in the A|P columns)
-      wait_bar(&misc->rdy_t, par, misc);
+      if (!ALONE) wait_bar(&misc->rdy_t, par, misc);  // (ALONE: the triangular and the output warps arrive on rdy_rhs)
       wait_bar(&misc->rdy_rhs, par, misc);
       tc_fence_after_sync();
       if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
-          mma_ts(tm + COL_U, tm + (kk < 4 ? COL_RO : COL_AP) + (kk & 3) * 8, desc_kmajor(sbase + OFF_TM + (kk & 3) * 32),
+          mma_ts(tm + COL_U<ALONE>, tm + (kk < 4 ? col_ro(n) : COL_RL) + (kk & 3) * 8, desc_kmajor(sbase + off_t(n) + (kk & 3) * 32),
                  ID_N32, kk != 0);
         mma_commit(&misc->bar_u);
       }
@@ -490,33 +643,41 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
       // MMA4 (high): O^T += U_hi^T P^T;  MMA5 (high): S'^T += U_hi^T Kh
       // U must have arrived in tensor memory before another product reads it as its A operand: the tensor pipe's issue
       // order does not see to that (it orders accumulators only).
-      wait_bar(&misc->bar_u, par, misc);
-      tc_fence_after_sync();
-      if (elect_one()) {
+      // ALONE: the state's product first, it is what the chain waits for; SHARED: the chain warps take the outputs next.
+      auto mma4 = [&](uint32_t u_t) {
         if (WITH_O) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            mma_ts(tm + COL_RO + 32, tm + COL_U + kk * 8, desc_kmajor(sbase + OFF_PM + kk * 32), ID_N32, true);
+            mma_ts(tm + col_ro(n) + 32, tm + u_t + kk * 8, desc_kmajor(sbase + OFF_PM + kk * 32), ID_N32, true);
         }
+      };
+      auto mma5 = [&](uint32_t u_t) {
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          mma_ts(tm + COL_S, tm + COL_U + kk * 8, desc_mn32(sbase + OFF_KHT + par * (128 * 128) + kk * 1024, 32 * 128), ID_N128_MN, true);
+          mma_ts(tm + COL_S, tm + u_t + kk * 8, desc_mn32(sbase + off_kht(n) + kk * 1024, 32 * 128), ID_N128_MN, true);
+      };
+      wait_bar(&misc->bar_u, par, misc);
+      tc_fence_after_sync();
+      if (elect_one()) {
+        if (!ALONE) mma4(COL_U<ALONE>);
+        mma5(COL_U<ALONE>);
       }
       __syncwarp();
       // MMA4 (low), MMA5 (low): the same with U_lo^T, which the chain warps wrote over the consumed RHS^T
       wait_bar(&misc->rdy_u, par, misc);
       tc_fence_after_sync();
       if (elect_one()) {
-        if (WITH_O) {
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_ts(tm + COL_RO + 32, tm + COL_RO + kk * 8, desc_kmajor(sbase + OFF_PM + kk * 32), ID_N32, true);
+        if (ALONE) {
+          mma5(col_ro(n));
+          mma_commit(&misc->bar_s[buf(n)]);
+          mma4(COL_U<ALONE>);
         }
+        mma4(col_ro(n));
         mma_commit(&misc->bar_o);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          mma_ts(tm + COL_S, tm + COL_RO + kk * 8, desc_mn32(sbase + OFF_KHT + par * (128 * 128) + kk * 1024, 32 * 128), ID_N128_MN, true);
-        mma_commit(&misc->bar_s);
+        if (!ALONE) {
+          mma5(col_ro(n));
+          mma_commit(&misc->bar_s[buf(n)]);
+        }
       }
       __syncwarp();
     }
@@ -556,25 +717,26 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
         ++v_unit;
       }
     };
-    // KDA: it also brings in beta, a chunk ahead (GDN: the producer warps, whose per-token factors contain it), and arrives on rdy_prep.
+    // KDA: it also brings in beta, a chunk ahead, and arrives on rdy_prep (ALONE: the MMA1 warp; GDN: the producer warps, whose per-token
+    // factors contain it).
     auto fetch_beta = [&]() {  // of the chunk whose copy comes next, lane = token
       const Unit &x = units[v_unit];
       return lane < x.n_tok - v_tok ? a.beta[(x.tok0 + v_tok + lane) * a.H_v + x.head] : 0.f;
     };
     if (all_chunks > 0) {
-      if (KDA) {
+      if (KDA && !ALONE) {
         beta_s[lane] = fetch_beta();
-        arrive_warp(&misc->rdy_prep, lane);
+        arrive_warp(&misc->rdy_prep[0], lane);
       }
       stage_v();
     }
     for (int n = 0; n < all_chunks; ++n) {
       const uint32_t par = n & 1;
       float beta_next = 0.f;
-      if (KDA && n + 1 < all_chunks) beta_next = fetch_beta();
-      wait_bar(&misc->bar_ap, par, misc);
+      if (KDA && !ALONE && n + 1 < all_chunks) beta_next = fetch_beta();
+      wait_bar(&misc->bar_ap[buf(n)], phase(n), misc);
       tc_fence_after_sync();
-      take_a_rows<KDA>(tm + COL_AP, 0, (KDA ? beta_s : bte1_s) + (n & 3) * C, e2_s + (n & 3) * C, LT, lane);
+      take_a_rows<KDA>(tm + col_ap(n), 0, (KDA ? beta_s : bte1_s) + (n % RING) * C, e2_s + (n % RING) * C, LT, lane);
       tc_fence_before_sync();
       asm volatile("bar.sync 3, 64;" ::: "memory");
       arrive_warp(&misc->a_taken, lane);  // the chain warps may reuse the A|P columns
@@ -606,13 +768,13 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
         warp_mm_store(Xm + 16, acc, 1.f, lane);
         // T -> tf32 operand tile, straight from the registers.  Its storage (shared with the P tile and the chain warps'
         // output tile) is free once the chain warps have copied the previous chunk's outputs out.
-        if (n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
+        if (!ALONE && n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
 #pragma unroll
         for (int rr = 0; rr < 16; ++rr)
-          *reinterpret_cast<uint32_t *>(smem + OFF_TM + sw128_offset(32, b * 16 + rr, b * 16 + cc)) = tf32_pre(xs[rr]);
+          *reinterpret_cast<uint32_t *>(smem + off_t(n) + sw128_offset(32, b * 16 + rr, b * 16 + cc)) = tf32_pre(xs[rr]);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
-          *reinterpret_cast<uint4 *>(smem + OFF_TM + sw128_offset(32, i * 8 + (lane >> 2), 16 + (lane & 3) * 4)) = make_uint4(0u, 0u, 0u, 0u);
+          *reinterpret_cast<uint4 *>(smem + off_t(n) + sw128_offset(32, i * 8 + (lane >> 2), 16 + (lane & 3) * 4)) = make_uint4(0u, 0u, 0u, 0u);
       }
       __syncwarp();
       {
@@ -621,17 +783,17 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
         const int g = lane >> 2, tig = lane & 3;
 #pragma unroll
         for (int nh = 0; nh < 2; ++nh) {
-          unsigned char *const p = smem + OFF_TM + sw128_offset(32, 16 + g, 8 * nh + 2 * tig);
+          unsigned char *const p = smem + off_t(n) + sw128_offset(32, 16 + g, 8 * nh + 2 * tig);
           *reinterpret_cast<uint2 *>(p) = make_uint2(tf32_pre(-acc2[nh][0]), tf32_pre(-acc2[nh][1]));
           *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(tf32_pre(-acc2[nh][2]), tf32_pre(-acc2[nh][3]));
         }
       }
       fence_smem_to_async();
-      arrive_warp(&misc->rdy_t, lane);  // -> MMA3
+      arrive_warp(ALONE ? &misc->rdy_rhs : &misc->rdy_t, lane);  // -> MMA3
       if (n + 1 < all_chunks) {  // once V has been read by every chain warp the next chunk's may land
-        if (KDA) {
-          beta_s[((n + 1) & 3) * C + lane] = beta_next;
-          arrive_warp(&misc->rdy_prep, lane);
+        if (KDA && !ALONE) {
+          beta_s[((n + 1) % RING) * C + lane] = beta_next;
+          arrive_warp(&misc->rdy_prep[0], lane);
         }
         wait_bar(&misc->rdy_rhs, par, misc);
         stage_v();
@@ -640,12 +802,91 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
     }
     // after a time-out the last copies of V may not have been waited for: they must have landed before the CTA leaves
     if (lane == 0 && misc->abort_flag && v_issued > 0) mbar_wait_bounded(&misc->v_full, (v_issued - 1) & 1, kMaxPolls);
+  } else if (ALONE && warp == WARP_MMA1) {
+    // ================================= MMA1, input copies (ALONE) =================================
+    // MMA1 goes out behind MMA2 of the chunk before, i.e. while the chain warps form its right-hand side.  By then A and P of two chunks
+    // ago, whose columns are written again, have been read.  Copies are two chunks ahead, a box per lane: KDA the log-decay by lanes 0-3;
+    // k by lanes 4, 5; q by lanes 6, 7.
+    const Unit &x = units[0];
+    const bool copies_g = KDA && lane < 4, copies_kq = lane >= 4 && lane < (WITH_O ? 8 : 6);
+    int issued = 0;
+    auto copy = [&](int n) {
+      if ((copies_g || copies_kq) && !misc->abort_flag) {
+        const int32_t z = static_cast<int32_t>(x.tok0 + n * C);
+        uint64_t *const full = copies_g ? &misc->g_full[buf(n)] : &misc->kq_full[buf(n)];
+        const uint32_t raw = sbase + (KDA ? off_kht(n) : off_kh(n)) + (lane & 1) * (RAW_ROWS * 128);
+        mbar_expect_tx(full, C * 128);
+        if (copies_g)
+          tma_load_3d(sbase + off_kh(n) + lane * (C * 128), &tmap_g, lane * 32, x.head, z, full);
+        else if (lane < 6)
+          tma_load_3d(raw, &tmap_k, (lane & 1) * 64, x.k_head, z, full);
+        else
+          tma_load_3d(raw + OFF_RAW_Q, &tmap_q, (lane & 1) * 64, x.k_head, z, full);
+        issued = n + 1;
+      }
+      __syncwarp();
+    };
+    for (int n = 0; n < 2 && n < all_chunks; ++n) copy(n);
+    // KDA: beta as well, lane = token, into its ring before MMA1 goes out (its readers wait for that product)
+    auto fetch_beta = [&](int n) { return lane < x.n_tok - n * C ? a.beta[(x.tok0 + n * C + lane) * a.H_v + x.head] : 0.f; };
+    float beta = KDA && all_chunks > 0 ? fetch_beta(0) : 0.f;
+    for (int n = 0; n < all_chunks; ++n) {
+      if (KDA) {
+        beta_s[(n % RING) * C + lane] = beta;
+        __syncwarp();
+        beta = fetch_beta(n + 1);
+      }
+      if (n > 0) wait_bar(&misc->bar_ro[buf(n - 1)], phase(n - 1), misc);
+      mma1(n);
+      take_a(n);
+      // MMA1 has read what the copies land on (KDA: the K-major Kh; GDN: raw k, q).  KDA, raw k, q: the MN-major tile, of which there are
+      // four, was read by MMA5 of two chunks ago, which the chain warps had seen complete before MMA2 of the chunk before.
+      if (n + 2 < all_chunks) copy(n + 2);
+    }
+    // after a time-out the last copies may not have been waited for: they must have landed before the CTA leaves
+    if (misc->abort_flag && issued > 0)
+      mbar_wait_bounded(copies_g ? &misc->g_full[buf(issued - 1)] : &misc->kq_full[buf(issued - 1)], phase(issued - 1), kMaxPolls);
+    __syncwarp();
+    // (after a time-out: as for the issuing warp)
+    if (misc->abort_flag) {
+      if (elect_one()) mma_commit(&misc->drain_1);
+      __syncwarp();
+      mbar_wait_bounded(&misc->drain_1, 0, kMaxPolls);
+    }
+    __syncwarp();
+  } else if (ALONE && warp >= WARP_O) {
+    // ================================= output warps (ALONE) =================================
+    // P and the outputs off the chain: P of the next chunk as soon as the products that read this one's have completed.
+    if (WITH_O && all_chunks > 0) {
+      const int ti = tid - WARP_O * 32;
+      OT *go = static_cast<OT *>(a.o) + (units[0].tok0 * a.H_v + units[0].head) * D;
+      if (sizeof(OT) == 2) go += (ti >> 4) * v_stride + (ti & 15) * 8;
+      auto next_p = [&](int n) {
+        if (quad >= 2) {
+          take_p(n, 0);
+          take_p(n, 1);
+        }
+        // -> MMA3, whose issue also says that the outputs up to chunk n - 2 have left tensor memory (there are three buffers)
+        arrive_warp(&misc->rdy_rhs, lane);
+      };
+      next_p(0);
+      const int n_tok = uni(units[0].n_tok);
+      for (int n = 0; n < all_chunks; ++n) {
+        wait_bar(&misc->bar_o, n & 1, misc);
+        if (n + 1 < all_chunks) next_p(n + 1);
+        asm volatile("bar.sync 6, 128;" ::: "memory");  // all have copied the previous chunk's out of the O tile
+        outputs(n, min(C, n_tok - n * C), go, 0, ti);
+        go += C * v_stride;
+        tc_fence_before_sync();
+      }
+    }
   } else if (warp >= 8) {
     // =============================== producer warps ===============================
     // warp = block of 32 channels; per half of the chunk, lane = (4 adjacent channels, 4 consecutive tokens), a 4 x 4
     // tile.  The midpoint is the end of the first half: first-half exponents are (local sum - the half's total),
     // second-half exponents the local sums themselves, so the halves are independent of one another.
-    const int pw = warp - 8;
+    const int pw = ALONE ? (warp & 3) : warp - 8;  // ALONE: warps 8-11 take the first half of the tokens, 12-15 the second
+    const int half_0 = ALONE ? (warp - 8) >> 2 : 0, half_n = ALONE ? half_0 + 1 : 2;
     const int cq = lane & 7, tg = lane >> 3;
     const int c0 = pw * 32 + cq * 4;
     // Inputs come by TMA a chunk ahead into tiles they will be overwritten with (KDA) or that are
@@ -655,7 +896,6 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
     //   raw k, q: two boxes each of 32 tokens x 64 channels.  KDA: into the MN-major Kh tile of the chunk's parity, written
     //   half by half once all producers have read that half (both layouts keep 16 tokens in 2 KB of every 4 KB).  GDN:
     //   the operand tile of MMA1 itself.
-    constexpr uint32_t RAW_ROWS = KDA ? 32 : 64, OFF_RAW_Q = KDA ? 2 * 32 * 128 : 32 * 128;
     int g_issued = 0, kq_issued = 0;
     // Each warp's first lane starts one box of each stream: a copy takes its issuing thread 200 to 300 cycles, and the warp that
     // issued all of them arrived 800 cycles behind the others.
@@ -668,22 +908,24 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
     };
     auto stage_kq = [&](int n) {
       if (!WITH_O && pw >= 2) return;
-      const uint32_t dst = sbase + (KDA ? OFF_KHT + (n & 1) * (128 * 128) : OFF_KQ16) + (pw & 1) * (RAW_ROWS * 128);
-      mbar_expect_tx(&misc->kq_full, C * 128);
+      const uint32_t dst = sbase + (KDA ? off_kht(n) : off_kh(n)) + (pw & 1) * (RAW_ROWS * 128);
+      uint64_t *const full = &misc->kq_full[0];
+      mbar_expect_tx(full, C * 128);
       if (pw < 2)
-        tma_load_3d(dst, &tmap_k, pw * 64, cp_k_head, cp_tok, &misc->kq_full);
+        tma_load_3d(dst, &tmap_k, pw * 64, cp_k_head, cp_tok, full);
       else
-        tma_load_3d(dst + OFF_RAW_Q, &tmap_q, (pw & 1) * 64, cp_k_head, cp_tok, &misc->kq_full);
+        tma_load_3d(dst + OFF_RAW_Q, &tmap_q, (pw & 1) * 64, cp_k_head, cp_tok, full);
       ++kq_issued;
     };
-    auto stage_g = [&]() {
-      mbar_expect_tx(&misc->g_full, C * 128);
-      tma_load_3d(sbase + OFF_KH + pw * (C * 128), &tmap_g, pw * 32, cp_head, cp_tok, &misc->g_full);
+    auto stage_g = [&](int n) {
+      uint64_t *const full = &misc->g_full[0];
+      mbar_expect_tx(full, C * 128);
+      tma_load_3d(sbase + off_kh(n) + pw * (C * 128), &tmap_g, pw * 32, cp_head, cp_tok, full);
       ++g_issued;
     };
-    if (lane == 0 && all_chunks > 0) {
+    if (!ALONE && lane == 0 && all_chunks > 0) {
       next_copies(units[0], 0);
-      if (KDA) stage_g();
+      if (KDA) stage_g(0);
       stage_kq(0);
     }
     // GDN, per-token scalars, by the first warp (lane = token): a chunk's go to their ring slots (the chain warps are at most two
@@ -702,7 +944,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
     //   MMA1 works on raw k, q (bf16 tile), MMA2 on raw k, q widened to tf32 containers, MMA5 on k_t e2_t;
     //   e1_t goes onto the rows of A, R and the outputs where they leave tensor memory, e2_j onto the columns of A, P.
     auto scalars = [&](int n, int u, int t0) {  // chunk n of the CTA: the tokens of unit u from t0 on
-      const int slot = (n & 3) * C + lane;
+      const int slot = (n % RING) * C + lane;
       const float beta = beta_next;
       beta_s[slot] = beta;
       float incl = gsc_next;
@@ -724,9 +966,9 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
       if (t0 == 0) post_prev = 0.f;
       const float f = ex2f((post_prev + tot0) * LOG2E);
       post_prev = tot1;
-      *reinterpret_cast<float4 *>(fac_s + (n & 1) * D + lane * 4) = make_float4(f, f, f, f);
+      *reinterpret_cast<float4 *>(fac_s + (n % FAC) * D + lane * 4) = make_float4(f, f, f, f);
       if (lane == 0) post_s[n & 3] = tot1;
-      arrive_warp(&misc->rdy_fac[n & 1], lane);
+      arrive_warp(&misc->rdy_fac[n % FAC], lane);
       t0 += C;
       if (t0 >= units[u].n_tok) {
         t0 = 0;
@@ -734,7 +976,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
       }
       if (n + 1 < all_chunks) fetch_scalars(units[u], t0);
     };
-    if (!KDA && pw == 0 && all_chunks > 0) {
+    if (!KDA && warp == 8 && all_chunks > 0) {
       fetch_scalars(units[0], 0);
       scalars(0, 0, 0);
     }
@@ -742,16 +984,20 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
     for (int n = 0, u = 0, t0 = 0; n < all_chunks; ++n) {
       const uint32_t par = n & 1;
       const int ntok = min(C, n_tok - t0);
-      unsigned char *kht_tile = smem + OFF_KHT + par * (128 * 128);
-      unsigned char *raw = KDA ? kht_tile : smem + OFF_KQ16;
-      if (!KDA) asm volatile("bar.sync 2, 128;" ::: "memory");   // the per-token factors are visible to all producer warps
+      unsigned char *kht_tile = smem + off_kht(n);
+      unsigned char *raw = KDA ? kht_tile : smem + off_kh(n);
+      unsigned char *const kq_tile = smem + off_kq(n), *const kh_tile = smem + off_kh(n);
+      // GDN: the per-token factors are visible to all producer warps.  ALONE: so is what the chunk before owes, and all have read that
+      // chunk's raw inputs
+      if (!KDA || ALONE) asm volatile("bar.sync 2, %0;" ::"n"(NP) : "memory");
       bool out_of_range = false;
-      wait_bar(&misc->kq_full, par, misc);
-      if (KDA) wait_bar(&misc->g_full, par, misc);
+      wait_bar(&misc->kq_full[buf(n)], phase(n), misc);
+      if (KDA) wait_bar(&misc->g_full[buf(n)], phase(n), misc);
+      if (ALONE && n > 1) wait_bar(&misc->bar_ro[buf(n)], phase(n - 2), misc);  // Kt/Qt of two chunks ago have been read
       const uint64_t l2e2 = pack2(LOG2E, LOG2E), comp2 = pack2(kLog2TruncComp, kLog2TruncComp);
       const uint64_t qs2 = pack2(a.q_scale, a.q_scale);
 #pragma unroll 1
-      for (int half = 0; half < 2; ++half) {
+      for (int half = half_0; half < half_n; ++half) {
         const int tr = half * 16 + tg * 4;
         // This lane's vectors (token tr + j): tr is a multiple of 4, so the row's part of a swizzle is an exclusive or with j.
         const uint32_t or0 = sw128_offset_bf16(RAW_ROWS, tr, c0), ok0 = sw128_offset(64, tr, c0), oh0 = sw128_offset(32, tr, c0),
@@ -777,7 +1023,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
         if constexpr (KDA) {
           float4 g4[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) g4[j] = *reinterpret_cast<const float4 *>(smem + OFF_KH + (oh0 ^ (j << 4)) + j * 128);
+          for (int j = 0; j < 4; ++j) g4[j] = *reinterpret_cast<const float4 *>(kh_tile + (oh0 ^ (j << 4)) + j * 128);
           if (left < 4) {
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -804,19 +1050,19 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
             // the first half's sums only: it is handed to the chain warps before the tiles are built.
             if (tg == 0) {
               const float4 pp = t0 > 0 ? *reinterpret_cast<const float4 *>(post_s + (par ^ 1) * D + c0) : make_float4(0.f, 0.f, 0.f, 0.f);
-              *reinterpret_cast<float4 *>(fac_s + par * D + c0) =
+              *reinterpret_cast<float4 *>(fac_s + (n % FAC) * D + c0) =
                   make_float4(ex2f((pp.x + tot[0]) * LOG2E), ex2f((pp.y + tot[1]) * LOG2E), ex2f((pp.z + tot[2]) * LOG2E),
                               ex2f((pp.w + tot[3]) * LOG2E));
             }
-            arrive_warp(&misc->rdy_fac[par], lane);
+            arrive_warp(&misc->rdy_fac[n % FAC], lane);
             ref01 = pack2(-tot[0] * LOG2E, -tot[1] * LOG2E);
             ref23 = pack2(-tot[2] * LOG2E, -tot[3] * LOG2E);
           } else if (tg == 0) {
             *reinterpret_cast<float4 *>(post_s + par * D + c0) = make_float4(tot[0], tot[1], tot[2], tot[3]);  // G_C - G_m
           }
-          asm volatile("bar.sync 2, 128;" ::: "memory");  // this half's raw k, q have been read: Kh may take their place
+          asm volatile("bar.sync %0, 128;" ::"r"(ALONE ? 4 + half : 2) : "memory");  // this half's raw k, q have been read: Kh may take their place
           // the Kt/Qt tile is free once MMA2 of the previous chunk has completed
-          if (n > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
+          if (!ALONE && n > 0 && half == 0) wait_bar(&misc->bar_ro[0], par ^ 1, misc);
           uint64_t run01 = pack2(run0[0], run0[1]), run23 = pack2(run0[2], run0[3]);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -836,7 +1082,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
             unpack2(mul2(k23, e1_23), kt[2], kt[3]);
             unpack2(mul2(k01, e2_01), kh[0], kh[1]);
             unpack2(mul2(k23, e2_23), kh[2], kh[3]);
-            unsigned char *pk = smem + OFF_KQ + (ok0 ^ (j << 4)) + j * 128;
+            unsigned char *pk = kq_tile + (ok0 ^ (j << 4)) + j * 128;
             if (WITH_O) {
               const uint64_t q01 = pack2(bf16lo(qw[j].x), bf16hi(qw[j].x)), q23 = pack2(bf16lo(qw[j].y), bf16hi(qw[j].y));
               float qt[4];
@@ -849,19 +1095,19 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
             // MN-major (MMA5 contracts over the tokens).  A tf32 MN-major operand has a swizzle of its own, so the two
             // tiles differ in where a vector lands, not in what it holds.
             const uint4 khv = make_uint4(tf32_pre(kh[0]), tf32_pre(kh[1]), tf32_pre(kh[2]), tf32_pre(kh[3]));
-            *reinterpret_cast<uint4 *>(smem + OFF_KH + (oh0 ^ (j << 4)) + j * 128) = khv;
+            *reinterpret_cast<uint4 *>(kh_tile + (oh0 ^ (j << 4)) + j * 128) = khv;
             *reinterpret_cast<uint4 *>(kht_tile + (om0 ^ (j << 5)) + j * 128) = khv;
           }
         } else {
-          if (n > 0 && half == 0) wait_bar(&misc->bar_ro, par ^ 1, misc);
+          if (!ALONE && n > 0 && half == 0) wait_bar(&misc->bar_ro[0], par ^ 1, misc);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            unsigned char *pk = smem + OFF_KQ + (ok0 ^ (j << 4)) + j * 128;
+            unsigned char *pk = kq_tile + (ok0 ^ (j << 4)) + j * 128;
             const uint4 kf = make_uint4(kw[j].x << 16, kw[j].x & 0xFFFF0000u, kw[j].y << 16, kw[j].y & 0xFFFF0000u);  // exact
             *reinterpret_cast<uint4 *>(pk) = kf;
             if (WITH_O)
               *reinterpret_cast<uint4 *>(pk + 32 * 128) = make_uint4(qw[j].x << 16, qw[j].x & 0xFFFF0000u, qw[j].y << 16, qw[j].y & 0xFFFF0000u);
-            const float e2 = e2_s[(n & 3) * C + tr + j];
+            const float e2 = e2_s[(n % RING) * C + tr + j];
             *reinterpret_cast<uint4 *>(kht_tile + (om0 ^ (j << 5)) + j * 128) =
                 make_uint4(tf32_pre(__uint_as_float(kf.x) * e2), tf32_pre(__uint_as_float(kf.y) * e2),
                            tf32_pre(__uint_as_float(kf.z) * e2), tf32_pre(__uint_as_float(kf.w) * e2));
@@ -871,40 +1117,43 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
       // the exponents of this chunk may have overflowed: the unit will not be written back
       if (KDA && out_of_range && tg == 0) misc->domain_flag[u & 3] = 1;
       fence_smem_to_async();
-      arrive_warp(&misc->rdy_prep, lane);  // -> MMA1
+      arrive_warp(&misc->rdy_prep[buf(n)], lane);  // -> MMA1
       t0 += C;
       if (t0 >= n_tok) {
         t0 = 0;
         ++u;
       }
       if (n + 1 < all_chunks) {
-        next_copies(units[u], t0);
-        n_tok = units[u].n_tok;
-        if (!KDA && pw == 0) scalars(n + 1, u, t0);
+        if (!ALONE) {
+          next_copies(units[u], t0);
+          n_tok = units[u].n_tok;
+        }
+        if (!KDA && warp == 8) scalars(n + 1, u, t0);
         // The next raw k, q (KDA) land once MMA5 of the previous chunk has read the Kh tile of that parity; the next
         // log-decay (KDA) or k, q (GDN) once MMA1 of this chunk has read the tile they go to.
-        if (KDA) {
-          if (n > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
+        if (KDA && !ALONE) {
+          if (n > 0) wait_bar(&misc->bar_s[0], par ^ 1, misc);
           if (lane == 0 && !misc->abort_flag) stage_kq(n + 1);
         }
-        wait_bar(&misc->bar_ap, par, misc);
-        if (lane == 0 && !misc->abort_flag) {
-          if (KDA) stage_g(); else stage_kq(n + 1);
+        if (!ALONE) {
+          wait_bar(&misc->bar_ap[0], par, misc);
+          if (lane == 0 && !misc->abort_flag) {
+            if (KDA) stage_g(n + 1); else stage_kq(n + 1);
+          }
         }
       }
     }
     // after a time-out the last copies may not have been waited for: they must have landed before the CTA leaves
     if (lane == 0 && misc->abort_flag) {
-      if (g_issued > 0) mbar_wait_bounded(&misc->g_full, (g_issued - 1) & 1, kMaxPolls);
-      if (kq_issued > 0) mbar_wait_bounded(&misc->kq_full, (kq_issued - 1) & 1, kMaxPolls);
+      if (g_issued > 0) mbar_wait_bounded(&misc->g_full[0], (g_issued - 1) & 1, kMaxPolls);
+      if (kq_issued > 0) mbar_wait_bounded(&misc->kq_full[0], (kq_issued - 1) & 1, kMaxPolls);
     }
   } else {
     // ================================= chain warps =================================
-    const int quad = warp & 3, colh = warp >> 2;                           // TMEM lane quadrant, column half
-    const uint32_t tlane = tm + (static_cast<uint32_t>(quad * 32) << 16);  // this warp's TMEM lanes
-    const int vrow = quad * 32 + lane;                                     // the TMEM lane this thread owns
+    const int colh = warp >> 2;            // column half
+    const int vrow = quad * 32 + lane;     // the TMEM lane this thread owns
 
-    const int g = lane >> 2, tig = lane & 3;
+    auto col_block = [&](int i) { return ALONE ? i * 64 + colh * 32 : colh * 64 + i * 32; };  // this warp's two blocks of 32 state columns
     int n = 0;  // index among the CTA's chunks
 #pragma unroll 1
     for (int u = 0; u < uni(misc->n_units); ++u) {
@@ -917,7 +1166,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
         // the start state goes into TMEM as it is; the first chunk's state pass scales it like any other.  (The state of the unit
         // before has been read out by the same threads.)
 #pragma unroll 1
-        for (int c0 = colh * 64; c0 < colh * 64 + 64; c0 += 32) {
+        for (int i = 0; i < 2; ++i) {
+          const int c0 = col_block(i);
           const float *const st_c = a.state + x.state + (c0 * D + vrow);
           uint32_t s[32];
           if (a.mode == DASC_REFRESH_CONTINUE) {
@@ -934,84 +1184,100 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
       for (int ch = 0; ch < n_chunks; ++ch, ++n) {
         const uint32_t par = n & 1;
         const int ntok = min(C, n_tok - ch * C);
-        const float *beta_c = beta_s + (n & 3) * C;
-        const float *fac_c = fac_s + par * D;
+        const float *beta_c = beta_s + (n % RING) * C;
+        const float *fac_c = fac_s + (n % FAC) * D;
         if (n + 1 == all_chunks && tid == 0) stream_order_release();  // one chunk (2.5 us) before the end: see launch.cuh
 
         // ---- (1) the previous chunk's state update is complete; this chunk's factors and tiles are ready ----
-        if (ch > 0) wait_bar(&misc->bar_s, par ^ 1, misc);
-        wait_bar(&misc->rdy_fac[par], (n >> 1) & 1, misc);
+        wait_bar(&misc->rdy_fac[n % FAC], (n / FAC) & 1, misc);
+        if (ch > 0) wait_bar(&misc->bar_s[buf(n - 1)], phase(n - 1), misc);
         tc_fence_after_sync();
 
         // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
         {
-          uint64_t f[8];
+          if constexpr (ALONE) {
+            // channels 0-63 first: MMA2 starts on them while 64-127 are scaled
+            uint32_t s[2][2][16];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const uint64_t *>(fac_c + colh * 64 + 8 * i + 2 * tig);
-#pragma unroll 1
-          for (uint32_t hh = 0; hh < 2; ++hh) {  // lanes 0-15, 16-31 of the quadrant
-            const uint32_t addr = tlane + (hh << 20) + COL_S + colh * 64;
-            uint32_t s[32];
-            tmem_ld_16x256b(addr, s);
+            for (uint32_t part = 0; part < 2; ++part)
+#pragma unroll
+              for (uint32_t hh = 0; hh < 2; ++hh) tmem_ld_16x256b(tlane + (hh << 20) + COL_S + part * 64 + colh * 32, s[part][hh]);
             tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              scale2(s[4 * i + 0], s[4 * i + 1], f[i]);
-              scale2(s[4 * i + 2], s[4 * i + 3], f[i]);
+            for (uint32_t part = 0; part < 2; ++part) {
+              const int c = part * 64 + colh * 32;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const uint64_t f = *reinterpret_cast<const uint64_t *>(fac_c + c + 8 * i + 2 * tig);
+#pragma unroll
+                for (uint32_t hh = 0; hh < 2; ++hh) {
+                  scale2(s[part][hh][4 * i + 0], s[part][hh][4 * i + 1], f);
+                  scale2(s[part][hh][4 * i + 2], s[part][hh][4 * i + 3], f);
+                }
+              }
+              if (part == 1) {  // the first part's stores have had the time of this scaling
+                tmem_st_wait();
+                tc_fence_before_sync();
+                arrive_warp(&misc->rdy_half, lane);  // -> MMA2's first half
+              }
+#pragma unroll
+              for (uint32_t hh = 0; hh < 2; ++hh) tmem_st_16x256b(tlane + (hh << 20) + COL_S + c, s[part][hh]);
             }
-            tmem_st_16x256b(addr, s);
+          } else {
+            uint64_t f[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) f[i] = *reinterpret_cast<const uint64_t *>(fac_c + colh * 64 + 8 * i + 2 * tig);
+#pragma unroll 1
+            for (uint32_t hh = 0; hh < 2; ++hh) {  // lanes 0-15, 16-31 of the quadrant
+              const uint32_t addr = tlane + (hh << 20) + COL_S + colh * 64;
+              uint32_t s[32];
+              tmem_ld_16x256b(addr, s);
+              tmem_ld_wait();
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                scale2(s[4 * i + 0], s[4 * i + 1], f[i]);
+                scale2(s[4 * i + 2], s[4 * i + 3], f[i]);
+              }
+              tmem_st_16x256b(addr, s);
+            }
           }
           tmem_st_wait();
         }
         tc_fence_before_sync();
         arrive_warp(&misc->rdy_state, lane);  // -> MMA2
 
-        // ---- (3) P = lower_incl_diag(Qt Kh^T) out of TMEM (rows 0-15, 16-31 are in the third and fourth quadrant) straight to
-        //          its operand tile.  GDN: the raw q_t . k_j gets its column factor e2_j here, the row factor e1_t is applied
-        //          to the outputs ----
-        if (WITH_O && quad >= 2) {
-          wait_bar(&misc->bar_ap, par, misc);
-          tc_fence_after_sync();
-          uint32_t x[8];
-          tmem_ld_16x256b(tlane + COL_AP + colh * 16, x);
-          if (n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);  // the previous chunk's outputs have left this storage
-          tmem_ld_wait();
-          const int t = (quad - 2) * 16 + g;
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int j = colh * 16 + 8 * i + 2 * tig;
-            float2 e = make_float2(kInvTruncComp, kInvTruncComp);
-            if constexpr (!KDA) {
-              const float2 e2 = *reinterpret_cast<const float2 *>(e2_s + (n & 3) * C + j);
-              e.x *= e2.x;
-              e.y *= e2.y;
-            }
-            unsigned char *const p = smem + OFF_PM + sw128_offset(32, t, j);
-            *reinterpret_cast<uint2 *>(p) = make_uint2(j <= t ? tf32_pre(__uint_as_float(x[4 * i]) * e.x) : 0u,
-                                                       j + 1 <= t ? tf32_pre(__uint_as_float(x[4 * i + 1]) * e.y) : 0u);
-            *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(j <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 2]) * e.x) : 0u,
-                                                              j + 1 <= t + 8 ? tf32_pre(__uint_as_float(x[4 * i + 3]) * e.y) : 0u);
-          }
-          fence_smem_to_async();
-        }
+        // ---- (3) P ----
+        if (!ALONE && WITH_O && quad >= 2) take_p(n, colh);
 
         // ---- (4) RHS^T = beta (V - R)^T as a tf32 pair: high over R^T, low in the consumed A|P columns ----
-        wait_bar(&misc->bar_ro, par, misc);
-        tc_fence_after_sync();
         // A's and P's columns are about to be overwritten: A's by warps that wait for its readers (the issuing warp read its rows
-        // before it issued MMA2), P's by the warps that read them
+        // before it issued MMA2), P's by the warps that read them.  (The wait that comes last in time is the last one.)
         wait_bar(&misc->a_taken, par, misc);
         wait_bar(&misc->v_full, par, misc);
         {
           const int tb = colh * 16;
-          // blocks of one ldmatrix: tokens 0-7 of the half with values 0-7, 8-15, tokens 8-15 with the same
+          // V and the per-token factors are fetched before the last wait.  Blocks of one ldmatrix: tokens 0-7 of the half with values
+          // 0-7, 8-15, tokens 8-15 with the same
           const int vt = tb + (lane >> 4) * 8 + (lane & 7);
+          uint32_t xx[2][8], vvv[2][4];
+          uint64_t beta2[2], e1c2[2];
+#pragma unroll
+          for (uint32_t hh = 0; hh < 2; ++hh)
+            ldmatrix_x4_trans(vvv[hh], sbase + OFF_V + (quad >> 1) * (C * 128) + vt * 128 +
+                                           ((((quad & 1) * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (vt & 7)) << 4));
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            beta2[i] = *reinterpret_cast<const uint64_t *>(beta_c + tb + i * 8 + 2 * tig);
+            if (!KDA) e1c2[i] = *reinterpret_cast<const uint64_t *>(e1c_s + (n % RING) * C + tb + i * 8 + 2 * tig);
+          }
+          wait_bar(&misc->bar_ro[buf(n)], phase(n), misc);
+          tc_fence_after_sync();
+#pragma unroll
+          for (uint32_t hh = 0; hh < 2; ++hh) tmem_ld_16x256b(tlane + (hh << 20) + col_ro(n) + tb, xx[hh]);
+          tmem_ld_wait();
 #pragma unroll
           for (uint32_t hh = 0; hh < 2; ++hh) {
-            uint32_t x[8], lo[8], vv[4];
-            tmem_ld_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
-            ldmatrix_x4_trans(vv, sbase + OFF_V + (quad >> 1) * (C * 128) + vt * 128 +
-                                      ((((quad & 1) * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (vt & 7)) << 4));
+            uint32_t(&x)[8] = xx[hh], (&vv)[4] = vvv[hh], lo[8];
             if (ntok < C) {
               // the boxes reached past the request's last token: those values are other tokens' (zeros past the end of the stream)
 #pragma unroll
@@ -1021,14 +1287,12 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
                 else if (t + 1 >= ntok) vv[i] &= 0xFFFFu;
               }
             }
-            tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              const int t = tb + (i >> 1) * 8 + 2 * tig;
               uint64_t r = pack2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
               // GDN: the product is k_t S' on the raw keys; its row factor e1_t (with the truncation compensation) comes here
-              if constexpr (!KDA) r = mul2(*reinterpret_cast<const uint64_t *>(e1c_s + (n & 3) * C + t), r);
-              r = mul2(*reinterpret_cast<const uint64_t *>(beta_c + t), sub2(pack2(bf16lo(vv[i]), bf16hi(vv[i])), r));
+              if constexpr (!KDA) r = mul2(e1c2[i >> 1], r);
+              r = mul2(beta2[i >> 1], sub2(pack2(bf16lo(vv[i]), bf16hi(vv[i])), r));
               // the high part is the value itself, which the tensor core truncates on reading; the low part the exact rest
               float r0, r1;
               unpack2(r, r0, r1);
@@ -1038,8 +1302,8 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
               lo[2 * i] = tf32_pre(r0);
               lo[2 * i + 1] = tf32_pre(r1);
             }
-            tmem_st_16x256b(tlane + (hh << 20) + COL_RO + tb, x);
-            tmem_st_16x256b(tlane + (hh << 20) + COL_AP + tb, lo);
+            tmem_st_16x256b(tlane + (hh << 20) + col_ro(n) + tb, x);
+            tmem_st_16x256b(tlane + (hh << 20) + COL_RL + tb, lo);
           }
           tmem_st_wait();
         }
@@ -1053,72 +1317,24 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
         {
           const int tb = colh * 16;
           uint32_t x[16];
-          tmem_ld16(tlane + COL_U + tb, x);
+          tmem_ld16(tlane + COL_U<ALONE> + tb, x);
           tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < 16; ++j)
             x[j] = tf32_pre(__uint_as_float(x[j]) - __uint_as_float(x[j] & 0xFFFFE000u));
-          tmem_st16(tlane + COL_RO + tb, x);
+          tmem_st16(tlane + col_ro(n) + tb, x);
           tmem_st_wait();
         }
         tc_fence_before_sync();
         arrive_warp(&misc->rdy_u, lane);  // -> MMA4, MMA5
 
-        // ---- (6) outputs of this chunk ----
-        wait_bar(&misc->bar_o, par, misc);
-        tc_fence_after_sync();
-        if (WITH_O) {
-          const int tb = colh * 16;
-          const int ot = tb + (lane >> 4) * 8 + (lane & 7);  // blocks of one stmatrix: as for V
-          uint32_t xx[2][8];
-          tmem_ld_16x256b(tlane + COL_RO + 32 + tb, xx[0]);
-          tmem_ld_16x256b(tlane + (1u << 20) + COL_RO + 32 + tb, xx[1]);
-          tmem_ld_wait();
-#pragma unroll
-          for (uint32_t hh = 0; hh < 2; ++hh) {
-            uint32_t(&x)[8] = xx[hh];
-            if constexpr (!KDA) {
-              // GDN: the accumulated q_t (S' + sum_j e2_j k_j u_j^T) still lacks its row factor e1_t, the query scale and
-              // the truncation compensation
-#pragma unroll
-              for (int i = 0; i < 2; ++i) {
-                const float2 e = *reinterpret_cast<const float2 *>(e1c_s + (n & 3) * C + tb + 8 * i + 2 * tig);
-                x[4 * i + 0] = __float_as_uint(__uint_as_float(x[4 * i + 0]) * (e.x * a.q_scale));
-                x[4 * i + 1] = __float_as_uint(__uint_as_float(x[4 * i + 1]) * (e.y * a.q_scale));
-                x[4 * i + 2] = __float_as_uint(__uint_as_float(x[4 * i + 2]) * (e.x * a.q_scale));
-                x[4 * i + 3] = __float_as_uint(__uint_as_float(x[4 * i + 3]) * (e.y * a.q_scale));
-              }
-            }
-            if constexpr (sizeof(OT) == 2) {
-              uint32_t w[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) w[i] = pack_bf16x2(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
-              stmatrix_x4_trans(sbase + OFF_TM + ot * 256 + (((quad * 4 + hh * 2 + ((lane >> 3) & 1)) ^ (ot & 7)) << 4), w[0], w[1], w[2], w[3]);
-            } else {
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int t = tb + (i >> 1) * 8 + 2 * tig, v = quad * 32 + hh * 16 + (i & 1) * 8 + g;
-                if (t < ntok) go[t * v_stride + v] = __uint_as_float(x[2 * i]);
-                if (t + 1 < ntok) go[(t + 1) * v_stride + v] = __uint_as_float(x[2 * i + 1]);
-              }
-            }
-          }
-          if constexpr (sizeof(OT) == 2) {
-            // through shared memory (the T and P tiles are free now) so that global stores are 16 bytes wide
-            sync_chain();
-            const int j = tid & 15;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const int t = (tid >> 4) + 16 * i;
-              if (t < ntok)
-                *reinterpret_cast<uint4 *>(go + i * 16 * v_stride) =
-                    *reinterpret_cast<const uint4 *>(smem + OFF_TM + t * 256 + ((j ^ (t & 7)) << 4));
-            }
-          }
-          go += C * v_stride;
+        // ---- (6) outputs of this chunk (without outputs MMA5 is waited for here as well) ----
+        if (!ALONE) {
+          outputs(n, ntok, go, colh, tid);
+          if (WITH_O) go += C * v_stride;
+          tc_fence_before_sync();
+          arrive_warp(&misc->tp_free, lane);  // this thread is done with the T|P|O tile region
         }
-        tc_fence_before_sync();
-        arrive_warp(&misc->tp_free, lane);  // this thread is done with the T|P|O tile region
       }
       // ---- final state: the factor still owed, then write back ----
       // Which of this warp's rows are written, a bit each, fetched before the waits: looked up row by row beside the stores, the
@@ -1128,12 +1344,12 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const uint8_t *keep = a.row_keep + x.keep_row;
-        rows[i] = __ballot_sync(0xffffffffu, a.mode == DASC_REFRESH_CONTINUE || !keep[colh * 64 + i * 32 + lane]);
+        rows[i] = __ballot_sync(0xffffffffu, a.mode == DASC_REFRESH_CONTINUE || !keep[col_block(i) + lane]);
       }
       // post_s of the last chunk is visible: its writers arrived on rdy_prep, which the issuing warp waited for before it met the
       // triangular warp, which arrived on a_taken, which these warps have waited for.  (Waiting for rdy_prep itself here could wait for
       // the wrong phase: the next unit's tiles can be complete by now.)
-      if (n_chunks > 0) wait_bar(&misc->bar_s, (n - 1) & 1, misc);
+      if (n_chunks > 0) wait_bar(&misc->bar_s[buf(n - 1)], phase(n - 1), misc);
       if (tid < D) fin_s[tid] = n_chunks > 0 ? ex2f(post_s[KDA ? ((n - 1) & 1) * D + tid : (n - 1) & 3] * LOG2E) : 1.f;
       sync_chain();
       tc_fence_after_sync();
@@ -1147,7 +1363,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
       } else {
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
-          const int c0 = colh * 64 + i * 32;
+          const int c0 = col_block(i);
           const uint32_t write = i == 0 ? rows[0] : rows[1];
           float *const st_c = a.state + x.state + (c0 * D + vrow);
           const float *const fin_c = fin_s + c0;
@@ -1168,7 +1384,7 @@ __global__ void __launch_bounds__(NT, 2) refresh_chunked_kernel(const __grid_con
   }
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == WARP_MMA) tmem_dealloc(tm, TMEM_COLS);
+  if (warp == WARP_MMA) tmem_dealloc(tm, F::TMEM_COLS);
   if (tid == 0 && misc->abort_flag) atomicExch(static_cast<uint32_t *>(a.workspace), 1u);  // a wait ran out
 }
 
@@ -1257,12 +1473,24 @@ int64_t grid_for(const DascRefreshArgs &a, int64_t n_units) {
   return even && g < n_units ? g : n_units;
 }
 
+// With at most a CTA per SM the time is the chain of one CTA: hand-offs, not any unit of the SM, bound it.  The ALONE form takes off
+// the chain what need not be on it: producers with twice the warps, running up to two chunks ahead of the chain into second (MN-major Kh:
+// fourth) buffers; MMA1, the copies of the inputs, P and the outputs in warps of their own (one warp that issued all products was busy all of
+// the time: 100 to 120 cycles per barrier, 40 per product); MMA2 started on the first half of the scaled state; the state's product ahead of
+// the outputs'.  A chunk takes 3.8 k cycles instead of 4.8 k (GDN 3.5 k, 4.5 k), from cold inputs 4.0 k instead of 5.6 k.
+// Measured, us, SHARED / ALONE, 256 tokens (GDN): 8 units 27.3 / 23.4 (23.6 / 21.7), 80 units 32.2 / 25.7 (24.0 / 22.3), 148 units 40.1 / 31.9
+// (32.7 / 28.6), state only 35.0 / 24.8; 148 units of 1 .. 599 tokens 72.5 / 60.0; 152 units 44.2 / 48.2 (35.5 / 43.4): the line is where a
+// second CTA per SM begins to be needed.
+constexpr int64_t kAloneUnits = 148;
+
 template <bool KDA, typename OT, bool WITH_O>
 int launch(DascRefreshArgs a, void *stream) {
-  auto kern = refresh_chunked_kernel<KDA, OT, WITH_O>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(SMEM_ALLOC));
-  if (e != cudaSuccess) return static_cast<int>(e);
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
+  const bool alone = n_units <= kAloneUnits;
+  auto kern = alone ? refresh_chunked_kernel<KDA, OT, WITH_O, true> : refresh_chunked_kernel<KDA, OT, WITH_O, false>;
+  const uint32_t smem = alone ? SMEM_ALONE : SMEM_BYTES;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return static_cast<int>(e);
   if (n_units == 0) return cudaSuccess;
   if (n_units > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
   a.ordered = ordered(a);
@@ -1286,7 +1514,8 @@ int launch(DascRefreshArgs a, void *stream) {
       (WITH_O && !make_map(&tmap_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.q, a.H_k, 2)) ||
       (KDA && !make_map(&tmap_g, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.g, a.H_v, 4)))
     return static_cast<int>(cudaErrorInvalidValue);
-  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(grid_for(a, n_units))), dim3(NT), SMEM_ALLOC, stream, a, tmap_q, tmap_k, tmap_v, tmap_g));
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(alone ? n_units : grid_for(a, n_units))),
+                                          dim3(alone ? Form<true>::NT : Form<false>::NT), smem, stream, a, tmap_q, tmap_k, tmap_v, tmap_g));
 }
 
 }  // namespace
