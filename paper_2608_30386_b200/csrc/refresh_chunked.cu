@@ -54,7 +54,7 @@ using namespace tc5;
 constexpr int C = 32;          // chunk length
 constexpr int D = 128;         // d_k = d_v
 constexpr int NCH = 256;       // chain threads (warps 0-7)
-// Two forms.  SHARED: two CTAs per SM.  ALONE (see kAloneUnits): one, with more warps and second buffers, so that the tiles, MMA1 and T of
+// Two forms.  SHARED: two CTAs per SM.  ALONE (see alone_for): one, with more warps and second buffers, so that the tiles, MMA1 and T of
 // the next chunk are made while the chain is in this one, and the outputs leave meanwhile.
 template <bool ALONE>
 struct Form {
@@ -155,7 +155,7 @@ struct Misc {
   uint64_t v_full;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;   // a bounded wait ran out: every later wait of this CTA returns at once
-  int32_t n_units, all_chunks;    // this CTA's units (those that have tokens listed first) and the chunks of all of them
+  int32_t n_units, n_replayed, all_chunks;  // this CTA's units, those of them that have tokens (listed first), the chunks of all
   volatile uint32_t domain_flag[4];  // a half-chunk decay sum left the range the midpoint factors can carry; by unit index mod 4
 };
 static_assert(sizeof(Misc) <= 320, "Misc outgrew its shared-memory slot");
@@ -346,7 +346,9 @@ __device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
 
 // WITH_O = false is the state-only variant (no outputs wanted): q is never read, the Qt rows, P and the
 // output product are left out.
-template <bool KDA, typename OT, bool WITH_O, bool ALONE>
+// WALK = false: one unit per CTA, known at compile time (grid_for left the grid at that; always so where ALONE): the bookkeeping between
+// units costs 1 to 4 % of a chunk where there is none to do.
+template <bool KDA, typename OT, bool WITH_O, bool ALONE, bool WALK>
 __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunked_kernel(const __grid_constant__ DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
                                                                 const __grid_constant__ CUtensorMap tmap_k,
                                                                 const __grid_constant__ CUtensorMap tmap_v,
@@ -413,11 +415,11 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     tmem_alloc(&misc->tmem_base, F::TMEM_COLS);
     tmem_relinquish();
   }
-  // This CTA's units, a lane of one warp each: every gridDim.x-th, there and back (see grid_for).  Which they are is worked out
+  // This CTA's units, a lane of one warp each: every gridDim.x-th, there and back (see grid_for; one where WALK is false).  Which they are is worked out
   // before the wait for earlier work, their tokens and state are looked up behind it.
   if (warp == WARP_T) {
     const int64_t idx = static_cast<int64_t>(lane) * gridDim.x + ((lane & 1) ? gridDim.x - 1u - blockIdx.x : blockIdx.x);
-    bool here = lane < (ALONE ? 1 : kMaxWalk) && idx < static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
+    bool here = lane < (WALK ? kMaxWalk : 1) && idx < static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
     const uint32_t row = static_cast<uint32_t>(idx) / a.H_v;  // (the host sees to it that units fit 31 bits)
     Unit x;
     x.head = static_cast<int32_t>(static_cast<uint32_t>(idx) - row * a.H_v);
@@ -447,6 +449,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     const int chunks = __reduce_add_sync(0xffffffffu, here ? (x.n_tok + C - 1) / C : 0);
     if (lane == 0) {
       misc->n_units = __popc(with | without);
+      misc->n_replayed = __popc(with);
       misc->all_chunks = chunks;
     }
   } else {
@@ -697,31 +700,35 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     // This warp also starts the copies of V, a chunk ahead: two boxes of 32 tokens x 64 values with the 128-byte swizzle (no bank
     // conflicts for the 8 x 8 blocks it is read in).  Started by two of the chain warps they held those up for 280 cycles of every
     // chunk; here they fall into the wait for the next A (0.3 to 1 % of a launch).
-    int v_issued = 0, v_unit = 0, v_tok = 0;  // copies started; the next one's unit and first token in it
+    int v_issued = 0, v_unit = 0;                  // copies started; the next one's unit,
+    int v_tok = 0, v_n = 0, v_row = 0, v_head = 0;  // its first token in that, of how many, and its coordinates
+    auto next_v = [&]() {
+      v_tok = 0;
+      v_n = units[v_unit].n_tok;
+      v_row = static_cast<int32_t>(units[v_unit].tok0);
+      v_head = units[v_unit].head;
+    };
+    if (all_chunks > 0) next_v();
     auto stage_v = [&]() {  // (the copies by the first lane)
-      const Unit &x = units[v_unit];
       if (lane == 0 && !misc->abort_flag) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           mbar_expect_tx(&misc->v_full, C * 128);
-          tma_load_3d(sbase + OFF_V + i * (C * 128), &tmap_v, i * 64, x.head, static_cast<int32_t>(x.tok0 + v_tok), &misc->v_full);
+          tma_load_3d(sbase + OFF_V + i * (C * 128), &tmap_v, i * 64, v_head, v_row, &misc->v_full);
         }
         // the state that the unit starts from, 64 KB in one piece, is brought into L2 meanwhile
-        if (v_tok == 0 && v_issued > 0 && a.mode == DASC_REFRESH_CONTINUE)
-          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.state + x.state), "n"(D * D * 4) : "memory");
+        if (WALK && v_tok == 0 && v_issued > 0 && a.mode == DASC_REFRESH_CONTINUE)
+          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.state + units[v_unit].state), "n"(D * D * 4) : "memory");
         ++v_issued;
       }
       v_tok += C;
-      if (v_tok >= x.n_tok) {
-        v_tok = 0;
-        ++v_unit;
-      }
+      v_row += C;
+      if (WALK && v_tok >= v_n && ++v_unit < misc->n_replayed) next_v();
     };
     // KDA: it also brings in beta, a chunk ahead, and arrives on rdy_prep (ALONE: the MMA1 warp; GDN: the producer warps, whose per-token
     // factors contain it).
     auto fetch_beta = [&]() {  // of the chunk whose copy comes next, lane = token
-      const Unit &x = units[v_unit];
-      return lane < x.n_tok - v_tok ? a.beta[(x.tok0 + v_tok + lane) * a.H_v + x.head] : 0.f;
+      return lane < v_n - v_tok ? a.beta[static_cast<int64_t>(v_row + lane) * a.H_v + v_head] : 0.f;
     };
     if (all_chunks > 0) {
       if (KDA && !ALONE) {
@@ -970,7 +977,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       if (lane == 0) post_s[n & 3] = tot1;
       arrive_warp(&misc->rdy_fac[n % FAC], lane);
       t0 += C;
-      if (t0 >= units[u].n_tok) {
+      if (WALK && t0 >= units[u].n_tok) {
         t0 = 0;
         ++u;
       }
@@ -1119,15 +1126,14 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       fence_smem_to_async();
       arrive_warp(&misc->rdy_prep[buf(n)], lane);  // -> MMA1
       t0 += C;
-      if (t0 >= n_tok) {
+      cp_tok += C;
+      if (WALK && t0 >= n_tok && n + 1 < all_chunks) {
         t0 = 0;
         ++u;
+        next_copies(units[u], 0);
+        n_tok = units[u].n_tok;
       }
       if (n + 1 < all_chunks) {
-        if (!ALONE) {
-          next_copies(units[u], t0);
-          n_tok = units[u].n_tok;
-        }
         if (!KDA && warp == 8) scalars(n + 1, u, t0);
         // The next raw k, q (KDA) land once MMA5 of the previous chunk has read the Kh tile of that parity; the next
         // log-decay (KDA) or k, q (GDN) once MMA1 of this chunk has read the tile they go to.
@@ -1156,7 +1162,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     auto col_block = [&](int i) { return ALONE ? i * 64 + colh * 32 : colh * 64 + i * 32; };  // this warp's two blocks of 32 state columns
     int n = 0;  // index among the CTA's chunks
 #pragma unroll 1
-    for (int u = 0; u < uni(misc->n_units); ++u) {
+    for (int u = 0; u < (WALK ? uni(misc->n_units) : min(uni(misc->n_units), 1)); ++u) {
       const Unit &x = units[u];
       // where this thread's part of the outputs of a chunk starts (bf16: 16 bytes of every 16th token; fp32: see below)
       OT *go = WITH_O ? static_cast<OT *>(a.o) + (x.tok0 * a.H_v + x.head) * D : nullptr;
@@ -1380,6 +1386,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
             if (write >> j & 1u) st_c[j * D] = __uint_as_float(s[j]) * fin_c[j];
         }
       }
+      if (!WALK) break;
     }
   }
   tc_fence_before_sync();
@@ -1460,17 +1467,31 @@ EncodeTiledFn encode_tiled_fn() {
 //    a unit each go to whichever CTA ends first: 2048 units of 1 .. 1023 tokens take 669 / 658 walked, 1600 of 1 .. 1199 596 / 601: little
 //    to gain where units are long.
 //  - requests that are not in order of length (more than kRefreshOrderMax): only if they are about equally long.
-constexpr int64_t kResident = 2 * 148, kWalkChunks = 64;
-int64_t grid_for(const DascRefreshArgs &a, int64_t n_units) {
+constexpr int64_t kSms = 148, kResident = 2 * kSms, kWalkChunks = 64;
+
+// What the host knows of a launch: the longest request (by the caller's bound) and all units together, in chunks (about: half a one
+// more per request).
+struct Load {
+  int64_t n_units, longest, per_head, chunks;
+  bool in_order;  // requests come longest first
+};
+Load load_of(const DascRefreshArgs &a) {
   const int64_t tokens = a.window > 0 ? std::min<int64_t>(a.total_tokens, static_cast<int64_t>(a.n_req) * a.window) : a.total_tokens;
-  const int64_t longest = (std::max(a.max_seqlen, 1) + C - 1) / C;
-  const int64_t per_head = tokens / C + a.n_req / 2;  // chunks, about: half a one more per request
-  const int64_t chunks = per_head * a.n_layers_in_call * a.H_v;
-  int64_t g = kResident * std::max<int64_t>((chunks + kResident * kWalkChunks - 1) / (kResident * kWalkChunks),
-                                            (n_units + kResident * kMaxWalk - 1) / (kResident * kMaxWalk));
-  const bool in_order = a.ordered || a.n_req == 1;
-  const bool even = in_order ? longest * 2 * g <= chunks : longest * a.n_req * 9 <= per_head * 10;
-  return even && g < n_units ? g : n_units;
+  Load l;
+  l.n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
+  l.longest = (std::max(a.max_seqlen, 1) + C - 1) / C;
+  l.per_head = tokens / C + a.n_req / 2;
+  l.chunks = l.per_head * a.n_layers_in_call * a.H_v;
+  l.in_order = a.ordered || a.n_req == 1;
+  return l;
+}
+
+int64_t grid_for(const DascRefreshArgs &a) {
+  const Load l = load_of(a);
+  const int64_t g = kResident * std::max<int64_t>((l.chunks + kResident * kWalkChunks - 1) / (kResident * kWalkChunks),
+                                                  (l.n_units + kResident * kMaxWalk - 1) / (kResident * kMaxWalk));
+  const bool even = l.in_order ? l.longest * 2 * g <= l.chunks : l.longest * a.n_req * 9 <= l.per_head * 10;
+  return even && g < l.n_units ? g : l.n_units;
 }
 
 // With at most a CTA per SM the time is the chain of one CTA: hand-offs, not any unit of the SM, bound it.  The ALONE form takes off
@@ -1481,19 +1502,26 @@ int64_t grid_for(const DascRefreshArgs &a, int64_t n_units) {
 // Measured, us, SHARED / ALONE, 256 tokens (GDN): 8 units 27.3 / 23.4 (23.6 / 21.7), 80 units 32.2 / 25.7 (24.0 / 22.3), 148 units 40.1 / 31.9
 // (32.7 / 28.6), state only 35.0 / 24.8; 148 units of 1 .. 599 tokens 72.5 / 60.0; 152 units 44.2 / 48.2 (35.5 / 43.4): the line is where a
 // second CTA per SM begins to be needed.
-constexpr int64_t kAloneUnits = 148;
+// Up to twice as many units as well where one request is longer than an SM's share of all: they are placed longest first, and the
+// time is that request's.  SHARED / ALONE: 256 units of 1 .. 3801 tokens 376 / 317, 280 of 1 .. 1399 164 / 127, 192 of 1 .. 1199 125 / 94.
+bool alone_for(const DascRefreshArgs &a) {
+  const Load l = load_of(a);
+  return l.n_units <= kSms || (l.n_units <= kResident && l.in_order && l.chunks <= kSms * l.longest);
+}
 
 template <bool KDA, typename OT, bool WITH_O>
 int launch(DascRefreshArgs a, void *stream) {
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
-  const bool alone = n_units <= kAloneUnits;
-  auto kern = alone ? refresh_chunked_kernel<KDA, OT, WITH_O, true> : refresh_chunked_kernel<KDA, OT, WITH_O, false>;
+  a.ordered = ordered(a);
+  const bool alone = alone_for(a);
+  const int64_t grid = alone ? n_units : grid_for(a);
+  auto kern = alone ? refresh_chunked_kernel<KDA, OT, WITH_O, true, false>
+              : grid < n_units ? refresh_chunked_kernel<KDA, OT, WITH_O, false, true> : refresh_chunked_kernel<KDA, OT, WITH_O, false, false>;
   const uint32_t smem = alone ? SMEM_ALONE : SMEM_BYTES;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return static_cast<int>(e);
   if (n_units == 0) return cudaSuccess;
   if (n_units > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
-  a.ordered = ordered(a);
   const int prep = dasc_launch_refresh_prep(a, stream);
   if (prep != 0) return prep;
   // tensor maps of the token streams [Lc*T tokens][heads][128]: boxes of 32 tokens x one head x 128 bytes of channels with
@@ -1514,7 +1542,7 @@ int launch(DascRefreshArgs a, void *stream) {
       (WITH_O && !make_map(&tmap_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.q, a.H_k, 2)) ||
       (KDA && !make_map(&tmap_g, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, a.g, a.H_v, 4)))
     return static_cast<int>(cudaErrorInvalidValue);
-  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(alone ? n_units : grid_for(a, n_units))),
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(grid)),
                                           dim3(alone ? Form<true>::NT : Form<false>::NT), smem, stream, a, tmap_q, tmap_k, tmap_v, tmap_g));
 }
 
