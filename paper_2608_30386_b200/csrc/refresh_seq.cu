@@ -472,26 +472,398 @@ int launch(const DascRefreshArgs &a, void *stream) {
   return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(grid)), dim3(NCOL / COLS * SL + NHELP), smem, stream, a));
 }
 
-// Columns do not interact, so units that leave SMs idle are split by columns: parts of 8 (16 at d = 32) with 16 (8) lanes per
-// column and warps of their own for the conversions while that gives at most two CTAs per SM (beyond, the conversions, which
-// every part repeats, cost more than the shorter chain saves); at d = 128 halves while those fit one CTA per SM.
-// B200, 128 fp32 tokens, microseconds split / whole on both sides of each line (KDA; GDN the same within 2 us where not given):
+// ---------------------------------------------------------------------------------------------
+// Four tokens at a time, for the forms that are split by columns because units are few: there the serial chain is all there is.
+// With D_t the product of the decays of the block's tokens up to t, and everything else over the block's tokens j < t or j <= t,
+//   r_t = (D_t k_t)^T S_0 + sum_j c_tj u_j        c_tj = k_t^T Diag(alpha_{j+1} ... alpha_t) k_j
+//   o_t = (D_t q_t)^T S_0 + sum_j p_tj u_j        p_tj = q_t^T Diag(alpha_{j+1} ... alpha_t) k_j
+//   S_4 = Diag(D_3) S_0 + sum_j w_j u_j^T         w_j = Diag(alpha_{j+1} ... alpha_3) k_j
+// so that the four dot products of a lane and their shuffles run side by side and one chain of multiply-adds per block is left.  All
+// factors are products of at most two exponentials, of sums of the log-decay: no division, and half of the token-by-token form's error
+// against fp64 (4 units of 64 x 64, 64 tokens: state 6.2e-7 -> 3.0e-7, outputs 3.5e-7 -> 2.0e-7), whose decays multiply up one token at
+// a time.  The helper warps form D k, D q, w and the 16 coefficients of a block, a group of tokens ahead; they and the replaying warps
+// share the SM's issue slots, which is what bounds a group now (about 95 ns per token at d = 64, 135 before).  More helper warps, or
+// copies and outputs in warps of their own, gained nothing.
+// ---------------------------------------------------------------------------------------------
+constexpr int NB = TB / 4;  // blocks of a group
+constexpr int NRAW = 4;     // groups whose raw rows are in shared memory
+
+template <int DK, int NCOL, int SL, typename IO, bool KDA>
+struct BlockSmem {
+  // raw staging, three groups ahead of the one that is being converted: a group takes less than a trip to memory
+  alignas(16) IO q[NRAW][TB][DK];
+  alignas(16) IO k[NRAW][TB][DK];
+  alignas(16) IO v[NRAW][TB][NCOL];
+  alignas(16) float g[NRAW][TB][KDA ? DK : 4];
+  alignas(16) float beta[NRAW][TB];
+  struct Group {
+    alignas(16) float kf[TB][DK];  // D k
+    alignas(16) float qf[TB][DK];  // D q
+    alignas(16) float wf[TB][DK];
+    alignas(16) float df[NB][DK];  // D_3
+    alignas(16) float cf[NB][2][16];  // two shares of c_10, c_20, c_21, c_30, c_31, c_32, p_00, p_10, p_11, p_20 ... p_33
+    alignas(16) float vf[TB][NCOL];
+    alignas(16) float bf[TB];
+    alignas(16) float of[TB][NCOL][SL];  // SL shares of each output
+  } grp[2];
+};
+
+template <int DK, int DV, int NCOL, int SL, int NHELP, typename IO, typename OT, bool KDA>
+__device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int unit, int part, unsigned char *smem_raw) {
+  constexpr int NC = NCOL * SL;    // threads that replay tokens, a column per SL lanes
+  constexpr int NV = DK / SL / 4;  // groups of four rows held by one lane
+  using Smem = BlockSmem<DK, NCOL, SL, IO, KDA>;
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+  const int tid = threadIdx.x;
+  const bool helper = tid >= NC;
+  const int ht = tid - NC;  // index among the helpers
+  const int slice = tid % SL, col = tid / SL;
+
+  const int h = unit % a.H_v;
+  const int lc = (unit / a.H_v) % a.n_layers_in_call;
+  const int r = unit / (a.H_v * a.n_layers_in_call);
+  const int hk = h / (a.H_v / a.H_k);
+  const int layer = a.layer_begin + lc;
+  const int64_t t_begin = a.tok_begin ? a.tok_begin[r] : a.cu_seqlens[r];
+  const int n_tok = static_cast<int>(a.cu_seqlens[r + 1] - t_begin);
+  if (n_tok <= 0 && a.mode == DASC_REFRESH_CONTINUE) return;
+
+  float *st = a.state + static_cast<int64_t>(a.req_idx[r]) * a.req_stride + static_cast<int64_t>(layer) * a.layer_stride +
+              static_cast<int64_t>(h) * DK * DV + part * NCOL;
+  const int64_t tok0 = static_cast<int64_t>(lc) * a.total_tokens + t_begin;
+  const IO *gq = static_cast<const IO *>(a.q) + (tok0 * a.H_k + hk) * DK;
+  const IO *gk = static_cast<const IO *>(a.k) + (tok0 * a.H_k + hk) * DK;
+  const IO *gv = static_cast<const IO *>(a.v) + (tok0 * a.H_v + h) * DV + part * NCOL;
+  const float *gg = a.g + (tok0 * a.H_v + h) * (KDA ? DK : 1);
+  const float *gb = a.beta + tok0 * a.H_v + h;
+  OT *go = a.o ? static_cast<OT *>(a.o) + (tok0 * a.H_v + h) * DV + part * NCOL : nullptr;
+  const int64_t qk_stride = static_cast<int64_t>(a.H_k) * DK, v_stride = static_cast<int64_t>(a.H_v) * DV;
+  const int64_t g_stride = static_cast<int64_t>(a.H_v) * (KDA ? DK : 1), b_stride = a.H_v;
+  const int n_grp = n_tok > 0 ? (n_tok + TB - 1) / TB : 0;
+
+  // raw rows of a group -> shared memory; consecutive threads take 16-byte vectors of all streams
+  auto stage = [&](int grp) {
+    const int t_lo = grp * TB, buf = grp % NRAW;
+    const int cnt = min(TB, n_tok - t_lo);  // (none past the end: an empty group is committed)
+    constexpr int QV = DK * sizeof(IO) / 16, VV = NCOL * sizeof(IO) / 16, GV = KDA ? DK * 4 / 16 : 1;
+    for (int i = ht; i < cnt * QV; i += NHELP) {
+      const int t = i / QV, j = i % QV;
+      if (go)
+        cp_async16(reinterpret_cast<char *>(&sm.q[buf][t][0]) + j * 16, reinterpret_cast<const char *>(gq + (t_lo + t) * qk_stride) + j * 16);
+      cp_async16(reinterpret_cast<char *>(&sm.k[buf][t][0]) + j * 16, reinterpret_cast<const char *>(gk + (t_lo + t) * qk_stride) + j * 16);
+    }
+    for (int i = ht; i < cnt * VV; i += NHELP) {
+      const int t = i / VV, j = i % VV;
+      cp_async16(reinterpret_cast<char *>(&sm.v[buf][t][0]) + j * 16, reinterpret_cast<const char *>(gv + (t_lo + t) * v_stride) + j * 16);
+    }
+    if constexpr (KDA) {
+      for (int i = ht; i < cnt * GV; i += NHELP) {
+        const int t = i / GV, j = i % GV;
+        cp_async16(reinterpret_cast<char *>(&sm.g[buf][t][0]) + j * 16, reinterpret_cast<const char *>(gg + (t_lo + t) * g_stride) + j * 16);
+      }
+    } else {
+      for (int t = ht; t < cnt; t += NHELP) cp_async4(&sm.g[buf][t][0], gg + (t_lo + t) * g_stride);
+    }
+    for (int t = ht; t < cnt; t += NHELP) cp_async4(&sm.beta[buf][t], gb + (t_lo + t) * b_stride);
+    cp_async_commit();
+  };
+  // raw -> what the replaying lanes read.  Tokens past the end of the request: k = q = v = beta = 0, alpha = 1.
+  auto convert = [&](int grp) {
+    const int buf = grp % NRAW, cnt = min(TB, n_tok - grp * TB);
+    typename Smem::Group &G = sm.grp[grp & 1];
+    constexpr int PER = DK < NHELP / NB ? DK : NHELP / NB;  // threads of a block
+    static_assert(PER % 32 == 0 && PER <= 64 && DK % PER == 0);
+    if (ht < NB * PER) {
+      const int b = ht / PER;
+      float x[16] = {};
+      // products of decays, mostly as exponentials of sums: at most two of them multiplied instead of four
+      float dd[4], a1, a2, a3, a12, a23, a13;
+      auto decays = [&](int c) {
+        float g[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) g[t] = b * 4 + t < cnt ? sm.g[buf][b * 4 + t][c] : 0.f;
+        const float g23 = g[2] + g[3];
+        a1 = expf(g[1]), a2 = expf(g[2]), a3 = expf(g[3]), a12 = expf(g[1] + g[2]), a23 = expf(g23), a13 = expf(g[1] + g23);
+        dd[0] = expf(g[0]), dd[1] = dd[0] * a1, dd[2] = dd[0] * a12, dd[3] = dd[0] * a13;
+      };
+      if constexpr (!KDA) decays(0);
+#pragma unroll
+      for (int c = ht % PER; c < DK; c += PER) {
+        if constexpr (KDA) decays(c);
+        float k[4], q[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int tt = b * 4 + t;
+          const bool in = tt < cnt;
+          k[t] = in ? io_to_float<IO>(sm.k[buf][tt][c]) : 0.f;
+          q[t] = in && go ? io_to_float<IO>(sm.q[buf][tt][c]) * a.q_scale : 0.f;
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          G.kf[b * 4 + t][c] = k[t] * dd[t];
+          if (go) G.qf[b * 4 + t][c] = q[t] * dd[t];
+        }
+        // from[t][j]: k_j carried from token j to token t
+        const float k01 = k[0] * a1, k02 = k[0] * a12, k03 = k[0] * a13, k12 = k[1] * a2, k13 = k[1] * a23, k23 = k[2] * a3;
+        G.wf[b * 4 + 0][c] = k03;
+        G.wf[b * 4 + 1][c] = k13;
+        G.wf[b * 4 + 2][c] = k23;
+        G.wf[b * 4 + 3][c] = k[3];
+        G.df[b][c] = dd[3];
+        x[0] = fmaf(k[1], k01, x[0]);
+        x[1] = fmaf(k[2], k02, x[1]);
+        x[2] = fmaf(k[2], k12, x[2]);
+        x[3] = fmaf(k[3], k03, x[3]);
+        x[4] = fmaf(k[3], k13, x[4]);
+        x[5] = fmaf(k[3], k23, x[5]);
+        x[6] = fmaf(q[0], k[0], x[6]);
+        x[7] = fmaf(q[1], k01, x[7]);
+        x[8] = fmaf(q[1], k[1], x[8]);
+        x[9] = fmaf(q[2], k02, x[9]);
+        x[10] = fmaf(q[2], k12, x[10]);
+        x[11] = fmaf(q[2], k[2], x[11]);
+        x[12] = fmaf(q[3], k03, x[12]);
+        x[13] = fmaf(q[3], k13, x[13]);
+        x[14] = fmaf(q[3], k23, x[14]);
+        x[15] = fmaf(q[3], k[3], x[15]);
+      }
+      // the warp's sums, number i in lanes 2i and 2i + 1
+      const int lane = ht & 31;
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) {
+        const bool up = (lane & (2 * w)) != 0;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+          const float give = up ? x[i] : x[i + w];
+          x[i] = (up ? x[i + w] : x[i]) + __shfl_xor_sync(0xffffffffu, give, 2 * w);
+        }
+      }
+      x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+      if ((lane & 1) == 0) G.cf[b][ht % PER / 32][lane / 2] = x[0];
+      if (PER == 32 && (lane & 1) == 1) G.cf[b][1][lane / 2] = 0.f;
+    }
+    for (int i = ht; i < TB * NCOL; i += NHELP) {
+      const int t = i / NCOL, c = i % NCOL;
+      G.vf[t][c] = t < cnt ? io_to_float<IO>(sm.v[buf][t][c]) : 0.f;
+    }
+    for (int t = ht; t < TB; t += NHELP) G.bf[t] = t < cnt ? sm.beta[buf][t] : 0.f;
+  };
+  // the outputs of a group, 16 bytes of `OT` per store
+  auto flush = [&](int grp) {
+    if (!go) return;
+    constexpr int OV = 16 / sizeof(OT);
+    const int t_lo = grp * TB, cnt = min(TB, n_tok - t_lo);
+    const typename Smem::Group &G = sm.grp[grp & 1];
+    for (int i = ht; i < cnt * (NCOL / OV); i += NHELP) {
+      const int t = i / (NCOL / OV), j = i % (NCOL / OV) * OV;
+      alignas(16) OT w[OV];
+#pragma unroll
+      for (int e = 0; e < OV; ++e) {
+        const float4 *p = reinterpret_cast<const float4 *>(G.of[t][j + e]);
+        float4 s = p[0];
+#pragma unroll
+        for (int sl = 1; sl < SL / 4; ++sl) s = make_float4(s.x + p[sl].x, s.y + p[sl].y, s.z + p[sl].z, s.w + p[sl].w);
+        w[e] = float_to_io<OT>((s.x + s.y) + (s.z + s.w));
+      }
+      *reinterpret_cast<uint4 *>(go + (t_lo + t) * v_stride + j) = *reinterpret_cast<const uint4 *>(w);
+    }
+  };
+  // the oldest group but NRAW - 2 has landed, for all helpers (who are past the conversion whose raw rows are overwritten next)
+  auto landed = [&]() {
+    asm volatile("cp.async.wait_group %0;\n\tbar.sync 1, %1;" ::"n"(NRAW - 2), "n"(NHELP) : "memory");
+  };
+
+  if (helper) {
+    if (n_grp > 0) {
+#pragma unroll
+      for (int i = 0; i < NRAW - 1; ++i) stage(i);
+      landed();
+      convert(0);
+    }
+    __syncthreads();
+    for (int grp = 0; grp < n_grp; ++grp) {
+      // the group before goes out, the next one is converted, the one after that is fetched
+      if (grp + 1 < n_grp) {
+        stage(grp + NRAW - 1);
+        landed();
+        convert(grp + 1);
+      }
+      if (grp > 0) flush(grp - 1);
+      __syncthreads();
+    }
+    if (n_grp > 0) flush(n_grp - 1);
+    return;
+  }
+
+  // row pairs (4 (i SL + slice) + 2p, + 1) of this lane's column
+  uint64_t S[NV][2];
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const float *row = st + (4 * (i * SL + slice) + 2 * p) * DV + col;
+      S[i][p] = a.mode == DASC_REFRESH_CONTINUE ? pack2(row[0], row[DV]) : 0ull;
+    }
+  __syncthreads();
+  for (int grp = 0; grp < n_grp; ++grp) {
+    const int cnt = min(TB, n_tok - grp * TB);
+    // one token group before the end: see launch.cuh
+    if (grp + 1 == n_grp) stream_order_release();
+    typename Smem::Group &G = sm.grp[grp & 1];
+    // straight code for the whole group (tokens past its end are zeros), so that the outputs of a block fill the waits of the next one
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      ulonglong2 k[4][NV], w[4][NV], d[NV];
+      auto load = [&](ulonglong2(&x)[NV], const float *row) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) x[i] = (reinterpret_cast<const ulonglong2 *>(row) + slice)[i * SL];
+      };
+#pragma unroll
+      for (int t = 0; t < 4; ++t) load(k[t], G.kf[b * 4 + t]);
+      float v[4], cf[16];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) v[t] = G.vf[b * 4 + t][col];
+      const float4 be4 = *reinterpret_cast<const float4 *>(&G.bf[b * 4]);
+      const float be[4] = {be4.x, be4.y, be4.z, be4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 x = reinterpret_cast<const float4 *>(G.cf[b][0])[i], y = reinterpret_cast<const float4 *>(G.cf[b][1])[i];
+        cf[4 * i] = x.x + y.x;
+        cf[4 * i + 1] = x.y + y.y;
+        cf[4 * i + 2] = x.z + y.z;
+        cf[4 * i + 3] = x.w + y.w;
+      }
+      load(d, G.df[b]);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) load(w[t], G.wf[b * 4 + t]);
+      auto dot = [&](const ulonglong2(&x)[NV]) {
+        uint64_t acc0 = mul2(x[0].x, S[0][0]), acc1 = mul2(x[0].y, S[0][1]);
+#pragma unroll
+        for (int i = 1; i < NV; ++i) {
+          acc0 = fma2(x[i].x, S[i][0], acc0);
+          acc1 = fma2(x[i].y, S[i][1], acc1);
+        }
+        return sum2(add2(acc0, acc1));
+      };
+      float p[4], o[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) p[t] = dot(k[t]);
+      if (go) {  // this lane's shares of the outputs, from the state before the block
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          load(k[t], G.qf[b * 4 + t]);
+          o[t] = dot(k[t]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        S[i][0] = mul2(S[i][0], d[i].x);
+        S[i][1] = mul2(S[i][1], d[i].y);
+      }
+#pragma unroll
+      for (int dd = 1; dd < SL; dd <<= 1)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) p[t] += __shfl_xor_sync(0xffffffffu, p[t], dd);
+      // tokens past the end write nothing, whatever the state holds
+      float u[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        float x = v[t] - p[t];
+#pragma unroll
+        for (int j = 0; j < t; ++j) x = fmaf(-cf[t * (t - 1) / 2 + j], u[j], x);
+        u[t] = b * 4 + t < cnt ? be[t] * x : 0.f;
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const uint64_t uu = pack2(u[t], u[t]);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+          S[i][0] = fma2(w[t][i].x, uu, S[i][0]);
+          S[i][1] = fma2(w[t][i].y, uu, S[i][1]);
+        }
+      }
+      if (go) {
+        // the part of the block's own tokens goes into the first lane's share
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          float x = 0.f;
+#pragma unroll
+          for (int j = 0; j <= t; ++j) x = fmaf(cf[6 + t * (t + 1) / 2 + j], u[j], x);
+          if (slice == 0) o[t] += x;
+          // no "memory" clobber: the loads of the next block may be moved above these stores
+          asm volatile("st.shared.f32 [%0], %1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&G.of[b * 4 + t][col][slice]))), "f"(o[t]));
+        }
+      }
+    }
+    __syncthreads();
+  }
+
+  const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * DK;
+  const bool all_rows = a.mode == DASC_REFRESH_CONTINUE;
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const int row = 4 * (i * SL + slice) + 2 * p;
+      float lo, hi;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(S[i][p]));
+      float *d = st + row * DV + col;
+      if (all_rows || !keep[row]) d[0] = lo;
+      if (all_rows || !keep[row + 1]) d[DV] = hi;
+    }
+}
+
+template <int DK, int DV, int NCOL, int SL, int NHELP, typename IO, typename OT, bool KDA>
+__global__ void __launch_bounds__(NCOL *SL + NHELP) refresh_seq_blocks_kernel(DascRefreshArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  stream_order_wait();
+  constexpr int PARTS = DV / NCOL;
+  seq_unit_blocks<DK, DV, NCOL, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x) / PARTS, static_cast<int>(blockIdx.x) % PARTS, smem_raw);
+}
+
+template <int DK, int DV, int NCOL, int SL, int NHELP, typename IO, typename OT, bool KDA>
+int launch_blocks(const DascRefreshArgs &a, void *stream) {
+  constexpr size_t smem = sizeof(BlockSmem<DK, NCOL, SL, IO, KDA>);
+  auto kern = refresh_seq_blocks_kernel<DK, DV, NCOL, SL, NHELP, IO, OT, KDA>;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return static_cast<int>(e);
+  }
+  const int64_t n_ctas = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v * (DV / NCOL);
+  if (n_ctas == 0) return cudaSuccess;
+  if (n_ctas > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(n_ctas)), dim3(NCOL * SL + NHELP), smem, stream, a));
+}
+
+// Columns do not interact, so units that leave SMs idle are split by columns: parts of 8 (16 at d = 32) with warps of their own for
+// the conversions while that gives at most two CTAs per SM (beyond, the conversions, which every part repeats, cost more than the shorter
+// chain saves); at d = 128 halves while those fit one CTA per SM.  The parts replay four tokens at a time, with 8 lanes per column (4 at
+// d = 32): fewer shuffles, longer dot products.
+// B200, 128 fp32 tokens, microseconds split / whole on both sides of each line, token by token:
 //   d = 32   148 units 27 / 31, 149 units 45 / 35
 //   d = 64    37 units 29 / 42,  38 units 48 / 42 (GDN 37 / 41: its line would lie at 48 units)
 //   d = 128   18 units 60 / 89 (halves 59; GDN split 36, halves 58), 19 units 88 / 89 (59); halves 74 units 60 / 89, 75 units 116 / 91
+// Token by token / blocks of four with 16 / with 8 lanes per column (KDA unless GDN):
+//   d = 32    4 units 19.9 / 13.7 / 12.4 (4 lanes), 120 units 27.0 / 23.5 / 17.6
+//   d = 64    4 units 21.0 / 16.5 / 14.8, 16 units 21.1 / 16.6 / 15.2; two CTAs per SM: 20 units 29.0 / 26.9 / 28.5, 36 units 29.1 / 26.9 / 29.3
+//   d = 128   4 units 30.2 / 22.0 / 20.9, 8 units GDN 25.9 / 20.7 / 20.6; two CTAs per SM: 16 units 59.5 / 43.2 / 41.3, GDN 36.3 / 40.5 / 39.5,
+// hence 16 lanes for d = 64 and the old form for GDN at d = 128 where two CTAs share an SM.
 constexpr int64_t kSplitCtas = 296, kHalfCtas = 148;
 
 template <int D, typename IO, typename OT, bool KDA>
 int dispatch_split(const DascRefreshArgs &a, void *stream) {
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
   if constexpr (D == 32) {
-    if (!a.from_list && n_units * 2 <= kSplitCtas) return launch<32, 32, 16, 1, 8, 256, IO, OT, KDA>(a, stream);
+    if (!a.from_list && n_units * 2 <= kSplitCtas) return launch_blocks<32, 32, 16, 4, 256, IO, OT, KDA>(a, stream);
     return launch<32, 32, 32, 2, 8, 0, IO, OT, KDA>(a, stream);
   } else if constexpr (D == 64) {
-    if (!a.from_list && n_units * 8 <= kSplitCtas) return launch<64, 64, 8, 1, 16, 256, IO, OT, KDA>(a, stream);
+    if (!a.from_list && n_units * 8 <= kHalfCtas) return launch_blocks<64, 64, 8, 8, 256, IO, OT, KDA>(a, stream);
+    if (!a.from_list && n_units * 8 <= kSplitCtas) return launch_blocks<64, 64, 8, 16, 256, IO, OT, KDA>(a, stream);
     return launch<64, 64, 64, 4, 8, 128, IO, OT, KDA>(a, stream);
   } else {
-    if (!a.from_list && n_units * 16 <= kSplitCtas) return launch<128, 128, 8, 1, 16, 256, IO, OT, KDA>(a, stream);
+    if (!a.from_list && n_units * 16 <= (KDA ? kSplitCtas : kHalfCtas)) return launch_blocks<128, 128, 8, 8, 256, IO, OT, KDA>(a, stream);
+    if constexpr (!KDA)
+      if (!a.from_list && n_units * 16 <= kSplitCtas) return launch<128, 128, 8, 1, 16, 256, IO, OT, KDA>(a, stream);
     if (!a.from_list && n_units * 2 <= kHalfCtas) return launch<128, 128, 64, 4, 16, 128, IO, OT, KDA>(a, stream);
     return launch<128, 128, 128, 4, 16, 0, IO, OT, KDA>(a, stream);
   }

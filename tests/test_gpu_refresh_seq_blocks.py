@@ -1,0 +1,38 @@
+"""The column-split forms of the token-by-token kernel replay four tokens at a time: every tail of a block and of a group of 16,
+all dimensions and both lane counts, strong decay included, against the fp64 oracle at the fp32 tolerance."""
+import pytest
+import torch
+
+import oracle
+import paper_2608_30386_b200 as dasc
+from helpers import assert_refresh_close, make_refresh_case, run_refresh_gpu, run_refresh_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+# (dimension, value heads): with four requests 8 and 16 units (a CTA per SM at most), 20 and 36 (two)
+@pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
+@pytest.mark.parametrize("dim,heads", [(32, 2), (64, 2), (64, 4), (64, 8), (128, 2), (128, 4)])
+@pytest.mark.parametrize("lens", [[1, 2, 3, 4], [5, 15, 16, 17], [18, 33, 64, 0], [47, 65, 80, 31]])
+def test_tails_of_blocks_and_groups(kind, dim, heads, lens):
+    case = make_refresh_case(81, kind, 1, heads, heads // 2, dim, dim, lens, io_dtype=torch.float32, scope=dasc.SCOPE_LAYER, keep_ratio=0.5)
+    case.streams.g[:, 1::7] *= 40.0    # decays down to nothing between ordinary ones
+    case.streams.g[:, 3::11] = -200.0
+    ref_s, ref_o = run_refresh_oracle(case, q_scale=0.5)
+    got_s, got_o = run_refresh_gpu(case, algo=dasc.ALGO_SEQUENTIAL, q_scale=0.5)
+    assert_refresh_close(case, got_s, got_o, ref_s, ref_o, 1e-5)
+    ref_s, _ = run_refresh_oracle(case, mode=oracle.MODE_SCRATCH_MERGE_LOCAL, want_o=False)
+    got_s, _ = run_refresh_gpu(case, mode=dasc.REFRESH_SCRATCH_MERGE_LOCAL, algo=dasc.ALGO_SEQUENTIAL, want_o=False)
+    assert_refresh_close(case, got_s, None, ref_s, None, 1e-5)
+
+
+@pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
+@pytest.mark.parametrize("dim", [32, 64, 128])
+def test_bf16_streams_and_outputs(kind, dim):
+    # bf16 streams are exact in fp32, so the fp32 tolerance holds for the state; bf16 outputs are the fp32 ones rounded
+    case = make_refresh_case(82, kind, 1, 2, 1, dim, dim, [37, 6], scope=dasc.SCOPE_LAYER, keep_ratio=0.5)
+    ref_s, ref_o = run_refresh_oracle(case)
+    got_s, got_o = run_refresh_gpu(case, algo=dasc.ALGO_SEQUENTIAL)
+    assert_refresh_close(case, got_s, got_o, ref_s, ref_o, 1e-5)
+    _, got_b = run_refresh_gpu(case, algo=dasc.ALGO_SEQUENTIAL, o_dtype=torch.bfloat16)
+    assert torch.equal(torch.from_numpy(got_o).to(torch.bfloat16).float(), torch.from_numpy(got_b))
