@@ -3,8 +3,9 @@
 // log-decay g <= 0; it is the reference point for the chunked tensor-core kernel
 // and the path for shapes that kernel does not take.
 //
-// One CTA per (request, layer, value head), or per part of its columns.  Columns of the state do not interact, so there is no
-// barrier between tokens: a column's d_k entries live in the registers of SL adjacent lanes, and S^T k, S^T q are shuffles.
+// One CTA per (request, layer, value head), or per part of its columns when units are few (second half of the file).  Columns of the
+// state do not interact, so there is no barrier between tokens: a column's d_k entries live in the registers of SL adjacent lanes, and
+// S^T k, S^T q are shuffles.
 // Per token
 //   S   <- Diag(alpha_t) S                       (decay on the key-channel index)
 //   r   <- S^T k_t
@@ -15,9 +16,9 @@
 // stretch of k, q, alpha, and row pairs are the operand pairs of the packed fp32 instructions.  Bound: when units are few the
 // serial chain (a dot product and its shuffles per token; the next token's is started before this token's update, see
 // below), else instruction issue and the registers' share of the shared-memory bandwidth (128 bytes per cycle whatever is
-// broadcast, hence 4 columns per lane in the wide variants).
-// Measured on B200, fp32 (the form before: one column per thread and row half, a block barrier per token): 4 units of 64 x 64, 64
-// tokens 26.7 -> 12.6 us; 4 of 128 x 128 54 -> 17.4 us; 256 of 128 x 128, 256 tokens 407 -> 345 us; 8192 of them 11.2 -> 9.6 ms.
+// broadcast, hence 4 columns per lane).
+// Measured on B200, fp32 (the form before: one column per thread and row half, a block barrier per token): 256 units of 128 x 128, 256
+// tokens 407 -> 345 us; 8192 of them 11.2 -> 9.6 ms.
 // Token inputs are staged TB tokens at a time: raw rows by cp.async into a double
 // buffer, then converted once (bf16 -> fp32, alpha = exp(g)); outputs leave a group later, 16 bytes per store.  With NHELP > 0
 // that many extra threads do both, a group ahead of and a group behind the tokens being replayed.
@@ -92,12 +93,12 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   return r;
 }
 
-template <int DK, int NCOL, int NOP, bool AHEAD, typename IO, bool KDA>
+template <int DK, int DV, int NOP, bool AHEAD, typename IO, bool KDA>
 struct SeqSmem {
   // raw staging, double buffered
   alignas(16) IO q[2][TB][DK];
   alignas(16) IO k[2][TB][DK];
-  alignas(16) IO v[2][TB][NCOL];
+  alignas(16) IO v[2][TB][DV];
   alignas(16) float g[2][TB][KDA ? DK : 4];
   alignas(16) float beta[2][TB];
   // converted; two groups when extra warps convert the next one meanwhile
@@ -105,8 +106,8 @@ struct SeqSmem {
     alignas(16) float kf[TB][DK];
     alignas(16) float qf[TB][DK];
     alignas(16) float af[TB][KDA ? DK : 4];
-    alignas(16) float vf[TB][NCOL];
-    alignas(16) float of[TB][NCOL][NOP];  // NOP shares of each of the group's outputs
+    alignas(16) float vf[TB][DV];
+    alignas(16) float of[TB][DV][NOP];  // NOP shares of each of the group's outputs
     float bf[TB], cf[TB];                     // beta;  c_t = (alpha_t k_t) . k_{t-1}
   } grp[AHEAD ? 2 : 1];
 };
@@ -116,8 +117,6 @@ __device__ __forceinline__ void load_cols(float (&x)[COLS], const float *p) {
   if constexpr (COLS == 4) {
     const float4 v = *reinterpret_cast<const float4 *>(p);
     x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-  } else if constexpr (COLS == 1) {
-    x[0] = *p;
   } else {
     const float2 v = *reinterpret_cast<const float2 *>(p);
     x[0] = v.x; x[1] = v.y;
@@ -127,21 +126,19 @@ template <int COLS>
 __device__ __forceinline__ void store_cols(float *p, const float (&x)[COLS]) {
   if constexpr (COLS == 4)
     *reinterpret_cast<float4 *>(p) = make_float4(x[0], x[1], x[2], x[3]);
-  else if constexpr (COLS == 1)
-    *p = x[0];
   else
     *reinterpret_cast<float2 *>(p) = make_float2(x[0], x[1]);
 }
 
-// One (request, layer, value head) unit, or NCOL of its DV columns, replayed by the whole CTA; COLS columns per lane, SL lanes per column.
-template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
-__device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int part, unsigned char *smem_raw) {
-  constexpr int NC = NCOL / COLS * SL;      // threads that replay tokens
+// One (request, layer, value head) unit, replayed token by token by the whole CTA; COLS columns per lane, SL lanes per column.
+template <int DK, int DV, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
+__device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, unsigned char *smem_raw) {
+  constexpr int NC = DV / COLS * SL;      // threads that replay tokens
   constexpr int NT = NHELP > 0 ? NHELP : NC;  // threads that bring the tokens in and the outputs out
   constexpr int NV = DK / SL / 4;  // groups of four rows held by one lane
   constexpr int NOP = SL / COLS;
   constexpr bool AHEAD = NHELP > 0;
-  using Smem = SeqSmem<DK, NCOL, NOP, AHEAD, IO, KDA>;
+  using Smem = SeqSmem<DK, DV, NOP, AHEAD, IO, KDA>;
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
 
   const int tid = threadIdx.x;
@@ -163,14 +160,14 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
   if (n_tok <= 0 && a.mode == DASC_REFRESH_CONTINUE) return;
 
   float *st = a.state + static_cast<int64_t>(a.req_idx[r]) * a.req_stride + static_cast<int64_t>(layer) * a.layer_stride +
-              static_cast<int64_t>(h) * DK * DV + part * NCOL;
+              static_cast<int64_t>(h) * DK * DV;
   const int64_t tok0 = static_cast<int64_t>(lc) * a.total_tokens + t_begin;
   const IO *gq = static_cast<const IO *>(a.q) + (tok0 * a.H_k + hk) * DK;
   const IO *gk = static_cast<const IO *>(a.k) + (tok0 * a.H_k + hk) * DK;
-  const IO *gv = static_cast<const IO *>(a.v) + (tok0 * a.H_v + h) * DV + part * NCOL;
+  const IO *gv = static_cast<const IO *>(a.v) + (tok0 * a.H_v + h) * DV;
   const float *gg = a.g + (tok0 * a.H_v + h) * (KDA ? DK : 1);
   const float *gb = a.beta + tok0 * a.H_v + h;
-  OT *go = a.o ? static_cast<OT *>(a.o) + (tok0 * a.H_v + h) * DV + part * NCOL : nullptr;
+  OT *go = a.o ? static_cast<OT *>(a.o) + (tok0 * a.H_v + h) * DV : nullptr;
   const int64_t qk_stride = static_cast<int64_t>(a.H_k) * DK, v_stride = static_cast<int64_t>(a.H_v) * DV;
   const int64_t g_stride = static_cast<int64_t>(a.H_v) * (KDA ? DK : 1), b_stride = a.H_v;
 
@@ -178,7 +175,7 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
   auto stage = [&](int grp) {
     const int t_lo = grp * TB, buf = grp & 1;
     const int cnt = min(TB, n_tok - t_lo);
-    constexpr int QV = DK * sizeof(IO) / 16, VV = NCOL * sizeof(IO) / 16, GV = KDA ? DK * 4 / 16 : 1;
+    constexpr int QV = DK * sizeof(IO) / 16, VV = DV * sizeof(IO) / 16, GV = KDA ? DK * 4 / 16 : 1;
     for (int i = ht; i < cnt * QV; i += NT) {
       const int t = i / QV, j = i % QV;
       cp_async16(reinterpret_cast<char *>(&sm.q[buf][t][0]) + j * 16,
@@ -256,7 +253,7 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
       if (go) G.qf[t][c] = io_to_float<IO>(sm.q[buf][t][c]) * a.q_scale;
       if constexpr (KDA) G.af[t][c] = expf(sm.g[buf][t][c]);
     }
-    for (int i = ht; i < cnt * NCOL; i += NT) G.vf[i / NCOL][i % NCOL] = io_to_float<IO>(sm.v[buf][i / NCOL][i % NCOL]);
+    for (int i = ht; i < cnt * DV; i += NT) G.vf[i / DV][i % DV] = io_to_float<IO>(sm.v[buf][i / DV][i % DV]);
     for (int t = ht; t < cnt; t += NT) {
       G.bf[t] = sm.beta[buf][t];
       if constexpr (!KDA) G.af[t][0] = expf(sm.g[buf][t][0]);
@@ -278,8 +275,8 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
     constexpr int OV = 16 / sizeof(OT);
     const int t_lo = grp * TB, cnt = min(TB, n_tok - t_lo);
     const typename Smem::Group &G = sm.grp[AHEAD ? grp & 1 : 0];
-    for (int i = ht; i < cnt * (NCOL / OV); i += NT) {
-      const int t = i / (NCOL / OV), j = i % (NCOL / OV) * OV;
+    for (int i = ht; i < cnt * (DV / OV); i += NT) {
+      const int t = i / (DV / OV), j = i % (DV / OV) * OV;
       alignas(16) OT w[OV];
 #pragma unroll
       for (int e = 0; e < OV; ++e) {
@@ -377,7 +374,7 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
       uint64_t uu[COLS];
 #pragma unroll
       for (int c = 0; c < COLS; ++c) {
-        const float x = COLS == 1 ? u : __shfl_sync(0xffffffffu, u, (threadIdx.x & 31 & ~(COLS - 1)) + c);
+        const float x = __shfl_sync(0xffffffffu, u, (threadIdx.x & 31 & ~(COLS - 1)) + c);
         uu[c] = pack2(x, x);
       }
       float p = 0.f;
@@ -434,46 +431,45 @@ __device__ __forceinline__ void seq_unit(const DascRefreshArgs &a, int unit, int
     }
 }
 
-// grid = one CTA per unit and column part (from_list == 0), or a fixed grid whose CTAs walk the list of units that the
+// grid = one CTA per unit (from_list == 0), or a fixed grid whose CTAs walk the list of units that the
 // chunked kernel handed over (from_list == 1; the list and its length are in the workspace, written earlier on the same stream).
-template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
-__global__ void __launch_bounds__(NCOL / COLS *SL + NHELP) refresh_seq_kernel(DascRefreshArgs a) {
+template <int DK, int DV, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
+__global__ void __launch_bounds__(DV / COLS *SL + NHELP) refresh_seq_kernel(DascRefreshArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   stream_order_wait();
-  constexpr int PARTS = DV / NCOL;
   if (!a.from_list) {
-    seq_unit<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x) / PARTS, static_cast<int>(blockIdx.x) % PARTS, smem_raw);
+    seq_unit<DK, DV, COLS, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x), smem_raw);
     return;
   }
   uint32_t *ws = static_cast<uint32_t *>(a.workspace);
   const uint32_t listed = ws[2];
   const int n_list = static_cast<int>(listed < static_cast<uint32_t>(a.unit_list_cap) ? listed : a.unit_list_cap);
-  for (int i = blockIdx.x; i < n_list * PARTS; i += gridDim.x) {
-    seq_unit<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>(a, a.unit_list[i / PARTS], i % PARTS, smem_raw);
-    if (threadIdx.x == 0 && i % PARTS == 0) atomicAdd(ws + 3, 1u);
+  for (int i = blockIdx.x; i < n_list; i += gridDim.x) {
+    seq_unit<DK, DV, COLS, SL, NHELP, IO, OT, KDA>(a, a.unit_list[i], smem_raw);
+    if (threadIdx.x == 0) atomicAdd(ws + 3, 1u);
     __syncthreads();  // the next unit reuses the staging buffers
   }
 }
 
-template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
+template <int DK, int DV, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
 int launch(const DascRefreshArgs &a, void *stream) {
-  constexpr size_t smem = sizeof(SeqSmem<DK, NCOL, SL / COLS, (NHELP > 0), IO, KDA>);
-  auto kern = refresh_seq_kernel<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>;
+  constexpr size_t smem = sizeof(SeqSmem<DK, DV, SL / COLS, (NHELP > 0), IO, KDA>);
+  auto kern = refresh_seq_kernel<DK, DV, COLS, SL, NHELP, IO, OT, KDA>;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return static_cast<int>(e);
   }
-  const int64_t n_ctas = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v * (DV / NCOL);
+  const int64_t n_ctas = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
   if (n_ctas == 0) return cudaSuccess;
   if (n_ctas > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
   // a handed-over list is short (units outside the chunked kernel's range or below its length threshold): a grid
   // of a CTA per SM walks it, and costs next to nothing when the list is empty
   const int64_t grid = a.from_list ? (n_ctas < 148 ? n_ctas : 148) : n_ctas;
-  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(grid)), dim3(NCOL / COLS * SL + NHELP), smem, stream, a));
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(grid)), dim3(DV / COLS * SL + NHELP), smem, stream, a));
 }
 
 // ---------------------------------------------------------------------------------------------
-// Four tokens at a time, for the forms that are split by columns because units are few: there the serial chain is all there is.
+// Four tokens at a time, where no SM has more than one unit or part of one (d = 32: two): there the serial chain is all there is.
 // With D_t the product of the decays of the block's tokens up to t, and everything else over the block's tokens j < t or j <= t,
 //   r_t = (D_t k_t)^T S_0 + sum_j c_tj u_j        c_tj = k_t^T Diag(alpha_{j+1} ... alpha_t) k_j
 //   o_t = (D_t q_t)^T S_0 + sum_j p_tj u_j        p_tj = q_t^T Diag(alpha_{j+1} ... alpha_t) k_j
@@ -482,15 +478,16 @@ int launch(const DascRefreshArgs &a, void *stream) {
 // factors are products of at most two exponentials, of sums of the log-decay: no division, and half of the token-by-token form's error
 // against fp64 (4 units of 64 x 64, 64 tokens: state 6.2e-7 -> 3.0e-7, outputs 3.5e-7 -> 2.0e-7), whose decays multiply up one token at
 // a time.  The helper warps form D k, D q, w and the 16 coefficients of a block, a group of tokens ahead; they and the replaying warps
-// share the SM's issue slots, which is what bounds a group now (about 95 ns per token at d = 64, 135 before).  More helper warps, or
+// share the SM's issue slots, which is what bounds a group of narrow parts (about 95 ns per token at d = 64, 135 before); wide ones
+// are bound by the replaying lanes' operand reads.  More helper warps, or
 // copies and outputs in warps of their own, gained nothing.
 // ---------------------------------------------------------------------------------------------
 constexpr int NB = TB / 4;  // blocks of a group
-constexpr int NRAW = 4;     // groups whose raw rows are in shared memory
 
 template <int DK, int NCOL, int SL, typename IO, bool KDA>
 struct BlockSmem {
-  // raw staging, three groups ahead of the one that is being converted: a group takes less than a trip to memory
+  // raw staging, NRAW - 1 groups ahead of the one that is being converted: a group takes less than a trip to memory
+  static constexpr int NRAW = DK * NCOL <= 128 * 32 ? 4 : 3;
   alignas(16) IO q[NRAW][TB][DK];
   alignas(16) IO k[NRAW][TB][DK];
   alignas(16) IO v[NRAW][TB][NCOL];
@@ -508,16 +505,17 @@ struct BlockSmem {
   } grp[2];
 };
 
-template <int DK, int DV, int NCOL, int SL, int NHELP, typename IO, typename OT, bool KDA>
+template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
 __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int unit, int part, unsigned char *smem_raw) {
-  constexpr int NC = NCOL * SL;    // threads that replay tokens, a column per SL lanes
+  constexpr int NC = NCOL / COLS * SL;  // threads that replay tokens, COLS columns per SL lanes
   constexpr int NV = DK / SL / 4;  // groups of four rows held by one lane
   using Smem = BlockSmem<DK, NCOL, SL, IO, KDA>;
+  constexpr int NRAW = Smem::NRAW;
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   const int tid = threadIdx.x;
   const bool helper = tid >= NC;
   const int ht = tid - NC;  // index among the helpers
-  const int slice = tid % SL, col = tid / SL;
+  const int slice = tid % SL, col = tid / SL * COLS;
 
   const int h = unit % a.H_v;
   const int lc = (unit / a.H_v) % a.n_layers_in_call;
@@ -695,15 +693,17 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
     return;
   }
 
-  // row pairs (4 (i SL + slice) + 2p, + 1) of this lane's column
-  uint64_t S[NV][2];
+  // row pairs (4 (i SL + slice) + 2p, + 1) of this lane's columns
+  uint64_t S[COLS][NV][2];
 #pragma unroll
-  for (int i = 0; i < NV; ++i)
+  for (int e = 0; e < COLS; ++e)
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const float *row = st + (4 * (i * SL + slice) + 2 * p) * DV + col;
-      S[i][p] = a.mode == DASC_REFRESH_CONTINUE ? pack2(row[0], row[DV]) : 0ull;
-    }
+    for (int i = 0; i < NV; ++i)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const float *row = st + (4 * (i * SL + slice) + 2 * p) * DV + col + e;
+        S[e][i][p] = a.mode == DASC_REFRESH_CONTINUE ? pack2(row[0], row[DV]) : 0ull;
+      }
   __syncthreads();
   for (int grp = 0; grp < n_grp; ++grp) {
     const int cnt = min(TB, n_tok - grp * TB);
@@ -720,9 +720,11 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
       };
 #pragma unroll
       for (int t = 0; t < 4; ++t) load(k[t], G.kf[b * 4 + t]);
-      float v[4], cf[16];
+      float v[COLS][4], cf[16];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) v[t] = G.vf[b * 4 + t][col];
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int e = 0; e < COLS; ++e) v[e][t] = G.vf[b * 4 + t][col + e];
       const float4 be4 = *reinterpret_cast<const float4 *>(&G.bf[b * 4]);
       const float be[4] = {be4.x, be4.y, be4.z, be4.w};
 #pragma unroll
@@ -736,63 +738,77 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
       load(d, G.df[b]);
 #pragma unroll
       for (int t = 0; t < 4; ++t) load(w[t], G.wf[b * 4 + t]);
-      auto dot = [&](const ulonglong2(&x)[NV]) {
-        uint64_t acc0 = mul2(x[0].x, S[0][0]), acc1 = mul2(x[0].y, S[0][1]);
+      auto dot = [&](const ulonglong2(&x)[NV], int e) {
+        uint64_t acc0 = mul2(x[0].x, S[e][0][0]), acc1 = mul2(x[0].y, S[e][0][1]);
 #pragma unroll
         for (int i = 1; i < NV; ++i) {
-          acc0 = fma2(x[i].x, S[i][0], acc0);
-          acc1 = fma2(x[i].y, S[i][1], acc1);
+          acc0 = fma2(x[i].x, S[e][i][0], acc0);
+          acc1 = fma2(x[i].y, S[e][i][1], acc1);
         }
         return sum2(add2(acc0, acc1));
       };
-      float p[4], o[4];
+      float p[COLS][4], o[COLS][4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) p[t] = dot(k[t]);
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int e = 0; e < COLS; ++e) p[e][t] = dot(k[t], e);
       if (go) {  // this lane's shares of the outputs, from the state before the block
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           load(k[t], G.qf[b * 4 + t]);
-          o[t] = dot(k[t]);
+#pragma unroll
+          for (int e = 0; e < COLS; ++e) o[e][t] = dot(k[t], e);
         }
       }
 #pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        S[i][0] = mul2(S[i][0], d[i].x);
-        S[i][1] = mul2(S[i][1], d[i].y);
-      }
+      for (int e = 0; e < COLS; ++e)
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+          S[e][i][0] = mul2(S[e][i][0], d[i].x);
+          S[e][i][1] = mul2(S[e][i][1], d[i].y);
+        }
 #pragma unroll
       for (int dd = 1; dd < SL; dd <<= 1)
 #pragma unroll
-        for (int t = 0; t < 4; ++t) p[t] += __shfl_xor_sync(0xffffffffu, p[t], dd);
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int e = 0; e < COLS; ++e) p[e][t] += __shfl_xor_sync(0xffffffffu, p[e][t], dd);
       // tokens past the end write nothing, whatever the state holds
-      float u[4];
+      float u[COLS][4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        float x = v[t] - p[t];
+      for (int t = 0; t < 4; ++t)
 #pragma unroll
-        for (int j = 0; j < t; ++j) x = fmaf(-cf[t * (t - 1) / 2 + j], u[j], x);
-        u[t] = b * 4 + t < cnt ? be[t] * x : 0.f;
-      }
+        for (int e = 0; e < COLS; ++e) {
+          float x = v[e][t] - p[e][t];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const uint64_t uu = pack2(u[t], u[t]);
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-          S[i][0] = fma2(w[t][i].x, uu, S[i][0]);
-          S[i][1] = fma2(w[t][i].y, uu, S[i][1]);
+          for (int j = 0; j < t; ++j) x = fmaf(-cf[t * (t - 1) / 2 + j], u[e][j], x);
+          u[e][t] = b * 4 + t < cnt ? be[t] * x : 0.f;
         }
-      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int e = 0; e < COLS; ++e) {
+          const uint64_t uu = pack2(u[e][t], u[e][t]);
+#pragma unroll
+          for (int i = 0; i < NV; ++i) {
+            S[e][i][0] = fma2(w[t][i].x, uu, S[e][i][0]);
+            S[e][i][1] = fma2(w[t][i].y, uu, S[e][i][1]);
+          }
+        }
       if (go) {
         // the part of the block's own tokens goes into the first lane's share
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          float x = 0.f;
+        for (int t = 0; t < 4; ++t)
 #pragma unroll
-          for (int j = 0; j <= t; ++j) x = fmaf(cf[6 + t * (t + 1) / 2 + j], u[j], x);
-          if (slice == 0) o[t] += x;
-          // no "memory" clobber: the loads of the next block may be moved above these stores
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&G.of[b * 4 + t][col][slice]))), "f"(o[t]));
-        }
+          for (int e = 0; e < COLS; ++e) {
+            float x = 0.f;
+#pragma unroll
+            for (int j = 0; j <= t; ++j) x = fmaf(cf[6 + t * (t + 1) / 2 + j], u[e][j], x);
+            if (slice == 0) o[e][t] += x;
+            // no "memory" clobber: the loads of the next block may be moved above these stores
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&G.of[b * 4 + t][col + e][slice]))),
+                         "f"(o[e][t]));
+          }
       }
     }
     __syncthreads();
@@ -801,30 +817,33 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
   const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * DK;
   const bool all_rows = a.mode == DASC_REFRESH_CONTINUE;
 #pragma unroll
-  for (int i = 0; i < NV; ++i)
+  for (int e = 0; e < COLS; ++e)
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const int row = 4 * (i * SL + slice) + 2 * p;
-      float lo, hi;
-      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(S[i][p]));
-      float *d = st + row * DV + col;
-      if (all_rows || !keep[row]) d[0] = lo;
-      if (all_rows || !keep[row + 1]) d[DV] = hi;
-    }
+    for (int i = 0; i < NV; ++i)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const int row = 4 * (i * SL + slice) + 2 * p;
+        float lo, hi;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(S[e][i][p]));
+        float *d = st + row * DV + col + e;
+        if (all_rows || !keep[row]) d[0] = lo;
+        if (all_rows || !keep[row + 1]) d[DV] = hi;
+      }
 }
 
-template <int DK, int DV, int NCOL, int SL, int NHELP, typename IO, typename OT, bool KDA>
-__global__ void __launch_bounds__(NCOL *SL + NHELP) refresh_seq_blocks_kernel(DascRefreshArgs a) {
+template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
+__global__ void __launch_bounds__(NCOL / COLS *SL + NHELP) refresh_seq_blocks_kernel(DascRefreshArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   stream_order_wait();
   constexpr int PARTS = DV / NCOL;
-  seq_unit_blocks<DK, DV, NCOL, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x) / PARTS, static_cast<int>(blockIdx.x) % PARTS, smem_raw);
+  seq_unit_blocks<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>(a, static_cast<int>(blockIdx.x) / PARTS, static_cast<int>(blockIdx.x) % PARTS, smem_raw);
 }
 
-template <int DK, int DV, int NCOL, int SL, int NHELP, typename IO, typename OT, bool KDA>
+template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
 int launch_blocks(const DascRefreshArgs &a, void *stream) {
   constexpr size_t smem = sizeof(BlockSmem<DK, NCOL, SL, IO, KDA>);
-  auto kern = refresh_seq_blocks_kernel<DK, DV, NCOL, SL, NHELP, IO, OT, KDA>;
+  static_assert(smem <= 227 * 1024);
+  auto kern = refresh_seq_blocks_kernel<DK, DV, NCOL, COLS, SL, NHELP, IO, OT, KDA>;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return static_cast<int>(e);
@@ -832,40 +851,50 @@ int launch_blocks(const DascRefreshArgs &a, void *stream) {
   const int64_t n_ctas = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v * (DV / NCOL);
   if (n_ctas == 0) return cudaSuccess;
   if (n_ctas > 2147483647LL) return static_cast<int>(cudaErrorInvalidConfiguration);
-  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(n_ctas)), dim3(NCOL * SL + NHELP), smem, stream, a));
+  return static_cast<int>(launch_in_order(kern, dim3(static_cast<unsigned>(n_ctas)), dim3(NCOL / COLS * SL + NHELP), smem, stream, a));
 }
 
-// Columns do not interact, so units that leave SMs idle are split by columns: parts of 8 (16 at d = 32) with warps of their own for
-// the conversions while that gives at most two CTAs per SM (beyond, the conversions, which every part repeats, cost more than the shorter
-// chain saves); at d = 128 halves while those fit one CTA per SM.  The parts replay four tokens at a time, with 8 lanes per column (4 at
-// d = 32): fewer shuffles, longer dot products.
-// B200, 128 fp32 tokens, microseconds split / whole on both sides of each line, token by token:
-//   d = 32   148 units 27 / 31, 149 units 45 / 35
-//   d = 64    37 units 29 / 42,  38 units 48 / 42 (GDN 37 / 41: its line would lie at 48 units)
-//   d = 128   18 units 60 / 89 (halves 59; GDN split 36, halves 58), 19 units 88 / 89 (59); halves 74 units 60 / 89, 75 units 116 / 91
-// Token by token / blocks of four with 16 / with 8 lanes per column (KDA unless GDN):
-//   d = 32    4 units 19.9 / 13.7 / 12.4 (4 lanes), 120 units 27.0 / 23.5 / 17.6
-//   d = 64    4 units 21.0 / 16.5 / 14.8, 16 units 21.1 / 16.6 / 15.2; two CTAs per SM: 20 units 29.0 / 26.9 / 28.5, 36 units 29.1 / 26.9 / 29.3
-//   d = 128   4 units 30.2 / 22.0 / 20.9, 8 units GDN 25.9 / 20.7 / 20.6; two CTAs per SM: 16 units 59.5 / 43.2 / 41.3, GDN 36.3 / 40.5 / 39.5,
-// hence 16 lanes for d = 64 and the old form for GDN at d = 128 where two CTAs share an SM.
-constexpr int64_t kSplitCtas = 296, kHalfCtas = 148;
+// Columns do not interact, so units that leave SMs idle are split by columns: the widest parts that still have an SM each, down to 8
+// columns (16 at d = 32), replayed four tokens at a time.  Beyond a CTA per SM the conversions, which every part repeats, cost more
+// than the shorter chain saves.  From 32 columns on a part is bound by the operand reads of its replaying lanes (a warp's read costs its
+// registers' share, whatever is broadcast), so that two columns per lane and few lanes per column pay there; narrow
+// parts want the short dot products of 8 lanes.  d = 32 has operands small enough for two CTAs per SM.
+// B200, 128 fp32 tokens, microseconds, KDA / GDN; "before" is the token-by-token form, split where the line before lay:
+//   d = 32    4 units  16 columns 12.5 / 12.2, whole in blocks 15.6 / 15.5
+//           148        16 columns 17.6 / 17.0, whole in blocks 15.8 / 15.7
+//           152        16 columns 28.2 / 27.5, whole in blocks 30.4 / 30.1, before 35.7 / 36.0; 296 units 33.5, 30.8, 35.5; 304: 43.6, 45.2, 45.0
+//   d = 64   18        8 columns 15.2 / 14.7, 16: 18.5 / 18.1
+//            36        8 columns 26.9 / 26.4, 16: 18.5 / 18.0 (8 lanes 19.1 / 18.6), before 29.1
+//            74        16 columns 36.1 / 35.1, 32: 24.2 / 23.8 (2 columns per lane, 8 lanes 25.0 / 24.4), before 41.9 / 40.5
+//           148        32 columns 47.4 / 46.6, 64: 31.2 / 30.3 (1 per lane 41.6 / 41.3), before 42.2 / 41.0
+//           152        64 columns 56.9 / 55.7, before 57.5 / 55.2; 296 units 60.8 / 59.0, 57.6 / 55.4
+//   d = 128   8        8 columns 21.5 / 20.7, 16: 27.4 / 26.6
+//            18        8 columns 41.7 / 39.5, 16: 27.7 / 26.8, before 59.5 / 36.3
+//            36        16 columns 54.1 / 52.5, 32: 35.4 / 34.6 (1 per lane, 4 lanes 39.6 / 39.2), before 59.3 / 58.3
+//            74        32 columns 69.1 / 67.2, 64: 48.4 / 46.8 (8 lanes 56.1 / 55.1), before 59.4 / 58.5
+//            76        64 columns 87.9 / 86.4, whole in blocks 96.5 / 92.2, before 91.3 / 84.4; 148 units 95.2 / 92.3, 97.1 / 91.6, 89.6 / 83.0
+constexpr int64_t kSms = 148;
 
 template <int D, typename IO, typename OT, bool KDA>
 int dispatch_split(const DascRefreshArgs &a, void *stream) {
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
+  const auto fits = [&](int parts, int64_t ctas) { return !a.from_list && n_units * parts <= ctas; };
   if constexpr (D == 32) {
-    if (!a.from_list && n_units * 2 <= kSplitCtas) return launch_blocks<32, 32, 16, 4, 256, IO, OT, KDA>(a, stream);
-    return launch<32, 32, 32, 2, 8, 0, IO, OT, KDA>(a, stream);
+    if (fits(2, kSms)) return launch_blocks<32, 32, 16, 1, 4, 256, IO, OT, KDA>(a, stream);
+    if (fits(1, 2 * kSms)) return launch_blocks<32, 32, 32, 1, 4, 256, IO, OT, KDA>(a, stream);
+    return launch<32, 32, 2, 8, 0, IO, OT, KDA>(a, stream);
   } else if constexpr (D == 64) {
-    if (!a.from_list && n_units * 8 <= kHalfCtas) return launch_blocks<64, 64, 8, 8, 256, IO, OT, KDA>(a, stream);
-    if (!a.from_list && n_units * 8 <= kSplitCtas) return launch_blocks<64, 64, 8, 16, 256, IO, OT, KDA>(a, stream);
-    return launch<64, 64, 64, 4, 8, 128, IO, OT, KDA>(a, stream);
+    if (fits(8, kSms)) return launch_blocks<64, 64, 8, 1, 8, 256, IO, OT, KDA>(a, stream);
+    if (fits(4, kSms)) return launch_blocks<64, 64, 16, 1, 4, 256, IO, OT, KDA>(a, stream);
+    if (fits(2, kSms)) return launch_blocks<64, 64, 32, 1, 4, 256, IO, OT, KDA>(a, stream);
+    if (fits(1, kSms)) return launch_blocks<64, 64, 64, 2, 4, 256, IO, OT, KDA>(a, stream);
+    return launch<64, 64, 4, 8, 128, IO, OT, KDA>(a, stream);
   } else {
-    if (!a.from_list && n_units * 16 <= (KDA ? kSplitCtas : kHalfCtas)) return launch_blocks<128, 128, 8, 8, 256, IO, OT, KDA>(a, stream);
-    if constexpr (!KDA)
-      if (!a.from_list && n_units * 16 <= kSplitCtas) return launch<128, 128, 8, 1, 16, 256, IO, OT, KDA>(a, stream);
-    if (!a.from_list && n_units * 2 <= kHalfCtas) return launch<128, 128, 64, 4, 16, 128, IO, OT, KDA>(a, stream);
-    return launch<128, 128, 128, 4, 16, 0, IO, OT, KDA>(a, stream);
+    if (fits(16, kSms)) return launch_blocks<128, 128, 8, 1, 8, 256, IO, OT, KDA>(a, stream);
+    if (fits(8, kSms)) return launch_blocks<128, 128, 16, 1, 8, 256, IO, OT, KDA>(a, stream);
+    if (fits(4, kSms)) return launch_blocks<128, 128, 32, 2, 8, 256, IO, OT, KDA>(a, stream);
+    if (fits(2, kSms)) return launch_blocks<128, 128, 64, 2, 4, 256, IO, OT, KDA>(a, stream);
+    return launch<128, 128, 4, 16, 0, IO, OT, KDA>(a, stream);
   }
 }
 

@@ -1,5 +1,5 @@
-"""The column-split forms of the token-by-token kernel replay four tokens at a time: every tail of a block and of a group of 16,
-all dimensions and both lane counts, strong decay included, against the fp64 oracle at the fp32 tolerance."""
+"""Where units are few the fp32 refresh replays four tokens at a time: every tail of a block and of a group of 16,
+all dimensions and widths of the column parts, strong decay included, against the fp64 oracle at the fp32 tolerance."""
 import pytest
 import torch
 
@@ -10,9 +10,9 @@ from helpers import assert_refresh_close, make_refresh_case, run_refresh_gpu, ru
 pytestmark = pytest.mark.gpu
 
 
-# (dimension, value heads): with four requests 8 and 16 units (a CTA per SM at most), 20 and 36 (two)
+# (dimension, value heads), four requests: every width, from the narrowest parts (8 columns, 16 at d = 32) up to whole units
 @pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
-@pytest.mark.parametrize("dim,heads", [(32, 2), (64, 2), (64, 4), (64, 8), (128, 2), (128, 4)])
+@pytest.mark.parametrize("dim,heads", [(32, 2), (32, 20), (64, 2), (64, 8), (64, 18), (64, 20), (128, 2), (128, 4), (128, 8), (128, 18)])
 @pytest.mark.parametrize("lens", [[1, 2, 3, 4], [5, 15, 16, 17], [18, 33, 64, 0], [47, 65, 80, 31]])
 def test_tails_of_blocks_and_groups(kind, dim, heads, lens):
     case = make_refresh_case(81, kind, 1, heads, heads // 2, dim, dim, lens, io_dtype=torch.float32, scope=dasc.SCOPE_LAYER, keep_ratio=0.5)
