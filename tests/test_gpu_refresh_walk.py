@@ -29,7 +29,8 @@ def replay(case, bound, mode, o_dtype, algo=dasc.ALGO_AUTO):
 
 # units and lengths around what changes a walk: 2 and 3 units of 2 chunks each; single chunks, 16 units to a CTA and the step to a
 # larger grid behind it (296 x 16 = 4736 units); ragged with empty requests, requests of at most 8 tokens (handed over
-# from the middle of a walk) and full chunks; more requests than are put in order; outputs in both types and none
+# from the middle of a walk) and full chunks; more requests than are put in order; 1.3 and 1.4 units to a CTA of very
+# different lengths; outputs in both types and none
 @pytest.mark.parametrize("kind,L,H,lens,mode,o_dtype", [
     (dasc.KDA, 1, 8, [64] * 60, dasc.REFRESH_CONTINUE, torch.bfloat16),
     (dasc.GDN, 1, 8, [50] * 111, dasc.REFRESH_CONTINUE, torch.float32),
@@ -39,6 +40,8 @@ def replay(case, bound, mode, o_dtype, algo=dasc.ALGO_AUTO):
     (dasc.KDA, 2, 8, [1, 96, 0, 33, 8, 64, 9, 31] * 12, dasc.REFRESH_SCRATCH_MERGE_LOCAL, None),
     (dasc.GDN, 2, 8, [96, 32, 0, 95, 65, 97, 2] * 14, dasc.REFRESH_CONTINUE, torch.bfloat16),
     (dasc.KDA, 1, 4, [64] * 250, dasc.REFRESH_CONTINUE, torch.bfloat16),
+    (dasc.KDA, 1, 8, [129, 9, 33, 0, 64, 160, 17] * 7, dasc.REFRESH_CONTINUE, torch.float32),
+    (dasc.GDN, 1, 8, [300, 9, 33, 0, 64, 600, 17, 65, 8] * 6, dasc.REFRESH_SCRATCH_MERGE_LOCAL, None),
 ])
 def test_walked_units_match_units_of_their_own(kind, L, H, lens, mode, o_dtype):
     case = make_refresh_case(61, kind, L, H, H if kind == dasc.KDA else H // 2, 128, 128, lens, scope=dasc.SCOPE_LAYER, keep_ratio=0.4)
