@@ -1,5 +1,6 @@
 // Suffix refresh, chunked form, on the Blackwell tensor cores (tcgen05 + TMEM), warp-specialised:
-// 32-token chunks, two CTAs resident per SM, four roles per CTA, several units (request, layer, value head) per CTA one after another.
+// 32-token chunks, two CTAs resident per SM (or one with more warps, where a launch has no more), several units (request, layer, value
+// head) per CTA one after another.
 //
 // Eq. 1 (transposed orientation) over a chunk of C = 32 tokens starting from S_0, with
 // G_t the running sum of the log-decay inside the chunk and m the chunk midpoint:
@@ -26,15 +27,15 @@
 // MMA1 has; MMA5 contracts over the tokens and reads Kh as an MN-major operand from a second tile (tf32
 // MN-major operands have a swizzle of their own), which, read last, is double-buffered by chunk parity.
 //
-// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1090 us = 1.92 G token-heads/s = 60 % of the
-// rate at which HBM could bring its bytes (657 us), GDN 885 us = 2.37 G (46 %); 1685 and 1630 us in the form this one grew from.
-// No unit of the SM is at its limit: per chunk and SM (two CTAs) KDA takes 4.5 k cycles, of which the shared-memory data pipe
-// (load/store units and the tensor core's operand reads together) is busy 74 %, the issue slots 50 %, the tensor pipe 35 %; GDN
-// 3.7 k, 82 %, 47 %, 39 %; the state-only form 4.8 k at 2 to 4 chunks per unit, 59 %, 46 %, 24 %.  A CTA alone on its SM
-// completes a chunk every 4.8 k cycles (GDN 4.5 k), bound by its chain of hand-offs; the second CTA hides some of that
-// and the starts and ends of units.
+// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1058 us = 1.98 G token-heads/s = 62 % of the
+// rate at which HBM could bring its bytes (657 us), GDN 824 us = 2.54 G (50 %); 1685 and 1630 us in the form this one grew from, 1090 and
+// 885 with a CTA per unit.  What is nearest its limit is the SM's shared-memory data pipe (load/store units and the tensor core's operand
+// reads together): per chunk and SM (two CTAs) KDA takes 4.2 k cycles, of which that pipe is busy 81 %, the issue slots 52 %, the tensor
+// pipe 37 %; GDN 3.3 k, 93 %, 48 %, 43 %; the state-only form 3.6 k at 2 to 4 chunks per unit, 74 %, 53 %, 33 %.  A CTA alone
+// on its SM is bound by its chain of hand-offs: a chunk every 3.8 k cycles (GDN 3.5 k) in the form made for it (see alone_for), 4.8 k
+// in the other.
 // What it was before, in the order in which it was found: 103 cycles of issue per tensor-core instruction (behind
-// `lane == 0` instead of an elected lane), 119 KB of code in the instruction caches (now 56 KB), and 85 % of the
+// `lane == 0` instead of an elected lane), 119 KB of code in the instruction caches (half of that now), and 85 % of the
 // shared-memory pipe (8-byte accesses in 16-byte places, A padded to 128 rows, V and O value by value).
 // Under sustained load the part is at its 1000 W limit and runs this kernel at 1.7 instead of 1.965 GHz.
 #include <cuda.h>

@@ -1,4 +1,4 @@
-"""The token-by-token kernel has one variant per range of unit counts (columns split over CTAs, halves, whole units): each
+"""The token-by-token kernel has one variant per range of unit counts (columns split over CTAs, whole units in blocks of four, token by token): each
 at the edges of its token groups and on both sides of the counts where the choice changes, against the fp64 oracle."""
 import pytest
 import torch
