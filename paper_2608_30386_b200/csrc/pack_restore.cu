@@ -28,8 +28,9 @@ constexpr int kUnroll = 4;     // over {128..1024} x {1..16}
 // layers of 2 .. 48 heads, microseconds with 4 / 2 / 1 loads at so many blocks:
 //   store  312: 4.9 3.5 3.5   600: 6.0 5.2 5.4   744: 6.5 6.3 6.3   816: 6.8 6.7 6.7   888: 7.0 7.0 7.1   1176: 8.4 8.5 8.8
 //   load   480: 5.1 4.0 3.8   672: 5.9 5.4 5.0   768: 5.8 5.8 5.4   864: 6.0 6.1 5.8   960: 6.3 6.5 6.3   1152: 6.9 7.2 7.1
-// Both kernels gain nothing from fewer loads from about 888 blocks on.  Up to there a load alone does a little better with 1 than with 2
-// in this table, but among others on the stream it is the slower one: 2 / 1 loads at 672 blocks 3.75 / 3.91, 768 3.98 / 4.31, 864 4.28 / 4.70.
+// Both kernels gain nothing from fewer loads from about 888 blocks on.  Up to there a load from and to memory does a
+// little better with 1 than with 2 (back to back over 350 MB of states and slots: 768 blocks 5.6 / 6.0, 864 6.0 / 6.4), one whose slot and state
+// are still in L2 a little worse (4.3 / 4.0, 4.7 / 4.3).
 int unroll_for(uint64_t blocks) { return blocks <= 4 * 148 ? 1 : blocks <= 6 * 148 ? 2 : kUnroll; }
 
 enum class Layout { Ragged, Padded, TpBalanced };
