@@ -1357,7 +1357,9 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       // triangular warp, which arrived on a_taken, which these warps have waited for.  (Waiting for rdy_prep itself here could wait for
       // the wrong phase: the next unit's tiles can be complete by now.)
       if (n_chunks > 0) wait_bar(&misc->bar_s[buf(n - 1)], phase(n - 1), misc);
-      if (tid < D) fin_s[tid] = n_chunks > 0 ? ex2f(post_s[KDA ? ((n - 1) & 1) * D + tid : (n - 1) & 3] * LOG2E) : 1.f;
+      // A unit without tokens has no factor and must not touch fin_s: it meets no wait on the way here, so the slower chain warps can
+      // still be scaling the unit before.  (One with tokens has been through rdy_state, which all of them arrive on behind that.)
+      if (n_chunks > 0 && tid < D) fin_s[tid] = ex2f(post_s[KDA ? ((n - 1) & 1) * D + tid : (n - 1) & 3] * LOG2E);
       sync_chain();
       tc_fence_after_sync();
       // A unit whose decay left the range, or whose CTA gave up on a wait, is NOT written back: its stored state keeps
@@ -1374,17 +1376,18 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
           const uint32_t write = i == 0 ? rows[0] : rows[1];
           float *const st_c = a.state + x.state + (c0 * D + vrow);
           const float *const fin_c = fin_s + c0;
-          uint32_t s[32];
           if (n_chunks > 0) {
+            uint32_t s[32];
             tmem_ld32(tlane + COL_S + c0, s);
             tmem_ld_wait();
-          } else {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) s[j] = 0u;  // scratch mode with an empty suffix
+            for (int j = 0; j < 32; ++j)
+              if (write >> j & 1u) st_c[j * D] = __uint_as_float(s[j]) * fin_c[j];
+          } else {  // scratch mode with an empty suffix
+#pragma unroll 1
+            for (int j = 0; j < 32; ++j)
+              if (write >> j & 1u) st_c[j * D] = 0.f;
           }
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (write >> j & 1u) st_c[j * D] = __uint_as_float(s[j]) * fin_c[j];
         }
       }
       if (!WALK) break;

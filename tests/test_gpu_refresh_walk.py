@@ -7,7 +7,8 @@ import torch
 
 import oracle
 import paper_2608_30386_b200 as dasc
-from helpers import assert_refresh_close, make_refresh_case, run_refresh_oracle
+from helpers import RefreshCase, assert_refresh_close, make_plans, make_refresh_case, run_refresh_oracle
+from paper_2608_30386_b200 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -56,3 +57,49 @@ def test_walked_units_match_units_of_their_own(kind, L, H, lens, mode, o_dtype):
         merge = mode != dasc.REFRESH_CONTINUE
         ref_s, ref_o = run_refresh_oracle(case, mode=oracle.MODE_SCRATCH_MERGE_LOCAL if merge else oracle.MODE_CONTINUE, want_o=not merge)
         assert_refresh_close(case, walked[0].cpu().numpy(), None if merge else walked[1].cpu().numpy(), ref_s, ref_o, 1e-3)
+
+
+def _half_kept_case(kind, kept_half):
+    """Requests with and without tokens; KDA: nearly all rows of one half of the channels are retained, nearly none of the other."""
+    L, H, lens = 1, 8, [64, 0, 0, 40, 0, 33] * 24
+    gen = synth.generator(62)
+    if kind == dasc.KDA:
+        rates = torch.full((L, H, 128), 0.08)
+        rates[:, :, kept_half * 64:kept_half * 64 + 64] = 0.002
+        rates *= 1 + 0.01 * torch.rand(rates.shape, generator=gen)
+    else:
+        rates = synth.decay_rates(gen, L, H, 1, 0.01, 0.1)
+    plan, oplan = make_plans(kind, L, H, H if kind == dasc.KDA else H // 2, 128, 128, rates, sel=dasc.SEL_TOP_RATIO,
+                             scope=dasc.SCOPE_LAYER, keep_ratio=0.48)
+    cu = torch.zeros(len(lens) + 1, dtype=torch.int32)
+    cu[1:] = torch.cumsum(torch.tensor(lens), 0).to(torch.int32)
+    s = synth.token_streams(gen, kind, L, int(cu[-1]), H, H if kind == dasc.KDA else H // 2, 128, 128, rates)
+    for f in ("q", "k", "v", "g", "beta"):
+        setattr(s, f, getattr(s, f).to("cuda"))
+    state0 = synth.states(gen, (len(lens), L, H, 128, 128)).to("cuda")
+    return RefreshCase(kind, L, H, H if kind == dasc.KDA else H // 2, 128, 128, cu, s, state0, plan, oplan)
+
+
+def replay_static(case, bound, mode):
+    dev, n = case.state0.device, case.cu.numel() - 1
+    dense = case.H_v * 128 * 128
+    s, state = case.streams, case.state0.clone()
+    scratch = dasc.dasc_refresh_static(case.plan, state, dense, case.L * dense, torch.arange(n, dtype=torch.int32, device=dev), s.q, s.k,
+                                       s.v, s.g, s.beta, case.cu.to(dev), int(case.cu[-1]), bound, mode=mode)
+    torch.cuda.synchronize()
+    assert dasc.dasc_refresh_status(scratch) == 0
+    return state
+
+
+# Where the caller asks for the chunked kernel alone, requests without tokens stay in a CTA's list, behind those with tokens; in the
+# merge mode they have rows to write, and nothing to wait for before they do.  Chain warps of channels 0-63 and 64-127 then end the unit
+# before at different times.
+@pytest.mark.parametrize("kind,kept_half", [(dasc.KDA, 0), (dasc.KDA, 1), (dasc.GDN, 0)])
+def test_units_without_tokens_behind_others_in_a_walk(kind, kept_half):
+    case, mode = _half_kept_case(kind, kept_half), dasc.REFRESH_SCRATCH_MERGE_LOCAL
+    own = replay(case, LOOSE, mode, None, dasc.ALGO_CHUNKED)[0]
+    ref_s, _ = run_refresh_oracle(case, mode=oracle.MODE_SCRATCH_MERGE_LOCAL, want_o=False)
+    assert_refresh_close(case, own.cpu().numpy(), None, ref_s, None, 1e-3)
+    for _ in range(6):
+        assert torch.equal(replay(case, 64, mode, None, dasc.ALGO_CHUNKED)[0].view(torch.int32), own.view(torch.int32))
+    assert torch.equal(replay_static(case, 64, mode).view(torch.int32), replay_static(case, LOOSE, mode).view(torch.int32))
