@@ -537,10 +537,10 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     fence_smem_to_async();
   };
   // Outputs of chunk n, of which `ntok` tokens are the request's: one token half (SHARED: the warp's) or both
-  // by this warp, thread ti of those that take them.
+  // by this warp, thread ti of those that take them.  The caller has waited for bar_o; no second wait for it here, since in the ALONE form
+  // product 4 of the next chunk is on its way by then and could turn the parity first.
   auto outputs = [&](int n, int ntok, OT *go, int half_0, int ti) {
     constexpr int NTH = ALONE ? 128 : NCH;
-    wait_bar(&misc->bar_o, n & 1, misc);
     tc_fence_after_sync();
     if (WITH_O) {
 #pragma unroll
@@ -1337,6 +1337,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
 
         // ---- (6) outputs of this chunk (without outputs MMA5 is waited for here as well) ----
         if (!ALONE) {
+          wait_bar(&misc->bar_o, par, misc);
           outputs(n, ntok, go, colh, tid);
           if (WITH_O) go += C * v_stride;
           tc_fence_before_sync();
