@@ -133,7 +133,8 @@ struct Misc {
   // Each barrier completes one phase per chunk.  Where the arrivals are "per warp", a warp's first lane arrives for it.
   // tensor core -> chain warps (one tcgen05.commit each); bar_ap also releases the triangular and the issuing warp and the
   // next log-decay (KDA) or k, q (GDN), bar_ro the Kt/Qt tile, bar_s the Kh tile of its parity (KDA)
-  // (two of each where a phase can complete before all have waited for the one before: ALONE, by chunk parity)
+  // (two of each, by chunk parity, where a phase could complete before all have waited for the one before: all three in ALONE; bar_s in
+  // both forms, since the KDA producers wait for chunk n - 1's after they have handed over chunk n's tiles, which its products 5 need)
   uint64_t bar_ap[2], bar_ro[2], bar_s[2], bar_u, bar_o;
   // producer -> issuing warp: the tiles of a chunk are ready (per warp: 4 arrivals; KDA one more from the triangular warp, for beta)
   uint64_t rdy_prep[2];  // (ALONE: by chunk parity)
@@ -361,7 +362,8 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
   constexpr int NP = F::NP, WARP_T = F::WARP_T, WARP_MMA = F::WARP_MMA, WARP_O = F::WARP_O, WARP_MMA1 = F::WARP_MMA1, RING = F::RING, FAC = F::FAC;
   // where chunk n's buffer is, and the barrier and the parity that stand for it
   auto buf = [](int n) { return static_cast<uint32_t>(ALONE ? n & 1 : 0); };
-  auto phase = [](int n) { return static_cast<uint32_t>(ALONE ? (n >> 1) & 1 : n & 1); };
+  auto phase2 = [](int n) { return static_cast<uint32_t>((n >> 1) & 1); };  // of what there are two of
+  auto phase = [&](int n) { return ALONE ? phase2(n) : static_cast<uint32_t>(n & 1); };
   auto off_kq = [&](int n) { return OFF_KQ + buf(n) * (OFF_KQ_2 - OFF_KQ); };
   auto off_kh = [&](int n) { return OFF_KH + buf(n) * (OFF_KH_2 - OFF_KH); };  // GDN: raw k, q
   auto off_kht = [&](int n) { return OFF_KHT + (n & 1) * (128 * 128) + (ALONE && (n & 2) ? OFF_KHT_2 - OFF_KHT : 0u); };
@@ -390,10 +392,10 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       mbar_init(&misc->rdy_prep[i], NP / 32 + (KDA && !ALONE ? 1 : 0));
       mbar_init(&misc->bar_ap[i], 1);
       mbar_init(&misc->bar_ro[i], 1);
-      mbar_init(&misc->bar_s[i], 1);
       mbar_init(&misc->g_full[i], 4);
       mbar_init(&misc->kq_full[i], WITH_O ? 4 : 2);
     }
+    for (int i = 0; i < 2; ++i) mbar_init(&misc->bar_s[i], 1);
     for (int i = 0; i < FAC; ++i) mbar_init(&misc->rdy_fac[i], KDA ? 4 : 1);
     mbar_init(&misc->bar_u, 1);
     mbar_init(&misc->bar_o, 1);
@@ -673,14 +675,14 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       if (elect_one()) {
         if (ALONE) {
           mma5(col_ro(n));
-          mma_commit(&misc->bar_s[buf(n)]);
+          mma_commit(&misc->bar_s[par]);
           mma4(COL_U<ALONE>);
         }
         mma4(col_ro(n));
         mma_commit(&misc->bar_o);
         if (!ALONE) {
           mma5(col_ro(n));
-          mma_commit(&misc->bar_s[buf(n)]);
+          mma_commit(&misc->bar_s[par]);
         }
       }
       __syncwarp();
@@ -1139,7 +1141,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
         // The next raw k, q (KDA) land once MMA5 of the previous chunk has read the Kh tile of that parity; the next
         // log-decay (KDA) or k, q (GDN) once MMA1 of this chunk has read the tile they go to.
         if (KDA && !ALONE) {
-          if (n > 0) wait_bar(&misc->bar_s[0], par ^ 1, misc);
+          if (n > 0) wait_bar(&misc->bar_s[par ^ 1], phase2(n - 1), misc);
           if (lane == 0 && !misc->abort_flag) stage_kq(n + 1);
         }
         if (!ALONE) {
@@ -1197,7 +1199,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
 
         // ---- (1) the previous chunk's state update is complete; this chunk's factors and tiles are ready ----
         wait_bar(&misc->rdy_fac[n % FAC], (n / FAC) & 1, misc);
-        if (ch > 0) wait_bar(&misc->bar_s[buf(n - 1)], phase(n - 1), misc);
+        if (ch > 0) wait_bar(&misc->bar_s[(n - 1) & 1], phase2(n - 1), misc);
         tc_fence_after_sync();
 
         // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
@@ -1357,7 +1359,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       // post_s of the last chunk is visible: its writers arrived on rdy_prep, which the issuing warp waited for before it met the
       // triangular warp, which arrived on a_taken, which these warps have waited for.  (Waiting for rdy_prep itself here could wait for
       // the wrong phase: the next unit's tiles can be complete by now.)
-      if (n_chunks > 0) wait_bar(&misc->bar_s[buf(n - 1)], phase(n - 1), misc);
+      if (n_chunks > 0) wait_bar(&misc->bar_s[(n - 1) & 1], phase2(n - 1), misc);
       // A unit without tokens has no factor and must not touch fin_s: it meets no wait on the way here, so the slower chain warps can
       // still be scaling the unit before.  (One with tokens has been through rdy_state, which all of them arrive on behind that.)
       if (n_chunks > 0 && tid < D) fin_s[tid] = ex2f(post_s[KDA ? ((n - 1) & 1) * D + tid : (n - 1) & 3] * LOG2E);

@@ -72,8 +72,8 @@ class Order:
 
 
 def roles(alone, kda, with_o):
-    two = {b: 2 for b in ("rdy_prep", "bar_ap", "bar_ro", "bar_s", "g_full", "kq_full")} if alone else {}
-    x = Order({**two, "rdy_fac": 4 if alone else 2})
+    two = {b: 2 for b in ("rdy_prep", "bar_ap", "bar_ro", "g_full", "kq_full")} if alone else {}
+    x = Order({**two, "bar_s": 2, "rdy_fac": 4 if alone else 2})
     chain, producers, out = [f"chain {i}" for i in range(8)], [f"producer {i}" for i in range(8 if alone else 4)], [f"out {i}" for i in range(4)]
 
     def mma1(role, n):
@@ -216,7 +216,7 @@ def roles(alone, kda, with_o):
     return x
 
 
-FORMS = [(True, kda, with_o) for kda in (True, False) for with_o in (True, False)]
+FORMS = [(alone, kda, with_o) for alone in (True, False) for kda in (True, False) for with_o in (True, False)]
 
 
 @pytest.mark.parametrize("alone,kda,with_o", FORMS)
@@ -228,6 +228,7 @@ def test_every_wait_of_the_kernel_is_entered_above():
     text = re.sub(r"//.*", "", open(SOURCE).read())
     outputs = text[text.index("auto outputs ="):text.index("if (warp == WARP_MMA) {", text.index("auto outputs ="))]
     assert "wait_bar" not in outputs  # its callers wait, once per chunk
+    assert "for (int i = 0; i < 2; ++i) mbar_init(&misc->bar_s[i], 1);" in text  # two in both forms
     sites = defaultdict(int)
     for bar in re.findall(r"wait_bar\(&misc->(\w+)", text):
         sites[bar] += 1
