@@ -503,7 +503,9 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     if (ALONE && n > 0) wait_bar(&misc->rdy_rhs, (n - 1) & 1, misc);  // the triangular warp has read the chunk before's
     tc_fence_after_sync();
     take_a_rows<KDA>(tm + (32u << 16) + col_ap(n), 16, (KDA ? beta_s : bte1_s) + (n % RING) * C, e2_s + (n % RING) * C, LT, lane);
-    asm volatile("bar.arrive 3, 64;" ::: "memory");
+    // A full barrier on both sides: after a time-out no wait below keeps this warp from the next chunk, and a second bare arrival of its own
+    // would complete the barrier without the triangular warp, which would later wait for an arrival that never comes.
+    asm volatile("bar.sync 3, 64;" ::: "memory");
   };
   // where a chunk's raw k, q lie: rows of a 64-channel block, and q behind k
   constexpr uint32_t RAW_ROWS = KDA ? 32 : 64, OFF_RAW_Q = KDA ? 2 * 32 * 128 : 32 * 128;
