@@ -213,7 +213,7 @@ __device__ __forceinline__ void wait_bar(uint64_t *bar, uint32_t parity, Misc *m
       : "memory");
 }
 
-// The test hook's wait (one call site): `max_polls` non-blocking looks at the barrier, so that a short limit runs out
+// The test hook's wait: `max_polls` non-blocking looks at the barrier, so that a short limit runs out
 // whatever the time slice of a blocking poll is.
 __device__ __forceinline__ void wait_bar_short(uint64_t *bar, uint32_t parity, Misc *misc, uint32_t max_polls) {
   bool done = false;
@@ -472,10 +472,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
 
   auto mma1 = [&](int n) {
     // MMA1: [Kt;Qt] Kh^T, M = 64: 16 rows in each TMEM quadrant, A's in the first two, P's in the last two.
-    if (n == 0 && a.poll_limit_first_wait)
-      wait_bar_short(&misc->rdy_prep[buf(n)], phase(n), misc, a.poll_limit_first_wait);
-    else
-      wait_bar(&misc->rdy_prep[buf(n)], phase(n), misc);
+    wait_bar(&misc->rdy_prep[buf(n)], phase(n), misc);
     tc_fence_after_sync();
     if (elect_one()) {
       if constexpr (KDA) {
@@ -496,6 +493,11 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       mma_commit(&misc->bar_ap[buf(n)]);
     }
     __syncwarp();
+  };
+  // Test hook: a first, short wait for the tiles of the first chunk, by the warp that issues MMA1, as soon as nothing but copies that have
+  // just been started can have gone into them.
+  auto first_wait = [&]() {
+    if (a.poll_limit_first_wait && all_chunks > 0) wait_bar_short(&misc->rdy_prep[0], 0, misc, a.poll_limit_first_wait);
   };
   auto take_a = [&](int n) {
     // rows 16-31 of A are in this warp's quadrant: hand them to the triangular warp
@@ -603,6 +605,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
   if (warp == WARP_MMA) {
     // =========================== tensor-core issue warp ===========================
     // The whole warp walks the chunks and waits; an elected lane issues.
+    if (!ALONE) first_wait();
     for (int n = 0; n < all_chunks; ++n) {
       const uint32_t par = n & 1;
       if (!ALONE) {
@@ -839,6 +842,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       __syncwarp();
     };
     for (int n = 0; n < 2 && n < all_chunks; ++n) copy(n);
+    first_wait();
     // KDA: beta as well, lane = token, into its ring before MMA1 goes out (its readers wait for that product)
     auto fetch_beta = [&](int n) { return lane < x.n_tok - n * C ? a.beta[(x.tok0 + n * C + lane) * a.H_v + x.head] : 0.f; };
     float beta = KDA && all_chunks > 0 ? fetch_beta(0) : 0.f;

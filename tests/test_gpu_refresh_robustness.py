@@ -149,3 +149,33 @@ def test_refresh_window_checks_every_argument_before_it_writes_window_begin():
     assert e.value.status == binding.ERR_INVALID_ARG
     torch.cuda.synchronize()
     assert int(wb.item()) == -7 and torch.equal(state, case.state0)
+
+
+# alone on an SM, a CTA per unit with two CTAs per SM (the loose bound), and CTAs that replay three units
+@pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
+@pytest.mark.parametrize("with_o", [True, False])
+@pytest.mark.parametrize("heads,lens,bound", [(2, [32], 32), (8, [70, 33, 96] * 13, 1 << 30), (8, [64] * 111, 64)])
+def test_a_wait_that_runs_out_in_every_form(kind, with_o, heads, lens, bound):
+    case = make_refresh_case(47, kind, 1, heads, heads if kind == dasc.KDA else heads // 2, 128, 128, lens, scope=dasc.SCOPE_LAYER,
+                             keep_ratio=0.5)
+    dev, n, T = case.state0.device, len(lens), int(case.cu[-1])
+    s, ids = case.streams, torch.arange(n, dtype=torch.int32, device=dev)
+    ws = torch.zeros(dasc.dasc_refresh_workspace_bytes(case.plan, n, 1, dasc.ALGO_CHUNKED), dtype=torch.uint8, device=dev)
+    o = torch.zeros((1, T, heads, 128), device=dev) if with_o else None
+
+    def call(state):
+        dasc.dasc_refresh(case.plan, state, heads * 128 * 128, heads * 128 * 128, ids, s.q, s.k, s.v, s.g, s.beta, case.cu.to(dev), T,
+                          bound, o=o, algo=dasc.ALGO_CHUNKED, workspace=ws)
+        torch.cuda.synchronize()
+        return dasc.dasc_refresh_status(ws)
+
+    first = case.state0.clone()
+    assert call(first) == binding.OK
+    state = case.state0.clone()
+    try:
+        dasc.dasc_debug_set_refresh_poll_limit(1)
+        assert call(state) == binding.ERR_TIMEOUT
+    finally:
+        dasc.dasc_debug_set_refresh_poll_limit(0)
+    assert torch.equal(state, case.state0)                                # no unit was written back
+    assert call(state) == binding.OK and torch.equal(state, first)        # the next call finds nothing left over
