@@ -859,9 +859,10 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       // four, was read by MMA5 of two chunks ago, which the chain warps had seen complete before MMA2 of the chunk before.
       if (n + 2 < all_chunks) copy(n + 2);
     }
-    // after a time-out the last copies may not have been waited for: they must have landed before the CTA leaves
-    if (misc->abort_flag && issued > 0)
-      mbar_wait_bounded(copies_g ? &misc->g_full[buf(issued - 1)] : &misc->kq_full[buf(issued - 1)], phase(issued - 1), kMaxPolls);
+    // after a time-out the last copies, those of two chunks, may not have been waited for: they must have landed before the CTA leaves
+    if (misc->abort_flag)
+      for (int n = max(issued - 2, 0); n < issued; ++n)
+        mbar_wait_bounded(copies_g ? &misc->g_full[buf(n)] : &misc->kq_full[buf(n)], phase(n), kMaxPolls);
     __syncwarp();
     // (after a time-out: as for the issuing warp)
     if (misc->abort_flag) {

@@ -151,10 +151,11 @@ def test_refresh_window_checks_every_argument_before_it_writes_window_begin():
     assert int(wb.item()) == -7 and torch.equal(state, case.state0)
 
 
-# alone on an SM, a CTA per unit with two CTAs per SM (the loose bound), and CTAs that replay three units
+# alone on an SM (five chunks: copies of two are in flight when the wait runs out), a CTA per unit with two CTAs per SM (the loose
+# bound), and CTAs that replay three units
 @pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
 @pytest.mark.parametrize("with_o", [True, False])
-@pytest.mark.parametrize("heads,lens,bound", [(2, [32], 32), (8, [70, 33, 96] * 13, 1 << 30), (8, [64] * 111, 64)])
+@pytest.mark.parametrize("heads,lens,bound", [(2, [130], 130), (8, [70, 33, 96] * 13, 1 << 30), (8, [64] * 111, 64)])
 def test_a_wait_that_runs_out_in_every_form(kind, with_o, heads, lens, bound):
     case = make_refresh_case(47, kind, 1, heads, heads if kind == dasc.KDA else heads // 2, 128, 128, lens, scope=dasc.SCOPE_LAYER,
                              keep_ratio=0.5)
