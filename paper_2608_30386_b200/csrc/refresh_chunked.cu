@@ -684,7 +684,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
           mma4(COL_U<ALONE>);
         }
         mma4(col_ro(n));
-        mma_commit(&misc->bar_o);
+        if (WITH_O || !ALONE) mma_commit(&misc->bar_o);  // (only where someone waits for it: an arrival must not outlive the CTA)
         if (!ALONE) {
           mma5(col_ro(n));
           mma_commit(&misc->bar_s[par]);

@@ -21,6 +21,7 @@ class Order:
         self.split = split                      # barrier -> how many there are, taken by chunk index in turn
         self.before = defaultdict(set)          # operation or event -> what comes directly before it
         self.last, self.arrivals, self.waits, self.n = {}, defaultdict(list), [], 0
+        self.unwaited, self.waited = set(), set()
 
     def op(self, role):
         self.n += 1
@@ -36,10 +37,15 @@ class Order:
     def arrive(self, role, bar, chunk):
         self.arrivals[self.phase(bar, chunk)].append(self.op(role))
 
+    def later(self, role, bar, chunk):  # an arrival by the tensor core or a copy, some time after the role has asked for it
+        self.arrive(role, bar, chunk)
+        self.unwaited.add(self.phase(bar, chunk))
+
     def wait(self, role, bar, chunk):
         w = self.op(role)
         self.before[w].add(self.phase(bar, chunk))
         self.waits.append((w, role, bar, self.phase(bar, chunk)))
+        self.waited.add(self.phase(bar, chunk))
 
     def meet(self, role, name, chunk):  # a named barrier of the block
         event = ("named", name, chunk)
@@ -77,7 +83,7 @@ def roles(alone, kda, with_o):
 
     def mma1(role, n):
         x.wait(role, "rdy_prep", n)
-        x.arrive(role, "bar_ap", n)
+        x.later(role, "bar_ap", n)
 
     def take_a(role, n):
         x.wait(role, "bar_ap", n)
@@ -98,17 +104,17 @@ def roles(alone, kda, with_o):
             mma1("issue", n)
             take_a("issue", n)
         x.wait("issue", "rdy_state", n)
-        x.arrive("issue", "bar_ro", n)
+        x.later("issue", "bar_ro", n)
         if not alone:
             x.wait("issue", "rdy_t", n)
         x.wait("issue", "rdy_rhs", n)
-        x.arrive("issue", "bar_u", n)
+        x.later("issue", "bar_u", n)
         x.wait("issue", "bar_u", n)
         x.wait("issue", "rdy_u", n)
-        for bar in ("bar_s", "bar_o") if alone else ("bar_o", "bar_s"):
-            x.arrive("issue", bar, n)
+        for bar in ("bar_s", "bar_o")[:2 if with_o else 1] if alone else ("bar_o", "bar_s"):
+            x.later("issue", bar, n)
 
-    x.arrive("triangular", "v_full", 0)
+    x.later("triangular", "v_full", 0)
     if kda and not alone:
         x.arrive("triangular", "rdy_prep", 0)
     for n in range(CHUNKS):
@@ -122,12 +128,12 @@ def roles(alone, kda, with_o):
             if kda and not alone:
                 x.arrive("triangular", "rdy_prep", n + 1)
             x.wait("triangular", "rdy_rhs", n)
-            x.arrive("triangular", "v_full", n + 1)
+            x.later("triangular", "v_full", n + 1)
 
     if alone:
         def copy(n):
             for bar in ("g_full", "kq_full") if kda else ("kq_full",):
-                x.arrive("mma1", bar, n)
+                x.later("mma1", bar, n)
         copy(0)
         copy(1)
         for n in range(CHUNKS):
@@ -155,10 +161,10 @@ def roles(alone, kda, with_o):
     for i, role in enumerate(producers):
         def kq(n):
             if with_o or i & 3 < 2:
-                x.arrive(role, "kq_full", n)
+                x.later(role, "kq_full", n)
         if not alone:
             if kda:
-                x.arrive(role, "g_full", 0)
+                x.later(role, "g_full", 0)
             kq(0)
         if not kda and i == 0:
             x.arrive(role, "rdy_fac", 0)
@@ -188,7 +194,7 @@ def roles(alone, kda, with_o):
                 if not alone:
                     x.wait(role, "bar_ap", n)
                     if kda:
-                        x.arrive(role, "g_full", n + 1)
+                        x.later(role, "g_full", n + 1)
                     else:
                         kq(n + 1)
 
@@ -212,6 +218,7 @@ def roles(alone, kda, with_o):
                 if with_o:
                     x.meet(role, "O tile", n)
                 x.arrive(role, "tp_free", n)
+        x.wait(role, "bar_s", CHUNKS - 1)  # the end of the unit
     return x
 
 
@@ -223,6 +230,12 @@ def test_no_wait_can_be_overtaken(alone, kda, with_o):
     assert roles(alone, kda, with_o).overtaken() == set()
 
 
+@pytest.mark.parametrize("alone,kda,with_o", FORMS)
+def test_nothing_arrives_after_the_block_has_left(alone, kda, with_o):
+    x = roles(alone, kda, with_o)
+    assert x.unwaited <= x.waited
+
+
 def test_named_barriers_hold_every_warp_that_meets_there():
     # after a time-out the mbarriers hold nobody back any more; warps that only arrived would run ahead and complete a later phase alone
     assert "bar.arrive" not in re.sub(r"//.*", "", open(SOURCE).read())
@@ -232,6 +245,7 @@ def test_every_wait_of_the_kernel_is_entered_above():
     text = re.sub(r"//.*", "", open(SOURCE).read())
     outputs = text[text.index("auto outputs ="):text.index("if (warp == WARP_MMA) {", text.index("auto outputs ="))]
     assert "wait_bar" not in outputs  # its callers wait, once per chunk
+    assert re.findall(r"(?:if \(.*\) )?mma_commit\(&misc->bar_o\)", text) == ["if (WITH_O || !ALONE) mma_commit(&misc->bar_o)"]
     assert "for (int i = 0; i < 2; ++i) mbar_init(&misc->bar_s[i], 1);" in text  # two in both forms
     sites = defaultdict(int)
     for bar in re.findall(r"wait_bar\(&misc->(\w+)", text):
