@@ -186,8 +186,19 @@ __device__ __forceinline__ void arrive_warp(uint64_t *bar, int lane) {
   if (lane == 0) mbar_arrive(bar);
 }
 
-// barrier among the 256 chain threads only
-__device__ __forceinline__ void sync_chain() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// Barrier among the 256 chain threads: does the predicate hold for any of them?
+__device__ __forceinline__ bool any_chain(bool p) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "barrier.cta.red.or.pred.aligned q, 1, 256, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any)
+      : "r"(static_cast<uint32_t>(p))
+      : "memory");
+  return any != 0;
+}
 
 // What comes out of a broadcast shuffle the compiler may keep in uniform registers.
 __device__ __forceinline__ int uni(int x) { return __shfl_sync(0xffffffffu, x, 0); }
@@ -1370,15 +1381,17 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       // A unit without tokens has no factor and must not touch fin_s: it meets no wait on the way here, so the slower chain warps can
       // still be scaling the unit before.  (One with tokens has been through rdy_state, which all of them arrive on behind that.)
       if (n_chunks > 0 && tid < D) fin_s[tid] = ex2f(post_s[KDA ? ((n - 1) & 1) * D + tid : (n - 1) & 3] * LOG2E);
-      sync_chain();
+      // In a walk other roles are in the next unit and can run out of a wait there at any time, so what the barrier answers, not a look at
+      // the flag by each thread, says whether this unit is written: all of it or nothing.
+      const bool gave_up = any_chain(misc->abort_flag != 0);
       tc_fence_after_sync();
       // A unit whose decay left the range, or whose CTA gave up on a wait, is NOT written back: its stored state keeps
       // the bits it had before the call, so that it can be replayed by the exact kernel (or by the caller).
-      const bool bad = misc->abort_flag != 0 || misc->domain_flag[u & 3] != 0;
+      const bool bad = gave_up || misc->domain_flag[u & 3] != 0;
       // The flag of unit u - 1, which everyone has looked at, becomes that of unit u + 3, which the producer warps cannot have reached.
       if (tid == 0) misc->domain_flag[(u + 3) & 3] = 0;
       if (bad) {
-        if (tid == 0 && misc->abort_flag == 0) hand_over(a, x.index, true);
+        if (tid == 0 && !gave_up) hand_over(a, x.index, true);
       } else {
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
