@@ -438,6 +438,13 @@ dasc_status_t dasc_refresh_counters(const void *workspace, size_t workspace_byte
  * that a test can watch a bounded wait run out (DASC_ERR_TIMEOUT, the unit left
  * unwritten, the context still usable).  0 restores the normal limit.  Process-wide. */
 void dasc_debug_set_refresh_poll_limit(uint32_t polls);
+/* Test hook: the form of the chunked kernel that a call of these sizes gets, so that a test can say which
+ * one it is about.  units_per_req = layers in the call x value heads; window and max_seqlen as the kernel sees
+ * them (dasc_refresh: 0 and the caller's bound; dasc_refresh_window: the window twice).  Returns 0: one thread
+ * block per unit, two per SM; 1: blocks replay several units each; 2: one block per unit, alone on its SM.
+ * *n_blocks (may be NULL) = blocks of the launch.  Host arithmetic only. */
+int32_t dasc_debug_refresh_form(int32_t n_req, int32_t units_per_req, int64_t total_tokens, int32_t window,
+                                int32_t max_seqlen, int64_t *n_blocks);
 
 /*
  * Load path, suffix-refresh policy as the paper states it (Section 4.2, with the

@@ -36,7 +36,7 @@ EXPORTS = (
     "dasc_int8_slot_bytes", "dasc_pack_int8", "dasc_restore_int8",
     "dasc_padded_pool_floats", "dasc_pack_padded", "dasc_restore_padded", "dasc_checkpoint_bytes", "dasc_slot_budget",
     "dasc_tp_balance", "dasc_pack_tp", "dasc_restore_tp", "dasc_tp_head_permutation", "dasc_conv_store", "dasc_conv_load",
-    "dasc_refresh_counters", "dasc_debug_set_refresh_poll_limit",
+    "dasc_refresh_counters", "dasc_debug_set_refresh_poll_limit", "dasc_debug_refresh_form",
     "dasc_refresh_workspace_bytes", "dasc_refresh", "dasc_refresh_status", "dasc_refresh_window", "dasc_refresh_static",
     "dasc_status_string", "dasc_version",
 )
@@ -117,6 +117,8 @@ def lib() -> C.CDLL:
         L.dasc_refresh_counters.argtypes = [C.c_void_p, C.c_size_t, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
         L.dasc_debug_set_refresh_poll_limit.restype = None
         L.dasc_debug_set_refresh_poll_limit.argtypes = [C.c_uint32]
+        L.dasc_debug_refresh_form.restype = C.c_int32
+        L.dasc_debug_refresh_form.argtypes = [C.c_int32, C.c_int32, C.c_int64, C.c_int32, C.c_int32, C.POINTER(C.c_int64)]
         L.dasc_int8_slot_bytes.argtypes = [C.c_void_p, C.POINTER(C.c_size_t)]
         L.dasc_pack_int8.argtypes = L.dasc_pack.argtypes
         L.dasc_restore_int8.argtypes = L.dasc_restore.argtypes
@@ -484,6 +486,13 @@ def dasc_refresh_counters(workspace):
 def dasc_debug_set_refresh_poll_limit(polls: int):
     """Test hook: poll limit of the chunked kernel's first wait (0 = normal)."""
     lib().dasc_debug_set_refresh_poll_limit(int(polls))
+
+
+def dasc_debug_refresh_form(n_req: int, units_per_req: int, total_tokens: int, max_seqlen: int, window: int = 0):
+    """Test hook: (form, thread blocks) of the chunked kernel for a call of these sizes; forms as in dasc.h."""
+    blocks = C.c_int64()
+    form = lib().dasc_debug_refresh_form(n_req, units_per_req, total_tokens, window, max_seqlen, C.byref(blocks))
+    return int(form), int(blocks.value)
 
 
 def dasc_refresh_static(plan: Plan, state: torch.Tensor, layer_stride: int, req_stride: int, req_idx: torch.Tensor,

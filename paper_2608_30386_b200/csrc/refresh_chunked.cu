@@ -1512,7 +1512,7 @@ Load load_of(const DascRefreshArgs &a) {
   const int64_t tokens = a.window > 0 ? std::min<int64_t>(a.total_tokens, static_cast<int64_t>(a.n_req) * a.window) : a.total_tokens;
   Load l;
   l.n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
-  l.longest = (std::max(a.max_seqlen, 1) + C - 1) / C;
+  l.longest = (std::max<int64_t>(a.max_seqlen, 1) + C - 1) / C;  // (any int32 is a legal bound)
   l.per_head = tokens / C + a.n_req / 2;
   l.chunks = l.per_head * a.n_layers_in_call * a.H_v;
   l.in_order = a.ordered || a.n_req == 1;
@@ -1549,7 +1549,7 @@ int launch(DascRefreshArgs a, void *stream) {
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
   a.ordered = ordered(a);
   const bool alone = alone_for(a);
-  const int64_t grid = alone ? n_units : grid_for(a);
+  const int64_t grid = alone ? n_units : grid_for(a);  // (dasc_debug_refresh_form answers the same)
   auto kern = alone ? refresh_chunked_kernel<KDA, OT, WITH_O, true, false>
               : grid < n_units ? refresh_chunked_kernel<KDA, OT, WITH_O, false, true> : refresh_chunked_kernel<KDA, OT, WITH_O, false, false>;
   const uint32_t smem = alone ? SMEM_ALONE : SMEM_BYTES;
@@ -1597,6 +1597,23 @@ size_t dasc_refresh_chunked_workspace_bytes(int32_t n_req, int32_t n_layers_in_c
 }
 
 uint32_t g_dasc_debug_poll_limit = 0;
+
+int32_t dasc_debug_refresh_form(int32_t n_req, int32_t units_per_req, int64_t total_tokens, int32_t window, int32_t max_seqlen,
+                                int64_t *n_blocks) {
+  DascRefreshArgs a{};
+  a.n_req = n_req;
+  a.n_layers_in_call = 1;
+  a.H_v = units_per_req;
+  a.total_tokens = total_tokens;
+  a.window = window;
+  a.max_seqlen = max_seqlen;
+  a.ordered = ordered(a);
+  const int64_t n_units = static_cast<int64_t>(n_req) * units_per_req;
+  const bool alone = alone_for(a);
+  const int64_t grid = alone ? n_units : grid_for(a);
+  if (n_blocks) *n_blocks = grid;
+  return alone ? 2 : grid < n_units ? 1 : 0;
+}
 
 // Returns a cudaError_t as int, or -1 if this kernel does not take the request
 // (it needs d_k = d_v = 128 and bf16 token streams).
