@@ -1537,12 +1537,11 @@ int64_t grid_for(const DascRefreshArgs &a) {
 // Measured, us, SHARED / ALONE, 256 tokens (GDN): 8 units 27.3 / 23.4 (23.6 / 21.7), 80 units 32.2 / 25.7 (24.0 / 22.3), 148 units 40.1 / 31.9
 // (32.7 / 28.6), state only 35.0 / 24.8; 148 units of 1 .. 599 tokens 72.5 / 60.0; 152 units 44.2 / 48.2 (35.5 / 43.4): the line is where a
 // second CTA per SM begins to be needed.
-// Up to twice as many units as well where one request is longer than an SM's share of all: they are placed longest first, and the
-// time is that request's.  SHARED / ALONE: 256 units of 1 .. 3801 tokens 376 / 317, 280 of 1 .. 1399 164 / 127, 192 of 1 .. 1199 125 / 94.
-bool alone_for(const DascRefreshArgs &a) {
-  const Load l = load_of(a);
-  return l.n_units <= kSms || (l.n_units <= kResident && l.in_order && l.chunks <= kSms * l.longest);
-}
+// Between 148 and 296 units ALONE would still be the better one where one request is longer than an SM's share of all (192 units of
+// 1 .. 1199 tokens 125 / 94, 256 of 1 .. 799 100 / 77), but the host knows only a bound on that length, and where the bound is loose and the
+// lengths are even ALONE loses: 152 units of 40 tokens 16.9 / 20.9 (GDN 15.6 / 19.2), 296 of 300 tokens 52.9 / 64.6 (42.6 / 55.9), windows
+// of 512 tokens over 256 prefixes of 100 24.3 / 27.5 (21.7 / 25.6).
+bool alone_for(const DascRefreshArgs &a) { return load_of(a).n_units <= kSms; }
 
 template <bool KDA, typename OT, bool WITH_O>
 int launch(DascRefreshArgs a, void *stream) {

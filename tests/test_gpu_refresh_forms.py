@@ -1,6 +1,5 @@
-"""The chunked kernel has two forms: up to 148 units, and up to 296 where one request is longer than an SM's share, a CTA has an SM
-to itself, with second buffers and more warps; above, two CTAs share one.  Both sides of the lines against the oracle, at
-lengths around the boundaries of chunks."""
+"""The chunked kernel has two forms: up to 148 units a CTA has an SM to itself, with second buffers and more warps; above, two CTAs
+share one.  Both sides of the line against the oracle, at lengths around the boundaries of chunks."""
 import pytest
 import torch
 
@@ -15,7 +14,7 @@ LENS = [9, 31, 32, 33, 63, 64, 65, 97, 128, 129, 0, 161, 193, 225, 257, 288, 47]
 
 
 @pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
-@pytest.mark.parametrize("n_req", [17, 37, 38, 75])  # x 4 heads: 68, 148, 152 and 300 units, the last in the form for two CTAs
+@pytest.mark.parametrize("n_req", [17, 37, 38, 75])  # x 4 heads: 68, 148, 152 and 300 units, the last two in the form for two CTAs
 def test_both_sides_of_the_lines(kind, n_req):
     lens = (LENS * 5)[:n_req]
     case = make_refresh_case(71, kind, 1, 4, 4 if kind == dasc.KDA else 2, 128, 128, lens, scope=dasc.SCOPE_LAYER, keep_ratio=0.4)
@@ -32,7 +31,7 @@ def test_both_sides_of_the_lines(kind, n_req):
 
 @pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
 def test_even_requests_just_above_an_sm_each(kind):
-    # 152 units of the same length: the form for two CTAs (a request is no longer than an SM's share)
+    # 152 units of the same length: the form for two CTAs
     case = make_refresh_case(72, kind, 1, 4, 4 if kind == dasc.KDA else 2, 128, 128, [95] * 38, scope=dasc.SCOPE_LAYER, keep_ratio=0.4)
     ref_s, ref_o = run_refresh_oracle(case)
     got_s, got_o = run_refresh_gpu(case)

@@ -10,3 +10,13 @@ OWN, WALK, ALONE = 0, 1, 2
 @pytest.mark.parametrize("n_req,units", [(80, 8), (300, 8), (128, 24)])
 def test_a_bound_that_says_nothing_gives_every_unit_a_block(bound, n_req, units):
     assert dasc.dasc_debug_refresh_form(n_req, units, n_req * 200, bound) == (OWN, n_req * units)
+
+
+@pytest.mark.parametrize("kind_of_call", ["bound x 1", "bound x 4", "bound x 1000", "window"])
+@pytest.mark.parametrize("tokens", [9, 40, 95, 100, 300, 1000])
+def test_above_an_sm_each_the_bound_does_not_decide_for_one_block_per_sm(kind_of_call, tokens):
+    # even lengths, which the host cannot tell from one long request among short ones by any upper bound
+    for n_req in range(38, 75):  # x 4 heads: 152 .. 296 units
+        window = 512 if kind_of_call == "window" else 0
+        bound = window or tokens * int(kind_of_call.split()[-1])
+        assert dasc.dasc_debug_refresh_form(n_req, 4, n_req * tokens, bound, window) == (OWN, n_req * 4)
