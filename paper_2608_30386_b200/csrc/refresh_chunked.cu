@@ -1512,7 +1512,7 @@ Load load_of(const DascRefreshArgs &a) {
   const int64_t tokens = a.window > 0 ? std::min<int64_t>(a.total_tokens, static_cast<int64_t>(a.n_req) * a.window) : a.total_tokens;
   Load l;
   l.n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
-  l.longest = (std::max<int64_t>(a.max_seqlen, 1) + C - 1) / C;  // (any int32 is a legal bound)
+  l.longest = (std::max<int64_t>(std::min<int64_t>(a.max_seqlen, tokens), 1) + C - 1) / C;  // (any int32 is a legal bound)
   l.per_head = tokens / C + a.n_req / 2;
   l.chunks = l.per_head * a.n_layers_in_call * a.H_v;
   l.in_order = a.ordered || a.n_req == 1;
@@ -1541,7 +1541,19 @@ int64_t grid_for(const DascRefreshArgs &a) {
 // 1 .. 1199 tokens 125 / 94, 256 of 1 .. 799 100 / 77), but the host knows only a bound on that length, and where the bound is loose and the
 // lengths are even ALONE loses: 152 units of 40 tokens 16.9 / 20.9 (GDN 15.6 / 19.2), 296 of 300 tokens 52.9 / 64.6 (42.6 / 55.9), windows
 // of 512 tokens over 256 prefixes of 100 24.3 / 27.5 (21.7 / 25.6).
-bool alone_for(const DascRefreshArgs &a) { return load_of(a).n_units <= kSms; }
+// Its 58,880 registers leave no room for a block of the copy kernels beside it (one CTA of SHARED leaves 33,280), so a Store on another stream
+// has the SMs without a unit, and where there are few waits for the refresh to end.  Hence ALONE for long requests only on half of
+// the SMs, else up to kWalkChunks chunks: like the CTAs of a walk they are gone after an eighth of a millisecond.  A Store of 16
+// checkpoints (85 us by itself) / the refresh it started with, us until each has ended, SHARED and ALONE:
+//   64 units of 4096 tokens 133 / 424, 155 / 290;   128 units 175 / 431, 335 / 332;   148 units 201 / 535, 420 / 420;   148 units of
+//   2048 tokens 199 / 290, 274 / 271 (GDN 193 / 222, 256 / 258), of 1024 tokens 176 / 179, 197 / 197 (GDN 156 / 154, 185 / 185).
+// With registers capped at 72 (one block fits) the Store still ended at 435 beside 148 units and the refresh by itself took 1 to 6 % longer;
+// at 64, spilling, 382 and 50 %.  Two launches on two streams share the SMs as well in SHARED: 2 x 148 units of 256 tokens 50 / 57
+// (2048 tokens 336 / 303), but 2 x 100 units 41 / 37, 2 x 72 39 / 29.
+bool alone_for(const DascRefreshArgs &a) {
+  const Load l = load_of(a);
+  return l.n_units <= kSms / 2 || (l.n_units <= kSms && l.longest <= kWalkChunks);
+}
 
 template <bool KDA, typename OT, bool WITH_O>
 int launch(DascRefreshArgs a, void *stream) {

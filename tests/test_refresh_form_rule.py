@@ -20,3 +20,13 @@ def test_above_an_sm_each_the_bound_does_not_decide_for_one_block_per_sm(kind_of
         window = 512 if kind_of_call == "window" else 0
         bound = window or tokens * int(kind_of_call.split()[-1])
         assert dasc.dasc_debug_refresh_form(n_req, 4, n_req * tokens, bound, window) == (OWN, n_req * 4)
+
+
+def test_long_requests_leave_half_of_the_sms_to_other_streams():
+    for units in (1, 32, 74):
+        assert dasc.dasc_debug_refresh_form(1, units, 1 << 20, 1 << 20) == (ALONE, units)
+    for units in (75, 128, 148):
+        assert dasc.dasc_debug_refresh_form(1, units, 2048, 2048) == (ALONE, units)
+        assert dasc.dasc_debug_refresh_form(1, units, 2049, 2049) == (OWN, units)
+        assert dasc.dasc_debug_refresh_form(1, units, 300, 1 << 30) == (ALONE, units)  # no request is longer than all tokens
+    assert dasc.dasc_debug_refresh_form(1, 149, 300, 300) == (OWN, 149)
