@@ -117,6 +117,8 @@ __device__ __forceinline__ void load_cols(float (&x)[COLS], const float *p) {
   if constexpr (COLS == 4) {
     const float4 v = *reinterpret_cast<const float4 *>(p);
     x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+  } else if constexpr (COLS == 1) {
+    x[0] = *p;
   } else {
     const float2 v = *reinterpret_cast<const float2 *>(p);
     x[0] = v.x; x[1] = v.y;
@@ -126,6 +128,8 @@ template <int COLS>
 __device__ __forceinline__ void store_cols(float *p, const float (&x)[COLS]) {
   if constexpr (COLS == 4)
     *reinterpret_cast<float4 *>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  else if constexpr (COLS == 1)
+    *p = x[0];
   else
     *reinterpret_cast<float2 *>(p) = make_float2(x[0], x[1]);
 }
@@ -509,6 +513,12 @@ template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, ty
 __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int unit, int part, unsigned char *smem_raw) {
   constexpr int NC = NCOL / COLS * SL;  // threads that replay tokens, COLS columns per SL lanes
   constexpr int NV = DK / SL / 4;  // groups of four rows held by one lane
+  // Looks at whether any tokens are left, ahead of so many of a group's later blocks: a call of a few tokens does not replay blocks of
+  // nothing.  128 tokens' worth of wide parts does not notice them, narrow ones lose the overlap of a block with the next
+  // (4 units of 64 x 64, 250 tokens 26.7 us without, 27.6 with all three; of 128 x 128 38.2 without, 38.2 with one, 38.7 with two).
+  // us for one token, without / with: 148 units of 64 x 64 7.0 / 4.4, 74 of 128 x 128 9.3 / 5.8 (5.3 with two columns per load and store of
+  // the state), 4 of them 4.8 / 4.0.
+  constexpr int CHECKS = DK * NCOL >= 2048 ? NB - 1 : DK * NCOL < 1024 ? 0 : DK == 32 ? 1 : 2;
   using Smem = BlockSmem<DK, NCOL, SL, IO, KDA>;
   constexpr int NRAW = Smem::NRAW;
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -571,8 +581,7 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
     typename Smem::Group &G = sm.grp[grp & 1];
     constexpr int PER = DK < NHELP / NB ? DK : NHELP / NB;  // threads of a block
     static_assert(PER % 32 == 0 && PER <= 64 && DK % PER == 0);
-    if (ht < NB * PER) {
-      const int b = ht / PER;
+    if (const int b = ht / PER; b < NB && min(b, CHECKS) * 4 < cnt) {  // (what will be replayed; a warp's threads are in one block)
       float x[16] = {};
       // products of decays, mostly as exponentials of sums: at most two of them multiplied instead of four
       float dd[4], a1, a2, a3, a12, a23, a13;
@@ -696,23 +705,29 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
   // row pairs (4 (i SL + slice) + 2p, + 1) of this lane's columns
   uint64_t S[COLS][NV][2];
 #pragma unroll
-  for (int e = 0; e < COLS; ++e)
+  for (int i = 0; i < NV; ++i)
 #pragma unroll
-    for (int i = 0; i < NV; ++i)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const float *row = st + (4 * (i * SL + slice) + 2 * p) * DV + col + e;
-        S[e][i][p] = a.mode == DASC_REFRESH_CONTINUE ? pack2(row[0], row[DV]) : 0ull;
+    for (int p = 0; p < 2; ++p) {
+      const float *row = st + (4 * (i * SL + slice) + 2 * p) * DV + col;
+      float x[COLS] = {}, y[COLS] = {};
+      if (a.mode == DASC_REFRESH_CONTINUE) {
+        load_cols<COLS>(x, row);
+        load_cols<COLS>(y, row + DV);
       }
+#pragma unroll
+      for (int e = 0; e < COLS; ++e) S[e][i][p] = pack2(x[e], y[e]);
+    }
   __syncthreads();
   for (int grp = 0; grp < n_grp; ++grp) {
     const int cnt = min(TB, n_tok - grp * TB);
     // one token group before the end: see launch.cuh
     if (grp + 1 == n_grp) stream_order_release();
     typename Smem::Group &G = sm.grp[grp & 1];
-    // straight code for the whole group (tokens past its end are zeros), so that the outputs of a block fill the waits of the next one
+    // straight code for the whole group but for CHECKS (tokens past its end are zeros), so that the outputs of a block fill the waits of the
+    // next one
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
+      if (b > 0 && b <= CHECKS && b * 4 >= cnt) break;
       ulonglong2 k[4][NV], w[4][NV], d[NV];
       auto load = [&](ulonglong2(&x)[NV], const float *row) {
 #pragma unroll
@@ -817,18 +832,17 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
   const uint8_t *keep = a.row_keep + static_cast<int64_t>(layer) * a.rows_per_layer + static_cast<int64_t>(h) * DK;
   const bool all_rows = a.mode == DASC_REFRESH_CONTINUE;
 #pragma unroll
-  for (int e = 0; e < COLS; ++e)
+  for (int i = 0; i < NV; ++i)
 #pragma unroll
-    for (int i = 0; i < NV; ++i)
+    for (int p = 0; p < 2; ++p) {
+      const int row = 4 * (i * SL + slice) + 2 * p;
+      float lo[COLS], hi[COLS];
 #pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const int row = 4 * (i * SL + slice) + 2 * p;
-        float lo, hi;
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(S[e][i][p]));
-        float *d = st + row * DV + col + e;
-        if (all_rows || !keep[row]) d[0] = lo;
-        if (all_rows || !keep[row + 1]) d[DV] = hi;
-      }
+      for (int e = 0; e < COLS; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(lo[e]), "=f"(hi[e]) : "l"(S[e][i][p]));
+      float *d = st + row * DV + col;
+      if (all_rows || !keep[row]) store_cols<COLS>(d, lo);
+      if (all_rows || !keep[row + 1]) store_cols<COLS>(d + DV, hi);
+    }
 }
 
 template <int DK, int DV, int NCOL, int COLS, int SL, int NHELP, typename IO, typename OT, bool KDA>
@@ -880,8 +894,11 @@ int dispatch_split(const DascRefreshArgs &a, void *stream) {
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
   const auto fits = [&](int parts, int64_t ctas) { return !a.from_list && n_units * parts <= ctas; };
   if constexpr (D == 32) {
-    if (fits(2, kSms)) return launch_blocks<32, 32, 16, 1, 4, 256, IO, OT, KDA>(a, stream);
-    if (fits(1, 2 * kSms)) return launch_blocks<32, 32, 32, 1, 4, 256, IO, OT, KDA>(a, stream);
+    // A few tokens end sooner without helper warps and groups of 16: us for 1 / 5 / 16 / 24 tokens, 296 units 7.3 / 7.5 / 7.8 / 10.9 in blocks,
+    // 3.9 / 4.7 / 6.9 / 9.1 token by token (64: 17.6, 19.1); 148 units 4.0 / 4.1 / 4.2 / 5.9 and 3.8 / 3.9 / 6.0 / 7.8.
+    const bool few = a.max_seqlen <= (n_units > kSms ? 24 : 5);
+    if (!few && fits(2, kSms)) return launch_blocks<32, 32, 16, 1, 4, 256, IO, OT, KDA>(a, stream);
+    if (!few && fits(1, 2 * kSms)) return launch_blocks<32, 32, 32, 1, 4, 256, IO, OT, KDA>(a, stream);
     return launch<32, 32, 2, 8, 0, IO, OT, KDA>(a, stream);
   } else if constexpr (D == 64) {
     if (fits(8, kSms)) return launch_blocks<64, 64, 8, 1, 8, 256, IO, OT, KDA>(a, stream);

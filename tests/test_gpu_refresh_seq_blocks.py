@@ -36,3 +36,17 @@ def test_bf16_streams_and_outputs(kind, dim):
     assert_refresh_close(case, got_s, got_o, ref_s, ref_o, 1e-5)
     _, got_b = run_refresh_gpu(case, algo=dasc.ALGO_SEQUENTIAL, o_dtype=torch.bfloat16)
     assert torch.equal(torch.from_numpy(got_o).to(torch.bfloat16).float(), torch.from_numpy(got_b))
+
+
+# Calls of a few tokens: blocks of a group that have none are left out in the wider parts, so nothing that lies in their place may be
+# read.  Every length up to a group and one over, behind a long request (whose blocks were in the same buffers) and alone
+@pytest.mark.parametrize("kind", [dasc.KDA, dasc.GDN])
+@pytest.mark.parametrize("dim,heads", [(32, 2), (32, 37), (32, 74), (64, 2), (64, 8), (64, 18), (64, 36), (128, 2), (128, 4), (128, 8), (128, 18)])
+@pytest.mark.parametrize("lens", [[1, 4], [5, 8], [9, 12], [13, 16], [16 + 1, 16 + 4], [32 + 5, 32 + 9], [2, 26], [1, 1]])
+def test_calls_of_a_few_tokens(kind, dim, heads, lens):
+    case = make_refresh_case(83, kind, 1, heads, heads // 2 if heads % 2 == 0 else heads, dim, dim, lens, io_dtype=torch.float32,
+                             scope=dasc.SCOPE_LAYER, keep_ratio=0.5)
+    ref_s, ref_o = run_refresh_oracle(case)
+    for _ in range(2):
+        got_s, got_o = run_refresh_gpu(case, algo=dasc.ALGO_SEQUENTIAL)
+        assert_refresh_close(case, got_s, got_o, ref_s, ref_o, 1e-5)
