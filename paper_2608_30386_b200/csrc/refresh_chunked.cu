@@ -1496,10 +1496,12 @@ EncodeTiledFn encode_tiled_fn() {
 //  - requests that are not in order of length (more than kRefreshOrderMax): only if they are about equally long.
 //  - up to two units per CTA, taken there and back, are what blocks of a unit each would come to as well (the shortest of the first G
 //    with the longest of the rest), whatever the lengths, so only the start of the second one is saved; but the CTAs that have one
-//    unit pay 1 to 4 % for the walk.  Hence from 1.4 units per CTA on (1.3 with short requests), where lengths differ.  us, a CTA per unit /
-//    walked, requests of 1 .. 2 n - 1 tokens, KDA: 424 units, n = 56 40.7 / 37.8, n = 300 94.8 / 90.5, 480 units, n = 128 63.9 / 59.6, n = 600 195 /
+//    unit pay 1 to 4 % for the walk.  Hence from 1.5 units per CTA on (1.3 with short requests), where lengths differ.  us, a CTA per unit /
+//    walked, requests of 1 .. 2 n - 1 tokens, KDA: 424 units, n = 56 40.7 / 37.8, 480 units, n = 128 63.9 / 59.6, n = 600 195 /
 //    170, 592 units, n = 128 75.8 / 68.8, n = 1000 361 / 322 (GDN 286 / 259); 392 units, n = 56 39.9 / 35.8 but n = 1000 233 / 247; 344 units 2 % more.
-//    Of 108 such launches at 424 .. 576 units ten lost, two of them more than 1 % (1.8, 9).  Equal lengths: 392 units GDN of 300 tokens 65.5 / 75.5.
+//    By the bound alone lengths may differ where they are equal, and with 1.4 units per CTA equal long ones lose: bounds of twice the
+//    length, 424 units of 700 tokens 170 / 190 (GDN 128 / 147), 448 of 700 192.5 / 193.5 (150 / 149), 464 of 300 99.2 / 98.2; short ones at most
+//    7 %: 388 units of 95 tokens 35.1 / 35.1 (28.3 / 30.4), 412 of 40 27.8 / 26.7 (23.3 / 24.1).
 constexpr int64_t kSms = 148, kResident = 2 * kSms, kWalkChunks = 64;
 
 // What the host knows of a launch: the longest request (by the caller's bound) and all units together, in chunks (about: half a one
@@ -1524,7 +1526,7 @@ int64_t grid_for(const DascRefreshArgs &a) {
   const int64_t g = kResident * std::max<int64_t>((l.chunks + kResident * kWalkChunks - 1) / (kResident * kWalkChunks),
                                                   (l.n_units + kResident * kMaxWalk - 1) / (kResident * kMaxWalk));
   const bool even = l.in_order ? l.longest * 2 * g <= l.chunks : l.longest * a.n_req * 9 <= l.per_head * 10;
-  const bool two = l.in_order && l.n_units <= 2 * kResident && l.n_units * 10 >= kResident * (l.longest * 4 <= kWalkChunks ? 13 : 14) &&
+  const bool two = l.in_order && l.n_units <= 2 * kResident && l.n_units * 10 >= kResident * (l.longest * 4 <= kWalkChunks ? 13 : 15) &&
                    l.longest <= kWalkChunks && l.longest * a.n_req * 2 >= l.per_head * 3;
   return (even || two) && g < l.n_units ? g : l.n_units;
 }

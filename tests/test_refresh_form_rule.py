@@ -30,3 +30,9 @@ def test_long_requests_leave_half_of_the_sms_to_other_streams():
         assert dasc.dasc_debug_refresh_form(1, units, 2049, 2049) == (OWN, units)
         assert dasc.dasc_debug_refresh_form(1, units, 300, 1 << 30) == (ALONE, units)  # no request is longer than all tokens
     assert dasc.dasc_debug_refresh_form(1, 149, 300, 300) == (OWN, 149)
+
+
+@pytest.mark.parametrize("tokens", [300, 700, 1000])
+def test_a_bound_of_twice_the_length_does_not_make_blocks_walk_where_that_could_lose(tokens):
+    for n_req, form in ((104, OWN), (106, OWN), (110, OWN), (111, WALK), (120, WALK), (148, WALK)):  # x 4 heads: 416 .. 592 units
+        assert dasc.dasc_debug_refresh_form(n_req, 4, n_req * tokens, 2 * tokens)[0] == form
