@@ -581,7 +581,7 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
     typename Smem::Group &G = sm.grp[grp & 1];
     constexpr int PER = DK < NHELP / NB ? DK : NHELP / NB;  // threads of a block
     static_assert(PER % 32 == 0 && PER <= 64 && DK % PER == 0);
-    if (const int b = ht / PER; b < NB && min(b, CHECKS) * 4 < cnt) {  // (what will be replayed; a warp's threads are in one block)
+    if (const int b = ht / PER; b < NB && (CHECKS == 0 || min(b, CHECKS) * 4 < cnt)) {  // (what will be replayed; a warp's threads are in one block)
       float x[16] = {};
       // products of decays, mostly as exponentials of sums: at most two of them multiplied instead of four
       float dd[4], a1, a2, a3, a12, a23, a13;
