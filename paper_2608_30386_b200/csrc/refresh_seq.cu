@@ -117,8 +117,6 @@ __device__ __forceinline__ void load_cols(float (&x)[COLS], const float *p) {
   if constexpr (COLS == 4) {
     const float4 v = *reinterpret_cast<const float4 *>(p);
     x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-  } else if constexpr (COLS == 1) {
-    x[0] = *p;
   } else {
     const float2 v = *reinterpret_cast<const float2 *>(p);
     x[0] = v.x; x[1] = v.y;
@@ -709,13 +707,17 @@ __device__ __forceinline__ void seq_unit_blocks(const DascRefreshArgs &a, int un
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
       const float *row = st + (4 * (i * SL + slice) + 2 * p) * DV + col;
-      float x[COLS] = {}, y[COLS] = {};
-      if (a.mode == DASC_REFRESH_CONTINUE) {
-        load_cols<COLS>(x, row);
-        load_cols<COLS>(y, row + DV);
-      }
+      if constexpr (COLS == 1) {  // (as below it took 0.07 us of the 8.7 us of 4 units of 64 x 64, 64 tokens)
+        S[0][i][p] = a.mode == DASC_REFRESH_CONTINUE ? pack2(row[0], row[DV]) : 0ull;
+      } else {
+        float x[COLS] = {}, y[COLS] = {};
+        if (a.mode == DASC_REFRESH_CONTINUE) {
+          load_cols<COLS>(x, row);
+          load_cols<COLS>(y, row + DV);
+        }
 #pragma unroll
-      for (int e = 0; e < COLS; ++e) S[e][i][p] = pack2(x[e], y[e]);
+        for (int e = 0; e < COLS; ++e) S[e][i][p] = pack2(x[e], y[e]);
+      }
     }
   __syncthreads();
   for (int grp = 0; grp < n_grp; ++grp) {
