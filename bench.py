@@ -52,8 +52,8 @@ CHUNKED_FLOPS_PER_TOKEN_HEAD = 180224   # tf32 flops the chunked kernel issues p
 # algorithmic write bytes for all three kernels).  profiles/traffic_kda_serving.md has the numbers.
 NCU_CAPTURE = {  # kernel: (dram__bytes_read.sum, lts__t_sectors_srcunit_tex_op_write.sum, algorithmic bytes of that launch)
     "pack": (153370624, 4783104, 306118656),
-    "restore": (153463296, 12582912, 555712512),
-    "refresh_chunked": (1412594688, 18874368, 2016411648),
+    "restore": (153511168, 12582912, 555712512),
+    "refresh_chunked": (1413344000, 18874368, 2016411648),
 }
 NCU_TRAFFIC_OVER_ALGORITHMIC = {k: (rd + 32 * wr) / alg for k, (rd, wr, alg) in NCU_CAPTURE.items()}
 

@@ -376,7 +376,9 @@ dasc_status_t dasc_restore_int8(const dasc_plan_t *plan, const void *pool_base,
  *   cu_seqlens DEVICE int32[n_req+1], ascending from 0: request r owns tokens
  *          [cu_seqlens[r], cu_seqlens[r+1]) of every layer; empty ranges are allowed.
  *   req_idx    DEVICE int32[n_req]: which dense state each request updates (distinct).
- *   max_seqlen an upper bound on any request's token count (sizes the launch).
+ *   max_seqlen an upper bound on any request's token count.  It does not limit what is
+ *          replayed; it helps to pick the kernel's form, so a tight bound can be faster (a
+ *          loose one leaves calls of many short requests without the form made for them).
  *
  * mode CONTINUE: S_0 is the state as stored (for instance just restored);
  *   every unit is written back.  This continues the recurrence.
@@ -410,7 +412,8 @@ dasc_status_t dasc_restore_int8(const dasc_plan_t *plan, const void *pool_base,
  *   NULL when that size is 0.
  * Errors: bad arguments -> no launch.  A bounded device-side wait that runs
  *   out sets the first header word (DASC_ERR_TIMEOUT): the CTA that gave up
- *   skips the rest of its work and leaves its unit's stored state untouched.
+ *   skips the rest of its work and leaves the stored states of the unit it was
+ *   replaying, and of those it had yet to replay, untouched.
  *   Read the flags with dasc_refresh_status after synchronising the stream.
  */
 dasc_status_t dasc_refresh_workspace_bytes(const dasc_plan_t *plan, int32_t n_req, int32_t n_layers_in_call,
@@ -434,9 +437,10 @@ dasc_status_t dasc_refresh_status(const void *workspace, size_t workspace_bytes)
 dasc_status_t dasc_refresh_counters(const void *workspace, size_t workspace_bytes, int32_t *handed_over,
                                     int32_t *replayed_exactly);
 /* Test hook, not for production use: when `polls` != 0 the chunked kernel's
- * issuing warp gives its very first wait of every CTA only that many polls, so
- * that a test can watch a bounded wait run out (DASC_ERR_TIMEOUT, the unit left
- * unwritten, the context still usable).  0 restores the normal limit.  Process-wide. */
+ * issuing warp begins every CTA with a wait of only that many polls, for tiles
+ * that cannot be there yet, so that a test can watch a bounded wait run out
+ * (DASC_ERR_TIMEOUT, its units left unwritten, the context still usable).
+ * 0 restores the normal limit.  Process-wide. */
 void dasc_debug_set_refresh_poll_limit(uint32_t polls);
 /* Test hook: the form of the chunked kernel that a call of these sizes gets, so that a test can say which
  * one it is about.  units_per_req = layers in the call x value heads; window and max_seqlen as the kernel sees

@@ -27,11 +27,11 @@
 // MMA1 has; MMA5 contracts over the tokens and reads Kh as an MN-major operand from a second tile (tf32
 // MN-major operands have a swizzle of their own), which, read last, is double-buffered by chunk parity.
 //
-// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1058 us = 1.98 G token-heads/s = 62 % of the
-// rate at which HBM could bring its bytes (657 us), GDN 824 us = 2.54 G (50 %); 1685 and 1630 us in the form this one grew from, 1090 and
+// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1035 us = 2.03 G token-heads/s = 63 % of the
+// rate at which HBM could bring its bytes (657 us), GDN 816 us = 2.57 G (50 %); 1685 and 1630 us in the form this one grew from, 1090 and
 // 885 with a CTA per unit.  What is nearest its limit is the SM's shared-memory data pipe (load/store units and the tensor core's operand
-// reads together): per chunk and SM (two CTAs) KDA takes 4.2 k cycles, of which that pipe is busy 81 %, the issue slots 52 %, the tensor
-// pipe 37 %; GDN 3.3 k, 93 %, 48 %, 43 %; the state-only form 3.6 k at 2 to 4 chunks per unit, 74 %, 53 %, 33 %.  A CTA alone
+// reads together): per chunk and SM (two CTAs) KDA takes 4.1 k cycles, of which that pipe is busy 83 %, the issue slots 51 %, the tensor
+// pipe 38 %; GDN 3.2 k, 95 %, 48 %, 44 %; the state-only form 3.5 k at 2 to 4 chunks per unit, 76 %, 52 %, 34 %.  A CTA alone
 // on its SM is bound by its chain of hand-offs: a chunk every 3.8 k cycles (GDN 3.5 k) in the form made for it (see alone_for), 4.8 k
 // in the other.
 // What it was before, in the order in which it was found: 103 cycles of issue per tensor-core instruction (behind
@@ -139,8 +139,8 @@ struct Misc {
   // producer -> issuing warp: the tiles of a chunk are ready (per warp: 4 arrivals; KDA one more from the triangular warp, for beta)
   uint64_t rdy_prep[2];  // (ALONE: by chunk parity)
   // producer -> chain warps: the state factors of a chunk are ready (KDA per warp: 4 arrivals; GDN the first warp only: 1)
-  // One barrier per chunk parity: the producer may hand over the factors of chunk n+1 before the chain warps
-  // have waited for those of chunk n, and a single barrier cannot tell phases two apart.
+  // One barrier per chunk parity (ALONE: by chunk index mod 4): the producer may hand over the factors of chunk n+1 (n+3) before the chain
+  // warps have waited for those of chunk n, and a single barrier cannot tell phases two apart.
   uint64_t rdy_fac[4];
   // chain warps -> issuing warp (per warp: 8 arrivals each)
   uint64_t rdy_state, rdy_half, rdy_rhs, rdy_u;  // (rdy_half, ALONE: the first half of the state's channels)
@@ -1488,7 +1488,8 @@ EncodeTiledFn encode_tiled_fn() {
 // Measured, us, a CTA per unit / this rule (KDA unless GDN): 4096 units of 1 .. 128 tokens, state only 253 / 223; 8192 of 64 tokens, state
 // only 379 / 309; 7680 of 16 tokens, state only 255 / 182; 8192 of 256 tokens 1128 / 1090 (GDN 1007 / 956).
 // Where the lines lie:
-//  - at most kWalkChunks chunks per CTA (a quarter of a millisecond): work of other streams is placed when CTAs end.  One grid of
+//  - kWalkChunks chunks per CTA on average, by the estimate of Load (a quarter of a millisecond; lengths just above a multiple of a chunk, or
+//    uneven ones, can give a CTA half as many more): work of other streams is placed when CTAs end.  One grid of
 //    resident CTAs, whatever they have to do, gains nothing more where there are more chunks than that (1365, GDN 1101).
 //  - no request longer than half of a CTA's share by the caller's bound, since here a CTA's units are fixed beforehand, while blocks of
 //    a unit each go to whichever CTA ends first: 2048 units of 1 .. 1023 tokens take 669 / 658 walked, 1600 of 1 .. 1199 596 / 601: little
@@ -1535,7 +1536,7 @@ int64_t grid_for(const DascRefreshArgs &a) {
 // the chain what need not be on it: producers with twice the warps, running up to two chunks ahead of the chain into second (MN-major Kh:
 // fourth) buffers; MMA1, the copies of the inputs, P and the outputs in warps of their own (one warp that issued all products was busy all of
 // the time: 100 to 120 cycles per barrier, 40 per product); MMA2 started on the first half of the scaled state; the state's product ahead of
-// the outputs'.  A chunk takes 3.8 k cycles instead of 4.8 k (GDN 3.5 k, 4.5 k), from cold inputs 4.0 k instead of 5.6 k.
+// the outputs'.  A chunk takes 3.8 k cycles instead of 4.8 k (GDN 3.5 k, 4.5 k), from cold inputs instead of 5.6 k.
 // Measured, us, SHARED / ALONE, 256 tokens (GDN): 8 units 27.3 / 23.4 (23.6 / 21.7), 80 units 32.2 / 25.7 (24.0 / 22.3), 148 units 40.1 / 31.9
 // (32.7 / 28.6), state only 35.0 / 24.8; 148 units of 1 .. 599 tokens 72.5 / 60.0; 152 units 44.2 / 48.2 (35.5 / 43.4): the line is where a
 // second CTA per SM begins to be needed.
