@@ -361,7 +361,11 @@ __device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
 // output product are left out.
 // WALK = false: one unit per CTA, known at compile time (grid_for left the grid at that; always so where ALONE): the bookkeeping between
 // units costs 1 to 4 % of a chunk where there is none to do.
-template <bool KDA, typename OT, bool WITH_O, bool ALONE, bool WALK>
+// ZERO: the merge mode, whose units start from zero.  Their first chunk, one of about three in a window of 128 tokens, needs no state pass and no
+// product 2, and its product 5 replaces what the accumulator holds.  32 requests of 1 .. 128 tokens x 4 layers x 32 heads, KDA: 204.8 -> 200.1,
+// 199.3 -> 188.2 us (two runs).  For calls without outputs, the load policy's, and at compile time: as flags in the issuing warp's loop it cost
+// every other call 1 to 3 %.
+template <bool KDA, typename OT, bool WITH_O, bool ALONE, bool WALK, bool ZERO>
 __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunked_kernel(const __grid_constant__ DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
                                                                 const __grid_constant__ CUtensorMap tmap_k,
                                                                 const __grid_constant__ CUtensorMap tmap_v,
@@ -617,8 +621,15 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     // =========================== tensor-core issue warp ===========================
     // The whole warp walks the chunks and waits; an elected lane issues.
     if (!ALONE) first_wait();
+    int left = 0, next_u = 0;  // ZERO: chunks left of the unit; the unit behind it
     for (int n = 0; n < all_chunks; ++n) {
       const uint32_t par = n & 1;
+      bool zero = false;  // this chunk's start state is zero, and nothing has been written where it would be
+      if (ZERO) {
+        zero = left == 0;
+        if (zero) left = (uni(units[next_u++].n_tok) + C - 1) / C;
+        --left;
+      }
       if (!ALONE) {
         mma1(n);
         take_a(n);
@@ -637,13 +648,13 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
         wait_bar(&misc->bar_ap[buf(n)], phase(n), misc);  // the tiles of this chunk are there: the warp that issued MMA1 has waited for them
         wait_bar(&misc->rdy_half, par, misc);
         tc_fence_after_sync();
-        if (elect_one()) mma2(0, 2);
+        if (!zero && elect_one()) mma2(0, 2);
         __syncwarp();
       }
       wait_bar(&misc->rdy_state, par, misc);
       tc_fence_after_sync();
       if (elect_one()) {
-        mma2(ALONE ? 2 : 0, 4);
+        if (!zero) mma2(ALONE ? 2 : 0, 4);
         mma_commit(&misc->bar_ro[buf(n)]);
       }
       __syncwarp();
@@ -673,16 +684,16 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
             mma_ts(tm + col_ro(n) + 32, tm + u_t + kk * 8, desc_kmajor(sbase + OFF_PM + kk * 32), ID_N32, true);
         }
       };
-      auto mma5 = [&](uint32_t u_t) {
+      auto mma5 = [&](uint32_t u_t, bool add) {
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          mma_ts(tm + COL_S, tm + u_t + kk * 8, desc_mn32(sbase + off_kht(n) + kk * 1024, 32 * 128), ID_N128_MN, true);
+          mma_ts(tm + COL_S, tm + u_t + kk * 8, desc_mn32(sbase + off_kht(n) + kk * 1024, 32 * 128), ID_N128_MN, add || kk != 0);
       };
       wait_bar(&misc->bar_u, par, misc);
       tc_fence_after_sync();
       if (elect_one()) {
         if (!ALONE) mma4(COL_U<ALONE>);
-        mma5(COL_U<ALONE>);
+        mma5(COL_U<ALONE>, !zero);
       }
       __syncwarp();
       // MMA4 (low), MMA5 (low): the same with U_lo^T, which the chain warps wrote over the consumed RHS^T
@@ -690,14 +701,14 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       tc_fence_after_sync();
       if (elect_one()) {
         if (ALONE) {
-          mma5(col_ro(n));
+          mma5(col_ro(n), true);
           mma_commit(&misc->bar_s[par]);
           mma4(COL_U<ALONE>);
         }
         mma4(col_ro(n));
         if (WITH_O || !ALONE) mma_commit(&misc->bar_o);  // (only where someone waits for it: an arrival must not outlive the CTA)
         if (!ALONE) {
-          mma5(col_ro(n));
+          mma5(col_ro(n), true);
           mma_commit(&misc->bar_s[par]);
         }
       }
@@ -1189,7 +1200,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       OT *go = WITH_O ? static_cast<OT *>(a.o) + (x.tok0 * a.H_v + x.head) * D : nullptr;
       if (WITH_O && sizeof(OT) == 2) go += (tid >> 4) * v_stride + (tid & 15) * 8;
       const int n_tok = uni(x.n_tok), n_chunks = (n_tok + C - 1) / C;
-      if (n_chunks > 0) {
+      if (!ZERO && n_chunks > 0) {
         // the start state goes into TMEM as it is; the first chunk's state pass scales it like any other.  (The state of the unit
         // before has been read out by the same threads.)
 #pragma unroll 1
@@ -1197,7 +1208,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
           const int c0 = col_block(i);
           const float *const st_c = a.state + x.state + (c0 * D + vrow);
           uint32_t s[32];
-          if (a.mode == DASC_REFRESH_CONTINUE) {
+          if (!ZERO && a.mode == DASC_REFRESH_CONTINUE) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) s[j] = __float_as_uint(st_c[j * D]);
           } else {
@@ -1221,7 +1232,12 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
         tc_fence_after_sync();
 
         // ---- (2) state pass (columns = channels, half of them per warp): scale the state to this chunk's midpoint ----
-        {
+        if (ZERO && ch == 0) {
+          if (ALONE) {
+            tc_fence_before_sync();
+            arrive_warp(&misc->rdy_half, lane);
+          }
+        } else {
           if constexpr (ALONE) {
             // channels 0-63 first: MMA2 starts on them while 64-127 are scaled
             uint32_t s[2][2][16];
@@ -1302,6 +1318,10 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
 #pragma unroll
           for (uint32_t hh = 0; hh < 2; ++hh) tmem_ld_16x256b(tlane + (hh << 20) + col_ro(n) + tb, xx[hh]);
           tmem_ld_wait();
+          if (ZERO && ch == 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) xx[0][i] = xx[1][i] = 0u;  // no product 2
+          }
 #pragma unroll
           for (uint32_t hh = 0; hh < 2; ++hh) {
             uint32_t(&x)[8] = xx[hh], (&vv)[4] = vvv[hh], lo[8];
@@ -1558,14 +1578,15 @@ bool alone_for(const DascRefreshArgs &a) {
   return l.n_units <= kSms / 2 || (l.n_units <= kSms && l.longest <= kWalkChunks);
 }
 
-template <bool KDA, typename OT, bool WITH_O>
+template <bool KDA, typename OT, bool WITH_O, bool ZERO = false>
 int launch(DascRefreshArgs a, void *stream) {
   const int64_t n_units = static_cast<int64_t>(a.n_req) * a.n_layers_in_call * a.H_v;
   a.ordered = ordered(a);
   const bool alone = alone_for(a);
   const int64_t grid = alone ? n_units : grid_for(a);  // (dasc_debug_refresh_form answers the same)
-  auto kern = alone ? refresh_chunked_kernel<KDA, OT, WITH_O, true, false>
-              : grid < n_units ? refresh_chunked_kernel<KDA, OT, WITH_O, false, true> : refresh_chunked_kernel<KDA, OT, WITH_O, false, false>;
+  auto kern = alone ? refresh_chunked_kernel<KDA, OT, WITH_O, true, false, ZERO>
+              : grid < n_units ? refresh_chunked_kernel<KDA, OT, WITH_O, false, true, ZERO>
+                               : refresh_chunked_kernel<KDA, OT, WITH_O, false, false, ZERO>;
   const uint32_t smem = alone ? SMEM_ALONE : SMEM_BYTES;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return static_cast<int>(e);
@@ -1636,6 +1657,8 @@ int dasc_launch_refresh_chunked(const DascRefreshArgs &a_in, void *stream) {
   DascRefreshArgs a = a_in;
   a.poll_limit_first_wait = __atomic_load_n(&g_dasc_debug_poll_limit, __ATOMIC_RELAXED);
   const bool kda = a.kind == DASC_KDA;
+  if (!a.o && a.mode == DASC_REFRESH_SCRATCH_MERGE_LOCAL)
+    return kda ? launch<true, __nv_bfloat16, false, true>(a, stream) : launch<false, __nv_bfloat16, false, true>(a, stream);
   if (!a.o) return kda ? launch<true, __nv_bfloat16, false>(a, stream) : launch<false, __nv_bfloat16, false>(a, stream);
   if (a.o_bf16) return kda ? launch<true, __nv_bfloat16, true>(a, stream) : launch<false, __nv_bfloat16, true>(a, stream);
   return kda ? launch<true, float, true>(a, stream) : launch<false, float, true>(a, stream);
