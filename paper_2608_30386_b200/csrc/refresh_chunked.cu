@@ -72,7 +72,8 @@ struct Form {
   static constexpr int FAC = ALONE ? 4 : 2;              // state factors, by chunk index mod FAC
   static constexpr uint32_t TMEM_COLS = ALONE ? 512 : 256;
 };
-constexpr int LDX = 36;        // row pitch (floats) of the fp32 triangular work matrices
+// row pitches (floats) of the fp32 triangular work matrices: A^T (KDA) and X; -A (GDN)
+constexpr int LDX = 36, LDL = 40;
 
 // TMEM columns; RO: R^T 32 columns | (Qt S')^T 32; RL: the right-hand side's low part (SHARED: over the consumed A|P)
 constexpr uint32_t COL_S = 0, COL_AP = 128;
@@ -88,8 +89,8 @@ constexpr uint32_t OFF_KH = OFF_KHT + 2 * 128 * 128;    // [4][32 rows][128 B]  
 constexpr uint32_t OFF_TM = OFF_KH + 4 * 32 * 128;      // [1][32 rows][128 B]  T[t][i]; TM|PM later the bf16 O tile
 constexpr uint32_t OFF_PM = OFF_TM + 32 * 128;          // [1][32 rows][128 B]  P[t][i]
 constexpr uint32_t OFF_V = OFF_PM + 32 * 128;           // [2][32 rows][128 B] V[t][v] bf16
-constexpr uint32_t OFF_L = OFF_V + C * D * 2;           // [32][LDX] fp32 A^T (entries on and above A's diagonal are not used)
-constexpr uint32_t OFF_X = OFF_L + C * LDX * 4;         // [32][LDX] fp32 X = (I + A)^-1
+constexpr uint32_t OFF_L = OFF_V + C * D * 2;           // fp32 A^T [32][LDX], GDN -A [32][LDL] (entries on and above A's diagonal are not used)
+constexpr uint32_t OFF_X = OFF_L + C * LDL * 4;         // [32][LDX] fp32 X = (I + A)^-1
 constexpr uint32_t OFF_FAC = OFF_X + C * LDX * 4;       // [2][128] fp32 state factor per channel, by chunk parity
 constexpr uint32_t OFF_POST = OFF_FAC + 2 * D * 4;      // log-factor owed after a chunk: KDA [2][128] fp32 by chunk parity, GDN [4] by chunk index mod 4
 constexpr uint32_t OFF_BETA = OFF_POST + 2 * D * 4;     // [4][32] fp32, by chunk index mod 4 (written well ahead)
@@ -327,25 +328,30 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return w;
 }
 
-// Rows row0 .. row0 + 15 of A = strict_lower(Kt Kh^T) * beta out of tensor memory (`taddr`: first lane of the warp's quadrant),
-// transposed into LT.  KDA: the decay is inside the product, whose Kt rows carry the truncation compensation; `rowf` = beta.
-// GDN: the product is the raw k_t . k_j and the decay exp(G_t - G_j) = e1_t e2_j is applied here; `rowf` = beta e1, `colf` = e2.
+// Rows row0 .. row0 + 15 of A = strict_lower(Kt Kh^T) * beta out of tensor memory (`taddr`: first lane of the warp's quadrant).
+// KDA: transposed into L; the decay is inside the product, whose Kt rows carry the truncation compensation; `rowf` = beta.
+// GDN: -A into L; the product is the raw k_t . k_j and the decay exp(G_t - G_j) = e1_t e2_j is applied here; `rowf` = beta e1, `colf` = e2.
 template <bool KDA>
-__device__ __forceinline__ void take_a_rows(uint32_t taddr, int row0, const float *rowf, const float *colf, float *LT, int lane) {
+__device__ __forceinline__ void take_a_rows(uint32_t taddr, int row0, const float *rowf, const float *colf, float *L, int lane) {
   const int g = lane >> 2, tig = lane & 3;
   uint32_t x[16];
   tmem_ld_16x256b(taddr, x);
-  const float f0 = rowf[row0 + g] * (KDA ? kInvTruncComp : 1.f), f1 = rowf[row0 + g + 8] * (KDA ? kInvTruncComp : 1.f);
+  const float f0 = rowf[row0 + g] * (KDA ? kInvTruncComp : -1.f), f1 = rowf[row0 + g + 8] * (KDA ? kInvTruncComp : -1.f);
   tmem_ld_wait();
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    float2 e = make_float2(1.f, 1.f);
-    if constexpr (!KDA) e = *reinterpret_cast<const float2 *>(colf + 8 * i + 2 * tig);
-    float *d = LT + (8 * i + 2 * tig) * LDX + row0 + g;
-    d[0] = __uint_as_float(x[4 * i]) * (f0 * e.x);
-    d[LDX] = __uint_as_float(x[4 * i + 1]) * (f0 * e.y);
-    d[8] = __uint_as_float(x[4 * i + 2]) * (f1 * e.x);
-    d[LDX + 8] = __uint_as_float(x[4 * i + 3]) * (f1 * e.y);
+    if constexpr (KDA) {
+      float *d = L + (8 * i + 2 * tig) * LDX + row0 + g;
+      d[0] = __uint_as_float(x[4 * i]) * f0;
+      d[LDX] = __uint_as_float(x[4 * i + 1]) * f0;
+      d[8] = __uint_as_float(x[4 * i + 2]) * f1;
+      d[LDX + 8] = __uint_as_float(x[4 * i + 3]) * f1;
+    } else {
+      const uint64_t e = *reinterpret_cast<const uint64_t *>(colf + 8 * i + 2 * tig);
+      uint64_t *const d = reinterpret_cast<uint64_t *>(L + (row0 + g) * LDL + 8 * i + 2 * tig);
+      d[0] = mul2(pack2(__uint_as_float(x[4 * i]), __uint_as_float(x[4 * i + 1])), mul2(pack2(f0, f0), e));
+      d[4 * LDL] = mul2(pack2(__uint_as_float(x[4 * i + 2]), __uint_as_float(x[4 * i + 3])), mul2(pack2(f1, f1), e));
+    }
   }
 }
 
@@ -386,7 +392,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
   auto col_ap = [&](int n) { return COL_AP + buf(n) * 32; };
   auto col_ro = [&](int n) { return COL_RO<ALONE> + (ALONE ? static_cast<uint32_t>(n) % 3u * 64 : 0u); };
   constexpr uint32_t COL_RL = ALONE ? 416 : COL_AP, OFF_O = ALONE ? OFF_OUT_2 : OFF_TM;
-  float *LT = reinterpret_cast<float *>(smem + OFF_L);
+  float *Lm = reinterpret_cast<float *>(smem + OFF_L);
   float *Xm = reinterpret_cast<float *>(smem + OFF_X);
   float *fac_s = reinterpret_cast<float *>(smem + (ALONE ? OFF_FAC_2 : OFF_FAC));
   float *post_s = reinterpret_cast<float *>(smem + OFF_POST);
@@ -519,7 +525,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     wait_bar(&misc->bar_ap[buf(n)], phase(n), misc);
     if (ALONE && n > 0) wait_bar(&misc->rdy_rhs, (n - 1) & 1, misc);  // the triangular warp has read the chunk before's
     tc_fence_after_sync();
-    take_a_rows<KDA>(tm + (32u << 16) + col_ap(n), 16, (KDA ? beta_s : bte1_s) + (n % RING) * C, e2_s + (n % RING) * C, LT, lane);
+    take_a_rows<KDA>(tm + (32u << 16) + col_ap(n), 16, (KDA ? beta_s : bte1_s) + (n % RING) * C, e2_s + (n % RING) * C, Lm, lane);
     // A full barrier on both sides: after a time-out no wait below keeps this warp from the next chunk, and a second bare arrival of its own
     // would complete the barrier without the triangular warp, which would later wait for an arrival that never comes.
     asm volatile("bar.sync 3, 64;" ::: "memory");
@@ -773,56 +779,150 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       if (KDA && !ALONE && n + 1 < all_chunks) beta_next = fetch_beta();
       wait_bar(&misc->bar_ap[buf(n)], phase(n), misc);
       tc_fence_after_sync();
-      take_a_rows<KDA>(tm + col_ap(n), 0, (KDA ? beta_s : bte1_s) + (n % RING) * C, e2_s + (n % RING) * C, LT, lane);
+      take_a_rows<KDA>(tm + col_ap(n), 0, (KDA ? beta_s : bte1_s) + (n % RING) * C, e2_s + (n % RING) * C, Lm, lane);
       tc_fence_before_sync();
       asm volatile("bar.sync 3, 64;" ::: "memory");
       arrive_warp(&misc->a_taken, lane);  // the chain warps may reuse the A|P columns
-      // diagonal 16x16 blocks: lane (block b, column cc) solves (I + L_bb) x = e_cc, column by column: every row that a new
-      // entry of x acts on is updated at once, so the serial chain is one multiply-add per row
-      {
-        const int b = lane >> 4, cc = lane & 15;
-        const float *Lb = LT + (b * 16) * LDX + b * 16;
-        float xs[16];
+      // X = (I + A)^-1, then T, to its tf32 operand tile straight from the registers.  The tile's storage (shared with the P tile and the chain
+      // warps' output tile) is free once the chain warps have copied the previous chunk's outputs out.
+      auto storage_free = [&]() {
+        if (!ALONE && n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
+      };
+      // Where two CTAs share an SM T is the last operand of MMA3 to be ready, and how long it takes is this warp's count of instructions.  GDN
+      // by rows of X, some forty fewer than by columns (us, by columns / by rows: 152 units of 256 tokens 32.4 / 31.4, 296 of 300 40.5 / 39.1, 424 of
+      // 300 74.6 / 65.5, 296 of 1 .. 1999 157 / 152; ALONE: 148 of 512 43.2 / 41.2, 4 of 2000 116.8 / 115.5).  KDA by columns: by rows SHARED
+      // gained at most 2 %, and 148 units of 512 tokens went from 48.9 to 43.7, but calls of few units, whose other roles are not held up by
+      // memory, got slower, 4 of 2000 125.5 -> 131.1, 32 of 509 38.7 -> 39.6, wherever in the chunk this step was put.  In between, 8x8
+      // diagonal blocks and products of hi / lo pairs: KDA 4 of 2000 128.4, but GDN 152 of 256 33.2, 424 of 300 75.7.
+      if constexpr (KDA) {
+        // diagonal 16x16 blocks: lane (block b, column cc) solves (I + L_bb) x = e_cc, column by column: every row that a new
+        // entry of x acts on is updated at once, so the serial chain is one multiply-add per row
+        {
+          const int b = lane >> 4, cc = lane & 15;
+          const float *Lb = Lm + (b * 16) * LDX + b * 16;
+          float xs[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) xs[i] = i == cc ? 1.f : 0.f;
+          for (int i = 0; i < 16; ++i) xs[i] = i == cc ? 1.f : 0.f;
 #pragma unroll
-        for (int j = 0; j < 15; ++j) {
+          for (int j = 0; j < 15; ++j) {
 #pragma unroll
-          for (int r4 = (j + 1) / 4 * 4; r4 < 16; r4 += 4) {
-            const float4 l4 = *reinterpret_cast<const float4 *>(Lb + j * LDX + r4);
-            if (r4 + 0 > j) xs[r4 + 0] = fmaf(-l4.x, xs[j], xs[r4 + 0]);
-            if (r4 + 1 > j) xs[r4 + 1] = fmaf(-l4.y, xs[j], xs[r4 + 1]);
-            if (r4 + 2 > j) xs[r4 + 2] = fmaf(-l4.z, xs[j], xs[r4 + 2]);
-            if (r4 + 3 > j) xs[r4 + 3] = fmaf(-l4.w, xs[j], xs[r4 + 3]);
+            for (int r4 = (j + 1) / 4 * 4; r4 < 16; r4 += 4) {
+              const float4 l4 = *reinterpret_cast<const float4 *>(Lb + j * LDX + r4);
+              if (r4 + 0 > j) xs[r4 + 0] = fmaf(-l4.x, xs[j], xs[r4 + 0]);
+              if (r4 + 1 > j) xs[r4 + 1] = fmaf(-l4.y, xs[j], xs[r4 + 1]);
+              if (r4 + 2 > j) xs[r4 + 2] = fmaf(-l4.z, xs[j], xs[r4 + 2]);
+              if (r4 + 3 > j) xs[r4 + 3] = fmaf(-l4.w, xs[j], xs[r4 + 3]);
+            }
+          }
+#pragma unroll
+          for (int rr = 0; rr < 16; ++rr) Xm[(b * 16 + rr) * LDX + b * 16 + cc] = xs[rr];
+          __syncwarp();
+          // off-diagonal block: X_10 = -X_11 (L_10 X_00); the product L_10 X_00 is parked in the unused block (0,1)
+          float acc[2][4] = {};
+          warp_mm_acc<true>(acc, Lm + 16, Xm, lane);
+          warp_mm_store(Xm + 16, acc, 1.f, lane);
+          storage_free();
+#pragma unroll
+          for (int rr = 0; rr < 16; ++rr)
+            *reinterpret_cast<uint32_t *>(smem + off_t(n) + sw128_offset(32, b * 16 + rr, b * 16 + cc)) = tf32_pre(xs[rr]);
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            *reinterpret_cast<uint4 *>(smem + off_t(n) + sw128_offset(32, i * 8 + (lane >> 2), 16 + (lane & 3) * 4)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        __syncwarp();
+        {
+          float acc2[2][4] = {};
+          warp_mm_acc<false>(acc2, Xm + 16 * LDX + 16, Xm + 16, lane);
+          const int g = lane >> 2, tig = lane & 3;
+#pragma unroll
+          for (int nh = 0; nh < 2; ++nh) {
+            unsigned char *const p = smem + off_t(n) + sw128_offset(32, 16 + g, 8 * nh + 2 * tig);
+            *reinterpret_cast<uint2 *>(p) = make_uint2(tf32_pre(-acc2[nh][0]), tf32_pre(-acc2[nh][1]));
+            *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(tf32_pre(-acc2[nh][2]), tf32_pre(-acc2[nh][3]));
           }
         }
-#pragma unroll
-        for (int rr = 0; rr < 16; ++rr) Xm[(b * 16 + rr) * LDX + b * 16 + cc] = xs[rr];
-        __syncwarp();
-        // off-diagonal block: X_10 = -X_11 (L_10 X_00); the product L_10 X_00 is parked in the unused block (0,1)
-        float acc[2][4] = {};
-        warp_mm_acc<true>(acc, LT + 16, Xm, lane);
-        warp_mm_store(Xm + 16, acc, 1.f, lane);
-        // T -> tf32 operand tile, straight from the registers.  Its storage (shared with the P tile and the chain warps'
-        // output tile) is free once the chain warps have copied the previous chunk's outputs out.
-        if (!ALONE && n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
-#pragma unroll
-        for (int rr = 0; rr < 16; ++rr)
-          *reinterpret_cast<uint32_t *>(smem + off_t(n) + sw128_offset(32, b * 16 + rr, b * 16 + cc)) = tf32_pre(xs[rr]);
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-          *reinterpret_cast<uint4 *>(smem + off_t(n) + sw128_offset(32, i * 8 + (lane >> 2), 16 + (lane & 3) * 4)) = make_uint4(0u, 0u, 0u, 0u);
-      }
-      __syncwarp();
-      {
-        float acc2[2][4] = {};
-        warp_mm_acc<false>(acc2, Xm + 16 * LDX + 16, Xm + 16, lane);
+      } else {
+        // By rows: lane (block b, row i) solves x (I + A_bb) = e_i, from the diagonal down: all entries that a new one acts on are updated at
+        // once, in pairs, so the serial chain is one multiply-add per entry, and a lane's entries leave 16 bytes at a time.
         const int g = lane >> 2, tig = lane & 3;
+        {
+          const int b = lane >> 4, row = lane & 15;
+          const float *const Lb = Lm + (b * 16) * LDL + b * 16;
+          uint64_t x[8];
 #pragma unroll
-        for (int nh = 0; nh < 2; ++nh) {
-          unsigned char *const p = smem + off_t(n) + sw128_offset(32, 16 + g, 8 * nh + 2 * tig);
-          *reinterpret_cast<uint2 *>(p) = make_uint2(tf32_pre(-acc2[nh][0]), tf32_pre(-acc2[nh][1]));
-          *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(tf32_pre(-acc2[nh][2]), tf32_pre(-acc2[nh][3]));
+          for (int p = 0; p < 8; ++p) x[p] = pack2(2 * p == row ? 1.f : 0.f, 2 * p + 1 == row ? 1.f : 0.f);
+#pragma unroll
+          for (int k = 15; k > 0; --k) {
+            float lo, hi;
+            unpack2(x[k >> 1], lo, hi);
+            const float f = k & 1 ? hi : lo;
+            const uint64_t f2 = pack2(f, f);
+#pragma unroll
+            for (int j4 = 0; j4 < k; j4 += 4) {
+              const ulonglong2 l = *reinterpret_cast<const ulonglong2 *>(Lb + k * LDL + j4);
+#pragma unroll
+              for (int p = 0; p < 2; ++p) {
+                const int j = j4 + 2 * p;
+                const uint64_t l2 = p ? l.y : l.x;
+                if (j + 1 < k) {
+                  x[j >> 1] = fma2(f2, l2, x[j >> 1]);
+                } else if (j < k) {  // the pair of entry k itself: its first entry only
+                  float l0, l1;
+                  unpack2(l2, l0, l1);
+                  x[j >> 1] = pack2(fmaf(f, l0, lo), hi);
+                }
+              }
+            }
+          }
+          float xs[16];
+#pragma unroll
+          for (int p = 0; p < 8; ++p) unpack2(x[p], xs[2 * p], xs[2 * p + 1]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<float4 *>(Xm + lane * LDX + b * 16 + 4 * q) = make_float4(xs[4 * q], xs[4 * q + 1], xs[4 * q + 2], xs[4 * q + 3]);
+          storage_free();
+          const uint32_t t0 = sw128_offset(32, lane, b * 16);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<uint4 *>(smem + off_t(n) + (t0 ^ (q << 4))) =
+                make_uint4(tf32_pre(xs[4 * q]), tf32_pre(xs[4 * q + 1]), tf32_pre(xs[4 * q + 2]), tf32_pre(xs[4 * q + 3]));
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            *reinterpret_cast<uint4 *>(smem + off_t(n) + sw128_offset(32, i * 8 + (lane >> 2), 16 + (lane & 3) * 4)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        __syncwarp();
+        // off-diagonal block: X_10 = X_11 (-A_10 X_00).  The inner product transposed, and the contraction index of a slice of 8 taken as
+        // 2 tig, 2 tig + 1: its accumulators are then the outer product's second operand as they are.
+        {
+          float m[2][4] = {}, acc[2][4] = {};  // m[half of A_10's rows]: rows = columns of X_00, columns = rows of A_10
+#pragma unroll
+          for (int kh = 0; kh < 2; ++kh) {
+            const float *const x0 = Xm + (8 * kh + 2 * tig) * LDX + g;
+            const uint32_t af[4] = {tf32_pre(x0[0]), tf32_pre(x0[8]), tf32_pre(x0[LDX]), tf32_pre(x0[LDX + 8])};
+#pragma unroll
+            for (int rh = 0; rh < 2; ++rh) {
+              const float2 l10 = *reinterpret_cast<const float2 *>(Lm + (16 + 8 * rh + g) * LDL + 8 * kh + 2 * tig);
+              const uint32_t bf[2] = {tf32_pre(l10.x), tf32_pre(l10.y)};
+              mma_tf32_16x8x8(m[rh], af, bf);
+            }
+          }
+#pragma unroll
+          for (int kh = 0; kh < 2; ++kh) {
+            const float *const x1 = Xm + (16 + g) * LDX + 16 + 8 * kh + 2 * tig;
+            const float2 r0 = *reinterpret_cast<const float2 *>(x1), r1 = *reinterpret_cast<const float2 *>(x1 + 8 * LDX);
+            const uint32_t af[4] = {tf32_pre(r0.x), tf32_pre(r1.x), tf32_pre(r0.y), tf32_pre(r1.y)};
+#pragma unroll
+            for (int ch = 0; ch < 2; ++ch) {
+              const uint32_t bf[2] = {tf32_pre(m[kh][2 * ch]), tf32_pre(m[kh][2 * ch + 1])};
+              mma_tf32_16x8x8(acc[ch], af, bf);
+            }
+          }
+#pragma unroll
+          for (int ch = 0; ch < 2; ++ch) {
+            unsigned char *const p = smem + off_t(n) + sw128_offset(32, 16 + g, 8 * ch + 2 * tig);
+            *reinterpret_cast<uint2 *>(p) = make_uint2(tf32_pre(acc[ch][0]), tf32_pre(acc[ch][1]));
+            *reinterpret_cast<uint2 *>(p + 1024) = make_uint2(tf32_pre(acc[ch][2]), tf32_pre(acc[ch][3]));
+          }
         }
       }
       fence_smem_to_async();
