@@ -641,8 +641,10 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
         take_a(n);
       }
       // MMA2: S'^T [Kt;Qt]^T, the fp32 state read as a tf32 operand
+      // (GDN in ALONE unrolled by two: 4 units of 2000 tokens 115.2 -> 112.5 us, 32 of 509 35.1 -> 34.3, 148 of 512 41.1 -> 40.9.  KDA by four: 4 of 2000
+      // 126.4 -> 124.5, but 148 of 512 48.3 -> 49.1.  SHARED keeps its code small.)
       auto mma2 = [&](int kb_0, int kb_n) {
-#pragma unroll 1
+#pragma unroll ALONE && !KDA ? 2 : 1
         for (int kb = kb_0; kb < kb_n; ++kb) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
