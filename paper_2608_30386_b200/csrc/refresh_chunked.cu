@@ -734,7 +734,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     // ================================ triangular warp ================================
     // T = (I + A)^-1 depends on the token inputs only, so it is formed off the chain: rows 0-15 of A out of TMEM (this
     // warp's quadrant; the issuing warp brings rows 16-31), 16x16 diagonal blocks by fp32 substitution, the off-diagonal
-    // block by mma.sync products.
+    // block by mma.sync products.  (GDN: by rows of the inverse and from -A, KDA by its columns and from A^T: see below.)
     // This warp also starts the copies of V, a chunk ahead: two boxes of 32 tokens x 64 values with the 128-byte swizzle (no bank
     // conflicts for the 8 x 8 blocks it is read in).  Started by two of the chain warps they held those up for 280 cycles of every
     // chunk; here they fall into the wait for the next A (0.3 to 1 % of a launch).
