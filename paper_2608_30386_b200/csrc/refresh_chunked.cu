@@ -28,11 +28,11 @@
 // MN-major operands have a swizzle of their own), which, read last, is double-buffered by chunk parity.
 //
 // Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1035 us = 2.03 G token-heads/s = 63 % of the
-// rate at which HBM could bring its bytes (657 us), GDN 816 us = 2.57 G (50 %); 1685 and 1630 us in the form this one grew from, 1090 and
+// rate at which HBM could bring its bytes (657 us), GDN 816 us = 2.57 G (50 %; since then 2 % less); 1685 and 1630 us in the form this one grew from, 1090 and
 // 885 with a CTA per unit.  What is nearest its limit is the SM's shared-memory data pipe (load/store units and the tensor core's operand
 // reads together): per chunk and SM (two CTAs) KDA takes 4.1 k cycles, of which that pipe is busy 83 %, the issue slots 51 %, the tensor
-// pipe 38 %; GDN 3.2 k, 95 %, 48 %, 44 %; the state-only form 3.5 k at 2 to 4 chunks per unit, 76 %, 52 %, 34 %.  A CTA alone
-// on its SM is bound by its chain of hand-offs: a chunk every 3.8 k cycles (GDN 3.5 k) in the form made for it (see alone_for), 4.8 k
+// pipe 38 %; GDN 3.1 k, 97 %, 48 %, 46 %; the state-only form 3.4 k at 2 to 4 chunks per unit, 76 %, 53 %, 33 %.  A CTA alone
+// on its SM is bound by its chain of hand-offs: a chunk every 3.8 k cycles (GDN 3.4 k) in the form made for it (see alone_for), 4.8 k
 // in the other.
 // What it was before, in the order in which it was found: 103 cycles of issue per tensor-core instruction (behind
 // `lane == 0` instead of an elected lane), 119 KB of code in the instruction caches (half of that now), and 85 % of the
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
         if (!ALONE && n > 0) wait_bar(&misc->tp_free, par ^ 1, misc);
       };
       // Where two CTAs share an SM T is the last operand of MMA3 to be ready, and how long it takes is this warp's count of instructions.  GDN
-      // by rows of X, some forty fewer than by columns (us, by columns / by rows: 152 units of 256 tokens 32.4 / 31.4, 296 of 300 40.5 / 39.1, 424 of
+      // by rows of X, a chunk's 6195 warp instructions become 6037 (us, by columns / by rows: 152 units of 256 tokens 32.4 / 31.4, 296 of 300 40.5 / 39.1, 424 of
       // 300 74.6 / 65.5, 296 of 1 .. 1999 157 / 152; ALONE: 148 of 512 43.2 / 41.2, 4 of 2000 116.8 / 115.5).  KDA by columns: by rows SHARED
       // gained at most 2 %, and 148 units of 512 tokens went from 48.9 to 43.7, but calls of few units, whose other roles are not held up by
       // memory, got slower, 4 of 2000 125.5 -> 131.1, 32 of 509 38.7 -> 39.6, wherever in the chunk this step was put.  In between, 8x8
