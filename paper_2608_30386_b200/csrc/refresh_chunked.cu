@@ -738,21 +738,29 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
     // This warp also starts the copies of V, a chunk ahead: two boxes of 32 tokens x 64 values with the 128-byte swizzle (no bank
     // conflicts for the 8 x 8 blocks it is read in).  Started by two of the chain warps they held those up for 280 cycles of every
     // chunk; here they fall into the wait for the next A (0.3 to 1 % of a launch).
-    int v_issued = 0, v_unit = 0;                  // copies started; the next one's unit,
-    int v_tok = 0, v_n = 0, v_row = 0, v_head = 0;  // its first token in that, of how many, and its coordinates
+    // HELD: the next copy's unit in registers.  GDN looks it up where the copy is started in a walk, whose inverse by rows left no room for
+    // it (16 bytes spilled, 4 without outputs; 592 units of 1 .. 1199 tokens 143 us both ways); with a unit per CTA it is kept, since looked up it
+    // cost 1 % (296 units of 300 tokens 39.1 / 39.7 us).
+    constexpr bool HELD = KDA || !WALK;
+    int v_issued = 0, v_unit = 0, v_tok = 0;  // copies started; the next one's unit, its first token in that,
+    int v_n = 0, v_row = 0, v_head = 0;       // of how many, and its coordinates
     auto next_v = [&]() {
       v_tok = 0;
-      v_n = units[v_unit].n_tok;
-      v_row = static_cast<int32_t>(units[v_unit].tok0);
-      v_head = units[v_unit].head;
+      if (HELD) {
+        v_n = units[v_unit].n_tok;
+        v_row = static_cast<int32_t>(units[v_unit].tok0);
+        v_head = units[v_unit].head;
+      }
     };
     if (all_chunks > 0) next_v();
     auto stage_v = [&]() {  // (the copies by the first lane)
       if (lane == 0 && !misc->abort_flag) {
+        const Unit &x = units[v_unit];
+        const int head = HELD ? v_head : x.head, row = HELD ? v_row : static_cast<int32_t>(x.tok0) + v_tok;
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           mbar_expect_tx(&misc->v_full, C * 128);
-          tma_load_3d(sbase + OFF_V + i * (C * 128), &tmap_v, i * 64, v_head, v_row, &misc->v_full);
+          tma_load_3d(sbase + OFF_V + i * (C * 128), &tmap_v, i * 64, head, row, &misc->v_full);
         }
         // the state that the unit starts from, 64 KB in one piece, is brought into L2 meanwhile
         if (WALK && v_tok == 0 && v_issued > 0 && a.mode == DASC_REFRESH_CONTINUE)
@@ -760,8 +768,8 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
         ++v_issued;
       }
       v_tok += C;
-      v_row += C;
-      if (WALK && v_tok >= v_n && ++v_unit < misc->n_replayed) next_v();
+      if (HELD) v_row += C;
+      if (WALK && v_tok >= (HELD ? v_n : units[v_unit].n_tok) && ++v_unit < misc->n_replayed) next_v();
     };
     // KDA: it also brings in beta, a chunk ahead, and arrives on rdy_prep (ALONE: the MMA1 warp; GDN: the producer warps, whose per-token
     // factors contain it).
