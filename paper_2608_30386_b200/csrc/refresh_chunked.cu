@@ -370,7 +370,9 @@ __device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
 // ZERO: the merge mode, whose units start from zero.  Their first chunk, one of about three in a window of 128 tokens, needs no state pass and no
 // product 2, and its product 5 replaces what the accumulator holds.  32 requests of 1 .. 128 tokens x 4 layers x 32 heads, KDA: 204.8 -> 200.1,
 // 199.3 -> 188.2 us (two runs).  For calls without outputs, the load policy's, and at compile time: as flags in the issuing warp's loop it cost
-// every other call 1 to 3 %.
+// every other call 1 to 3 %.  Calls without outputs and without ZERO are of the continue mode only, and still look at a.mode: with the merge mode's
+// branches out at compile time GDN took 1 % less (296 units of 300 tokens 33.5 / 33.0 us), but KDA alone on an SM 2 % more (32 of 509 34.5 / 35.3, 148 of
+// 256 22.7 / 23.1), for no reason that the source shows; with a flag for both worked out once, KDA 2 % more and GDN the same.
 template <bool KDA, typename OT, bool WITH_O, bool ALONE, bool WALK, bool ZERO>
 __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunked_kernel(const __grid_constant__ DascRefreshArgs a, const __grid_constant__ CUtensorMap tmap_q,
                                                                 const __grid_constant__ CUtensorMap tmap_k,
@@ -1318,7 +1320,7 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
           const int c0 = col_block(i);
           const float *const st_c = a.state + x.state + (c0 * D + vrow);
           uint32_t s[32];
-          if (!ZERO && a.mode == DASC_REFRESH_CONTINUE) {
+          if (a.mode == DASC_REFRESH_CONTINUE) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) s[j] = __float_as_uint(st_c[j * D]);
           } else {
