@@ -27,13 +27,13 @@
 // MMA1 has; MMA5 contracts over the tokens and reads Kh as an MN-major operand from a second tile (tf32
 // MN-major operands have a swizzle of their own), which, read last, is double-buffered by chunk parity.
 //
-// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1035 us = 2.03 G token-heads/s = 63 % of the
-// rate at which HBM could bring its bytes (657 us), GDN 816 us = 2.57 G (50 %; since then 2 % less); 1685 and 1630 us in the form this one grew from, 1090 and
-// 885 with a CTA per unit.  What is nearest its limit is the SM's shared-memory data pipe (load/store units and the tensor core's operand
+// Bound, measured (B200, 64 requests x 256 tokens x 4 layers x 32 heads): KDA 1064 us = 1.97 G token-heads/s = 62 % of the
+// rate at which HBM could bring its bytes (657 us), GDN 825 us = 2.54 G (50 %; 849 with the inverse by columns), in single passes 0.1 s apart, which
+// the power limit leaves alone; 1685 and 1630 us in the form this one grew from, 1090 and 885 with a CTA per unit.  What is nearest its limit is the SM's shared-memory data pipe (load/store units and the tensor core's operand
 // reads together): per chunk and SM (two CTAs) KDA takes 4.1 k cycles, of which that pipe is busy 83 %, the issue slots 51 %, the tensor
 // pipe 38 %; GDN 3.1 k, 97 %, 48 %, 46 %; the state-only form 3.4 k at 2 to 4 chunks per unit, 76 %, 53 %, 33 %.  A CTA alone
-// on its SM is bound by its chain of hand-offs: a chunk every 3.8 k cycles (GDN 3.4 k) in the form made for it (see alone_for), 4.8 k
-// in the other.
+// on its SM is bound by its chain of hand-offs: a chunk every 3.7 k cycles (GDN 3.3 k) in the form made for it (see alone_for), 5.0 k
+// (3.8 k) in the other.
 // What it was before, in the order in which it was found: 103 cycles of issue per tensor-core instruction (behind
 // `lane == 0` instead of an elected lane), 119 KB of code in the instruction caches (half of that now), and 85 % of the
 // shared-memory pipe (8-byte accesses in 16-byte places, A padded to 128 rows, V and O value by value).
@@ -368,8 +368,7 @@ __device__ __forceinline__ void scale2(uint32_t &a, uint32_t &b, uint64_t f) {
 // WALK = false: one unit per CTA, known at compile time (grid_for left the grid at that; always so where ALONE): the bookkeeping between
 // units costs 1 to 4 % of a chunk where there is none to do.
 // ZERO: the merge mode, whose units start from zero.  Their first chunk, one of about three in a window of 128 tokens, needs no state pass and no
-// product 2, and its product 5 replaces what the accumulator holds.  32 requests of 1 .. 128 tokens x 4 layers x 32 heads, KDA: 204.8 -> 200.1,
-// 199.3 -> 188.2 us (two runs).  For calls without outputs, the load policy's, and at compile time: as flags in the issuing warp's loop it cost
+// product 2, and its product 5 replaces what the accumulator holds.  32 requests of 1 .. 128 tokens x 4 layers x 32 heads, KDA: 212.0 -> 205.8 us.  For calls without outputs, the load policy's, and at compile time: as flags in the issuing warp's loop it cost
 // every other call 1 to 3 %.  Calls without outputs and without ZERO are of the continue mode only, and still look at a.mode: with the merge mode's
 // branches out at compile time GDN took 1 % less (296 units of 300 tokens 33.5 / 33.0 us), but KDA alone on an SM 2 % more (32 of 509 34.5 / 35.3, 148 of
 // 256 22.7 / 23.1), for no reason that the source shows; with a flag for both worked out once, KDA 2 % more and GDN the same.
@@ -803,8 +802,8 @@ __global__ void __launch_bounds__(Form<ALONE>::NT, ALONE ? 1 : 2) refresh_chunke
       // Where two CTAs share an SM T is the last operand of MMA3 to be ready, and how long it takes is this warp's count of instructions.  GDN
       // by rows of X, a chunk's 6195 warp instructions become 6037 (us, by columns / by rows: 152 units of 256 tokens 32.4 / 31.4, 296 of 300 40.5 / 39.1, 424 of
       // 300 74.6 / 65.5, 296 of 1 .. 1999 157 / 152; ALONE: 148 of 512 43.2 / 41.2, 4 of 2000 116.8 / 115.5).  KDA by columns: by rows SHARED
-      // gained at most 2 %, and 148 units of 512 tokens went from 48.9 to 43.7, but calls of few units, whose other roles are not held up by
-      // memory, got slower, 4 of 2000 125.5 -> 131.1, 32 of 509 38.7 -> 39.6, wherever in the chunk this step was put.  In between, 8x8
+      // gained at most 2 %, and 148 units of 512 tokens went from 48.9 to 43.7, but calls of few units got slower, 4 of 2000 125.5 -> 131.1, 32 of
+      // 509 38.7 -> 39.6, wherever in the chunk this step was put (why is not known); and all forms have to give the same bits, so SHARED alone cannot have it.  In between, 8x8
       // diagonal blocks and products of hi / lo pairs: KDA 4 of 2000 128.4, but GDN 152 of 256 33.2, 424 of 300 75.7.
       if constexpr (KDA) {
         // diagonal 16x16 blocks: lane (block b, column cc) solves (I + L_bb) x = e_cc, column by column: every row that a new
@@ -1618,7 +1617,7 @@ EncodeTiledFn encode_tiled_fn() {
 // requests come longest first, each gets long and short ones, and adjacent heads still run side by side.  The grid is a
 // multiple of the CTAs that are resident at once, so that no last wave is nearly empty.
 // Measured, us, a CTA per unit / this rule (KDA unless GDN): 4096 units of 1 .. 128 tokens, state only 253 / 223; 8192 of 64 tokens, state
-// only 379 / 309; 7680 of 16 tokens, state only 255 / 182; 8192 of 256 tokens 1128 / 1090 (GDN 1007 / 956).
+// only 379 / 309; 7680 of 16 tokens, state only 255 / 182; 8192 of 256 tokens 1128 / 1090 (GDN 879 / 829), 4096 of 64 GDN 209 / 160.
 // Where the lines lie:
 //  - kWalkChunks chunks per CTA on average, by the estimate of Load (a quarter of a millisecond; lengths just above a multiple of a chunk, or
 //    uneven ones, can give a CTA half as many more): work of other streams is placed when CTAs end.  One grid of
@@ -1631,10 +1630,12 @@ EncodeTiledFn encode_tiled_fn() {
 //    with the longest of the rest), whatever the lengths, so only the start of the second one is saved; but the CTAs that have one
 //    unit pay 1 to 4 % for the walk.  Hence from 1.5 units per CTA on (1.3 with short requests), where lengths differ.  us, a CTA per unit /
 //    walked, requests of 1 .. 2 n - 1 tokens, KDA: 424 units, n = 56 40.7 / 37.8, 480 units, n = 128 63.9 / 59.6, n = 600 195 /
-//    170, 592 units, n = 128 75.8 / 68.8, n = 1000 361 / 322 (GDN 286 / 259); 392 units, n = 56 39.9 / 35.8 but n = 1000 233 / 247; 344 units 2 % more.
+//    170, 592 units, n = 128 75.8 / 68.8, n = 1000 361 / 322; 392 units, n = 56 39.9 / 35.8 but n = 1000 233 / 247; 344 units 2 % more.  GDN: 392 units, n = 56 35.2 / 32.3, n = 128
+//    45.9 / 40.1, n = 1000 170 / 173.5; 424, n = 56 37.1 / 34.6; 480, n = 128 50.7 / 47.5, n = 600 141 / 125; 592, n = 1000 262 / 233.
 //    By the bound alone lengths may differ where they are equal, and with 1.4 units per CTA equal long ones lose: bounds of twice the
-//    length, 424 units of 700 tokens 170 / 190 (GDN 128 / 147), 448 of 700 192.5 / 193.5 (150 / 149), 464 of 300 99.2 / 98.2; short ones at most
-//    7 %: 388 units of 95 tokens 35.1 / 35.1 (28.3 / 30.4), 412 of 40 27.8 / 26.7 (23.3 / 24.1).
+//    length, 424 units of 700 tokens 170 / 190 (GDN 126 / 144), 424 of 300 96.9 / 95.3 (65.0 / 71.6), 448 of 700 192.5 / 193.5 (144.6 / 144.0), 464 of 300
+//    99.2 / 98.2 (75.3 / 73.9); short ones at most 5 %: 388 units of 95 tokens 35.1 / 35.1 (28.3 / 29.5), 412 of 40 27.8 / 26.7 (23.5 / 23.8).  What that
+//    costs uneven lengths below 1.5 units per CTA: GDN, n = 300, 392 units 69.8 / 66.2, 424 73.8 / 67.2 (KDA 98.6 / 90.0).
 constexpr int64_t kSms = 148, kResident = 2 * kSms, kWalkChunks = 64;
 
 // What the host knows of a launch: the longest request (by the caller's bound) and all units together, in chunks (about: half a one
@@ -1668,20 +1669,20 @@ int64_t grid_for(const DascRefreshArgs &a) {
 // the chain what need not be on it: producers with twice the warps, running up to two chunks ahead of the chain into second (MN-major Kh:
 // fourth) buffers; MMA1, the copies of the inputs, P and the outputs in warps of their own (one warp that issued all products was busy all of
 // the time: 100 to 120 cycles per barrier, 40 per product); MMA2 started on the first half of the scaled state; the state's product ahead of
-// the outputs'.  A chunk takes 3.8 k cycles instead of 4.8 k (GDN 3.5 k, 4.5 k), from cold inputs instead of 5.6 k.
-// Measured, us, SHARED / ALONE, 256 tokens (GDN): 8 units 27.3 / 23.4 (23.6 / 21.7), 80 units 32.2 / 25.7 (24.0 / 22.3), 148 units 40.1 / 31.9
-// (32.7 / 28.6), state only 35.0 / 24.8; 148 units of 1 .. 599 tokens 72.5 / 60.0; 152 units 44.2 / 48.2 (35.5 / 43.4): the line is where a
-// second CTA per SM begins to be needed.
+// the outputs'.  A chunk takes 3.7 k cycles instead of 5.0 k (GDN 3.3 k, 3.8 k; from the times of 512 and 2048 tokens), KDA from cold inputs 5.6 k in SHARED.
+// Measured, us, SHARED / ALONE, 256 tokens (GDN): 8 units 27.3 / 23.4 (22.5 / 20.5), 80 units 27.7 / 23.4 (22.8 / 21.1), 148 units 33.3 / 27.0
+// (24.6 / 24.5), state only 29.8 / 22.6 (21.4 / 20.4); 148 units of 1 .. 599 tokens 68.3 / 57.6 (50.2 / 48.9), of 1000 tokens 116.0 / 87.2
+// (91.3 / 75.0); 152 units 37.9 / 43.5 (31.4 / 39.5): the line is where a second CTA per SM begins to be needed.
 // Between 148 and 296 units ALONE would still be the better one where one request is longer than an SM's share of all (192 units of
-// 1 .. 1199 tokens 125 / 94, 256 of 1 .. 799 100 / 77), but the host knows only a bound on that length, and where the bound is loose and the
-// lengths are even ALONE loses: 152 units of 40 tokens 16.9 / 20.9 (GDN 15.6 / 19.2), 296 of 300 tokens 52.9 / 64.6 (42.6 / 55.9), windows
-// of 512 tokens over 256 prefixes of 100 24.3 / 27.5 (21.7 / 25.6).
+// 1 .. 1199 tokens 123 / 95 (GDN 87 / 81), 256 of 1 .. 799 98.5 / 80.7 (63.4 / 62.5)), but the host knows only a bound on that length, and where the
+// bound is loose and the lengths are even ALONE loses: 152 units of 40 tokens 16.0 / 20.4 (14.2 / 18.8), 296 of 300 tokens 53.0 / 65.3 (38.9 / 54.0),
+// windows of 512 tokens over 256 prefixes of 100 20.9 / 27.2 (17.8 / 24.4).
 // Its 58,880 registers leave no room for a block of the copy kernels beside it (one CTA of SHARED leaves 33,280), so a Store on another stream
 // has the SMs without a unit, and where there are few waits for the refresh to end.  Hence ALONE for long requests only on half of
 // the SMs, else up to kWalkChunks chunks: like the CTAs of a walk they are gone after an eighth of a millisecond.  A Store of 16
 // checkpoints (85 us by itself) / the refresh it started with, us until each has ended, SHARED and ALONE:
 //   64 units of 4096 tokens 133 / 424, 155 / 290;   128 units 175 / 431, 335 / 332;   148 units 201 / 535, 420 / 420;   148 units of
-//   2048 tokens 199 / 290, 274 / 271 (GDN 193 / 222, 256 / 258), of 1024 tokens 176 / 179, 197 / 197 (GDN 156 / 154, 185 / 185).
+//   2048 tokens 199 / 250, 269 / 266 (GDN 193 / 203, 244 / 242), of 1024 tokens 175 / 174, 190 / 193 (GDN 156 / 154, 179 / 176).
 // With registers capped at 72 (one block fits) the Store still ended at 435 beside 148 units and the refresh by itself took 1 to 6 % longer;
 // at 64, spilling, 382 and 50 %.  Two launches on two streams share the SMs as well in SHARED: 2 x 148 units of 256 tokens 50 / 57
 // (2048 tokens 336 / 303), but 2 x 100 units 41 / 37, 2 x 72 39 / 29.

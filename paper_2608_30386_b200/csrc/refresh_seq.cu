@@ -479,10 +479,10 @@ int launch(const DascRefreshArgs &a, void *stream) {
 // so that the four dot products of a lane and their shuffles run side by side and one chain of multiply-adds per block is left.  All
 // factors are products of at most two exponentials, of sums of the log-decay: no division, and half of the token-by-token form's error
 // against fp64 (4 units of 64 x 64, 64 tokens: state 6.2e-7 -> 3.0e-7, outputs 3.5e-7 -> 2.0e-7), whose decays multiply up one token at
-// a time.  The helper warps form D k, D q, w and the 16 coefficients of a block, a group of tokens ahead; they and the replaying warps
-// share the SM's issue slots, which is what bounds a group of narrow parts (about 95 ns per token at d = 64, 135 before); wide ones
-// are bound by the replaying lanes' operand reads.  More helper warps, or
-// copies and outputs in warps of their own, gained nothing.
+// a time.  The helper warps form D k, D q, w and the 16 coefficients of a block, a group of tokens ahead.  Narrow parts take 95 ns per token at
+// d = 64 (135 before), 750 cycles per block.  No unit of the SM is at its limit then (4 units of 1024 tokens: issue slots 41 % busy, of the SM's
+// busiest quarter 53 %, the shared-memory pipe 62 %): what is left is the chain of a block and the hand-over of groups, whose shares have not been
+// told apart.  Wide parts are bound by the replaying lanes' operand reads.  More helper warps, or copies and outputs in warps of their own, gained nothing.
 // ---------------------------------------------------------------------------------------------
 constexpr int NB = TB / 4;  // blocks of a group
 
